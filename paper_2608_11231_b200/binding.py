@@ -1,9 +1,11 @@
-"""ctypes binding of the lkv C ABI (see include/lkv.h): argument marshalling only.
+"""Binding of the lkv C ABI (see include/lkv.h): argument marshalling only.
 
 Functions carry the names of the C entry points and take torch CUDA tensors for
 device buffers; torch is used for device memory and streams, nothing else.
-Every step of the computation runs in the CUDA library.  There is no fallback:
-if ``liblkv.so`` is missing, the first call raises.
+Every step of the computation runs in the CUDA library.  The calls of the request
+path are marshalled by the extension module ``_lkv_calls`` (csrc/py_calls.cpp),
+the rest through ctypes.  There is no fallback: if ``liblkv.so`` or the module is
+missing, the first call raises.
 """
 from __future__ import annotations
 
@@ -62,6 +64,22 @@ class LkvError(RuntimeError):
 
 
 _lib = None
+_calls = None
+
+
+def calls():
+    """The native call module, loaded with the library on first use.  Raises if it is missing: there is no other path."""
+    global _calls
+    if _calls is None:
+        load()
+        try:
+            from . import _lkv_calls as m
+        except ImportError as e:
+            raise RuntimeError("the call module _lkv_calls.so is missing or does not load: build it with "
+                               "`python -m paper_2608_11231_b200.build`") from e
+        m.setup(LkvError, workspace, _ws_cache, _host_i32)
+        _calls = m
+    return _calls
 
 
 def load() -> ctypes.CDLL:
@@ -198,30 +216,16 @@ def lkv_init_state(states: torch.Tensor, transitions: Optional[torch.Tensor], K:
                    S0: Optional[torch.Tensor] = None, *, family: int, chunk_ids=None, sel_index: int = 0,
                    compute: int = LKV_COMPUTE_AUTO, workspace_t: Optional[torch.Tensor] = None, stream=None):
     """State initialisation for one request.  states: pool [n, H, d_k, d_v]; returns S0 [H, d_k, d_v] fp32."""
-    ids = _host_i32(chunk_ids)
-    d, ws_t = _init_desc(states, family, compute, workspace_t, 1, int(K), ids, sel_index)
-    if S0 is None:
-        S0 = torch.empty(states.shape[1:], dtype=torch.float32, device=states.device)
-    st = load().lkv_init_state(_ptr(states), _ptr(transitions), int(K), int(mode), _ptr(S0), ctypes.byref(d),
-                               _stream(stream))
-    if st != LKV_OK:
-        raise LkvError(st, "lkv_init_state")
-    return S0
+    return (_calls or calls()).init_state(states, transitions, K, mode, S0, family, chunk_ids, sel_index, compute, workspace_t,
+                                          stream)
 
 
 def lkv_init_state_batched(states: torch.Tensor, transitions: Optional[torch.Tensor], chunk_ids, cu_k, n_req: int,
                            mode: int, sel_index=None, S0: Optional[torch.Tensor] = None, *, family: int,
                            compute: int = LKV_COMPUTE_AUTO, workspace_t: Optional[torch.Tensor] = None, stream=None):
     """State initialisation for n_req requests in one launch; returns S0 [n_req, H, d_k, d_v] fp32."""
-    ids, cu, sel = _host_i32(chunk_ids), _host_i32(cu_k), _host_i32(sel_index)
-    d, ws_t = _init_desc(states, family, compute, workspace_t, int(n_req), 0 if ids is None else ids.size)
-    if S0 is None:
-        S0 = torch.empty((n_req,) + tuple(states.shape[1:]), dtype=torch.float32, device=states.device)
-    st = load().lkv_init_state_batched(_ptr(states), _ptr(transitions), _hp(ids), _hp(cu), int(n_req), int(mode),
-                                       _hp(sel), _ptr(S0), ctypes.byref(d), _stream(stream))
-    if st != LKV_OK:
-        raise LkvError(st, "lkv_init_state_batched")
-    return S0
+    return (_calls or calls()).init_state_batched(states, transitions, chunk_ids, cu_k, n_req, mode, sel_index, S0, family,
+                                                  compute, workspace_t, stream)
 
 
 LKV_STATIC_MAX_INDEX = 16384
@@ -257,26 +261,8 @@ def lkv_gdn_fwd(q, k, v, g, beta, S0=None, o=None, S_T=None, *, cu_seqlens=None,
     Returns (o [T, H_v, d_v] in the dtype of v, or None with want_outputs=False; S_T [n_seq, H_v, d_k, d_v] in
     state_dtype (fp32 or bf16; the dtype of S_T if one is passed) or None).
     """
-    T, H_k, d_k = q.shape
-    _, H_v, d_v = v.shape
-    cu = _host_i32(cu_seqlens)
-    n_seq = 1 if cu is None else cu.size - 1
-    d = lkv_gdn_desc(T_total=T, n_seq=n_seq, cu_seqlens=None if cu is None else cu.ctypes.data, H_k=H_k, H_v=H_v,
-                     d_k=d_k, d_v=d_v, io_dtype=_dtype_code(v), compute=compute, scale=float(scale), state_dtype=0,
-                     workspace=None, workspace_bytes=0)
-    ws_t = workspace_t if workspace_t is not None else workspace(v.device, lkv_workspace_bytes(LKV_WS_GDN, d, n_seq))
-    d.workspace, d.workspace_bytes = ws_t.data_ptr(), ws_t.numel()
-    if o is None and want_outputs:
-        o = torch.empty_like(v)
-    if S_T is None and want_final_state:
-        S_T = torch.empty((n_seq, H_v, d_k, d_v), dtype=state_dtype, device=v.device)
-    if S_T is not None:
-        d.state_dtype = _dtype_code(S_T)
-    st = load().lkv_gdn_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(S0), _ptr(o), _ptr(S_T),
-                            ctypes.byref(d), _stream(stream))
-    if st != LKV_OK:
-        raise LkvError(st, "lkv_gdn_fwd")
-    return o, S_T
+    return (_calls or calls()).gdn_fwd(q, k, v, g, beta, S0, o, S_T, cu_seqlens, scale, compute, want_final_state, want_outputs,
+                                       state_dtype, workspace_t, stream)
 
 
 def lkv_gdn_fwd_segmented(q, k, v, g, beta, S0=None, o=None, S_T=None, *, n_segments: int, scale: float = 0.0,
@@ -311,25 +297,8 @@ def lkv_ssd_fwd(x, dt, A, B, C, S0=None, y=None, S_T=None, *, cu_seqlens=None, c
 
     Returns (y [T, H, P] in the dtype of x, S_T [n_seq, H, N, P] in state_dtype (fp32 or bf16) or None).
     """
-    T, H, P = x.shape
-    _, G, N = B.shape
-    cu = _host_i32(cu_seqlens)
-    n_seq = 1 if cu is None else cu.size - 1
-    d = lkv_ssd_desc(T_total=T, n_seq=n_seq, cu_seqlens=None if cu is None else cu.ctypes.data, H=H, P=P, N=N, G=G,
-                     io_dtype=_dtype_code(x), compute=compute, workspace=None, workspace_bytes=0)
-    ws_t = workspace_t if workspace_t is not None else workspace(x.device, lkv_workspace_bytes(LKV_WS_SSD, d, n_seq))
-    d.workspace, d.workspace_bytes = ws_t.data_ptr(), ws_t.numel()
-    if y is None and want_outputs:
-        y = torch.empty_like(x)
-    if S_T is None and want_final_state:
-        S_T = torch.empty((n_seq, H, N, P), dtype=state_dtype, device=x.device)
-    if S_T is not None:
-        d.state_dtype = _dtype_code(S_T)
-    st = load().lkv_ssd_fwd(_ptr(x), _ptr(dt), _ptr(A), _ptr(B), _ptr(C), _ptr(S0), _ptr(y), _ptr(S_T),
-                            ctypes.byref(d), _stream(stream))
-    if st != LKV_OK:
-        raise LkvError(st, "lkv_ssd_fwd")
-    return y, S_T
+    return (_calls or calls()).ssd_fwd(x, dt, A, B, C, S0, y, S_T, cu_seqlens, compute, want_final_state, want_outputs,
+                                       state_dtype, workspace_t, stream)
 
 
 def lkv_init_state_fold(states: torch.Tensor, k, g, beta, cu_tokens, K: int, chunk_ids=None,
@@ -396,42 +365,13 @@ def lkv_gdn_chunk_artifacts(k, v, g, beta, states=None, transitions=None, *, cu_
                             compute: int = LKV_COMPUTE_AUTO, workspace_t: Optional[torch.Tensor] = None, stream=None):
     """S_local and T_C of every chunk (sequence of cu_seqlens) in one launch.  Returns (states, transitions),
     fp32 [n_seq, H_v, d, d] each."""
-    T, H_k, d_k = k.shape
-    _, H_v, d_v = v.shape
-    cu = _host_i32(cu_seqlens)
-    n_seq = 1 if cu is None else cu.size - 1
-    d = lkv_gdn_desc(T_total=T, n_seq=n_seq, cu_seqlens=None if cu is None else cu.ctypes.data, H_k=H_k, H_v=H_v,
-                     d_k=d_k, d_v=d_v, io_dtype=_dtype_code(k), compute=compute, scale=0.0, state_dtype=0,
-                     workspace=None, workspace_bytes=0)
-    ws_t = workspace_t if workspace_t is not None else workspace(k.device, lkv_workspace_bytes(LKV_WS_GDN, d, 2 * n_seq))
-    d.workspace, d.workspace_bytes = ws_t.data_ptr(), ws_t.numel()
-    if states is None:
-        states = torch.empty((n_seq, H_v, d_k, d_v), dtype=torch.float32, device=k.device)
-    if transitions is None:
-        transitions = torch.empty((n_seq, H_v, d_k, d_k), dtype=torch.float32, device=k.device)
-    st = load().lkv_gdn_chunk_artifacts(_ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(states), _ptr(transitions),
-                                        ctypes.byref(d), _stream(stream))
-    if st != LKV_OK:
-        raise LkvError(st, "lkv_gdn_chunk_artifacts")
-    return states, transitions
+    return (_calls or calls()).gdn_chunk_artifacts(k, v, g, beta, states, transitions, cu_seqlens, compute, workspace_t, stream)
 
 
 def lkv_mamba_chunk_logdecay(dt, A, logdecay=None, *, cu_seqlens=None, workspace_t: Optional[torch.Tensor] = None,
                              stream=None):
     """lambda[c][h] = A[h] * sum of dt over chunk c.  dt: [T, H] fp32; A: [H] fp32.  Returns [n_seq, H] fp32."""
-    T, H = dt.shape
-    cu = _host_i32(cu_seqlens)
-    n_seq = 1 if cu is None else cu.size - 1
-    d = lkv_ssd_desc(T_total=T, n_seq=n_seq, cu_seqlens=None if cu is None else cu.ctypes.data, H=H, P=1, N=1, G=1,
-                     io_dtype=LKV_DTYPE_F32, compute=LKV_COMPUTE_AUTO, workspace=None, workspace_bytes=0)
-    ws_t = workspace_t if workspace_t is not None else workspace(dt.device, lkv_workspace_bytes(LKV_WS_SSD, d, n_seq))
-    d.workspace, d.workspace_bytes = ws_t.data_ptr(), ws_t.numel()
-    if logdecay is None:
-        logdecay = torch.empty((n_seq, H), dtype=torch.float32, device=dt.device)
-    st = load().lkv_mamba_chunk_logdecay(_ptr(dt), _ptr(A), _ptr(logdecay), ctypes.byref(d), _stream(stream))
-    if st != LKV_OK:
-        raise LkvError(st, "lkv_mamba_chunk_logdecay")
-    return logdecay
+    return (_calls or calls()).mamba_chunk_logdecay(dt, A, logdecay, cu_seqlens, workspace_t, stream)
 
 
 def lkv_state_rel_error(S_init, S_ref, n_states: Optional[int] = None, rel_err=None, *, stream=None):

@@ -1,4 +1,4 @@
-"""In-tree build of the CUDA library: nvcc -> paper_2608_11231_b200/liblkv.so (sm_100a only)."""
+"""In-tree build: nvcc -> paper_2608_11231_b200/liblkv.so (sm_100a only), g++ -> _lkv_calls.so (the Python binding's hot calls)."""
 from __future__ import annotations
 
 import glob
@@ -10,6 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "liblkv.so")
+CALLS = os.path.join(HERE, "_lkv_calls.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -54,7 +55,25 @@ def build(verbose: bool = False, force: bool = False) -> str:
         raise RuntimeError("nvcc failed")
     if procs or not os.path.exists(LIB):
         subprocess.run([nvcc, "-shared", "-Wno-deprecated-gpu-targets", "-o", LIB, *objs], check=True)
+    build_calls(headers)
     return LIB
+
+
+def build_calls(headers) -> str:
+    """Compile csrc/py_calls.cpp against torch's headers and link it to liblkv.so beside it."""
+    src = os.path.join(CSRC, "py_calls.cpp")
+    if not _newer(src, CALLS, [h for h in headers if h.endswith(".h")]):
+        return CALLS
+    import sysconfig
+    from torch.utils import cpp_extension
+    libs = [p for p in cpp_extension.library_paths() if os.path.isdir(p)]
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-w", src, "-o", CALLS,
+                    *["-isystem" + p for p in [*cpp_extension.include_paths(), os.path.join(cuda, "include"),
+                                               sysconfig.get_paths()["include"]]],
+                    *["-L" + p for p in [HERE, *libs]], "-llkv", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
+                    "-Wl,-rpath,$ORIGIN", *["-Wl,-rpath," + p for p in libs]], check=True)
+    return CALLS
 
 
 if __name__ == "__main__":
