@@ -66,7 +66,7 @@ template <bool SBF16>
 __global__ void __launch_bounds__(kThreads, 1)
 init_gdn_exact_tensor_kernel(const __grid_constant__ InitArgs a, const __grid_constant__ CUtensorMap mapT) {
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    unsigned char *sm = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);   // an offset, not a cast: the compiler keeps shared-memory addressing
     // fullT: TMA transactions; roundT: the rounding warps are done with the stage; freeT: the MMAs of the step have read it;
     // e_ready[h]: warpgroup h has stored its half of the new operand; mma[h]: output half h of the step is complete
     __shared__ uint64_t bar_fullT[kStages], bar_roundT[kStages], bar_freeT[kStages], bar_eready[2], bar_mma[2];
