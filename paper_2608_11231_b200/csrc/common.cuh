@@ -90,6 +90,12 @@ struct SsdArgs {
     void *y;
     float *S_T;                  // final states, fp32 or (st_bf16) bf16 behind the same pointer
     int32_t st_bf16;
+    // One sequence cut into segments that run side by side (tensor-core scan only).  Sequences n_s0 .. start from S0_more
+    // (index seq - n_s0; nullptr = zero), final states are wanted of sequences st_first .. only (index seq - st_first), and
+    // lam, where given, gets the log-decay of every sequence and head.  A plain call has n_s0 = n_seq, st_first = 0, lam = nullptr.
+    int32_t n_s0, st_first;
+    const float *S0_more;
+    float *lam;
     int32_t n_seq, T_total, H, P, N, G;
     int32_t *status;
     IndexBlock<kScanIdxCap> cu;  // cu_seqlens[n_seq + 1]

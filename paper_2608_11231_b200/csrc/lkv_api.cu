@@ -181,6 +181,72 @@ void append_launch_order(std::vector<int32_t> &cu, int n_seq) {
     cu.insert(cu.end(), order.begin(), order.end());
 }
 
+int sm_count() {
+    static int cached[64];   // per device; the same value whoever writes it
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        cudaGetLastError();
+        return 148;
+    }
+    n = __atomic_load_n(&cached[dev], __ATOMIC_RELAXED);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            n = 148;
+        }
+        __atomic_store_n(&cached[dev], n, __ATOMIC_RELAXED);
+    }
+    return n;
+}
+
+// A single sequence fills (heads / 2) of the SMs (two heads per CTA) and is a chain of blocks.  Cut into segments, it runs as
+// three launches: the states the first segments reach on their own (no outputs: 2.0 K cycles a block against 3.2 K), the
+// composition of every segment's initial state (Eq. 6), all segments with outputs side by side.  Worth it from three
+// segments up -- two save 0.6 K cycles a block -- of at least 1024 tokens: the two more launches cost about 16 blocks.
+int ssd_segments(const lkv_ssd_desc *d, int n_seq) {
+    if (n_seq != 1 || d->io_dtype != LKV_DTYPE_BF16 || d->compute == LKV_COMPUTE_FP32 || d->H < 1 || d->G < 1 || d->H % d->G || d->P != 64 || d->N != 128)
+        return 1;
+    const int ctas = d->G * ((d->H / d->G + 1) / 2);
+    const int n = std::min({sm_count() / ctas, d->T_total / 1024, 16});
+    return n >= 3 ? n : 1;
+}
+// local states and log-decays of the first segments, initial states of all but the first
+size_t ssd_segment_scratch(const lkv_ssd_desc *d, int segs) {
+    if (segs < 2) return 0;
+    const size_t slot = sizeof(float) * static_cast<size_t>(d->H) * d->N * d->P;
+    return 2 * (segs - 1) * slot + align_up(sizeof(float) * static_cast<size_t>(segs - 1) * d->H, 256);
+}
+int ssd_segmented(SsdArgs a, int segs, char *scratch, cudaStream_t s) {
+    const size_t slot = static_cast<size_t>(a.H) * a.N * a.P;
+    float *local = reinterpret_cast<float *>(scratch), *init = local + (segs - 1) * slot, *lam = init + (segs - 1) * slot;
+    // whole blocks of 128 tokens
+    const int per = ((a.T_total + segs - 1) / segs + 127) / 128 * 128;
+    auto bounds = [&](SsdArgs &b, int n) {
+        b.n_seq = n;
+        b.cu.ptr = nullptr;
+        for (int i = 0; i <= n; ++i) b.cu.v[i] = static_cast<int32_t>(std::min<long long>(static_cast<long long>(i) * per, a.T_total));
+        for (int i = 0; i < n; ++i) b.cu.v[n + 1 + i] = i;
+    };
+    SsdArgs p1 = a;
+    bounds(p1, segs - 1);
+    p1.y = nullptr; p1.S_T = local; p1.st_bf16 = 0; p1.n_s0 = 1; p1.st_first = 0; p1.lam = lam;
+    if (launch_ssd_scan_tensor(p1, s) != cudaSuccess) return LKV_ERR_CUDA;
+    InitArgs c;
+    c.states = local; c.transitions = lam; c.S0 = init; c.n_req = segs - 1; c.H = a.H; c.d_k = a.N; c.d_v = a.P; c.n_chunks = segs - 1;
+    c.off_sel = -1; c.off_ids = segs; c.status = a.status; c.idx.ptr = nullptr;
+    int at = segs;
+    for (int r = 0; r < segs - 1; ++r) {
+        c.idx.v[r] = at - segs;
+        for (int j = 0; j <= r; ++j) c.idx.v[at++] = j;
+    }
+    c.idx.v[segs - 1] = at - segs;
+    if (launch_init_mamba_exact_stream(c, false, s) != cudaSuccess) return LKV_ERR_CUDA;
+    SsdArgs p3 = a;
+    bounds(p3, segs);
+    p3.n_s0 = 1; p3.S0_more = init; p3.st_first = segs - 1;
+    return launch_ssd_scan_tensor(p3, s) == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
+}
+
 }  // namespace
 
 extern "C" {
@@ -583,7 +649,12 @@ int lkv_ssd_fwd(const void *x, const float *dt, const float *A, const void *B, c
         if (!tensor_fits && !fp32_fits) return LKV_ERR_UNSUPPORTED;
         use_tensor = tensor_fits;
     }
+    a.n_s0 = d->n_seq; a.st_first = 0; a.S0_more = nullptr; a.lam = nullptr;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const int segs = use_tensor && S_T != S0 && y ? ssd_segments(d, d->n_seq) : 1;
+    const size_t head = ws_bytes_for(2 * d->n_seq + 1, kScanIdxCap);
+    if (segs > 1 && d->workspace_bytes >= head + ssd_segment_scratch(d, segs))
+        return ssd_segmented(a, segs, static_cast<char *>(d->workspace) + head, s);
     append_launch_order(cu, d->n_seq);
     st = place_indices(a.cu, cu, d->workspace, s);
     if (st != LKV_OK) return st;
@@ -595,8 +666,11 @@ size_t lkv_workspace_bytes(int which, const void *desc, int n_units, int n_index
     if (!desc || n_units < 0 || n_index < 0) return 0;
     switch (which) {
         case LKV_WS_INIT: return ws_bytes_for(2 * n_units + 1 + n_index, kInitIdxCap);
-        case LKV_WS_GDN:
-        case LKV_WS_SSD: return ws_bytes_for(2 * n_units + 1, kScanIdxCap);
+        case LKV_WS_GDN: return ws_bytes_for(2 * n_units + 1, kScanIdxCap);
+        case LKV_WS_SSD: {
+            const lkv_ssd_desc *d = static_cast<const lkv_ssd_desc *>(desc);
+            return ws_bytes_for(2 * n_units + 1, kScanIdxCap) + ssd_segment_scratch(d, ssd_segments(d, n_units));
+        }
         default: return 0;
     }
 }

@@ -1,22 +1,44 @@
 // Chunkwise Mamba-2 (SSD) scan on the 5th-generation tensor cores (Eq. 1 with Eq. 2), for
-// headdim P = 64, d_state N = 128 and bf16 x/B/C/y.  One CTA owns one (sequence, head) and walks
-// the sequence in blocks of 128 tokens with the N x P state carried on chip (fp32 in tensor memory,
-// a bf16 copy in shared memory as an MMA operand).  With l the running sum of dt * A_h inside the
-// block and S the incoming state, per block:
-//   (a) G      = C B^T                                   [128 x 128], K = N                 tcgen05
-//       G'_ti  = G_ti e^{l_t - l_i} dt_i  (i <= t), 0 otherwise -> bf16 operand in TMEM     epilogue warps
-//   (b) Yintra = G' X                                    [128 x 64],  K = 128 tokens         tcgen05 (A from TMEM)
-//   (c) Yinter = C S                                     [128 x 64],  K = N                  tcgen05
-//       y_t    = Yintra_t + e^{l_t} Yinter_t                                                 epilogue warps
-//   (d) S     <- e^{l_Q} S + B^T X~,  X~_i = e^{l_Q - l_i} dt_i x_i   [128 x 64], K = tokens   tcgen05
-//       (the state is pre-scaled in tensor memory, (d) accumulates onto it)                  state warps
-// Only (c) and (d) depend on the previous block: (a) of the next block is issued as soon as the mask
-// epilogue has drained G, so the epilogue warps never wait for the block-to-block chain
-// (d) -> state copy -> (c), (d); the scaled X~ of the next block is prepared while (d) runs.
-// A padded token has dt = 0.
-// Warps 0-7 epilogue (thread = token row, warpgroup = column half), 8-11 state copy (the only SIMT
-// work on the block-to-block chain), 12-15 per-block scalars and X~ (running ahead of the chain),
-// 16 TMA, 17 MMA issue.  All waits on mbarriers are bounded.
+// headdim P = 64, d_state N = 128 and bf16 x/B/C/y.  One CTA owns one sequence and TWO heads of one group and walks
+// the sequence in blocks of up to 128 tokens with the heads' states carried on chip.
+//
+// No decay appears inside a contraction.  With l the running sum of dt * A_h inside a block (in log2 units, n its last
+// token) and R a scale exponent of the block,
+//     y_t = 2^{l_t - R} [ sum_{i<=t} (C_t.B_i) X^_i  +  C_t S^ ],    X^_i = 2^{R - l_i} dt_i x_i,   S^ = 2^R S
+//     S  <- 2^{l_n - R} [ S^ + B^T X^ ]
+// so the token-by-token decay only scales the rows of X going in and the rows of y coming out,
+// and the masked product G = tril(C B^T) is the same matrix for every head of the group: it is formed once per CTA, with
+// nothing but the causal mask applied.  (The form with the decays inside, G'_ti = G_ti e^{l_t - l_i} dt_i, costs a mask of
+// 128 x 128 / 2 products and exponent factors per head and block; that, not the tensor cores, set the pace of this scan.)
+// The state as held, S^ + B^T X^, is the next block's S^ with R - l_n for R: it is multiplied by a power of two only when
+// that would pass kMaxScale, every block to every seventh with decays as strong as the benchmark's.
+// Scaling by powers of two commutes with rounding, and fp32 and bf16 have the same exponent range, so nothing is lost
+// while the exponents stay in range: a block ends before the token at which |l| would pass kMaxRange (it always keeps one
+// token).
+//
+// Everything is held transposed so that the tiles have M = 128 rows = 2 heads x 64 features (all 128 TMEM lanes):
+//   (G)    G     = C B^T                     [128 t x 128 i], K = n        tcgen05; tril -> bf16 tile in shared memory (prep warps)
+//   (Y2)   Y^T   = S^^T C^T                  [128 x 128 t], K = n          A = bf16 S^^T in tensor memory
+//   (S)    S^^T += X^^T B                    [128 x 128 n], K = tokens     A = X^^T in tensor memory
+//   (Y1)   Y^T  += X^^T G^T                  [128 x 128 t], K = tokens     A = X^^T in tensor memory (t < 64, i >= 64: skipped)
+//   X^^T   ldmatrix.trans out of the X tile, scaled, stored to tensor memory                        prep warps
+//   state  fp32 S^^T rescaled for the next block, bf16 copy beside it, both in tensor memory        state warps
+//   y      Y^T scaled by 2^{l_t - r}, transposed by stmatrix into a tile that TMA stores            output warps
+// X^ goes to tensor memory rather than back into its tile: the X tile is free for the next block at once, and the SM's
+// shared-memory port (128 bytes per clock, the scarcest thing on chip here) is spared the write-back and three reads.
+// The chain from block to block is (Y2), (S) -> state pass; X^, G and the outputs hang off it.
+//
+// Bound: per block the CTA takes in 96 KB (B, C, two X tiles) and writes 32 KB; an SM takes in about 40 bytes per clock
+// from L2, 2.4 K cycles, and the copy bandwidth of the memory gives 2.9 K for the X and y bytes alone.  Measured: 3.2 K
+// cycles a block on an idle GPU, 3.4 K on a full one, 2.0 K without outputs (one head per CTA and the decays inside the
+// mask took 7.7 K for the same two heads).  32 sequences x 4096 tokens x 80 heads: 1370 -> 725 us.
+//
+// The hot loops are rolled where they repeat: eight programs run side by side, each once per block, and fetched unrolled
+// (60 KB of code) every role took three to five times as long as its instructions (the scalar warp 5300 cycles for 250).
+//
+// Warps 0-7 outputs (warpgroup = half of the tokens), 8-15 state (warpgroup = half of n), 16-23 X^ (warpgroup = half of the
+// tokens) and then the mask, 24 TMA loads, 25 MMA issue of (S), 26 MMA issue of (G), (Y2), (Y1), 27 block limits and scalars.
+// All waits on mbarriers are bounded.
 #include <string.h>
 
 #include "common.cuh"
@@ -31,38 +53,65 @@ using namespace tc;
 constexpr int kP = 64;     // headdim
 constexpr int kN = 128;    // d_state
 constexpr int kQ = 128;    // tokens per block
-constexpr int kThreads = 576;
+constexpr int kThreads = 896;
 
 // shared-memory map (bytes, after 1024-byte alignment); every tile row is 128 bytes, 128-byte swizzle
-constexpr int kXTile = kQ * 128;            // X [128 tokens x 64 p]
-constexpr int kBTile = 2 * kQ * 128;        // B [B_kb0 | B_kb1], each [128 tokens x 64 n]
-constexpr int kCTile = 2 * kQ * 128;        // C likewise
-constexpr int kStageBytes = kXTile + kBTile + kCTile;   // 80 KB
-constexpr int kOffX2 = 2 * kStageBytes;     // X~ [128 tokens x 64 p], double-buffered
-constexpr int kOffHb = kOffX2 + 2 * kXTile; // bf16 state [128 n x 64 p]
-constexpr int kOffSc = kOffHb + kN * 128;   // per-block scalars, three buffers
-constexpr int kScFloats = 5 * kQ + 4;       // l2 = l log2(e), e^{l}, s = e^{l_Q - l} dt, f = e^{l_ref - l} dt, dt, flag
+constexpr int kTile = kQ * 128;                  // [128 rows x 64 bf16]
+constexpr int kBCStage = 4 * kTile;              // [B_nb0 | B_nb1 | C_nb0 | C_nb1], each [128 tokens x 64 n]
+constexpr int kOffX = 2 * kBCStage;              // X of the two heads, [128 tokens x 64 p] each
+constexpr int kOffY = kOffX + 2 * kTile;         // y likewise, staged for the TMA store; an output warp writes 64 tokens x 32 p
+constexpr int kOffG = kOffY + 2 * kTile;         // tril(G) bf16: columns i < 64 of all rows t (16 KB), then i >= 64 of rows t >= 64 (8 KB)
+constexpr int kOffSlot = kOffG + kTile + kTile / 2;
+constexpr int kSlots = 4;
+struct Slot {            // block descriptor
+    uint2 s[2][kQ / 2];  // 2^{R - l_t} dt_t of two tokens per head (0 beyond the block), as two bf16 parts: {high pair, low pair}
+    float e[2][kQ];      // 2^{l_t - R}
+    float f2[2], e2[2];  // exponents: R minus the R that the block before left, l_n - R
+    int start, n;        // first token, number of tokens
+    int pad[2];
+};
+constexpr int kSmemBytes = kOffSlot + kSlots * static_cast<int>(sizeof(Slot)) + 1024;
+static_assert(kSmemBytes + 512 <= 227 * 1024, "shared memory budget");
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kMaxGroupRange = 100.f;     // log2 units: above this the per-group factors could overflow
-constexpr int kSmemBytes = kOffSc + 3 * kScFloats * 4 + 1024;
-static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
+constexpr float kMaxRange = 200.f;               // log2 units of decay inside one block
+constexpr float kMaxScale = 104.f;               // 2^R - l_n at most: X^ and S^ grow to about 2^104 ...
+constexpr float kNewScale = 96.f;                // ... and a state that is scaled back starts from 2^-96 (104 + 96 = kMaxRange)
 
 // tensor-memory map (columns)
-constexpr uint32_t kTmG = 0;        // 128
-constexpr uint32_t kTmYa = 128;     // Yintra, 2 x 64
-constexpr uint32_t kTmYe = 256;     // Yinter, 2 x 64
-constexpr uint32_t kTmH = 384;      // 64
-constexpr uint32_t kTmGp = 448;     // G' as bf16 pairs: 128 K-elements in 64 columns
+constexpr uint32_t kTmS = 0;        // 128: S^^T fp32
+constexpr uint32_t kTmSb = 128;     // 64: S^^T as bf16 pairs (A operand of (Y2))
+constexpr uint32_t kTmX = 192;      // 64: X^^T as bf16 pairs (A operand of (S) and (Y1))
+constexpr uint32_t kTmY = 256;      // 128
+constexpr uint32_t kTmG = 384;      // 128
 constexpr uint32_t kTmemCols = 512;
 
 struct Bars {
-    uint64_t full_bc[2], full_x[2];                    // TMA transactions
-    uint64_t bc_free[2], ac_done, y_done, h_done[2];   // tcgen05.commit targets
-    uint64_t mg_ready, yo_done[3], ys_ready[2];        // 256 epilogue threads
-    uint64_t sc_ready[3], x2_ready[2], hb_ready;       // 128 threads (scalar warps; hb_ready: state warps)
+    // single-arrival barriers: TMA transactions and tcgen05.commit
+    uint64_t full_bc[2], full_x, g_done, y2_done, y_done, h_done, xs_free, xy_free;
+    // commits of (S) and (Y2) ((S) alone when no outputs are wanted)
+    uint64_t bc_free[2];
+    // one arrival per warp: the scalar warp
+    uint64_t sc_ready[kSlots];
+    // the eight output, state or prep warps
+    uint64_t y_free, hb_ready, x_free, x2_ready, mask_done;
+    // output and state warps (state warps alone when no outputs are wanted)
+    uint64_t slot_free[kSlots];
 };
+constexpr int kBars1 = 9;
+static_assert(sizeof(Bars) == 8 * (kBars1 + 2 + kSlots + 5 + kSlots), "barrier table");
 
 __device__ __forceinline__ void named_bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+// barrier over n threads that also tells whether any of them passed true
+__device__ __forceinline__ bool named_bar_or(int id, int n, bool p) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred a, b;\n\tsetp.ne.u32 a, %3, 0;\n\t"
+        "bar.red.or.pred b, %1, %2, a;\n\tselp.u32 %0, 1, 0, b;\n\t}"
+        : "=r"(r)
+        : "r"(id), "r"(n), "r"(p ? 1u : 0u)
+        : "memory");
+    return r != 0;
+}
 __device__ __forceinline__ uint32_t elect_one() {
     uint32_t e;
     asm volatile("{\n\t.reg .pred P1;\n\telect.sync _|P1, %1;\n\tselp.u32 %0, 1, 0, P1;\n\t}" : "=r"(e) : "r"(0xffffffffu));
@@ -72,415 +121,537 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t *>(&v);
 }
+__device__ __forceinline__ float2 f2(uint32_t x, uint32_t y) { return make_float2(__uint_as_float(x), __uint_as_float(y)); }
+// every lane takes the same decision although `dead` may change under the read
+__device__ __forceinline__ bool warp_dead(volatile int *dead) { return __any_sync(0xffffffffu, *dead != 0); }
+
+// One arrival for the whole warp, after every lane's work before it: an mbarrier takes the arrivals of the lanes of one
+// instruction one by one, each a turn at the shared-memory port (1700 a block where every thread arrives for itself).
+__device__ __forceinline__ void warp_arrive(uint64_t *bar) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// 32 columns n0 .. n0+31 of the state of this thread's lane (feature p of head h) as bf16 pairs for (Y2)
+__device__ __forceinline__ void copy_state32(uint32_t lane_base, int n0, const uint32_t (&rr)[32]) {
+    uint32_t w[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) w[c] = pack_bf16(__uint_as_float(rr[2 * c]), __uint_as_float(rr[2 * c + 1]));
+    tmem_st16(lane_base + kTmSb + n0 / 2, w);
+}
+// 64 columns of the fp32 state multiplied by 2^ex in place, in two steps: the factor may lie below the fp32 range where its
+// product with the state does not.  Not inlined: one block in several needs it.
+__device__ __noinline__ void scale_state64(uint32_t taddr, float ex) {
+    const float f = ex2(0.5f * ex);
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q) {
+        uint32_t rr[16];
+        tmem_ld16(taddr + 16 * q, rr);
+        tmem_ld_wait();
+#pragma unroll
+        for (int c = 0; c < 16; ++c) rr[c] = __float_as_uint(__uint_as_float(rr[c]) * f * f);
+        tmem_st16(taddr + 16 * q, rr);
+    }
+    tmem_st_wait();
+}
 
 __global__ void __launch_bounds__(kThreads, 1)
 ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant__ CUtensorMap mapX,
                        const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapC,
                        const __grid_constant__ CUtensorMap mapY) {
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    unsigned char *sm = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);   // an offset, not a cast: the compiler keeps shared-memory addressing
     __shared__ Bars bars;
     __shared__ uint32_t tmem_base;
     __shared__ volatile int dead;
-    __shared__ float scan_carry[4];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int h = blockIdx.x, seq = a.cu[a.n_seq + 1 + blockIdx.y];   // launch order: longest sequence first
-    const int grp = h / (a.H / a.G);
+    const int per_grp = a.H / a.G, pairs = (per_grp + 1) / 2;
+    const int grp = blockIdx.x / pairs, pr = blockIdx.x % pairs;
+    const int h0 = grp * per_grp + 2 * pr;
+    const bool two = 2 * pr + 1 < per_grp;   // the last head of an odd group is computed twice and stored once
+    const int h1 = h0 + (two ? 1 : 0);
+    const int seq = a.cu[a.n_seq + 1 + blockIdx.y];   // launch order: longest sequence first
     const int t_begin = a.cu[seq], t_end = a.cu[seq + 1];
-    const int nblk = (t_end - t_begin + kQ - 1) / kQ;
-    const size_t sbase = (static_cast<size_t>(seq) * a.H + h) * kN * kP;
+    // initial and final state of head h0; that of the other follows
+    const float *S0 = seq < a.n_s0 ? a.S0 : a.S0_more;
+    if (S0) S0 += (static_cast<size_t>(seq < a.n_s0 ? seq : seq - a.n_s0) * a.H + h0) * kN * kP;
+    float *ST = seq < a.st_first ? nullptr : a.S_T;
+    const size_t st_off = (static_cast<size_t>(seq - a.st_first) * a.H + h0) * kN * kP;
+    const bool has_y = a.y != nullptr;
 
-    if (nblk == 0) {  // empty sequence: hand the state through untouched
-        if (a.S_T && a.S_T != a.S0)
-            for (int e = tid; e < kN * kP; e += kThreads) store_state(a.S_T, a.st_bf16, sbase + e, a.S0 ? a.S0[sbase + e] : 0.f);
+    if (t_begin == t_end) {  // empty sequence: hand the states through untouched
+        if (ST && a.S_T != a.S0)
+            for (int e = tid; e < (two ? 2 : 1) * kN * kP; e += kThreads) store_state(ST, a.st_bf16, st_off + e, S0 ? S0[e] : 0.f);
         return;
     }
     if (tid == 0) {
         dead = 0;
-        uint64_t *b1 = &bars.full_bc[0];
-        for (int i = 0; i < 10; ++i) mbar_init(b1 + i, 1);
-        uint64_t *b256 = &bars.mg_ready;
-        for (int i = 0; i < 6; ++i) mbar_init(b256 + i, 256);
-        uint64_t *b128 = &bars.sc_ready[0];
-        for (int i = 0; i < 6; ++i) mbar_init(b128 + i, 128);
+        uint64_t *bp = &bars.full_bc[0];
+        for (int i = 0; i < kBars1; ++i) mbar_init(bp++, 1);
+        for (int i = 0; i < 2; ++i) mbar_init(bp++, has_y ? 2 : 1);
+        for (int i = 0; i < kSlots; ++i) mbar_init(bp++, 1);
+        for (int i = 0; i < 5; ++i) mbar_init(bp++, 8);
+        for (int i = 0; i < kSlots; ++i) mbar_init(bp++, has_y ? 16 : 8);
         mbar_fence_init();
     }
-    if (warp == 17) tmem_alloc(&tmem_base, kTmemCols);
+    if (warp == 0) tmem_alloc(&tmem_base, kTmemCols);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tm = tmem_base;
-    float *scal = reinterpret_cast<float *>(sm + kOffSc);
+    Slot *slots = reinterpret_cast<Slot *>(sm + kOffSlot);
+    const uint32_t lane_base = tm + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+    const int wg = warp >> 2, wq = warp & 3;
 
-    if (warp == 16) {
-        // ======================================================= TMA producer
-        if (lane == 0) {
-            tma_prefetch_desc(&mapX);
-            tma_prefetch_desc(&mapB);
-            tma_prefetch_desc(&mapC);
-            if (a.y) tma_prefetch_desc(&mapY);
-            for (int b = 0; b < nblk + 2; ++b) {
-                if (dead) break;   // a wait ran out: nothing more is issued
-                const int st = b & 1;
-                unsigned char *base = sm + st * kStageBytes;
-                const int row = t_begin + b * kQ;
-                // the two-stage ring cannot hide the DRAM latency of the tile loads: pull the tiles of block b+2 into L2 now
-                if (b + 2 < nblk) {
-                    tma_prefetch_l2_2d(&mapX, h * kP, row + 2 * kQ);
-                    for (int kb = 0; kb < 2; ++kb) {
-                        tma_prefetch_l2_2d(&mapB, grp * kN + kb * 64, row + 2 * kQ);
-                        tma_prefetch_l2_2d(&mapC, grp * kN + kb * 64, row + 2 * kQ);
-                    }
-                }
-                if (b < nblk) {
-                    // B and C of block b-2 are free after its (d)
-                    if (b >= 2) mbar_wait(&bars.bc_free[st], ((b - 2) >> 1) & 1, &dead, a.status);
-                    mbar_expect_tx(&bars.full_bc[st], kBTile + kCTile);
-                    for (int kb = 0; kb < 2; ++kb) {
-                        tma_load_2d(base + kXTile + kb * kQ * 128, &mapB, grp * kN + kb * 64, row, &bars.full_bc[st]);
-                        tma_load_2d(base + kXTile + kBTile + kb * kQ * 128, &mapC, grp * kN + kb * 64, row, &bars.full_bc[st]);
-                    }
-                }
-                if (b >= 2) {
-                    // the X tile of block b-2 now stages its y tile (whole blocks only): store it, then reuse the tile
-                    mbar_wait(&bars.ys_ready[st], ((b - 2) >> 1) & 1, &dead, a.status);
-                    if (a.y && row - kQ <= t_end && !dead) {
-                        tma_store_2d(&mapY, base, h * kP, row - 2 * kQ);
-                        tma_store_commit();
-                        tma_store_wait_read();
-                    }
-                }
-                if (b < nblk) {
-                    mbar_expect_tx(&bars.full_x[st], kXTile);
-                    tma_load_2d(base, &mapX, h * kP, row, &bars.full_x[st]);
-                }
-            }
-            tma_store_wait_all();
-        }
-    } else if (warp == 17) {
-        // ======================================================= MMA issuer (one elected thread)
-        if (elect_one()) {
-            constexpr uint32_t idA = umma_idesc(kFmtBF16, false, false, 128, 128);   // (a): C, B both K-major
-            constexpr uint32_t idC = umma_idesc(kFmtBF16, false, true, 128, 64);     // (c), (b): B operand MN-major
-            constexpr uint32_t idD = umma_idesc(kFmtBF16, true, true, 128, 64);      // (d): both MN-major
-            const uint64_t dHb = umma_desc(smem_u32(sm + kOffHb), 0, 1024);
-            // (a) G = C B^T of block b (both operands K-major)
-            auto issue_a = [&](int b) {
-                const uint32_t sbase_u = smem_u32(sm + (b & 1) * kStageBytes);
-                const uint64_t dBk = umma_desc(sbase_u + kXTile, 0, 1024);
-                const uint64_t dCk = umma_desc(sbase_u + kXTile + kBTile, 0, 1024);
+    if (warp == 27) {
+        // ======================================================= scalar warp: half-warp = head, lane = 8 tokens
+        const int hd = lane >> 4, hl = lane & 15;
+        const float Ah = a.A[hd ? h1 : h0] * kLog2e;
+        const float *dth = a.dt + (hd ? h1 : h0);
+        // dt of the next block and of the one after it (a load from DRAM takes as long as a block without outputs)
+        float dt[8], dt2[8];
+        auto fetch_dt = [&](float (&d)[8], int t0) {
+            const float *p = dth + static_cast<size_t>(t0 + 8 * hl) * a.H;
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const uint64_t off = ((k >> 2) * (kQ * 128) + (k & 3) * 32) >> 4;
-                    umma_bf16(tm + kTmG, dCk + off, dBk + off, idA, k > 0);
-                }
-                umma_commit(&bars.ac_done);
-            };
-            mbar_wait(&bars.full_bc[0], 0, &dead, a.status);
-            tc_fence_after_sync();
-            issue_a(0);
-            for (int b = 0; b < nblk; ++b) {
-                if (dead) break;   // a wait ran out: nothing more is issued
-                const uint32_t par = b & 1;
-                const uint32_t sbase_u = smem_u32(sm + (b & 1) * kStageBytes);
-                const uint64_t dX = umma_desc(sbase_u, 0, 1024);
-                const uint64_t dBm = umma_desc(sbase_u + kXTile, kQ * 128, 1024);          // B tile, MN-major view (n blocks 16 KB apart)
-                const uint64_t dCk = umma_desc(sbase_u + kXTile + kBTile, 0, 1024);
-                const uint64_t dX2 = umma_desc(smem_u32(sm + kOffX2 + (b & 1) * kXTile), 0, 1024);
-                mbar_wait(&bars.hb_ready, par, &dead, a.status);
-                if (b >= 2) mbar_wait(&bars.yo_done[(b - 2) % 3], ((b - 2) / 3) & 1, &dead, a.status);
-                tc_fence_after_sync();
-                // (c) Yinter = C S : A = C (K = n), B = bf16 state read MN-major (rows = n)
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    umma_bf16(tm + kTmYe + 64 * par, dCk + (((k >> 2) * (kQ * 128) + (k & 3) * 32) >> 4), dHb + ((k * 16 * 128) >> 4), idC, k > 0);
-                // (d) S += B^T X~ : A = B tile read MN-major (rows = tokens), B = X~ read MN-major
-                mbar_wait(&bars.x2_ready[b & 1], (b >> 1) & 1, &dead, a.status);
-                tc_fence_after_sync();
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    umma_bf16(tm + kTmH, dBm + ((k * 16 * 128) >> 4), dX2 + ((k * 16 * 128) >> 4), idD, true);
-                umma_commit(&bars.h_done[b & 1]);
-                umma_commit(&bars.bc_free[b & 1]);
-                // (b) Yintra = G' X : A = G' from tensor memory (8 columns per K-step of 16 tokens), B = X read MN-major
-                mbar_wait(&bars.mg_ready, par, &dead, a.status);
-                mbar_wait(&bars.full_x[b & 1], (b >> 1) & 1, &dead, a.status);
-                tc_fence_after_sync();
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    umma_bf16_ts(tm + kTmYa + 64 * par, tm + kTmGp + 8 * k, dX + ((k * 16 * 128) >> 4), idC, k > 0);
-                umma_commit(&bars.y_done);
-                // (a) of the next block: G has been drained by the mask epilogue of this one
-                if (b + 1 < nblk) {
-                    mbar_wait(&bars.full_bc[(b + 1) & 1], ((b + 1) >> 1) & 1, &dead, a.status);
-                    tc_fence_after_sync();
-                    issue_a(b + 1);
-                }
-            }
-        }
-    } else if (warp >= 12) {
-        // ======================================================= scalar warpgroup: thread = token; per-block scalars and X~, ahead of the chain
-        const int x = tid - 384;   // 0..127
-        const float Ah = a.A[h];
-        // dt of this thread's token in block b (0 beyond the sequence end); fetched one block before it is used
-        auto fetch_dt = [&](int b) {
-            const int t = t_begin + b * kQ + x;
-            return (b < nblk && t < t_end) ? a.dt[static_cast<size_t>(t) * a.H + h] : 0.f;
+            for (int j = 0; j < 8; ++j) d[j] = t0 + 8 * hl + j < t_end ? p[static_cast<size_t>(j) * a.H] : 0.f;
         };
-        float dt_next = fetch_dt(0);
-        auto prepare_scalars = [&](int b) {
-            float *dst = scal + (b % 3) * kScFloats;
-            const float dtv = dt_next;
-            dt_next = fetch_dt(b + 1);
-            float run = dtv * Ah;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const float up = __shfl_up_sync(0xffffffffu, run, o);
-                if (lane >= o) run += up;
-            }
-            if (lane == 31) scan_carry[warp & 3] = run;
-            named_bar_sync(1, 128);
-            for (int w = 0; w < (warp & 3); ++w) run += scan_carry[w];
-            const float l2 = run * kLog2e;
-            dst[x] = l2;
-            dst[kQ + x] = exp2f(l2);
-            dst[4 * kQ + x] = dtv;
-            named_bar_sync(1, 128);
-            dst[2 * kQ + x] = exp2f(dst[kQ - 1] - l2) * dtv;
-            // factor of column x relative to the first column of its group of 16 (>= 1 before dt)
-            const float rng = dst[x & ~15] - l2;
-            dst[3 * kQ + x] = exp2f(fminf(rng, 126.f)) * dtv;
-            // the fast epilogue is exact only while no group spans more than kMaxGroupRange
-            const unsigned bad = __ballot_sync(0xffffffffu, rng > kMaxGroupRange);
-            if (lane == 0) scan_carry[warp & 3] = bad ? 1.f : 0.f;
-            named_bar_sync(1, 128);
-            if (x == 0) dst[5 * kQ] = scan_carry[0] + scan_carry[1] + scan_carry[2] + scan_carry[3];
-            named_bar_sync(1, 128);
-            mbar_arrive(&bars.sc_ready[b % 3]);
-        };
-        // X~ row of token x of block b: s_x * X[x][:]
-        auto scaled_x = [&](int b) {
-            const float *sc = scal + (b % 3) * kScFloats;
-            mbar_wait(&bars.full_x[b & 1], (b >> 1) & 1, &dead, a.status);
-            const unsigned char *xt = sm + (b & 1) * kStageBytes;
-            unsigned char *x2 = sm + kOffX2 + (b & 1) * kXTile;
-            const float s = sc[2 * kQ + x];
-#pragma unroll
-            for (int c8 = 0; c8 < 8; ++c8) {
-                const uint32_t off = sw128_offset(x, c8);
-                const uint4 v = *reinterpret_cast<const uint4 *>(xt + off);
-                const uint32_t in[4] = {v.x, v.y, v.z, v.w};
-                uint32_t w[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    w[e] = pack_bf16(__uint_as_float(in[e] << 16) * s, __uint_as_float(in[e] & 0xFFFF0000u) * s);
-                *reinterpret_cast<uint4 *>(x2 + off) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-            fence_async_smem();
-            mbar_arrive(&bars.x2_ready[b & 1]);
-        };
-        for (int b = 0; b < nblk; ++b) {
-            // the scalar buffer of block b is the one block b-3 used: its outputs must be written
-            if (b >= 3) mbar_wait(&bars.yo_done[b % 3], ((b - 3) / 3) & 1, &dead, a.status);
-            prepare_scalars(b);
-            // the X~ buffer of block b was read by (d) of block b-2
-            if (b >= 2) mbar_wait(&bars.h_done[b & 1], ((b - 2) >> 1) & 1, &dead, a.status);
-            scaled_x(b);
-        }
-    } else if (warp >= 8) {
-        // ======================================================= state warpgroup: thread = state row n
-        const int x = tid - 256;   // 0..127
-        const uint32_t lane_base = tm + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-        // initial state: fp32 into tensor memory pre-scaled by e^{l_Q} of block 0, bf16 copy unscaled
-        mbar_wait(&bars.sc_ready[0], 0, &dead, a.status);
-        {
-            const float gq = scal[kQ + kQ - 1];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                uint32_t rr[32], sc[32];
-#pragma unroll
-                for (int c = 0; c < 32; ++c) {
-                    const float v = a.S0 ? a.S0[sbase + static_cast<size_t>(x) * kP + 32 * q + c] : 0.f;
-                    rr[c] = __float_as_uint(v);
-                    sc[c] = __float_as_uint(v * gq);
-                }
-                tmem_st32(lane_base + kTmH + 32 * q, sc);
-#pragma unroll
-                for (int c8 = 0; c8 < 4; ++c8) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) w[e] = pack_bf16(__uint_as_float(rr[8 * c8 + 2 * e]), __uint_as_float(rr[8 * c8 + 2 * e + 1]));
-                    *reinterpret_cast<uint4 *>(sm + kOffHb + sw128_offset(x, 4 * q + c8)) = make_uint4(w[0], w[1], w[2], w[3]);
-                }
-            }
-            tmem_st_wait();
-            fence_async_smem();
-            tc_fence_before_sync();
-            mbar_arrive(&bars.hb_ready);
-        }
-        for (int b = 0; b < nblk; ++b) {
-            // state after (d): copy for the next block's (c), pre-scale for its (d); or S_T at the end
-            const bool last = b + 1 == nblk;
-            if (!last) mbar_wait(&bars.sc_ready[(b + 1) % 3], ((b + 1) / 3) & 1, &dead, a.status);
-            const float gq = last ? 1.f : scal[((b + 1) % 3) * kScFloats + kQ + kQ - 1];
-            mbar_wait(&bars.h_done[b & 1], (b >> 1) & 1, &dead, a.status);
-            tc_fence_after_sync();
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                uint32_t rr[32];
-                tmem_ld32(lane_base + kTmH + 32 * q, rr);
-                tmem_ld_wait();
-                if (last) {
-                    if (a.S_T && !dead && a.st_bf16) {
-                        __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(a.S_T) + sbase + static_cast<size_t>(x) * kP + 32 * q;
-#pragma unroll
-                        for (int c = 0; c < 32; c += 8)
-                            *reinterpret_cast<uint4 *>(dst + c) =
-                                make_uint4(pack_bf16(__uint_as_float(rr[c]), __uint_as_float(rr[c + 1])), pack_bf16(__uint_as_float(rr[c + 2]), __uint_as_float(rr[c + 3])),
-                                           pack_bf16(__uint_as_float(rr[c + 4]), __uint_as_float(rr[c + 5])), pack_bf16(__uint_as_float(rr[c + 6]), __uint_as_float(rr[c + 7])));
-                    } else if (a.S_T && !dead) {
-#pragma unroll
-                        for (int c = 0; c < 32; c += 4)
-                            *reinterpret_cast<float4 *>(a.S_T + sbase + static_cast<size_t>(x) * kP + 32 * q + c) =
-                                make_float4(__uint_as_float(rr[c]), __uint_as_float(rr[c + 1]), __uint_as_float(rr[c + 2]), __uint_as_float(rr[c + 3]));
-                    }
-                } else {
-#pragma unroll
-                    for (int c8 = 0; c8 < 4; ++c8) {
-                        uint32_t w[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) w[e] = pack_bf16(__uint_as_float(rr[8 * c8 + 2 * e]), __uint_as_float(rr[8 * c8 + 2 * e + 1]));
-                        *reinterpret_cast<uint4 *>(sm + kOffHb + sw128_offset(x, 4 * q + c8)) = make_uint4(w[0], w[1], w[2], w[3]);
-                    }
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) rr[c] = __float_as_uint(__uint_as_float(rr[c]) * gq);
-                    tmem_st32(lane_base + kTmH + 32 * q, rr);
-                }
-            }
-            if (!last) {
-                tmem_st_wait();
-                fence_async_smem();
-                tc_fence_before_sync();
-                mbar_arrive(&bars.hb_ready);
-            }
-        }
-    } else {
-        // ======================================================= epilogue warpgroups: thread = token row t, warpgroup = column half
-        const int t = tid & 127;
-        const int half = warp >> 2;
-        const uint32_t lane_base = tm + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-        __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(a.y);
-        {
-            // operand columns above the diagonal for every row of this warp are never written again: zero them once
-            const uint32_t z[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-            for (int q = 0; q < 4; ++q)
-                if (64 * half + 16 * q > 32 * (warp & 3) + 31) tmem_st8(lane_base + kTmGp + 32 * half + 8 * q, z);
-            tmem_st_wait();
-        }
-        for (int b = 0; b < nblk; ++b) {
-            const float *sc = scal + (b % 3) * kScFloats;
-            mbar_wait(&bars.sc_ready[b % 3], (b / 3) & 1, &dead, a.status);
-            mbar_wait(&bars.ac_done, b & 1, &dead, a.status);
-            tc_fence_after_sync();
-            // G' row t, columns i = 64*half .. 64*half+63 -> bf16 pairs in TMEM columns 32*half .. 32*half+31 of the operand.
-            // ((b) of the previous block, which read that operand, completed before its y epilogue ran.)
-            // e^{l_t - l_i} dt_i = 2^{l2_t - l2_ref} * f_i with ref the first column of i's group of 16: one
-            // exponential per group instead of one per element (every factor is <= 1 where i <= t);
-            // blocks whose decay is too violent for that take the per-element path.
-            {
-                const float lt = sc[t];
-                const bool fast = sc[5 * kQ] == 0.f;
+        int t0 = t_begin;
+        float R = 0.f, total = 0.f;
+        fetch_dt(dt, t0);
+        fetch_dt(dt2, t0 + kQ);
+        // (never leaves the loop early: every pass advances t0 whatever the waits say)
 #pragma unroll 1
-                for (int q = 0; q < 4; ++q) {
-                    const int i0 = 64 * half + 16 * q;
-                    if (i0 > 32 * (warp & 3) + 31) break;   // above the diagonal for every row of this warp: stays zero
-                    uint32_t rr[16];
-                    tmem_ld16(lane_base + kTmG + 64 * half + 16 * q, rr);
-                    tmem_ld_wait();
-                    uint32_t w[8];
-                    if (fast) {
-                        float aa;
-                        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(aa) : "f"(fminf(lt - sc[i0], 0.f)));
-                        if (i0 + 15 <= 32 * (warp & 3)) {
-                            // the whole group lies below the diagonal for every row of this warp: no masking
+        for (int b = 0; t0 < t_end; ++b) {
+            float l2[8], dv[8];
 #pragma unroll
-                            for (int c = 0; c < 16; c += 4) {
-                                const float4 f = *reinterpret_cast<const float4 *>(sc + 3 * kQ + i0 + c);
-                                w[c / 2] = pack_bf16(__uint_as_float(rr[c]) * aa * f.x, __uint_as_float(rr[c + 1]) * aa * f.y);
-                                w[c / 2 + 1] = pack_bf16(__uint_as_float(rr[c + 2]) * aa * f.z, __uint_as_float(rr[c + 3]) * aa * f.w);
-                            }
-                        } else {
+            for (int j = 0; j < 8; ++j) dv[j] = dt[j];
+            int n = min(kQ, t_end - t0);
+            // the block ends before the first token whose decay leaves the range, in either head: then again without the rest
+#pragma unroll 1
+            for (;;) {
+                float run = 0.f;
 #pragma unroll
-                            for (int c = 0; c < 16; c += 4) {
-                                const float4 f = *reinterpret_cast<const float4 *>(sc + 3 * kQ + i0 + c);
-                                const float v0 = (i0 + c <= t) ? __uint_as_float(rr[c]) * aa * f.x : 0.f;
-                                const float v1 = (i0 + c + 1 <= t) ? __uint_as_float(rr[c + 1]) * aa * f.y : 0.f;
-                                const float v2 = (i0 + c + 2 <= t) ? __uint_as_float(rr[c + 2]) * aa * f.z : 0.f;
-                                const float v3 = (i0 + c + 3 <= t) ? __uint_as_float(rr[c + 3]) * aa * f.w : 0.f;
-                                w[c / 2] = pack_bf16(v0, v1);
-                                w[c / 2 + 1] = pack_bf16(v2, v3);
-                            }
-                        }
-                    } else {
+                for (int j = 0; j < 8; ++j) {
+                    run = fmaf(dv[j], Ah, run);
+                    l2[j] = run;
+                }
+                float tot = run;
 #pragma unroll
-                        for (int c = 0; c < 16; c += 2) {
-                            const float v0 = (i0 + c <= t) ? __uint_as_float(rr[c]) * exp2f(lt - sc[i0 + c]) * sc[4 * kQ + i0 + c] : 0.f;
-                            const float v1 = (i0 + c + 1 <= t) ? __uint_as_float(rr[c + 1]) * exp2f(lt - sc[i0 + c + 1]) * sc[4 * kQ + i0 + c + 1] : 0.f;
-                            w[c / 2] = pack_bf16(v0, v1);
-                        }
+                for (int o = 1; o < 16; o <<= 1) {
+                    const float up = __shfl_up_sync(0xffffffffu, tot, o, 16);
+                    if (hl >= o) tot += up;
+                }
+                const float before = tot - run;
+                int bad = kQ;
+#pragma unroll
+                for (int j = 7; j >= 0; --j) {
+                    l2[j] += before;
+                    if (fabsf(l2[j]) > kMaxRange) bad = 8 * hl + j;
+                }
+                unsigned any = __ballot_sync(0xffffffffu, bad < n);
+                if (!any || n == 1) break;
+#pragma unroll 1
+                for (; any; any &= any - 1) n = min(n, __shfl_sync(0xffffffffu, bad, __ffs(any) - 1));
+                n = max(n, 1);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (8 * hl + j >= n) dv[j] = 0.f;
+            }
+            const float ln = __shfl_sync(0xffffffffu, l2[7], 15, 16);   // tokens beyond the block have dt = 0
+            float Rn = R;
+            if (fabsf(R - ln) > kMaxScale) Rn = ln < 0.f ? -kNewScale : kNewScale;
+            if (fabsf(ln) > kMaxRange) Rn = rintf(ln);   // a single token of violent decay: nothing of the state is left
+            const int start = t0;
+            t0 += n;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) dt[j] = dt2[j];
+            if (n < kQ && t0 < t_end) fetch_dt(dt, t0);
+            fetch_dt(dt2, t0 + kQ);
+            if (b >= kSlots) mbar_wait(&bars.slot_free[b % kSlots], ((b - kSlots) / kSlots) & 1, &dead, a.status);
+            __syncwarp();
+            Slot &sl = slots[b % kSlots];
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                const float s0 = dv[j] * ex2(Rn - l2[j]), s1 = dv[j + 1] * ex2(Rn - l2[j + 1]);
+                hi[j / 2] = pack_bf16(s0, s1);
+                lo[j / 2] = pack_bf16(s0 - __uint_as_float(hi[j / 2] << 16), s1 - __uint_as_float(hi[j / 2] & 0xFFFF0000u));
+            }
+#pragma unroll
+            for (int j = 0; j < 8; j += 4) {
+                *reinterpret_cast<uint4 *>(&sl.s[hd][4 * hl + j / 2]) = make_uint4(hi[j / 2], lo[j / 2], hi[j / 2 + 1], lo[j / 2 + 1]);
+                *reinterpret_cast<float4 *>(&sl.e[hd][8 * hl + j]) = make_float4(ex2(l2[j] - Rn), ex2(l2[j + 1] - Rn), ex2(l2[j + 2] - Rn), ex2(l2[j + 3] - Rn));
+            }
+            if (hl == 0) {
+                sl.f2[hd] = Rn - R;
+                sl.e2[hd] = ln - Rn;
+                sl.start = start;
+                sl.n = n;
+            }
+            R = Rn - ln;
+            total += ln;
+            warp_arrive(&bars.sc_ready[b % kSlots]);
+        }
+        if (a.lam && hl == 0 && (hd == 0 || two)) a.lam[static_cast<size_t>(seq) * a.H + h0 + hd] = total / kLog2e;
+    } else if (warp >= 24) {
+        // ======================================================= single-issue roles.  The whole warp walks the loop and one elected lane
+        // issues: the operands of these instructions live in registers that the warp shares, so its lanes stay together.
+        int row = t_begin;
+        if (warp == 24) {
+            // ---- TMA: one load brings both 64-column halves of B or C, or X of both heads
+#pragma unroll 1
+            for (int b = 0; row < t_end; ++b) {
+                if (warp_dead(&dead)) break;   // a wait ran out: nothing more is issued
+                const int st = b & 1;
+                if (b >= 2) mbar_wait(&bars.bc_free[st], ((b - 2) >> 1) & 1, &dead, a.status);
+                __syncwarp();
+                if (elect_one()) {
+                    unsigned char *bc = sm + st * kBCStage;
+                    mbar_expect_tx(&bars.full_bc[st], has_y ? kBCStage : kBCStage / 2);
+                    tma_load_3d(bc, &mapB, row, 2 * grp, &bars.full_bc[st]);
+                    if (has_y) tma_load_3d(bc + 2 * kTile, &mapC, row, 2 * grp, &bars.full_bc[st]);
+                    // the ring cannot hide the DRAM latency of the tile loads: pull the tiles of block b+2 into L2 now
+                    if (row + 2 * kQ < t_end) {
+                        tma_prefetch_l2_3d(&mapX, row + 2 * kQ, h0);
+                        tma_prefetch_l2_3d(&mapB, row + 2 * kQ, 2 * grp);
+                        if (has_y) tma_prefetch_l2_3d(&mapC, row + 2 * kQ, 2 * grp);
                     }
-                    tmem_st8(lane_base + kTmGp + 32 * half + 8 * q, w);
+                }
+                __syncwarp();
+                if (b >= 1) mbar_wait(&bars.x_free, (b - 1) & 1, &dead, a.status);
+                __syncwarp();
+                if (elect_one()) {
+                    mbar_expect_tx(&bars.full_x, 2 * kTile);
+                    tma_load_3d(sm + kOffX, &mapX, row, h0, &bars.full_x);
+                }
+                __syncwarp();
+                // where the next block starts
+                mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
+                row += slots[b % kSlots].n;
+            }
+        } else if (warp == 25) {
+            // ---- MMA issue of (S)
+            constexpr uint32_t idS = umma_idesc(kFmtBF16, false, true, 128, 128);
+#pragma unroll 1
+            for (int b = 0; row < t_end; ++b) {
+                if (warp_dead(&dead)) break;
+                const int st = b & 1;
+                const uint64_t dB = umma_desc(smem_u32(sm + st * kBCStage), kTile, 1024);
+                mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
+                row += slots[b % kSlots].n;
+                mbar_wait(&bars.full_bc[st], (b >> 1) & 1, &dead, a.status);
+                mbar_wait(&bars.x2_ready, b & 1, &dead, a.status);
+                mbar_wait(&bars.hb_ready, b & 1, &dead, a.status);
+                __syncwarp();
+                tc_fence_after_sync();
+                if (elect_one()) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) umma_bf16_ts(tm + kTmS, tm + kTmX + 8 * k, dB + ((k * 16 * 128) >> 4), idS, true);
+                    umma_commit(&bars.h_done);
+                    umma_commit(&bars.xs_free);
+                    umma_commit(&bars.bc_free[st]);
+                }
+                __syncwarp();
+            }
+        } else if (has_y) {
+            // ---- MMA issue of (G) (both operands K-major; one block ahead), (Y2), (Y1)
+            constexpr uint32_t idG = umma_idesc(kFmtBF16, false, false, 128, 128);
+            constexpr uint32_t idY64 = umma_idesc(kFmtBF16, false, false, 128, 64);
+            const uint64_t dG = umma_desc(smem_u32(sm + kOffG), 0, 1024);
+#pragma unroll 1
+            for (int b = -1; b < 0 || row < t_end; ++b) {
+                if (warp_dead(&dead)) break;
+                bool last = false;
+                if (b >= 0) {
+                    const uint64_t dC = umma_desc(smem_u32(sm + (b & 1) * kBCStage + 2 * kTile), 0, 1024);
+                    mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
+                    row += slots[b % kSlots].n;
+                    last = row >= t_end;
+                    if (b >= 1) mbar_wait(&bars.y_free, (b - 1) & 1, &dead, a.status);
+                    mbar_wait(&bars.hb_ready, b & 1, &dead, a.status);
+                    __syncwarp();
+                    tc_fence_after_sync();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            umma_bf16_ts(tm + kTmY, tm + kTmSb + 8 * k, dC + (((k >> 2) * kTile + (k & 3) * 32) >> 4), idG, k > 0);
+                        umma_commit(&bars.y2_done);
+                        umma_commit(&bars.bc_free[b & 1]);
+                    }
+                    __syncwarp();
+                    mbar_wait(&bars.x2_ready, b & 1, &dead, a.status);
+                    mbar_wait(&bars.mask_done, b & 1, &dead, a.status);
+                    __syncwarp();
+                    tc_fence_after_sync();
+                    if (elect_one()) {
+                        // tokens i < 64 onto all t, then i >= 64 onto t >= 64
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) umma_bf16_ts(tm + kTmY, tm + kTmX + 8 * k, dG + ((k * 32) >> 4), idG, true);
+#pragma unroll
+                        for (int k = 4; k < 8; ++k)
+                            umma_bf16_ts(tm + kTmY + 64, tm + kTmX + 8 * k, dG + ((kTile + (k - 4) * 32) >> 4), idY64, true);
+                        umma_commit(&bars.y_done);
+                        umma_commit(&bars.xy_free);
+                    }
+                    __syncwarp();
+                }
+                if (!last) {   // (G) of block b+1: the mask warps have drained the G columns
+                    const uint32_t bc = smem_u32(sm + ((b + 1) & 1) * kBCStage);
+                    const uint64_t dB = umma_desc(bc, 0, 1024), dC = umma_desc(bc + 2 * kTile, 0, 1024);
+                    mbar_wait(&bars.full_bc[(b + 1) & 1], ((b + 1) >> 1) & 1, &dead, a.status);
+                    __syncwarp();
+                    tc_fence_after_sync();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const uint64_t off = ((k >> 2) * kTile + (k & 3) * 32) >> 4;
+                            umma_bf16(tm + kTmG, dC + off, dB + off, idG, k > 0);
+                        }
+                        umma_commit(&bars.g_done);
+                    }
+                    __syncwarp();
                 }
             }
+        }
+    } else if (wg >= 4) {
+        // ======================================================= prep: X^^T of 64 tokens; this warp: 32 features of one head
+        const int th = wg - 4, hd = wq >> 1;
+        const int m = lane >> 3, i = lane & 7;
+        const uint32_t zero = a.n_seq < 0 ? 1u : 0u;   // 0, which the compiler cannot know
+        // matrix m of a load: features 8 (m & 1) .., tokens 8 (m >> 1) ..
+        const uint32_t xrow = smem_u32(sm + kOffX + hd * kTile) + (64 * th + 8 * (m >> 1) + i) * 128;
+        // mask: row t of tril(G) -> bf16 operand tile, columns < 64 of row t and columns >= 64 of row t - 64
+        const int t = tid & 127;
+        unsigned char *g0 = sm + kOffG + t * 128, *g1 = g0 + kTile - 64 * 128;
+        if ((wq & 1) == 0 && th == 0) {   // the 32 columns right of this warp's diagonal block: zeros, never written again
+#pragma unroll
+            for (int c8 = 4; c8 < 8; ++c8) *reinterpret_cast<uint4 *>((wq ? g1 : g0) + ((c8 ^ (t & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        bool last = false;
+#pragma unroll 1
+        for (int b = 0; !last; ++b) {
+            if (warp_dead(&dead)) break;
+            mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
+            const Slot &sl = slots[b % kSlots];
+            last = sl.start + sl.n >= t_end;
+            mbar_wait(&bars.full_x, b & 1, &dead, a.status);
+            __syncwarp();
+            uint32_t w[2][16];
+#pragma unroll
+            for (int lh = 0; lh < 2; ++lh)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    ldmatrix_x4_trans(xrow + 16 * j * 128 + (((4 * (wq & 1) + 2 * lh + (m & 1)) ^ i) << 4), w[lh][4 * j], w[lh][4 * j + 1],
+                                      w[lh][4 * j + 2], w[lh][4 * j + 3]);
+            // x s with s = high + low part: two packed operations and one rounding that counts, where unpacking, fp32 products and
+            // packing take five
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const uint2 s2 = sl.s[hd][32 * th + 4 * k + (lane & 3)];
+                const __nv_bfloat162 sh = *reinterpret_cast<const __nv_bfloat162 *>(&s2.x), sl2 = *reinterpret_cast<const __nv_bfloat162 *>(&s2.y);
+#pragma unroll
+                for (int lh = 0; lh < 2; ++lh)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        __nv_bfloat162 *x = reinterpret_cast<__nv_bfloat162 *>(&w[lh][2 * k + e]);
+                        *x = __hfma2(*x, sh, __hmul2(*x, sl2));
+                    }
+            }
+            // The tile may be overwritten once its loads have RETURNED, not once they are issued: the assembler may hold their first
+            // use back past the arrival, and under load they have come back later than the next tile (seen: single rows of the
+            // next block).  So the arrival's address takes a zero that is made of one result of every load.
+            uint32_t any = 0;
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) any |= w[0][j] | w[1][j];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.x_free + (any & zero));
+            if (b >= 1) {   // (S) and (Y1) have read the X^ before
+                mbar_wait(&bars.xs_free, (b - 1) & 1, &dead, a.status);
+                if (has_y) mbar_wait(&bars.xy_free, (b - 1) & 1, &dead, a.status);
+            }
+            __syncwarp();
+            tc_fence_after_sync();
+#pragma unroll
+            for (int lh = 0; lh < 2; ++lh) tmem_st_16x128b_x8(lane_base + (static_cast<uint32_t>(16 * lh) << 16) + kTmX + 32 * th, w[lh]);
             tmem_st_wait();
             tc_fence_before_sync();
-            mbar_arrive(&bars.mg_ready);
-            // y_t[p] = Yintra + e^{l_t} Yinter, p = 32*half .. 32*half+31
-            mbar_wait(&bars.y_done, b & 1, &dead, a.status);
-            tc_fence_after_sync();
-            {
-                uint32_t ya[32], ye[32];
-                tmem_ld32(lane_base + kTmYa + 64 * (b & 1) + 32 * half, ya);
-                tmem_ld32(lane_base + kTmYe + 64 * (b & 1) + 32 * half, ye);
-                tmem_ld_wait();
-                const float et = sc[kQ + t];
-                const int row0 = t_begin + b * kQ;
-                uint32_t w[16];
+            warp_arrive(&bars.x2_ready);
+            if (has_y) {
+                // mask, 32 columns at a time: the two warps of a lane quarter take every other one; the last holds the diagonal.
+                // ((Y1) of the block before has read the tile: waited for above.)
+                mbar_wait(&bars.g_done, b & 1, &dead, a.status);
+                __syncwarp();
+                tc_fence_after_sync();
+#pragma unroll 1
+                for (int q = th; q <= wq; q += 2) {
+                    uint32_t rr[32], wm[16];
+                    tmem_ld32(lane_base + kTmG + 32 * q, rr);
+                    tmem_ld_wait();
 #pragma unroll
-                for (int c = 0; c < 32; c += 2)
-                    w[c / 2] = pack_bf16(__uint_as_float(ya[c]) + et * __uint_as_float(ye[c]),
-                                         __uint_as_float(ya[c + 1]) + et * __uint_as_float(ye[c + 1]));
-                if (!a.y) {
-                    // no outputs wanted (final states only)
-                } else if (row0 + kQ <= t_end) {
-                    // whole block inside the sequence: stage the y tile in this block's X tile ((b) has read it) in
-                    // the layout of the tensor map and let the TMA warp store it -- full 128-byte rows
-                    // instead of 32 scattered 16-byte pieces per warp instruction
-                    unsigned char *ys = sm + (b & 1) * kStageBytes;
+                    for (int e = 0; e < 16; ++e) wm[e] = pack_bf16(__uint_as_float(rr[2 * e]), __uint_as_float(rr[2 * e + 1]));
+                    if (q == wq) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) wm[e] = 2 * e + 1 <= lane ? wm[e] : (2 * e <= lane ? wm[e] & 0xffffu : 0u);
+                    }
+                    unsigned char *row = q < 2 ? g0 : g1;
 #pragma unroll
                     for (int c8 = 0; c8 < 4; ++c8)
-                        *reinterpret_cast<uint4 *>(ys + sw128_offset(t, 4 * half + c8)) = make_uint4(w[4 * c8], w[4 * c8 + 1], w[4 * c8 + 2], w[4 * c8 + 3]);
-                    fence_async_smem();
-                } else {
-                    const int tok = row0 + t;
-                    if (tok < t_end && !dead) {
-                        __nv_bfloat16 *dst = y + (static_cast<size_t>(tok) * a.H + h) * kP + 32 * half;
-#pragma unroll
-                        for (int c8 = 0; c8 < 4; ++c8)
-                            *reinterpret_cast<uint4 *>(dst + 8 * c8) = make_uint4(w[4 * c8], w[4 * c8 + 1], w[4 * c8 + 2], w[4 * c8 + 3]);
-                    }
+                        *reinterpret_cast<uint4 *>(row + (((4 * (q & 1) + c8) ^ (t & 7)) << 4)) = make_uint4(wm[4 * c8], wm[4 * c8 + 1], wm[4 * c8 + 2], wm[4 * c8 + 3]);
                 }
-                mbar_arrive(&bars.ys_ready[b & 1]);
+                fence_async_smem();
+                tc_fence_before_sync();
+                warp_arrive(&bars.mask_done);
             }
-            tc_fence_before_sync();
-            mbar_arrive(&bars.yo_done[b % 3]);
         }
+    } else if (wg >= 2) {
+        // ======================================================= state: lane = (head, p), warpgroup = 64 columns n
+        const int x = tid & 127, hd = x >> 6, n0 = 64 * (wg - 2);
+        const size_t mine = (hd && two ? static_cast<size_t>(kN) * kP : 0) + static_cast<size_t>(n0) * kP + (x & 63);
+        {
+            // initial state, scaled by 2^R of block 0
+#pragma unroll 1
+            for (int q = 0; q < 2; ++q) {
+                uint32_t rr[32];
+#pragma unroll
+                for (int c = 0; c < 32; ++c) rr[c] = S0 ? __float_as_uint(S0[mine + (32 * q + c) * kP]) : 0u;
+                if (q == 0) mbar_wait(&bars.sc_ready[0], 0, &dead, a.status);
+                __syncwarp();
+                const float f = ex2(slots[0].f2[hd]);
+#pragma unroll
+                for (int c = 0; c < 32; ++c) rr[c] = __float_as_uint(__uint_as_float(rr[c]) * f);
+                tmem_st32(lane_base + kTmS + n0 + 32 * q, rr);
+                copy_state32(lane_base, n0 + 32 * q, rr);
+            }
+            tmem_st_wait();
+            tc_fence_before_sync();
+            warp_arrive(&bars.hb_ready);
+        }
+        bool last = false;
+#pragma unroll 1
+        for (int b = 0; !last; ++b) {
+            if (warp_dead(&dead)) break;
+            mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
+            const Slot &sl = slots[b % kSlots];
+            last = sl.start + sl.n >= t_end;
+            float ex = sl.e2[hd];
+            if (!last) {
+                mbar_wait(&bars.sc_ready[(b + 1) % kSlots], ((b + 1) / kSlots) & 1, &dead, a.status);
+                ex = slots[(b + 1) % kSlots].f2[hd];
+            }
+            mbar_wait(&bars.h_done, b & 1, &dead, a.status);
+            if (has_y) mbar_wait(&bars.y2_done, b & 1, &dead, a.status);   // the bf16 copy has been read
+            __syncwarp();
+            tc_fence_after_sync();
+            if (ex != 0.f) scale_state64(lane_base + kTmS + n0, ex);
+            __syncwarp();
+            if (last) {
+                const bool store = ST && (hd == 0 || two) && !warp_dead(&dead);
+#pragma unroll 1
+                for (int q = 0; q < 8; ++q) {
+                    uint32_t rr[8];
+                    tmem_ld8(lane_base + kTmS + n0 + 8 * q, rr);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        if (store) store_state(ST, a.st_bf16, st_off + mine + static_cast<size_t>(8 * q + c) * kP, __uint_as_float(rr[c]));
+                }
+            } else {
+#pragma unroll 1
+                for (int q = 0; q < 2; ++q) {
+                    uint32_t rr[32];
+                    tmem_ld32(lane_base + kTmS + n0 + 32 * q, rr);
+                    tmem_ld_wait();
+                    copy_state32(lane_base, n0 + 32 * q, rr);
+                }
+                tmem_st_wait();
+                tc_fence_before_sync();
+                warp_arrive(&bars.hb_ready);
+            }
+            warp_arrive(&bars.slot_free[b % kSlots]);
+        }
+    } else if (has_y) {
+        // ======================================================= outputs of 64 tokens; this warp: 32 features of one head
+        const int th = wg, hd = wq >> 1;
+        const int m = lane >> 3, i = lane & 7;
+        // staging rows [token][128 bytes = 64 features], this warp's four 16-byte pieces of each;
+        // matrix m of a store: features 8 (m & 1) .., tokens 8 (m >> 1) ..
+        unsigned char *ys = sm + kOffY + hd * kTile + 64 * th * 128;
+        const uint32_t srow = smem_u32(ys) + (8 * (m >> 1) + i) * 128;
+        bool last = false;
+#pragma unroll 1
+        for (int b = 0; !last; ++b) {
+            mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
+            const Slot &sl = slots[b % kSlots];
+            const int start = sl.start, n = sl.n;
+            last = start + n >= t_end;
+            mbar_wait(&bars.y_done, b & 1, &dead, a.status);
+            __syncwarp();
+            tc_fence_after_sync();
+            // all of Y leaves tensor memory (packed: 32 registers) before the stage is needed, which the store of the block before
+            // may still be reading
+            uint32_t w[2][16];
+            const float *e0 = &sl.e[hd][64 * th + 2 * (lane & 3)];
+#pragma unroll
+            for (int lh = 0; lh < 2; ++lh) {
+                uint32_t r[32];
+                tmem_ld_16x256b_x8(lane_base + (static_cast<uint32_t>(16 * lh) << 16) + kTmY + 64 * th, r);
+                tmem_ld_wait();
+                if (lh == 1) {
+                    tc_fence_before_sync();
+                    warp_arrive(&bars.y_free);
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {   // 8 tokens
+                    const float2 e = *reinterpret_cast<const float2 *>(e0 + 8 * k);
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)   // (scalar multiplies: packed ones cost register moves here)
+                        w[lh][2 * k + u] = pack_bf16(__uint_as_float(r[4 * k + 2 * u]) * e.x, __uint_as_float(r[4 * k + 2 * u + 1]) * e.y);
+                }
+            }
+            warp_arrive(&bars.slot_free[b % kSlots]);
+            // the eight warps leave together if a wait ran out
+            if (warp == 0 && elect_one()) tma_store_wait_read();
+            if (named_bar_or(1, 256, dead != 0)) break;
+#pragma unroll
+            for (int lh = 0; lh < 2; ++lh)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)   // 16 tokens
+                    stmatrix_x4_trans(srow + 16 * kk * 128 + (((4 * (wq & 1) + 2 * lh + (m & 1)) ^ i) << 4), w[lh][4 * kk], w[lh][4 * kk + 1],
+                                      w[lh][4 * kk + 2], w[lh][4 * kk + 3]);
+            if (n == kQ && two) {
+                fence_async_smem();
+                named_bar_sync(2, 256);
+                if (warp == 0 && elect_one()) {
+                    tma_store_3d(&mapY, sm + kOffY, start, h0);
+                    tma_store_commit();
+                }
+            } else if (hd == 0 || two) {
+                // a block that is not whole, or whose second head is not wanted: rows straight to global memory
+                __syncwarp();
+                const size_t tstride = static_cast<size_t>(a.H) * kP;
+                __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(a.y) + static_cast<size_t>(start + 64 * th + i) * tstride +
+                                     static_cast<size_t>(h0 + hd) * kP + 32 * (wq & 1) + 8 * m;
+                const unsigned char *src = ys + i * 128 + (((4 * (wq & 1) + m) ^ i) << 4);
+                const int left = min(64, n - 64 * th);
+#pragma unroll 1
+                for (int j = i; j < left; j += 8, src += 8 * 128, dst += 8 * tstride)   // lane = row i of 8, piece m of this warp's four
+                    *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(src);
+                fence_async_smem();
+            }
+        }
+        if (warp == 0 && elect_one()) tma_store_wait_all();
     }
     grace_after_timeout(&dead);
+    __syncwarp();   // the warps of the single-thread roles come back together before the warp-aligned instructions below
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 17) tmem_dealloc(tm, kTmemCols);
+    if (warp == 0) tmem_dealloc(tm, kTmemCols);
 }
 
 }  // namespace
@@ -498,15 +669,16 @@ cudaError_t launch_ssd_scan_tensor(const SsdArgs &a, cudaStream_t s) {
         // cannot be encoded)
         memset(&mapX, 0, sizeof(mapX));
         mapB = mapC = mapY = mapX;
-    } else if (!make_tensor_map_2d(&mapX, a.x, 2, x_inner, rows, x_inner * 2, 64, kQ, true) ||
-        !make_tensor_map_2d(&mapB, a.B, 2, bc_inner, rows, bc_inner * 2, 64, kQ, true) ||
-        !make_tensor_map_2d(&mapC, a.C, 2, bc_inner, rows, bc_inner * 2, 64, kQ, true) ||
-        (a.y && !make_tensor_map_2d(&mapY, a.y, 2, x_inner, rows, x_inner * 2, 64, kQ, true)))
+    } else if (!make_tensor_map_cols64(&mapX, a.x, x_inner, rows, x_inner * 2, kQ, 2) ||
+               !make_tensor_map_cols64(&mapB, a.B, bc_inner, rows, bc_inner * 2, kQ, 2) ||
+               !make_tensor_map_cols64(&mapC, a.C, bc_inner, rows, bc_inner * 2, kQ, 2) ||
+               !make_tensor_map_cols64(&mapY, a.y ? a.y : a.x, x_inner, rows, x_inner * 2, kQ, 2)) {
         return cudaErrorInvalidValue;
-    if (!a.y) mapY = mapX;   // never used by the kernel then
+    }
     cudaError_t e = cudaFuncSetAttribute(ssd_scan_tensor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
-    ssd_scan_tensor_kernel<<<dim3(a.H, a.n_seq), kThreads, kSmemBytes, s>>>(a, mapX, mapB, mapC, mapY);
+    const int pairs = (a.H / a.G + 1) / 2;
+    ssd_scan_tensor_kernel<<<dim3(a.G * pairs, a.n_seq), kThreads, kSmemBytes, s>>>(a, mapX, mapB, mapC, mapY);
     return cudaGetLastError();
 }
 

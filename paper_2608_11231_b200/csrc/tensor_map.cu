@@ -38,4 +38,18 @@ bool make_tensor_map_2d(CUtensorMap *map, const void *base, int elem_bytes, uint
     return r == CUDA_SUCCESS;
 }
 
+bool make_tensor_map_cols64(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, uint64_t row_stride_bytes,
+                            uint32_t box_rows, uint32_t box_blocks) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t gdim[3] = {64, rows, inner / 64};
+    const cuuint64_t gstride[2] = {row_stride_bytes, 128};
+    const cuuint32_t box[3] = {64, box_rows, box_blocks};
+    const cuuint32_t estride[3] = {1, 1, 1};
+    const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), gdim, gstride, box, estride,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS;
+}
+
 }  // namespace lkv

@@ -1,0 +1,57 @@
+"""Mamba-2 scan at the edges of its blocks: lengths around the 64- and 128-token tiles, groups with an odd number of heads,
+decays that end blocks early in one head of a pair, and one sequence long enough to be scanned in segments."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import TOL_BF16, dev, host, maxrel_per_head
+from paper_2608_11231_b200 import binding as b
+from paper_2608_11231_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H, G, lens, decay", [
+    (3, 1, [1, 63, 64, 65, 127, 128, 129, 255, 257], 1.0),       # odd head count, every remainder that matters
+    (6, 2, [200, 128, 640], 1.0),                                # odd heads per group: pairs do not straddle groups
+    (4, 1, [700, 130], np.array([0.05, 20.0, 1.0, 200.0])),      # mild and violent heads in one CTA: blocks end early
+    (80, 1, [300], 0.02),                                        # benchmark shape, weak decay
+    (4, 1, [3333], 0.3),                                         # one long sequence: segments
+])
+@pytest.mark.parametrize("outputs", [True, False])
+def test_ssd_scan_block_edges(H, G, lens, decay, outputs):
+    import torch
+    rng = np.random.default_rng(H * 1000 + lens[0])
+    P, N = 64, 128
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    A = (wl.ssd_A(rng, H) * decay).astype(np.float32)
+    tok = wl.ssd_tokens(rng, int(cu[-1]), H, P, N, G)
+    S0 = rng.standard_normal((len(lens), H, N, P)).astype(np.float32)
+    bf = torch.bfloat16
+    y, ST = b.lkv_ssd_fwd(dev(tok["x"], bf), dev(tok["dt"]), dev(A), dev(tok["B"], bf), dev(tok["C"], bf), dev(S0),
+                          cu_seqlens=cu if len(lens) > 1 else None, want_outputs=outputs)
+    y = host(y) if outputs else None
+    ST = host(ST)
+    for s in range(len(lens)):
+        sl = slice(cu[s], cu[s + 1])
+        y_ref, ST_ref = oracle.ssd_seq(tok["x"][sl], tok["dt"][sl], A, tok["B"][sl], tok["C"][sl], S0[s])
+        assert maxrel_per_head(ST[s], ST_ref, 0) <= TOL_BF16
+        if outputs:
+            assert maxrel_per_head(y[sl], y_ref, 1) <= TOL_BF16
+
+
+def test_ssd_scan_results_repeat_on_a_full_gpu():
+    """Every SM busy, loads from DRAM: the same inputs give the same bits (a tile released before it is read does not)."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rn = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    H, n, L = 80, 16, 2000
+    T = n * L
+    bf = torch.bfloat16
+    args = (rn(T, H, 64).to(bf), torch.nn.functional.softplus(-2.0 + 0.5 * rn(T, H)), -torch.exp(2.0 * torch.rand(H, generator=gen, device="cuda")),
+            (rn(T, 1, 128) / 128 ** 0.5).to(bf), (rn(T, 1, 128) / 128 ** 0.5).to(bf))
+    cu = (np.arange(n + 1) * L).astype(np.int32)
+    y0, S0 = b.lkv_ssd_fwd(*args, cu_seqlens=cu)
+    for _ in range(10):
+        y, S = b.lkv_ssd_fwd(*args, cu_seqlens=cu)
+        assert torch.equal(y, y0) and torch.equal(S, S0)
