@@ -80,6 +80,11 @@ struct GdnArgs {
     // (the ranges of sequences 0 .. tr_first-1); a plain call has n_ranges = tr_first = n_seq.
     int32_t n_ranges, tr_first, tr_src0;
     float *tr_out;               // where transition sequence tr_first + i stores its final state (index i), or nullptr: S_T like the others
+    // One sequence cut into segments that run side by side (tensor-core scan only).  Sequences n_s0 .. start from S0_more (index
+    // seq - n_s0; nullptr = zero), final states are wanted of sequences st_first .. only (index seq - st_first).  A plain call
+    // has n_s0 = n_seq, st_first = 0.
+    int32_t n_s0, st_first;
+    const float *S0_more;
     int32_t *status;
     IndexBlock<kScanIdxCap> cu;  // cu_seqlens[n_seq + 1], then the launch order: sequence of grid row y at [n_seq + 1 + y]
 };

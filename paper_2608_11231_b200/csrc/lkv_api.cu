@@ -325,6 +325,7 @@ static int gdn_impl(const void *q, const void *k, const void *v, const float *g,
     a.scale = d->scale != 0.f ? d->scale : 1.0f / sqrtf(static_cast<float>(d->d_k));
     a.s0_identity = transition ? 1 : 0;
     a.n_ranges = n_ranges; a.tr_first = n_ranges; a.tr_src0 = what == 3 ? 1 : 0; a.tr_out = tr_out;
+    a.n_s0 = d->n_seq; a.st_first = 0; a.S0_more = nullptr;
     a.status = static_cast<int32_t *>(d->workspace);
     const bool io_bf16 = d->io_dtype == LKV_DTYPE_BF16;
     const bool tensor_fits = gdn_scan_tensor_supported(a, io_bf16);

@@ -74,8 +74,8 @@ constexpr int kSmemBytes = kOffSlot + kSlots * static_cast<int>(sizeof(Slot)) + 
 static_assert(kSmemBytes + 512 <= 227 * 1024, "shared memory budget");
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kMaxRange = 200.f;               // log2 units of decay inside one block
-constexpr float kMaxScale = 104.f;               // 2^R - l_n at most: X^ and S^ grow to about 2^104 ...
-constexpr float kNewScale = 96.f;                // ... and a state that is scaled back starts from 2^-96 (104 + 96 = kMaxRange)
+constexpr float kMaxScale = 104.f;               // R - l_n at most: X^ and S^ grow to about 2^104.  A state that is scaled back starts
+                                                 // from R = 0, or from below (to -96) where the block's own decay leaves no other choice
 
 // tensor-memory map (columns)
 constexpr uint32_t kTmS = 0;        // 128: S^^T fp32
@@ -122,15 +122,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t *>(&v);
 }
 __device__ __forceinline__ float2 f2(uint32_t x, uint32_t y) { return make_float2(__uint_as_float(x), __uint_as_float(y)); }
-// every lane takes the same decision although `dead` may change under the read
-__device__ __forceinline__ bool warp_dead(volatile int *dead) { return __any_sync(0xffffffffu, *dead != 0); }
 
-// One arrival for the whole warp, after every lane's work before it: an mbarrier takes the arrivals of the lanes of one
-// instruction one by one, each a turn at the shared-memory port (1700 a block where every thread arrives for itself).
-__device__ __forceinline__ void warp_arrive(uint64_t *bar) {
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
-}
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -265,7 +257,7 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
             }
             const float ln = __shfl_sync(0xffffffffu, l2[7], 15, 16);   // tokens beyond the block have dt = 0
             float Rn = R;
-            if (fabsf(R - ln) > kMaxScale) Rn = ln < 0.f ? -kNewScale : kNewScale;
+            if (fabsf(R - ln) > kMaxScale) Rn = ln < 0.f ? fminf(0.f, floorf(kMaxScale + ln)) : fmaxf(0.f, ceilf(ln - kMaxScale));
             if (fabsf(ln) > kMaxRange) Rn = rintf(ln);   // a single token of violent decay: nothing of the state is left
             const int start = t0;
             t0 += n;

@@ -33,6 +33,12 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// One arrival for the whole warp, after every lane's work before it: an mbarrier takes the arrivals of the lanes of one
+// instruction one by one, each a turn at the shared-memory port.
+__device__ __forceinline__ void warp_arrive(uint64_t *bar) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -87,6 +93,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     if (mbar_try_wait(bar, parity)) return true;
     return mbar_wait_slow(smem_u32(bar), parity, dead, status, limit);
 }
+
+// Has a wait run out?  Every lane takes the same decision although `dead` may change under the read
+__device__ __forceinline__ bool warp_dead(volatile int *dead) { return __any_sync(0xffffffffu, *dead != 0); }
 
 // After a wait has run out the threads that issue tile loads stop issuing (they test the flag once per block; an MMA
 // issuer may run through its remaining blocks without waiting, its products read whatever the tiles hold).  This pause,
