@@ -32,7 +32,10 @@
  *     `stream` is capturing.
  *   - The caller owns every buffer.  The library allocates nothing, frees
  *     nothing and keeps no pointer after a call returns; scratch lives in a
- *     caller-provided workspace whose size lkv_workspace_bytes() reports.
+ *     caller-provided workspace whose size lkv_workspace_bytes() reports.  For
+ *     a scan of one long sequence that size includes room for the states of
+ *     the segments it is cut into when SMs would be idle; with a smaller
+ *     workspace such a call runs as one piece.
  *     A workspace must not be shared by calls that can overlap on the GPU.
  *   - Calls are asynchronous on `stream` (a cudaStream_t passed as void*,
  *     NULL = the legacy default stream).  They do not synchronise.

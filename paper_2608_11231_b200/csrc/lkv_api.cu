@@ -247,6 +247,81 @@ int ssd_segmented(SsdArgs a, int segs, char *scratch, cudaStream_t s) {
     return launch_ssd_scan_tensor(p3, s) == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
 }
 
+// The same for the GDN scan (one head per CTA), where the first pass also computes the transitions of the segments between the
+// first and the last: n segments are (2 n - 3) H_v CTAs there and n H_v in the last pass.  Two ways to stay within one round
+// of CTAs: n equal segments, or one of the segments with a transition half as long as the others, so that its two CTAs of a
+// head follow one another on one SM (n - 1/2 segments' worth of tokens; at H_v = 32 on 148 SMs n = 4, against 3 equal ones).
+// Both passes take as long as the longest segment; the composition, the launches and the fill of another pipeline cost about
+// 14 blocks of 64 tokens.
+struct GdnCut {
+    int n, full;   // segments, tokens of a full one; segment n - 2 may be shorter
+};
+GdnCut gdn_cut(const lkv_gdn_desc *d, int n_seq) {
+    const GdnCut whole{1, 0};
+    if (n_seq != 1 || d->io_dtype != LKV_DTYPE_BF16 || d->compute == LKV_COMPUTE_FP32 || d->H_v < 1 || d->d_k != 128 || d->d_v != 128 || d->T_total < 1024)
+        return whole;
+    const int slots = sm_count() / d->H_v;
+    const int equal = std::min((slots + 3) / 2, slots), halved = std::min((slots + 4) / 2, slots);
+    const int blocks = (d->T_total + 63) / 64;
+    GdnCut c = whole;
+    int longest;   // blocks of a full segment
+    if (halved > equal && halved >= 3) {
+        longest = (2 * blocks + 2 * halved - 2) / (2 * halved - 1);
+        c.n = halved;
+    } else {
+        longest = equal > 0 ? (blocks + equal - 1) / equal : blocks;
+        c.n = equal;
+    }
+    c.n = std::min(c.n, 16);
+    c.full = 64 * longest;
+    return c.n >= 3 && blocks - 2 * longest > 14 && static_cast<long long>(c.full) * c.n < d->T_total + 2ll * c.full ? c : whole;
+}
+// local states and transitions of all segments but the last, initial states of all but the first
+size_t gdn_segment_scratch(const lkv_gdn_desc *d, GdnCut c) {
+    if (c.n < 2) return 0;
+    return 3 * static_cast<size_t>(c.n - 1) * sizeof(float) * d->H_v * d->d_k * d->d_v;
+}
+int gdn_segmented(GdnArgs a, GdnCut c, char *scratch, cudaStream_t s) {
+    const int n = c.n, m = n - 1;
+    const size_t slot = static_cast<size_t>(a.H_v) * a.d_k * a.d_v;
+    float *local = reinterpret_cast<float *>(scratch), *trans = local + m * slot, *init = trans + m * slot;
+    // whole blocks; the last segment is full, the one before it takes what is left
+    int at[17];
+    for (int i = 0; i < n - 2; ++i) at[i] = i * c.full;
+    at[n - 2] = (n - 2) * c.full;
+    at[n] = a.T_total;
+    at[n - 1] = std::max(at[n - 2], (a.T_total - c.full + 63) / 64 * 64);
+    auto ranges = [&](GdnArgs &b, int k, int n_tr) {
+        b.cu.ptr = nullptr;
+        b.n_ranges = b.tr_first = k;
+        b.n_seq = k + n_tr;
+        for (int i = 0; i <= k; ++i) b.cu.v[i] = at[i];
+        auto len = [&](int sq) { const int r = sq < k ? sq : sq - k + b.tr_src0; return at[r + 1] - at[r]; };
+        int32_t *order = b.cu.v + k + 1;
+        for (int i = 0; i < b.n_seq; ++i) order[i] = i;
+        std::stable_sort(order, order + b.n_seq, [&](int32_t x, int32_t y) { return len(x) > len(y); });
+    };
+    GdnArgs p1 = a;
+    p1.tr_src0 = 1;
+    ranges(p1, m, m - 1);
+    p1.o = nullptr; p1.S_T = local; p1.st_bf16 = 0; p1.n_s0 = 1; p1.tr_out = trans + slot;   // transition of segment j at trans + j slots
+    if (launch_gdn_scan_tensor(p1, s) != cudaSuccess) return LKV_ERR_CUDA;
+    InitArgs k;
+    k.states = local; k.transitions = trans; k.S0 = init; k.n_req = m; k.H = a.H_v; k.d_k = a.d_k; k.d_v = a.d_v; k.n_chunks = m;
+    k.off_sel = -1; k.off_ids = n; k.status = a.status; k.idx.ptr = nullptr;
+    int ids = n;
+    for (int r = 0; r < m; ++r) {
+        k.idx.v[r] = ids - n;
+        for (int j = 0; j <= r; ++j) k.idx.v[ids++] = j;
+    }
+    k.idx.v[m] = ids - n;
+    if (launch_init_gdn_exact_tensor(k, false, s) != cudaSuccess) return LKV_ERR_CUDA;
+    GdnArgs p3 = a;
+    ranges(p3, n, 0);
+    p3.n_s0 = 1; p3.S0_more = init; p3.st_first = n - 1;
+    return launch_gdn_scan_tensor(p3, s) == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
+}
+
 }  // namespace
 
 extern "C" {
@@ -342,6 +417,12 @@ static int gdn_impl(const void *q, const void *k, const void *v, const float *g,
         use_tensor = tensor_fits;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // A long sequence that leaves SMs idle runs in segments (a caller whose workspace is smaller than
+    // lkv_workspace_bytes() asked for gets the plain scan; S_T on top of S0 would be written while S0 is read)
+    const GdnCut cut = use_tensor && what == 0 && S_T != S0 && o ? gdn_cut(d, d->n_seq) : GdnCut{1, 0};
+    const size_t head = ws_bytes_for(2 * d->n_seq + 1, kScanIdxCap);
+    if (cut.n > 1 && d->workspace_bytes >= head + gdn_segment_scratch(d, cut))
+        return gdn_segmented(a, cut, static_cast<char *>(d->workspace) + head, s);
     if (what >= 3) {
         // launch order over all sequences, longest first; transition sequence j runs over range j - m + (1 or 0)
         std::vector<int32_t> order(d->n_seq);
@@ -667,7 +748,10 @@ size_t lkv_workspace_bytes(int which, const void *desc, int n_units, int n_index
     if (!desc || n_units < 0 || n_index < 0) return 0;
     switch (which) {
         case LKV_WS_INIT: return ws_bytes_for(2 * n_units + 1 + n_index, kInitIdxCap);
-        case LKV_WS_GDN: return ws_bytes_for(2 * n_units + 1, kScanIdxCap);
+        case LKV_WS_GDN: {
+            const lkv_gdn_desc *d = static_cast<const lkv_gdn_desc *>(desc);
+            return ws_bytes_for(2 * n_units + 1, kScanIdxCap) + gdn_segment_scratch(d, gdn_cut(d, n_units));
+        }
         case LKV_WS_SSD: {
             const lkv_ssd_desc *d = static_cast<const lkv_ssd_desc *>(desc);
             return ws_bytes_for(2 * n_units + 1, kScanIdxCap) + ssd_segment_scratch(d, ssd_segments(d, n_units));
