@@ -64,6 +64,8 @@ struct InitArgs {
     __device__ __forceinline__ int sel(int r, int K) const { return off_sel < 0 ? K - 1 : idx[off_sel + r]; }
 };
 
+int sm_count();   // of the current device
+
 struct GdnArgs {
     const void *q, *k, *v;
     const float *g, *beta, *S0;

@@ -2,6 +2,8 @@
 // (Eq. 6 as the chain of Eq. 5) for Mamba-2 (scalar decay, HBM-bound) and for GDN in
 // plain fp32 FMA (the tight-tolerance / small-shape path; the tensor-core path for
 // d_k = d_v = 128 lives in init_gdn_tensor.cu).
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace lkv {
@@ -106,27 +108,31 @@ __global__ void __launch_bounds__(256) init_mamba_exact_kernel(const __grid_cons
 }
 
 // ---------------------------------------------------------------- GDN exact composition, fp32 FMA
-// One CTA owns kTN columns of one head's state for one request: the chain
+// One CTA owns TN columns of one head's state for one request: the chain
 // S <- T_{c_j} S + S_{c_j} acts on the left, so columns never mix.  The current column
-// block sits in shared memory; T_j streams through shared memory kTM rows at a time.
-constexpr int kTN = 32;  // state columns per CTA
-constexpr int kTM = 32;  // transition rows staged per step
+// block sits in shared memory; T_j streams through a ring in shared memory kTM rows at a time, copied asynchronously several
+// tiles ahead (a step waited for global memory twice before;
+// the measured figures stand at the scan, gdn_scan_fp32.cu).
+constexpr int kTM = 32;        // transition rows per stage
+constexpr int kMaxStages = 6;
+// row stride (floats) of a staged transition: 16-byte rows, successive rows four banks apart
+__host__ __device__ constexpr int t_stride(int dk) { return (((dk + 3) / 4) | 1) * 4; }
 
-template <bool BF16>
-__global__ void __launch_bounds__(256) init_gdn_exact_fp32_kernel(const __grid_constant__ InitArgs a) {
-    extern __shared__ float smem[];
-    const int dk = a.d_k, dv = a.d_v;
-    float *Scur = smem;                 // [dk][kTN]
-    float *Snew = Scur + dk * kTN;      // [dk][kTN]
-    float *Tt = Snew + dk * kTN;        // [kTM][dk + 1]
-    const int tstride = dk + 1;
-    const int col0 = blockIdx.x * kTN;
+template <bool BF16, int TN>
+__global__ void __launch_bounds__(256) init_gdn_exact_fp32_kernel(const __grid_constant__ InitArgs a, int stages) {
+    constexpr int RG = 256 / TN, U = kTM / RG;   // thread (rg, c) has rows rg, rg + RG, ... of column c
+    extern __shared__ __align__(16) float smem[];
+    const int dk = a.d_k, dv = a.d_v, ts = t_stride(dk);
+    float *Tt = smem;                           // stages x [kTM][ts]
+    float *Scur = Tt + stages * kTM * ts;       // [dk][TN]
+    float *Snew = Scur + dk * TN;               // [dk][TN]
+    const int col0 = blockIdx.x * TN;
     const int h = blockIdx.y, r = blockIdx.z;
     const int k0 = a.cu_k(r), K = a.cu_k(r + 1) - k0;
     const size_t ss = static_cast<size_t>(dk) * dv;
-    const int tid = threadIdx.x;
-    const int c = tid % kTN;   // column inside the block
-    const int rg = tid / kTN;  // row group 0..7
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c = tid % TN;    // column inside the block
+    const int rg = tid / TN;   // row group
     const bool col_ok = col0 + c < dv;
 
     auto load_state = [&](int chunk, int i) -> float {
@@ -135,39 +141,88 @@ __global__ void __launch_bounds__(256) init_gdn_exact_fp32_kernel(const __grid_c
         if (BF16) return __bfloat162float(static_cast<const __nv_bfloat16 *>(a.states)[off]);
         return static_cast<const float *>(a.states)[off];
     };
-
-    for (int i = rg; i < dk; i += 8) Scur[i * kTN + c] = (K > 0) ? load_state(a.id(k0), i) : 0.f;
-    __syncthreads();
-    for (int j = 1; j < K; ++j) {
-        const int chunk = a.id(k0 + j);
-        const float *Tj = a.transitions + (static_cast<size_t>(chunk) * a.H + h) * dk * dk;
-        for (int i0 = 0; i0 < dk; i0 += kTM) {
-            for (int idx = tid; idx < kTM * dk; idx += 256) {
-                const int ii = idx / dk, m = idx % dk;
-                Tt[ii * tstride + m] = (i0 + ii < dk) ? __ldg(Tj + static_cast<size_t>(i0 + ii) * dk + m) : 0.f;
+    // tile x of the sequence of all transitions, kTM rows each, into its stage: one asynchronous copy group per tile
+    const int tiles = (dk + kTM - 1) / kTM, total = (K > 1 ? K - 1 : 0) * tiles;
+    const bool vec = dk % 4 == 0;
+    auto fetch = [&](int x) {
+        if (x < total) {
+            const int i0 = (x % tiles) * kTM;
+            const float *Tj = a.transitions + (static_cast<size_t>(a.id(k0 + 1 + x / tiles)) * a.H + h) * dk * dk;
+            float *st = Tt + (x % stages) * kTM * ts;
+            for (int ii = warp; ii < kTM && i0 + ii < dk; ii += 8) {
+                const float *src = Tj + static_cast<size_t>(i0 + ii) * dk;
+                const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(st + ii * ts));
+                if (vec)
+                    for (int m = 4 * lane; m < dk; m += 128) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 4 * m), "l"(src + m) : "memory");
+                else
+                    for (int m = lane; m < dk; m += 32) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4 * m), "l"(src + m) : "memory");
             }
-            __syncthreads();
-            // thread (rg, c) produces rows i0 + rg, i0 + rg + 8, ... of column c
-            float acc[kTM / 8];
-#pragma unroll
-            for (int u = 0; u < kTM / 8; ++u) acc[u] = 0.f;
-            for (int m = 0; m < dk; ++m) {
-                const float s = Scur[m * kTN + c];
-#pragma unroll
-                for (int u = 0; u < kTM / 8; ++u) acc[u] = fmaf(Tt[(rg + 8 * u) * tstride + m], s, acc[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < kTM / 8; ++u) {
-                const int i = i0 + rg + 8 * u;
-                if (i < dk) Snew[i * kTN + c] = acc[u] + load_state(chunk, i);
-            }
-            __syncthreads();
         }
-        float *t = Scur; Scur = Snew; Snew = t;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int x = 0; x < stages - 1; ++x) fetch(x);
+#pragma unroll 4
+    for (int i = rg; i < dk; i += RG) Scur[i * TN + c] = (K > 0) ? load_state(a.id(k0), i) : 0.f;
+    for (int x = 0; x < total; ++x) {
+        const int i0 = (x % tiles) * kTM, chunk = a.id(k0 + 1 + x / tiles);
+        float acc[U], add[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {   // in flight while the tile is waited for
+            const int i = i0 + rg + RG * u;
+            add[u] = i < dk ? load_state(chunk, i) : 0.f;
+            acc[u] = 0.f;
+        }
+        if (stages > 1) fetch(x + stages - 1);   // into the stage that every thread left at the end of the last round
+        else fetch(x);
+        switch (stages) {
+            case 1: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
+            case 2: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
+            case 3: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
+            case 4: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+            case 5: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+            default: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
+        }
+        __syncthreads();
+        const float *st = Tt + (x % stages) * kTM * ts;
+        const int dk4 = dk & ~3;
+        for (int m = 0; m < dk4; m += 4) {
+            float s[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[e] = Scur[(m + e) * TN + c];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const float4 t = *reinterpret_cast<const float4 *>(st + (rg + RG * u) * ts + m);
+                acc[u] = fmaf(t.x, s[0], acc[u]); acc[u] = fmaf(t.y, s[1], acc[u]);
+                acc[u] = fmaf(t.z, s[2], acc[u]); acc[u] = fmaf(t.w, s[3], acc[u]);
+            }
+        }
+        for (int m = dk4; m < dk; ++m)
+#pragma unroll
+            for (int u = 0; u < U; ++u) acc[u] = fmaf(st[(rg + RG * u) * ts + m], Scur[m * TN + c], acc[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + rg + RG * u;
+            if (i < dk) Snew[i * TN + c] = acc[u] + add[u];
+        }
+        __syncthreads();
+        if (x % tiles == tiles - 1) { float *t = Scur; Scur = Snew; Snew = t; }
     }
+    if (total == 0) __syncthreads();
     if (col_ok)
-        for (int i = rg; i < dk; i += 8)
-            a.S0[(static_cast<size_t>(r) * a.H + h) * ss + static_cast<size_t>(i) * dv + col0 + c] = Scur[i * kTN + c];
+#pragma unroll 4
+        for (int i = rg; i < dk; i += RG)
+            a.S0[(static_cast<size_t>(r) * a.H + h) * ss + static_cast<size_t>(i) * dv + col0 + c] = Scur[i * TN + c];
+}
+
+template <bool BF16, int TN>
+cudaError_t launch_gdn_fp32(const InitArgs &a, cudaStream_t s) {
+    const size_t state = 2 * static_cast<size_t>(a.d_k) * TN * sizeof(float), stage = static_cast<size_t>(kTM) * t_stride(a.d_k) * sizeof(float);
+    const int stages = static_cast<int>(std::min<size_t>(kMaxStages, (227 * 1024 - state) / stage));
+    const size_t smem = state + stages * stage;
+    const cudaError_t e = cudaFuncSetAttribute(init_gdn_exact_fp32_kernel<BF16, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    init_gdn_exact_fp32_kernel<BF16, TN><<<dim3((a.d_v + TN - 1) / TN, a.H, a.n_req), 256, smem, s>>>(a, stages);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -190,20 +245,13 @@ cudaError_t launch_init_mamba_exact(const InitArgs &a, bool pool_bf16, cudaStrea
     return cudaGetLastError();
 }
 
+// 32 columns of the state per CTA, or 8 where that many CTAs still find an SM each (a step is then a quarter of the work: what
+// a small call waits for); 8 also where the rows are so long that two copies of 32 columns leave no room for a stage.
 cudaError_t launch_init_gdn_exact_fp32(const InitArgs &a, bool pool_bf16, cudaStream_t s) {
-    const size_t smem = (static_cast<size_t>(2) * a.d_k * kTN + static_cast<size_t>(kTM) * (a.d_k + 1)) * sizeof(float);
-    dim3 grid((a.d_v + kTN - 1) / kTN, a.H, a.n_req);
-    cudaError_t e;
-    if (pool_bf16) {
-        e = cudaFuncSetAttribute(init_gdn_exact_fp32_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        init_gdn_exact_fp32_kernel<true><<<grid, 256, smem, s>>>(a);
-    } else {
-        e = cudaFuncSetAttribute(init_gdn_exact_fp32_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        init_gdn_exact_fp32_kernel<false><<<grid, 256, smem, s>>>(a);
-    }
-    return cudaGetLastError();
+    const long long narrow = static_cast<long long>((a.d_v + 7) / 8) * a.H * a.n_req;
+    const bool wide_fits = (2 * static_cast<size_t>(a.d_k) * 32 + kTM * static_cast<size_t>(t_stride(a.d_k))) * sizeof(float) <= 227 * 1024;
+    if (narrow <= sm_count() || !wide_fits) return pool_bf16 ? launch_gdn_fp32<true, 8>(a, s) : launch_gdn_fp32<false, 8>(a, s);
+    return pool_bf16 ? launch_gdn_fp32<true, 32>(a, s) : launch_gdn_fp32<false, 32>(a, s);
 }
 
 namespace {

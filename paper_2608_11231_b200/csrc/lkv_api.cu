@@ -9,6 +9,24 @@
 
 using namespace lkv;
 
+int lkv::sm_count() {
+    static int cached[64];   // per device; the same value whoever writes it
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        cudaGetLastError();
+        return 148;
+    }
+    n = __atomic_load_n(&cached[dev], __ATOMIC_RELAXED);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            n = 148;
+        }
+        __atomic_store_n(&cached[dev], n, __ATOMIC_RELAXED);
+    }
+    return n;
+}
+
 namespace {
 
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -179,24 +197,6 @@ void append_launch_order(std::vector<int32_t> &cu, int n_seq) {
     std::stable_sort(order.begin(), order.end(),
                      [&](int32_t x, int32_t y) { return cu[x + 1] - cu[x] > cu[y + 1] - cu[y]; });
     cu.insert(cu.end(), order.begin(), order.end());
-}
-
-int sm_count() {
-    static int cached[64];   // per device; the same value whoever writes it
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
-        cudaGetLastError();
-        return 148;
-    }
-    n = __atomic_load_n(&cached[dev], __ATOMIC_RELAXED);
-    if (n == 0) {
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-            cudaGetLastError();
-            n = 148;
-        }
-        __atomic_store_n(&cached[dev], n, __ATOMIC_RELAXED);
-    }
-    return n;
 }
 
 // A single sequence fills (heads / 2) of the SMs (two heads per CTA) and is a chain of blocks.  Cut into segments, it runs as
