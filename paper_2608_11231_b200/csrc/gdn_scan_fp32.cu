@@ -14,7 +14,7 @@
 // A small call is one CTA per head and a chain of blocks: what counts is the time of one block, and there the reads of shared
 // memory (one per FMA in the direct form).  So the products work on register tiles (2 x 2 tokens, four tokens or rows per
 // value read) with 16-byte reads along the contraction, the running sum is a warp scan, and the substitution hands u_i round
-// by shuffles instead of leaving 31 dependent sums to one thread.Measured on B200 with two heads of
+// by shuffles instead of leaving 31 dependent sums to one thread.  Measured on B200 with two heads of
 // 64 x 64: the composition of four chunks and a scan of 64 tokens, 69.7 -> 28.7 us for the two calls (register tiles and four
 // times the CTAs).
 #include "common.cuh"
@@ -47,6 +47,8 @@ __global__ void __launch_bounds__(256) gdn_scan_fp32_kernel(const __grid_constan
     float *ec = bs + kC;                   // [kC]   e^{cg_C - cg_i}
     float *S = ec + kC;                    // [dk][VC]
     float *Us = S + dk * VC;               // [kC][kLdU]   right-hand side, then u
+    pdl_launch();
+    pdl_wait();
 
     const int h = blockIdx.x, seq = a.cu[a.n_ranges + 1 + blockIdx.y];   // launch order: longest sequence first
     const bool tr = seq >= a.tr_first;                                    // transition sequence
@@ -265,8 +267,7 @@ cudaError_t launch(const GdnArgs &a, cudaStream_t s) {
     const size_t smem = smem_bytes(a.d_k, VC);
     cudaError_t e = cudaFuncSetAttribute(gdn_scan_fp32_kernel<T, VC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    gdn_scan_fp32_kernel<T, VC><<<dim3(a.H_v, a.n_seq, a.d_v / VC), 256, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(gdn_scan_fp32_kernel<T, VC>, dim3(a.H_v, a.n_seq, a.d_v / VC), 256, smem, s, a);
 }
 
 // Columns per CTA: all of them when heads and sequences fill the GPU; otherwise halved as long as that still finds idle SMs.

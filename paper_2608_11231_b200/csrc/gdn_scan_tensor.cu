@@ -346,6 +346,8 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
     __shared__ volatile int dead;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_launch();
+    if (a.cu.ptr) pdl_wait();   // the index list is in global memory
     const int h = blockIdx.x, seq = a.cu[a.n_ranges + 1 + blockIdx.y];   // launch order: longest sequence first
     const bool tr = seq >= a.tr_first;                                    // transition sequence
     const int rg = tr ? seq - a.tr_first + a.tr_src0 : seq;
@@ -368,6 +370,7 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
     const bool has_v = a.v != nullptr && !tr, has_o = a.o != nullptr && !tr;
 
     if (nblk == 0) {  // empty sequence: hand the state through untouched
+        pdl_wait();
         const float *S0 = initial_state();
         size_t obase;
         float *ST = final_state(obase);
@@ -389,6 +392,7 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
         mbar_fence_init();
     }
     if (warp == 0) tmem_alloc(&tmem_base, kTmemCols);
+    pdl_wait();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -1067,8 +1071,7 @@ cudaError_t launch_gdn_scan_tensor(const GdnArgs &a, cudaStream_t s) {
     if (!a.o) mapO = mapK;
     cudaError_t e = cudaFuncSetAttribute(gdn_scan_tensor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
-    gdn_scan_tensor_kernel<<<dim3(a.H_v, a.n_seq), kThreads, kSmemBytes, s>>>(a, mapQ, mapK, mapV, mapO);
-    return cudaGetLastError();
+    return launch_chained(gdn_scan_tensor_kernel, dim3(a.H_v, a.n_seq), kThreads, kSmemBytes, s, a, mapQ, mapK, mapV, mapO);
 }
 
 }  // namespace lkv

@@ -75,11 +75,14 @@ init_gdn_exact_tensor_kernel(const __grid_constant__ InitArgs a, const __grid_co
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int h = blockIdx.x, r = blockIdx.y;
+    pdl_launch();
+    if (a.idx.ptr) pdl_wait();   // the index list is in global memory
     const int k0 = a.cu_k(r), K = a.cu_k(r + 1) - k0;
     constexpr size_t ss = static_cast<size_t>(kD) * kD;
     float *out = a.S0 + (static_cast<size_t>(r) * a.H + h) * ss;
 
     if (K == 0) {  // empty request: zero state
+        pdl_wait();
         for (int e = tid * 4; e < kD * kD; e += kThreads * 4) *reinterpret_cast<float4 *>(out + e) = make_float4(0.f, 0.f, 0.f, 0.f);
         return;
     }
@@ -91,6 +94,7 @@ init_gdn_exact_tensor_kernel(const __grid_constant__ InitArgs a, const __grid_co
     }
     constexpr int kMmaWarp = (kEpiThreads + kRoundThreads) / 32, kTmaWarp = kMmaWarp + 1;
     if (warp == kMmaWarp) tmem_alloc(&tmem_base, kTmemCols);
+    pdl_wait();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -245,13 +249,12 @@ cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cuda
     if (pool_bf16) {
         e = cudaFuncSetAttribute(init_gdn_exact_tensor_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         if (e != cudaSuccess) return e;
-        init_gdn_exact_tensor_kernel<true><<<dim3(a.H, a.n_req), kThreads, kSmemBytes, s>>>(a, mapT);
+        return launch_chained(init_gdn_exact_tensor_kernel<true>, dim3(a.H, a.n_req), kThreads, kSmemBytes, s, a, mapT);
     } else {
         e = cudaFuncSetAttribute(init_gdn_exact_tensor_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         if (e != cudaSuccess) return e;
-        init_gdn_exact_tensor_kernel<false><<<dim3(a.H, a.n_req), kThreads, kSmemBytes, s>>>(a, mapT);
+        return launch_chained(init_gdn_exact_tensor_kernel<false>, dim3(a.H, a.n_req), kThreads, kSmemBytes, s, a, mapT);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace lkv

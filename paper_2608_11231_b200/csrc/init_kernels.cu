@@ -47,6 +47,8 @@ __device__ __forceinline__ void store_vec(float *dst, const float (&v)[E]) {
 template <bool BF16>
 __global__ void __launch_bounds__(256) init_single_kernel(const __grid_constant__ InitArgs a, size_t state_elems) {
     using PV = PoolVec<BF16>;
+    pdl_launch();
+    pdl_wait();
     const int r = blockIdx.y;
     const int k0 = a.cu_k(r), k1 = a.cu_k(r + 1);
     const size_t e = (static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x) * PV::kElems;
@@ -72,6 +74,8 @@ __global__ void __launch_bounds__(256) init_mamba_exact_kernel(const __grid_cons
     using PV = PoolVec<BF16>;
     constexpr int E = PV::kElems;
     constexpr int kUnroll = 8;
+    pdl_launch();
+    pdl_wait();
     const int r = blockIdx.y;
     const int k0 = a.cu_k(r), K = a.cu_k(r + 1) - k0;
     const size_t e = (static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x) * E;
@@ -128,6 +132,8 @@ __global__ void __launch_bounds__(256) init_gdn_exact_fp32_kernel(const __grid_c
     float *Snew = Scur + dk * TN;               // [dk][TN]
     const int col0 = blockIdx.x * TN;
     const int h = blockIdx.y, r = blockIdx.z;
+    pdl_launch();
+    pdl_wait();
     const int k0 = a.cu_k(r), K = a.cu_k(r + 1) - k0;
     const size_t ss = static_cast<size_t>(dk) * dv;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -221,8 +227,7 @@ cudaError_t launch_gdn_fp32(const InitArgs &a, cudaStream_t s) {
     const size_t smem = state + stages * stage;
     const cudaError_t e = cudaFuncSetAttribute(init_gdn_exact_fp32_kernel<BF16, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    init_gdn_exact_fp32_kernel<BF16, TN><<<dim3((a.d_v + TN - 1) / TN, a.H, a.n_req), 256, smem, s>>>(a, stages);
-    return cudaGetLastError();
+    return launch_chained(init_gdn_exact_fp32_kernel<BF16, TN>, dim3((a.d_v + TN - 1) / TN, a.H, a.n_req), 256, smem, s, a, stages);
 }
 
 }  // namespace
@@ -231,18 +236,14 @@ cudaError_t launch_init_single(const InitArgs &a, bool pool_bf16, cudaStream_t s
     const size_t elems = static_cast<size_t>(a.H) * a.d_k * a.d_v;
     const int per = pool_bf16 ? 8 : 4;
     dim3 grid(static_cast<unsigned>((elems / per + 255) / 256), a.n_req);
-    if (pool_bf16) init_single_kernel<true><<<grid, 256, 0, s>>>(a, elems);
-    else init_single_kernel<false><<<grid, 256, 0, s>>>(a, elems);
-    return cudaGetLastError();
+    return launch_chained(pool_bf16 ? init_single_kernel<true> : init_single_kernel<false>, grid, 256, 0, s, a, elems);
 }
 
 cudaError_t launch_init_mamba_exact(const InitArgs &a, bool pool_bf16, cudaStream_t s) {
     const size_t elems = static_cast<size_t>(a.H) * a.d_k * a.d_v;
     const int per = pool_bf16 ? 8 : 4;
     dim3 grid(static_cast<unsigned>((elems / per + 255) / 256), a.n_req);
-    if (pool_bf16) init_mamba_exact_kernel<true><<<grid, 256, 0, s>>>(a, elems, a.d_k * a.d_v);
-    else init_mamba_exact_kernel<false><<<grid, 256, 0, s>>>(a, elems, a.d_k * a.d_v);
-    return cudaGetLastError();
+    return launch_chained(pool_bf16 ? init_mamba_exact_kernel<true> : init_mamba_exact_kernel<false>, grid, 256, 0, s, a, elems, a.d_k * a.d_v);
 }
 
 // 32 columns of the state per CTA, or 8 where that many CTAs still find an SM each (a step is then a quarter of the work: what
@@ -263,6 +264,8 @@ __global__ void mamba_logdecay_kernel(const __grid_constant__ SsdArgs a, float *
     const int h = blockIdx.x * 32 + (threadIdx.x & 31);
     const int part = threadIdx.x >> 5, nparts = blockDim.x >> 5;
     __shared__ float red[8][32];
+    pdl_launch();
+    pdl_wait();
     const int t0 = a.cu[seq], t1 = a.cu[seq + 1];
     float acc = 0.f;
     if (h < a.H)
@@ -279,8 +282,7 @@ __global__ void mamba_logdecay_kernel(const __grid_constant__ SsdArgs a, float *
 }  // namespace
 
 cudaError_t launch_mamba_logdecay(const SsdArgs &a, float *logdecay, cudaStream_t s) {
-    mamba_logdecay_kernel<<<dim3((a.H + 31) / 32, a.n_seq), 256, 0, s>>>(a, logdecay);
-    return cudaGetLastError();
+    return launch_chained(mamba_logdecay_kernel, dim3((a.H + 31) / 32, a.n_seq), 256, 0, s, a, logdecay);
 }
 
 namespace {

@@ -58,6 +58,8 @@ init_mamba_exact_stream_kernel(const __grid_constant__ InitArgs a, size_t state_
         }
         mbar_fence_init();
     }
+    pdl_launch();
+    pdl_wait();
     __syncthreads();
     const int n_units = a.n_req * tiles_per_state;
     const int pieces_per_state = static_cast<int>(state_elems / kPieceElems);
@@ -178,8 +180,7 @@ static cudaError_t launch_stream(const InitArgs &a, int sms, cudaStream_t s) {
     auto kern = init_mamba_exact_stream_kernel<BF16, PER>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kConsumers + 32, kSmemBytes, s>>>(a, elems, a.d_k * a.d_v, tiles);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, kConsumers + 32, kSmemBytes, s, a, elems, a.d_k * a.d_v, tiles);
 }
 
 cudaError_t launch_init_mamba_exact_stream(const InitArgs &a, bool pool_bf16, cudaStream_t s) {

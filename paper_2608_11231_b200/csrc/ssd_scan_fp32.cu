@@ -29,6 +29,8 @@ __global__ void __launch_bounds__(256) ssd_scan_fp32_kernel(const __grid_constan
     float *Gm = Xs + kQ * P;          // [kQ][kQ+1]
     float *ls = Gm + kQ * (kQ + 1);   // [kQ]
     float *dts = ls + kQ;             // [kQ]
+    pdl_launch();
+    pdl_wait();
 
     const int h = blockIdx.x, seq = a.cu[a.n_seq + 1 + blockIdx.y];   // launch order: longest sequence first
     const int grp = h / (a.H / a.G);
@@ -121,8 +123,7 @@ cudaError_t launch(const SsdArgs &a, cudaStream_t s) {
     const size_t smem = smem_bytes(a.N, P);
     cudaError_t e = cudaFuncSetAttribute(ssd_scan_fp32_kernel<T, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    ssd_scan_fp32_kernel<T, P><<<dim3(a.H, a.n_seq), 256, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(ssd_scan_fp32_kernel<T, P>, dim3(a.H, a.n_seq), 256, smem, s, a);
 }
 
 template <typename T>

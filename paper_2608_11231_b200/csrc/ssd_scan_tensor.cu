@@ -168,6 +168,8 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
     const int h0 = grp * per_grp + 2 * pr;
     const bool two = 2 * pr + 1 < per_grp;   // the last head of an odd group is computed twice and stored once
     const int h1 = h0 + (two ? 1 : 0);
+    pdl_launch();
+    if (a.cu.ptr) pdl_wait();   // the index list is in global memory
     const int seq = a.cu[a.n_seq + 1 + blockIdx.y];   // launch order: longest sequence first
     const int t_begin = a.cu[seq], t_end = a.cu[seq + 1];
     // initial and final state of head h0; that of the other follows
@@ -178,6 +180,7 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
     const bool has_y = a.y != nullptr;
 
     if (t_begin == t_end) {  // empty sequence: hand the states through untouched
+        pdl_wait();
         if (ST && a.S_T != a.S0)
             for (int e = tid; e < (two ? 2 : 1) * kN * kP; e += kThreads) store_state(ST, a.st_bf16, st_off + e, S0 ? S0[e] : 0.f);
         return;
@@ -193,6 +196,7 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
         mbar_fence_init();
     }
     if (warp == 0) tmem_alloc(&tmem_base, kTmemCols);
+    pdl_wait();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -670,8 +674,7 @@ cudaError_t launch_ssd_scan_tensor(const SsdArgs &a, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(ssd_scan_tensor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     const int pairs = (a.H / a.G + 1) / 2;
-    ssd_scan_tensor_kernel<<<dim3(a.G * pairs, a.n_seq), kThreads, kSmemBytes, s>>>(a, mapX, mapB, mapC, mapY);
-    return cudaGetLastError();
+    return launch_chained(ssd_scan_tensor_kernel, dim3(a.G * pairs, a.n_seq), kThreads, kSmemBytes, s, a, mapX, mapB, mapC, mapY);
 }
 
 }  // namespace lkv
