@@ -917,25 +917,29 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
         // ======================================================= chain warpgroups: lane = state column j, `half` = token / row half
         const int j = tid & 127, half = warp >> 2;
         const uint32_t lane_base = tm + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-        // initial state: S0[m][j], m = 64*half..+63 -> TMEM (fp32, pre-scaled by gam_C of block 0) and bf16 pairs
-        mbar_wait(&bars.gb_ready[0], 0, &dead, a.status);
+        // initial state: S0[m][j], m = 64*half..+63 -> TMEM (fp32, times 2^R of block 0) and bf16 pairs.  All of it is asked for at
+        // once, and before the block's scalars are waited for: 16 values a thread in registers, the others into L2 (16 requests
+        // of up to 128 tokens: 56.6 -> 55.4 us).
         {
-            const float fc = ex2(0.5f * gb[kGbExp]), fa = ex2(0.5f * gb[kGbExp + 1]);
             const float *S0 = s0_id ? nullptr : initial_state();
-            const float *S0p = S0 ? S0 + static_cast<size_t>(64 * half) * kD + j : nullptr;
+            if (S0) {
+                S0 += static_cast<size_t>(64 * half) * kD;
+                for (int i = j >> 2; i < 48; i += 32) prefetch_l2(S0 + (16 + i) * kD + 32 * (j & 3));
+                S0 += j;
+            }
 #pragma unroll 1
             for (int q = 0; q < 4; ++q) {
                 float v[16];
+                if (S0) {   // one branch for the sixteen loads: they are in flight together
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) v[c] = S0[(16 * q + c) * kD];
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) v[c] = s0_id && 64 * half + 16 * q + c == j ? 1.f : 0.f;
+                }
+                if (q == 0) mbar_wait(&bars.gb_ready[0], 0, &dead, a.status);
+                const float fc = ex2(0.5f * gb[kGbExp]), fa = ex2(0.5f * gb[kGbExp + 1]);
                 uint32_t rr[16], w[8];
-#pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const int m = 64 * half + 16 * q + c;
-                    v[c] = s0_id && m == j ? 1.f : 0.f;
-                }
-                if (S0p) {   // one branch for the sixteen loads: all of them in flight together
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) v[c] = S0p[(16 * q + c) * kD];
-                }
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
                     rr[c] = __float_as_uint(v[c] * fa * fa);
