@@ -50,6 +50,7 @@ template <int CAP>
 int place_indices(IndexBlock<CAP> &blk, const std::vector<int32_t> &ints, void *workspace, cudaStream_t s) {
     if (static_cast<int>(ints.size()) <= CAP) {
         blk.ptr = nullptr;
+        blk.n = static_cast<int32_t>(ints.size());
         if (!ints.empty()) memcpy(blk.v, ints.data(), sizeof(int32_t) * ints.size());
         return LKV_OK;
     }
@@ -66,6 +67,7 @@ int place_indices(IndexBlock<CAP> &blk, const std::vector<int32_t> &ints, void *
         return LKV_ERR_CUDA;
     }
     blk.ptr = dst;
+    blk.n = 0;
     return LKV_OK;
 }
 
@@ -224,6 +226,7 @@ int ssd_segmented(SsdArgs a, int segs, char *scratch, cudaStream_t s) {
     auto bounds = [&](SsdArgs &b, int n) {
         b.n_seq = n;
         b.cu.ptr = nullptr;
+        b.cu.n = 2 * n + 1;
         for (int i = 0; i <= n; ++i) b.cu.v[i] = static_cast<int32_t>(std::min<long long>(static_cast<long long>(i) * per, a.T_total));
         for (int i = 0; i < n; ++i) b.cu.v[n + 1 + i] = i;
     };
@@ -240,6 +243,7 @@ int ssd_segmented(SsdArgs a, int segs, char *scratch, cudaStream_t s) {
         for (int j = 0; j <= r; ++j) c.idx.v[at++] = j;
     }
     c.idx.v[segs - 1] = at - segs;
+    c.idx.n = at;
     if (launch_init_mamba_exact_stream(c, false, s) != cudaSuccess) return LKV_ERR_CUDA;
     SsdArgs p3 = a;
     bounds(p3, segs);
@@ -295,6 +299,7 @@ int gdn_segmented(GdnArgs a, GdnCut c, char *scratch, cudaStream_t s) {
         b.cu.ptr = nullptr;
         b.n_ranges = b.tr_first = k;
         b.n_seq = k + n_tr;
+        b.cu.n = k + 1 + b.n_seq;
         for (int i = 0; i <= k; ++i) b.cu.v[i] = at[i];
         auto len = [&](int sq) { const int r = sq < k ? sq : sq - k + b.tr_src0; return at[r + 1] - at[r]; };
         int32_t *order = b.cu.v + k + 1;
@@ -315,6 +320,7 @@ int gdn_segmented(GdnArgs a, GdnCut c, char *scratch, cudaStream_t s) {
         for (int j = 0; j <= r; ++j) k.idx.v[ids++] = j;
     }
     k.idx.v[m] = ids - n;
+    k.idx.n = ids;
     if (launch_init_gdn_exact_tensor(k, false, s) != cudaSuccess) return LKV_ERR_CUDA;
     GdnArgs p3 = a;
     ranges(p3, n, 0);
