@@ -33,7 +33,8 @@
 //
 // What bounds it: neither a pipe (tensor 36 %, issue slots 39 % with every SM busy) nor one chain, but the latency of about
 // 6 K instructions per block in ten programs that share an SM: mask 1.7 K cycles, inverse 3.0 K, chain 2.1 K of a block period of
-// 3.3 K.  Hence small rolled loops, fp16 storage of what is an fp16 operand, ldmatrix / movmatrix instead of fp32 round trips, and
+// 3.3 K -- and instruction fetch: 5 KB less code in the issuing and scalar warps (each piece of code once, its loop started a
+// block early instead of a copy before it) took 32 x 4096 tokens from 992 to 940 us.  Hence small rolled loops, fp16 storage of what is an fp16 operand, ldmatrix / movmatrix instead of fp32 round trips, and
 // few warps: outputs in a warpgroup of their own, or the last merge of the inverse moved to the W warps, made every program slower
 // (8 % and 17 % on one sequence).  Measured on B200, 32 value heads: one sequence of 8192 tokens 311 -> 254 us, 32 x 4096 tokens
 // 1172 -> 982 us against the form that gates the products and solves for u in the chain (three conversions).
@@ -317,6 +318,12 @@ __device__ __noinline__ void rescale_state(uint32_t tm_s, uint32_t tm_sb, float 
         tmem_st16(tm_s + 16 * q, rr);
     }
 }
+// Empty sequence: the initial state (the identity, S0, or zero) and what is to be added, as the final state
+__device__ __noinline__ void hand_through(float *ST, size_t obase, int st_bf16, bool id, const float *S0, const float *add) {
+#pragma unroll 1
+    for (int e = threadIdx.x; e < kD * kD; e += kThreads)
+        store_state(ST, st_bf16, obase + e, (id ? (e / kD == e % kD ? 1.f : 0.f) : (S0 ? S0[e] : 0.f)) + (add ? add[e] : 0.f));
+}
 // Exact block: u_t[j] of 32 tokens -> Uw = w o u as bf16 pairs over the first 16 of these 32 columns, u over the rest
 __device__ __noinline__ void u_operands_exact(uint32_t taddr, const float *w) {
     uint32_t rr[32], p[8];
@@ -371,14 +378,11 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
 
     if (nblk == 0) {  // empty sequence: hand the state through untouched
         pdl_wait();
-        const float *S0 = initial_state();
         size_t obase;
         float *ST = final_state(obase);
+        const float *S0 = initial_state();
         if (ST && (ST != a.S0 || s0_id || a.S_add))
-            for (int e = tid; e < kD * kD; e += kThreads)
-                store_state(ST, a.st_bf16, obase + e,
-                            (s0_id ? (e / kD == e % kD ? 1.f : 0.f) : (S0 ? S0[e] : 0.f)) +
-                                (a.S_add ? a.S_add[sbase + e] : 0.f));
+            hand_through(ST, obase, a.st_bf16, s0_id, s0_id ? nullptr : S0, a.S_add ? a.S_add + sbase : nullptr);
         return;
     }
     if (tid == 0) {
@@ -455,11 +459,13 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
                 bv.y = a.beta[static_cast<size_t>(t + 1) * a.H_v + h];
             }
         };
-        float2 gv_next, bv_next;
-        fetch_gb(0, gv_next, bv_next);
+        float2 gv_next = make_float2(0.f, 0.f), bv_next = gv_next;
         float R = 0.f;   // the state is held times 2^R
 #pragma unroll 1
-        for (int b = 0; b < nblk; ++b) {
+        for (int b = -1; b < nblk; ++b) {
+            const float2 gv = gv_next, bv = bv_next;
+            fetch_gb(b + 1, gv_next, bv_next);   // in flight while this block is prepared
+            if (b < 0) continue;
             if (warp_dead(&dead)) break;   // a wait ran out: nothing more is issued
             const int s4 = b % kQKStages;
             const int row = t_begin + b * kC;
@@ -488,8 +494,6 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
             }
             __syncwarp();
             float *sc = gb + (b & 3) * kGbFloats;
-            const float2 gv = gv_next, bv = bv_next;
-            fetch_gb(b + 1, gv_next, bv_next);   // in flight while this block is prepared
             float run = gv.x + gv.y;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -532,13 +536,7 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
             }
             __syncwarp();
         };
-#pragma unroll 1
-        for (int b = 0; b <= nblk; ++b) {
-            if (warp_dead(&dead)) break;   // a wait ran out: nothing more is issued
-            if (b == nblk) {
-                issue_w(b - 1);
-                break;
-            }
+        auto issue_g = [&](int b) {
             const int s3 = b % kQKStages;
             // (1) of block b: the mask epilogue of block b-1 has drained the G columns
             if (b >= 1) {
@@ -558,6 +556,11 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
                 umma_commit(&bars.g_done);
             }
             __syncwarp();
+        };
+#pragma unroll 1
+        for (int b = 0; b <= nblk; ++b) {
+            if (warp_dead(&dead)) break;   // a wait ran out: nothing more is issued
+            if (b < nblk) issue_g(b);
             if (b >= 1) issue_w(b - 1);
         }
     } else if (warp == 17) {
@@ -584,10 +587,7 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
             }
             __syncwarp();
         };
-        issue_3a(0);
-#pragma unroll 1
-        for (int b = 0; b < nblk; ++b) {
-            if (warp_dead(&dead)) break;
+        auto chain_block = [&](int b) {
             const uint32_t par = b & 1;
             const uint32_t qk = smem_u32(sm + (b % kQKStages) * kQKStage);
             const uint64_t dQ = umma_desc(qk, 0, 1024), dKmn = umma_desc(qk + kC * 128, 2 * kC * 128, 1024);
@@ -645,6 +645,11 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
                 umma_commit(&bars.o_mma_done[par]);
             }
             __syncwarp();
+        };
+#pragma unroll 1
+        for (int b = -1; b < nblk; ++b) {
+            if (warp_dead(&dead)) break;
+            if (b >= 0) chain_block(b);
             if (b + 1 < nblk) issue_3a(b + 1);
         }
     } else if (warp >= 20) {
