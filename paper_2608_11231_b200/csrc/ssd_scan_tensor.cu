@@ -94,7 +94,8 @@ struct Bars {
     uint64_t sc_ready[kSlots];
     // the eight output, state or prep warps
     uint64_t y_free, hb_ready, x_free, x2_ready, mask_done;
-    // output and state warps (state warps alone when no outputs are wanted)
+    // readers of a block descriptor that nothing later waits for: the output and state warps (state warps alone when no outputs are
+    // wanted) and the TMA warp.  (The other readers are done before the products that the state and the outputs wait for.)
     uint64_t slot_free[kSlots];
 };
 constexpr int kBars1 = 9;
@@ -192,7 +193,7 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
         for (int i = 0; i < 2; ++i) mbar_init(bp++, has_y ? 2 : 1);
         for (int i = 0; i < kSlots; ++i) mbar_init(bp++, 1);
         for (int i = 0; i < 5; ++i) mbar_init(bp++, 8);
-        for (int i = 0; i < kSlots; ++i) mbar_init(bp++, has_y ? 16 : 8);
+        for (int i = 0; i < kSlots; ++i) mbar_init(bp++, has_y ? 17 : 9);
         mbar_fence_init();
     }
     if (warp == 0) tmem_alloc(&tmem_base, kTmemCols);
@@ -330,6 +331,7 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
                 // where the next block starts
                 mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
                 row += slots[b % kSlots].n;
+                warp_arrive(&bars.slot_free[b % kSlots]);
             }
         } else if (warp == 25) {
             // ---- MMA issue of (S)
