@@ -820,8 +820,8 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
 #pragma unroll 1
         for (int b = 0; b < nblk; ++b) {
             const float *sc = gb + (b & 3) * kGbFloats;
-            mbar_wait(&bars.gb_ready[b & 3], (b >> 2) & 1, &dead, a.status);
-            const bool exact = sc[kGbExp + 3] != 0.f;
+            // (Without outputs the warps of Ps leave the scalars alone: nothing that frees their buffer would wait for that read.)
+            if (x >= kC || has_o) mbar_wait(&bars.gb_ready[b & 3], (b >> 2) & 1, &dead, a.status);
             if (x < kC) {
                 // rows of Ps, the diagonal included.  The buffer is free once (7) of block b-2 has read it.
                 if (b >= 2 && has_o) mbar_wait(&bars.p_free[b & 1], ((b - 2) >> 1) & 1, &dead, a.status);
@@ -830,6 +830,7 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
                 tc_fence_after_sync();
                 unsigned char *ps = sm + kOffP + (b & 1) * (kC * 128);
                 if (has_o) {
+                    const bool exact = sc[kGbExp + 3] != 0.f;
                     // column groups above the diagonal for every row of this warp are never touched
 #pragma unroll 1
                     for (int q = 0; 16 * q <= row_hi; ++q) {
@@ -855,6 +856,7 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
                 fence_async_smem();
                 warp_arrive(&bars.p_ready[b & 1]);
             } else {
+                const bool exact = sc[kGbExp + 3] != 0.f;
                 // rows of A, strictly lower.  F is free once block b-2 has been inverted, D once the diagonal blocks of block b-1 are.
                 if (b >= 2) mbar_wait(&bars.m_ready[b & 1], ((b - 2) >> 1) & 1, &dead, a.status);
                 if (b >= 1) mbar_wait(&bars.d_free, (b - 1) & 1, &dead, a.status);
