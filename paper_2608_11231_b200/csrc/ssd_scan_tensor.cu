@@ -421,7 +421,6 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
         // ======================================================= prep: X^^T of 64 tokens; this warp: 32 features of one head
         const int th = wg - 4, hd = wq >> 1;
         const int m = lane >> 3, i = lane & 7;
-        const uint32_t zero = a.n_seq < 0 ? 1u : 0u;   // 0, which the compiler cannot know
         // matrix m of a load: features 8 (m & 1) .., tokens 8 (m >> 1) ..
         const uint32_t xrow = smem_u32(sm + kOffX + hd * kTile) + (64 * th + 8 * (m >> 1) + i) * 128;
         // mask: row t of tril(G) -> bf16 operand tile, columns < 64 of row t and columns >= 64 of row t - 64
@@ -463,12 +462,12 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
             }
             // The tile may be overwritten once its loads have RETURNED, not once they are issued: the assembler may hold their first
             // use back past the arrival, and under load they have come back later than the next tile (seen: single rows of the
-            // next block).  So the arrival's address takes a zero that is made of one result of every load.
+            // next block).  So which lane arrives depends on one result of every load of every lane.
             uint32_t any = 0;
 #pragma unroll
             for (int j = 0; j < 16; j += 4) any |= w[0][j] | w[1][j];
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bars.x_free + (any & zero));
+            const uint32_t odd = __ballot_sync(0xffffffffu, any & 1u);
+            if (lane == (odd ? __ffs(odd) - 1 : 0)) mbar_arrive(&bars.x_free);
             if (b >= 1) {   // (S) and (Y1) have read the X^ before
                 mbar_wait(&bars.xs_free, (b - 1) & 1, &dead, a.status);
                 if (has_y) mbar_wait(&bars.xy_free, (b - 1) & 1, &dead, a.status);
