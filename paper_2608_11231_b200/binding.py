@@ -168,15 +168,25 @@ def _hp(a: Optional[np.ndarray]):
 
 
 _ws_cache = {}
+_ws_replaced = []
 _err_ws_cache = {}
 
 
 def workspace(device, nbytes: int) -> torch.Tensor:
-    """A zero-initialised, cached device workspace of at least nbytes (one per device and stream)."""
+    """A zero-initialised, cached device workspace of at least nbytes (one per device and stream).
+
+    A workspace that has become too small is replaced but not given back: a CUDA graph captured with it, or a call that another
+    thread has in flight, still writes there.  Sizes at least double, so that all the replaced ones together are smaller than
+    the one in use.
+    """
     key = (torch.device(device).index, torch.cuda.current_stream().cuda_stream)
     ws = _ws_cache.get(key)
     if ws is None or ws.numel() < nbytes:
-        ws = torch.zeros(max(int(nbytes), 4096), dtype=torch.uint8, device=device)
+        size = max(int(nbytes), 4096)
+        if ws is not None:
+            size = max(size, 2 * ws.numel())
+            _ws_replaced.append(ws)
+        ws = torch.zeros(size, dtype=torch.uint8, device=device)
         _ws_cache[key] = ws
     return ws
 
