@@ -17,6 +17,8 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <mutex>
+
 #include "../../include/lkv.h"
 
 namespace {
@@ -154,6 +156,25 @@ void check(int st, const char *where) {
     throw Failed{};
 }
 
+// The C call with the interpreter lock released, as ctypes does it: a launch into a full stream queue blocks, and so does the copy
+// of a long index list; the engine's other threads run on meanwhile.  The arguments are plain C values by then, what they
+// point to is held by the caller's frame.  A call may be several launches that pass data through the workspace, and threads that
+// share a stream share its workspace: calls on one workspace take turns (the lock is picked by the workspace's address).
+template <typename... P, typename... A>
+void call(const char *where, const void *workspace, int (*f)(P...), A... args) {
+    static std::mutex turns[64];
+    int st;
+    {
+        struct Released {
+            PyThreadState *state = PyEval_SaveThread();
+            ~Released() { PyEval_RestoreThread(state); }
+        } released;
+        std::lock_guard<std::mutex> turn(turns[(reinterpret_cast<uintptr_t>(workspace) >> 9) % 64]);
+        st = f(args...);
+    }
+    check(st, where);
+}
+
 int to_int(PyObject *o) {
     PyObject *i = PyNumber_Long(o);
     if (!i) throw Failed{};
@@ -253,7 +274,8 @@ PyObject *init_state(PyObject *, PyObject *const *a, Py_ssize_t n) {
         Output S0;
         if (a[4] != Py_None) S0.given(a[4]);
         else S0.make(new_tensor(states.sizes().slice(1), at::kFloat, states));
-        check(lkv_init_state(ptr_of(a[0]), ptr_of(a[1]), K, to_int(a[3]), S0.ptr, &d, stream_of(a[10])), "lkv_init_state");
+        call("lkv_init_state", d.workspace, lkv_init_state, ptr_of(a[0]), ptr_of(a[1]), K, to_int(a[3]), S0.ptr, &d,
+             stream_of(a[10]));
         return S0.take();
     });
 }
@@ -270,9 +292,8 @@ PyObject *init_state_batched(PyObject *, PyObject *const *a, Py_ssize_t n) {
         Output S0;
         if (a[7] != Py_None) S0.given(a[7]);
         else S0.make(new_tensor({n_req, states.size(1), states.size(2), states.size(3)}, at::kFloat, states));
-        check(lkv_init_state_batched(ptr_of(a[0]), ptr_of(a[1]), ids.data(), cu.data(), n_req, to_int(a[5]), sel.data(), S0.ptr,
-                                     &d, stream_of(a[11])),
-              "lkv_init_state_batched");
+        call("lkv_init_state_batched", d.workspace, lkv_init_state_batched, ptr_of(a[0]), ptr_of(a[1]), ids.data(), cu.data(),
+             n_req, to_int(a[5]), sel.data(), S0.ptr, &d, stream_of(a[11]));
         return S0.take();
     });
 }
@@ -311,10 +332,9 @@ PyObject *gdn_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
         if (a[7] != Py_None) S_T.given(a[7]);
         else if (PyObject_IsTrue(a[11]) == 1) S_T.make(new_tensor({d.n_seq, d.H_v, d.d_k, d.d_v}, scalar_type_of(a[13]), v));
         if (S_T.obj) d.state_dtype = dtype_code(THPVariable_Unpack(S_T.obj));
-        check(lkv_gdn_fwd(ptr_of(a[0]), ptr_of(a[1]), ptr_of(a[2]), static_cast<float *>(ptr_of(a[3])),
-                          static_cast<float *>(ptr_of(a[4])), static_cast<float *>(ptr_of(a[5])), o.ptr, S_T.ptr, &d,
-                          stream_of(a[15])),
-              "lkv_gdn_fwd");
+        call("lkv_gdn_fwd", d.workspace, lkv_gdn_fwd, ptr_of(a[0]), ptr_of(a[1]), ptr_of(a[2]),
+             static_cast<float *>(ptr_of(a[3])), static_cast<float *>(ptr_of(a[4])), static_cast<float *>(ptr_of(a[5])), o.ptr,
+             S_T.ptr, &d, stream_of(a[15]));
         return pair(o, S_T);
     });
 }
@@ -334,10 +354,9 @@ PyObject *gdn_chunk_artifacts(PyObject *, PyObject *const *a, Py_ssize_t n) {
         else S.make(new_tensor({d.n_seq, d.H_v, d.d_k, d.d_v}, at::kFloat, k));
         if (a[5] != Py_None) T.given(a[5]);
         else T.make(new_tensor({d.n_seq, d.H_v, d.d_k, d.d_k}, at::kFloat, k));
-        check(lkv_gdn_chunk_artifacts(ptr_of(a[0]), ptr_of(a[1]), static_cast<float *>(ptr_of(a[2])),
-                                      static_cast<float *>(ptr_of(a[3])), static_cast<float *>(S.ptr),
-                                      static_cast<float *>(T.ptr), &d, stream_of(a[9])),
-              "lkv_gdn_chunk_artifacts");
+        call("lkv_gdn_chunk_artifacts", d.workspace, lkv_gdn_chunk_artifacts, ptr_of(a[0]), ptr_of(a[1]),
+             static_cast<float *>(ptr_of(a[2])), static_cast<float *>(ptr_of(a[3])), static_cast<float *>(S.ptr),
+             static_cast<float *>(T.ptr), &d, stream_of(a[9]));
         return pair(S, T);
     });
 }
@@ -367,9 +386,9 @@ PyObject *ssd_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
         if (a[7] != Py_None) S_T.given(a[7]);
         else if (PyObject_IsTrue(a[10]) == 1) S_T.make(new_tensor({d.n_seq, d.H, d.N, d.P}, scalar_type_of(a[12]), x));
         if (S_T.obj) d.state_dtype = dtype_code(THPVariable_Unpack(S_T.obj));
-        check(lkv_ssd_fwd(ptr_of(a[0]), static_cast<float *>(ptr_of(a[1])), static_cast<float *>(ptr_of(a[2])), ptr_of(a[3]),
-                          ptr_of(a[4]), static_cast<float *>(ptr_of(a[5])), y.ptr, S_T.ptr, &d, stream_of(a[14])),
-              "lkv_ssd_fwd");
+        call("lkv_ssd_fwd", d.workspace, lkv_ssd_fwd, ptr_of(a[0]), static_cast<float *>(ptr_of(a[1])),
+             static_cast<float *>(ptr_of(a[2])), ptr_of(a[3]), ptr_of(a[4]), static_cast<float *>(ptr_of(a[5])), y.ptr,
+             S_T.ptr, &d, stream_of(a[14]));
         return pair(y, S_T);
     });
 }
@@ -391,9 +410,8 @@ PyObject *mamba_chunk_logdecay(PyObject *, PyObject *const *a, Py_ssize_t n) {
         Output out;
         if (a[2] != Py_None) out.given(a[2]);
         else out.make(new_tensor({d.n_seq, d.H}, at::kFloat, dt));
-        check(lkv_mamba_chunk_logdecay(static_cast<float *>(ptr_of(a[0])), static_cast<float *>(ptr_of(a[1])),
-                                       static_cast<float *>(out.ptr), &d, stream_of(a[5])),
-              "lkv_mamba_chunk_logdecay");
+        call("lkv_mamba_chunk_logdecay", d.workspace, lkv_mamba_chunk_logdecay, static_cast<float *>(ptr_of(a[0])),
+             static_cast<float *>(ptr_of(a[1])), static_cast<float *>(out.ptr), &d, stream_of(a[5]));
         return out.take();
     });
 }
