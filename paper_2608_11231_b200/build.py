@@ -29,7 +29,7 @@ def build(verbose: bool = False, force: bool = False) -> str:
     """Compile every .cu under csrc/ and link liblkv.so; returns the library path."""
     nvcc = os.environ.get("NVCC", "nvcc")
     os.makedirs(OBJ, exist_ok=True)
-    headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(HERE, "..", "include", "*.h"))
+    headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(HERE, "..", "include", "*.h"))
     objs, procs = [], []
     sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     # one stale source means a full rebuild (a few seconds): the library is never a mix of objects from different states

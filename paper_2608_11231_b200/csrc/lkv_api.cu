@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "segments.h"
 
 using namespace lkv;
 
@@ -202,15 +203,15 @@ void append_launch_order(std::vector<int32_t> &cu, int n_seq) {
 }
 
 // A single sequence fills (heads / 2) of the SMs (two heads per CTA) and is a chain of blocks.  Cut into segments, it runs as
-// three launches: the states the first segments reach on their own (no outputs: 2.0 K cycles a block against 3.2 K), the
-// composition of every segment's initial state (Eq. 6), all segments with outputs side by side.  Worth it from three
-// segments up -- two save 0.6 K cycles a block -- of at least 1024 tokens: the two more launches cost about 16 blocks.
-int ssd_segments(const lkv_ssd_desc *d, int n_seq) {
-    if (n_seq != 1 || d->io_dtype != LKV_DTYPE_BF16 || d->compute == LKV_COMPUTE_FP32 || d->H < 1 || d->G < 1 || d->H % d->G || d->P != 64 || d->N != 128)
-        return 1;
-    const int ctas = d->G * ((d->H / d->G + 1) / 2);
-    const int n = std::min({sm_count() / ctas, d->T_total / 1024, 16});
-    return n >= 3 ? n : 1;
+// three launches: the states the first segments reach on their own (no outputs), the composition of every segment's initial
+// state (Eq. 6), all segments with outputs side by side.
+constexpr int kSsdBlock = 128, kGdnBlock = 64;   // tokens
+Cut ssd_cut(const lkv_ssd_desc *d, int n_seq) {
+    if (n_seq != 1 || d->io_dtype != LKV_DTYPE_BF16 || d->compute == LKV_COMPUTE_FP32 || d->H < 1 || d->G < 1 || d->H % d->G ||
+        d->P != 64 || d->N != 128 || d->T_total < 1)
+        return Cut{1, {0}};
+    const int pairs = d->G * ((d->H / d->G + 1) / 2);
+    return ssd_cut_blocks((d->T_total - 1) / kSsdBlock + 1, pairs, sm_count());
 }
 // local states and log-decays of the first segments, initial states of all but the first
 size_t ssd_segment_scratch(const lkv_ssd_desc *d, int segs) {
@@ -218,16 +219,15 @@ size_t ssd_segment_scratch(const lkv_ssd_desc *d, int segs) {
     const size_t slot = sizeof(float) * static_cast<size_t>(d->H) * d->N * d->P;
     return 2 * (segs - 1) * slot + align_up(sizeof(float) * static_cast<size_t>(segs - 1) * d->H, 256);
 }
-int ssd_segmented(SsdArgs a, int segs, char *scratch, cudaStream_t s) {
+int ssd_segmented(SsdArgs a, const Cut &cut, char *scratch, cudaStream_t s) {
+    const int segs = cut.n;
     const size_t slot = static_cast<size_t>(a.H) * a.N * a.P;
     float *local = reinterpret_cast<float *>(scratch), *init = local + (segs - 1) * slot, *lam = init + (segs - 1) * slot;
-    // whole blocks of 128 tokens
-    const int per = ((a.T_total + segs - 1) / segs + 127) / 128 * 128;
     auto bounds = [&](SsdArgs &b, int n) {
         b.n_seq = n;
         b.cu.ptr = nullptr;
         b.cu.n = 2 * n + 1;
-        for (int i = 0; i <= n; ++i) b.cu.v[i] = static_cast<int32_t>(std::min<long long>(static_cast<long long>(i) * per, a.T_total));
+        for (int i = 0; i <= n; ++i) b.cu.v[i] = std::min<long long>(kSsdBlock * static_cast<long long>(cut.at[i]), a.T_total);
         for (int i = 0; i < n; ++i) b.cu.v[n + 1 + i] = i;
     };
     SsdArgs p1 = a;
@@ -252,49 +252,23 @@ int ssd_segmented(SsdArgs a, int segs, char *scratch, cudaStream_t s) {
 }
 
 // The same for the GDN scan (one head per CTA), where the first pass also computes the transitions of the segments between the
-// first and the last: n segments are (2 n - 3) H_v CTAs there and n H_v in the last pass.  Two ways to stay within one round
-// of CTAs: n equal segments, or one of the segments with a transition half as long as the others, so that its two CTAs of a
-// head follow one another on one SM (n - 1/2 segments' worth of tokens; at H_v = 32 on 148 SMs n = 4, against 3 equal ones).
-// Both passes take as long as the longest segment; the composition, the launches and the fill of another pipeline cost about
-// 14 blocks of 64 tokens.
-struct GdnCut {
-    int n, full;   // segments, tokens of a full one; segment n - 2 may be shorter
-};
-GdnCut gdn_cut(const lkv_gdn_desc *d, int n_seq) {
-    const GdnCut whole{1, 0};
-    if (n_seq != 1 || d->io_dtype != LKV_DTYPE_BF16 || d->compute == LKV_COMPUTE_FP32 || d->H_v < 1 || d->d_k != 128 || d->d_v != 128 || d->T_total < 1024)
-        return whole;
-    const int slots = sm_count() / d->H_v;
-    const int equal = std::min((slots + 3) / 2, slots), halved = std::min((slots + 4) / 2, slots);
-    const int blocks = (d->T_total + 63) / 64;
-    GdnCut c = whole;
-    int longest;   // blocks of a full segment
-    if (halved > equal && halved >= 3) {
-        longest = (2 * blocks + 2 * halved - 2) / (2 * halved - 1);
-        c.n = halved;
-    } else {
-        longest = equal > 0 ? (blocks + equal - 1) / equal : blocks;
-        c.n = equal;
-    }
-    c.n = std::min(c.n, 16);
-    c.full = 64 * longest;
-    return c.n >= 3 && blocks - 2 * longest > 14 && static_cast<long long>(c.full) * c.n < d->T_total + 2ll * c.full ? c : whole;
+// first and the last.
+Cut gdn_cut(const lkv_gdn_desc *d, int n_seq) {
+    if (n_seq != 1 || d->io_dtype != LKV_DTYPE_BF16 || d->compute == LKV_COMPUTE_FP32 || d->d_k != 128 || d->d_v != 128 || d->T_total < 1)
+        return Cut{1, {0}};
+    return gdn_cut_blocks((d->T_total - 1) / kGdnBlock + 1, d->H_v, sm_count());
 }
 // local states and transitions of all segments but the last, initial states of all but the first
-size_t gdn_segment_scratch(const lkv_gdn_desc *d, GdnCut c) {
+size_t gdn_segment_scratch(const lkv_gdn_desc *d, const Cut &c) {
     if (c.n < 2) return 0;
     return 3 * static_cast<size_t>(c.n - 1) * sizeof(float) * d->H_v * d->d_k * d->d_v;
 }
-int gdn_segmented(GdnArgs a, GdnCut c, char *scratch, cudaStream_t s) {
+int gdn_segmented(GdnArgs a, const Cut &c, char *scratch, cudaStream_t s) {
     const int n = c.n, m = n - 1;
     const size_t slot = static_cast<size_t>(a.H_v) * a.d_k * a.d_v;
     float *local = reinterpret_cast<float *>(scratch), *trans = local + m * slot, *init = trans + m * slot;
-    // whole blocks; the last segment is full, the one before it takes what is left
-    int at[17];
-    for (int i = 0; i < n - 2; ++i) at[i] = i * c.full;
-    at[n - 2] = (n - 2) * c.full;
-    at[n] = a.T_total;
-    at[n - 1] = std::max(at[n - 2], (a.T_total - c.full + 63) / 64 * 64);
+    int at[kMaxSegments + 1];
+    for (int i = 0; i <= n; ++i) at[i] = std::min<long long>(kGdnBlock * static_cast<long long>(c.at[i]), a.T_total);
     auto ranges = [&](GdnArgs &b, int k, int n_tr) {
         b.cu.ptr = nullptr;
         b.n_ranges = b.tr_first = k;
@@ -425,7 +399,7 @@ static int gdn_impl(const void *q, const void *k, const void *v, const float *g,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // A long sequence that leaves SMs idle runs in segments (a caller whose workspace is smaller than
     // lkv_workspace_bytes() asked for gets the plain scan; S_T on top of S0 would be written while S0 is read)
-    const GdnCut cut = use_tensor && what == 0 && S_T != S0 && o ? gdn_cut(d, d->n_seq) : GdnCut{1, 0};
+    const Cut cut = use_tensor && what == 0 && S_T != S0 && o ? gdn_cut(d, d->n_seq) : Cut{1, {0}};
     const size_t head = ws_bytes_for(2 * d->n_seq + 1, kScanIdxCap);
     if (cut.n > 1 && d->workspace_bytes >= head + gdn_segment_scratch(d, cut))
         return gdn_segmented(a, cut, static_cast<char *>(d->workspace) + head, s);
@@ -739,10 +713,10 @@ int lkv_ssd_fwd(const void *x, const float *dt, const float *A, const void *B, c
     }
     a.n_s0 = d->n_seq; a.st_first = 0; a.S0_more = nullptr; a.lam = nullptr;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int segs = use_tensor && S_T != S0 && y ? ssd_segments(d, d->n_seq) : 1;
+    const Cut cut = use_tensor && S_T != S0 && y ? ssd_cut(d, d->n_seq) : Cut{1, {0}};
     const size_t head = ws_bytes_for(2 * d->n_seq + 1, kScanIdxCap);
-    if (segs > 1 && d->workspace_bytes >= head + ssd_segment_scratch(d, segs))
-        return ssd_segmented(a, segs, static_cast<char *>(d->workspace) + head, s);
+    if (cut.n > 1 && d->workspace_bytes >= head + ssd_segment_scratch(d, cut.n))
+        return ssd_segmented(a, cut, static_cast<char *>(d->workspace) + head, s);
     append_launch_order(cu, d->n_seq);
     st = place_indices(a.cu, cu, d->workspace, s);
     if (st != LKV_OK) return st;
@@ -760,7 +734,7 @@ size_t lkv_workspace_bytes(int which, const void *desc, int n_units, int n_index
         }
         case LKV_WS_SSD: {
             const lkv_ssd_desc *d = static_cast<const lkv_ssd_desc *>(desc);
-            return ws_bytes_for(2 * n_units + 1, kScanIdxCap) + ssd_segment_scratch(d, ssd_segments(d, n_units));
+            return ws_bytes_for(2 * n_units + 1, kScanIdxCap) + ssd_segment_scratch(d, ssd_cut(d, n_units).n);
         }
         default: return 0;
     }
