@@ -291,10 +291,11 @@ int lkv_gdn_fwd(const void *q, const void *k, const void *v, const float *g, con
  * Same arguments and results as lkv_gdn_fwd (results equal up to the rounding of the composition, which uses the
  * arithmetic of d->compute: tf32 products under AUTO / TENSOR at d = 128); requires d->n_seq == 1, d_k == d_v,
  * state_dtype fp32.  scratch: device, 16-byte aligned, >= lkv_gdn_segmented_scratch_bytes(d, n_segments) bytes, owned by
- * the caller.  n_segments == 1 is lkv_gdn_fwd itself; n_segments == 0 lets the library choose (as many segments as keep
- * both scanning passes within one round of CTAs on the current GPU, none shorter than 512 tokens; the scratch-size call
- * makes the same choice).  Five stream operations besides the three kernel launches
- * (memsets / device copies of single states).  (The paper has no counterpart: its prefill is the plain scan.)
+ * the caller.  n_segments == 1 is lkv_gdn_fwd itself; n_segments == 0 lets the library choose: where the tensor-core scan
+ * runs, the very segments that lkv_gdn_fwd takes with a workspace of lkv_workspace_bytes() (the same results bit for bit; this
+ * call then differs in where the scratch comes from), otherwise as many as keep both scanning passes within one round of
+ * CTAs on the current GPU, none shorter than 512 tokens; the scratch-size call makes the same choice.  Three kernel launches,
+ * and a device copy of one state where S_T is S0.  (The paper has no counterpart: its prefill is the plain scan.)
  */
 int lkv_gdn_fwd_segmented(const void *q, const void *k, const void *v, const float *g, const float *beta,
                           const float *S0, void *o, void *S_T, const lkv_gdn_desc *d, int n_segments,

@@ -48,15 +48,19 @@ __device__ __forceinline__ void store_state(float *S_T, int st_bf16, size_t idx,
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... Params, typename... Args>
-cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const Args &...args) {
+cudaError_t launch_kernel(bool early, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const Args &...args) {
     static_assert((std::is_same<Params, Args>::value && ...), "the arguments are passed by address");
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
     void *p[] = {const_cast<void *>(static_cast<const void *>(&args))...};
     return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), p);
+}
+template <typename... Params, typename... Args>
+cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const Args &...args) {
+    return launch_kernel(true, kernel, grid, block, smem, s, args...);
 }
 
 // Small host-checked index arrays travel to the device inside the kernel parameters
@@ -130,7 +134,7 @@ struct GdnArgsBase {
     // (the ranges of sequences 0 .. tr_first-1); a plain call has n_ranges = tr_first = n_seq.
     int32_t n_ranges, tr_first, tr_src0;
     float *tr_out;               // where transition sequence tr_first + i stores its final state (index i), or nullptr: S_T like the others
-    // One sequence cut into segments that run side by side (tensor-core scan only).  Sequences n_s0 .. start from S0_more (index
+    // One sequence cut into segments that run side by side.  Sequences n_s0 .. start from S0_more (index
     // seq - n_s0; nullptr = zero), final states are wanted of sequences st_first .. only (index seq - st_first).  A plain call
     // has n_s0 = n_seq, st_first = 0.
     int32_t n_s0, st_first;
@@ -178,7 +182,8 @@ bool init_mamba_stream_supported(const InitArgs &a, bool pool_bf16);
 cudaError_t launch_init_mamba_exact_stream(const InitArgs &a, bool pool_bf16, cudaStream_t s);
 cudaError_t launch_init_gdn_exact_fp32(const InitArgs &a, bool pool_bf16, cudaStream_t s);
 bool init_gdn_exact_tensor_supported(const InitArgs &a, bool pool_bf16);
-cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cudaStream_t s);
+// early = false: not before the kernel ahead of it on the stream has left the GPU
+cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cudaStream_t s, bool early = true);
 
 bool gdn_scan_fp32_supported(int d_k, int d_v);
 cudaError_t launch_gdn_scan_fp32(const GdnArgs &a, bool io_bf16, cudaStream_t s);

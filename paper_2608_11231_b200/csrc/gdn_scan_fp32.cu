@@ -62,16 +62,20 @@ __global__ void __launch_bounds__(256) gdn_scan_fp32_kernel(const __grid_constan
     const T *k = static_cast<const T *>(a.k);
     const T *v = tr ? nullptr : static_cast<const T *>(a.v);
     T *o = tr ? nullptr : static_cast<T *>(a.o);
-    const size_t sbase = (static_cast<size_t>(seq) * a.H_v + h) * dk * dv + j0;
-    float *ST = (tr && a.tr_out) ? a.tr_out : a.S_T;   // final state of this sequence
-    const size_t obase = (tr && a.tr_out) ? (static_cast<size_t>(seq - a.tr_first) * a.H_v + h) * dk * dv + j0 : sbase;
+    // where this sequence's initial state lies (nullptr = zero) and where its final state goes (nullptr = nowhere)
+    auto state_at = [&](int i) { return (static_cast<size_t>(i) * a.H_v + h) * dk * dv + j0; };
+    const bool more = seq >= a.n_s0, own = tr && a.tr_out != nullptr;
+    const float *S0 = more ? a.S0_more : a.S0;
+    float *ST = own ? a.tr_out : seq >= a.st_first ? a.S_T : nullptr;
+    const size_t obase = state_at(own ? seq - a.tr_first : seq - a.st_first);
 
-    if (a.s0_identity || tr || !a.S0) {
+    if (a.s0_identity || tr || !S0) {
         const bool id = a.s0_identity || tr;
         for (int m = tg; m < dk; m += NG) S[m * VC + j] = id && m == j0 + j ? 1.f : 0.f;
     } else {
+        S0 += state_at(more ? seq - a.n_s0 : seq);
 #pragma unroll 4
-        for (int m = tg; m < dk; m += NG) S[m * VC + j] = a.S0[sbase + static_cast<size_t>(m) * dv + j];
+        for (int m = tg; m < dk; m += NG) S[m * VC + j] = S0[static_cast<size_t>(m) * dv + j];
     }
     for (int t = warp; t < kC; t += 8)
         for (int m = dk + lane; m < ks; m += 32) Qs[t * ks + m] = Ks[t * ks + m] = 0.f;
@@ -252,7 +256,7 @@ __global__ void __launch_bounds__(256) gdn_scan_fp32_kernel(const __grid_constan
         for (int m = tg; m < dk; m += NG) {
             const size_t e = static_cast<size_t>(m) * dv + j;
             float x = S[m * VC + j];
-            if (a.S_add) x += a.S_add[sbase + e];
+            if (a.S_add) x += a.S_add[state_at(seq) + e];
             store_state(ST, a.st_bf16, obase + e, x);
         }
     }

@@ -241,7 +241,7 @@ bool init_gdn_exact_tensor_supported(const InitArgs &a, bool) {
            static_cast<long long>(a.n_chunks) * a.H * kD < (1ll << 31);
 }
 
-cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cudaStream_t s) {
+cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cudaStream_t s, bool early) {
     CUtensorMap mapT;
     const uint64_t rows = static_cast<uint64_t>(a.n_chunks) * a.H * kD;
     if (!make_tensor_map_2d(&mapT, a.transitions, 4, kD, rows, kD * 4, 32, kD, true)) return cudaErrorInvalidValue;
@@ -250,7 +250,7 @@ cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cuda
         auto kernel = pool_bf16 ? init_gdn_exact_tensor_kernel<true, Args> : init_gdn_exact_tensor_kernel<false, Args>;
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         if (e != cudaSuccess) return e;
-        return launch_chained(kernel, dim3(a.H, a.n_req), kThreads, kSmemBytes, s, x, mapT);
+        return launch_kernel(early, kernel, dim3(a.H, a.n_req), kThreads, kSmemBytes, s, x, mapT);
     });
 }
 

@@ -206,6 +206,11 @@ void append_launch_order(std::vector<int32_t> &cu, int n_seq) {
 // three launches: the states the first segments reach on their own (no outputs), the composition of every segment's initial
 // state (Eq. 6), all segments with outputs side by side.
 constexpr int kSsdBlock = 128, kGdnBlock = 64;   // tokens
+std::vector<int32_t> segment_tokens(const Cut &c, int block, int T_total) {
+    std::vector<int32_t> at(c.n + 1);
+    for (int i = 0; i <= c.n; ++i) at[i] = std::min<long long>(static_cast<long long>(block) * c.at[i], T_total);
+    return at;
+}
 Cut ssd_cut(const lkv_ssd_desc *d, int n_seq) {
     if (n_seq != 1 || d->io_dtype != LKV_DTYPE_BF16 || d->compute == LKV_COMPUTE_FP32 || d->H < 1 || d->G < 1 || d->H % d->G ||
         d->P != 64 || d->N != 128 || d->T_total < 1)
@@ -223,11 +228,12 @@ int ssd_segmented(SsdArgs a, const Cut &cut, char *scratch, cudaStream_t s) {
     const int segs = cut.n;
     const size_t slot = static_cast<size_t>(a.H) * a.N * a.P;
     float *local = reinterpret_cast<float *>(scratch), *init = local + (segs - 1) * slot, *lam = init + (segs - 1) * slot;
+    const std::vector<int32_t> tokens = segment_tokens(cut, kSsdBlock, a.T_total);
     auto bounds = [&](SsdArgs &b, int n) {
         b.n_seq = n;
         b.cu.ptr = nullptr;
         b.cu.n = 2 * n + 1;
-        for (int i = 0; i <= n; ++i) b.cu.v[i] = std::min<long long>(kSsdBlock * static_cast<long long>(cut.at[i]), a.T_total);
+        for (int i = 0; i <= n; ++i) b.cu.v[i] = tokens[i];
         for (int i = 0; i < n; ++i) b.cu.v[n + 1 + i] = i;
     };
     SsdArgs p1 = a;
@@ -259,47 +265,54 @@ Cut gdn_cut(const lkv_gdn_desc *d, int n_seq) {
     return gdn_cut_blocks((d->T_total - 1) / kGdnBlock + 1, d->H_v, sm_count());
 }
 // local states and transitions of all segments but the last, initial states of all but the first
-size_t gdn_segment_scratch(const lkv_gdn_desc *d, const Cut &c) {
-    if (c.n < 2) return 0;
-    return 3 * static_cast<size_t>(c.n - 1) * sizeof(float) * d->H_v * d->d_k * d->d_v;
+size_t gdn_segment_scratch(const lkv_gdn_desc *d, int n) {
+    if (n < 2) return 0;
+    return 3 * static_cast<size_t>(n - 1) * sizeof(float) * d->H_v * d->d_k * d->d_v;
 }
-int gdn_segmented(GdnArgs a, const Cut &c, char *scratch, cudaStream_t s) {
-    const int n = c.n, m = n - 1;
+// at: first tokens of the n segments and T_total, whole blocks.  tensor: the scans run on the tensor cores, and so does the
+// composition unless the call asked for fp32 arithmetic.
+// own_cut: the library chose the segments, so the passes fill the GPU.  A number of the caller's may leave a third of it idle: then
+// the composition does not start early, because its waiting CTAs would hold the free SMs and leave the last pass packed onto
+// neighbouring SMs, which share an instruction cache (3 segments of 16384 tokens, 32 heads: 339 us against 316; at the
+// library's own cut, 4 segments there, 283 against 286).
+int gdn_segmented(const GdnArgs &a, const lkv_gdn_desc *d, const std::vector<int32_t> &at, bool own_cut, bool tensor, void *scratch, cudaStream_t s) {
+    const int n = static_cast<int>(at.size()) - 1, m = n - 1;
+    const bool io_bf16 = d->io_dtype == LKV_DTYPE_BF16;
     const size_t slot = static_cast<size_t>(a.H_v) * a.d_k * a.d_v;
-    float *local = reinterpret_cast<float *>(scratch), *trans = local + m * slot, *init = trans + m * slot;
-    int at[kMaxSegments + 1];
-    for (int i = 0; i <= n; ++i) at[i] = std::min<long long>(kGdnBlock * static_cast<long long>(c.at[i]), a.T_total);
-    auto ranges = [&](GdnArgs &b, int k, int n_tr) {
-        b.cu.ptr = nullptr;
+    float *local = static_cast<float *>(scratch), *trans = local + m * slot, *init = trans + m * slot;
+    // the scan over the first k segments as sequences and n_tr transition sequences
+    auto scan = [&](GdnArgs &b, int k, int n_tr) {
         b.n_ranges = b.tr_first = k;
         b.n_seq = k + n_tr;
-        b.cu.n = k + 1 + b.n_seq;
-        for (int i = 0; i <= k; ++i) b.cu.v[i] = at[i];
+        std::vector<int32_t> ints(at.begin(), at.begin() + k + 1), order(b.n_seq);
         auto len = [&](int sq) { const int r = sq < k ? sq : sq - k + b.tr_src0; return at[r + 1] - at[r]; };
-        int32_t *order = b.cu.v + k + 1;
         for (int i = 0; i < b.n_seq; ++i) order[i] = i;
-        std::stable_sort(order, order + b.n_seq, [&](int32_t x, int32_t y) { return len(x) > len(y); });
+        std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return len(x) > len(y); });
+        ints.insert(ints.end(), order.begin(), order.end());
+        const int st = place_indices(b.cu, ints, d->workspace, s);
+        if (st != LKV_OK) return st;
+        return (tensor ? launch_gdn_scan_tensor(b, s) : launch_gdn_scan_fp32(b, io_bf16, s)) == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
     };
     GdnArgs p1 = a;
     p1.tr_src0 = 1;
-    ranges(p1, m, m - 1);
     p1.o = nullptr; p1.S_T = local; p1.st_bf16 = 0; p1.n_s0 = 1; p1.tr_out = trans + slot;   // transition of segment j at trans + j slots
-    if (launch_gdn_scan_tensor(p1, s) != cudaSuccess) return LKV_ERR_CUDA;
+    int st = scan(p1, m, std::max(m - 1, 0));
+    if (st != LKV_OK) return st;
     InitArgs k;
     k.states = local; k.transitions = trans; k.S0 = init; k.n_req = m; k.H = a.H_v; k.d_k = a.d_k; k.d_v = a.d_v; k.n_chunks = m;
-    k.off_sel = -1; k.off_ids = n; k.status = a.status; k.idx.ptr = nullptr;
-    int ids = n;
-    for (int r = 0; r < m; ++r) {
-        k.idx.v[r] = ids - n;
-        for (int j = 0; j <= r; ++j) k.idx.v[ids++] = j;
+    k.off_sel = -1; k.off_ids = n; k.status = a.status;
+    std::vector<int32_t> ints(n);
+    for (int r = 0; r < m; ++r) {   // segment r + 1 starts from segments 0 .. r
+        ints[r + 1] = ints[r] + r + 1;
+        for (int j = 0; j <= r; ++j) ints.push_back(j);
     }
-    k.idx.v[m] = ids - n;
-    k.idx.n = ids;
-    if (launch_init_gdn_exact_tensor(k, false, s) != cudaSuccess) return LKV_ERR_CUDA;
+    st = place_indices(k.idx, ints, d->workspace, s);
+    if (st != LKV_OK) return st;
+    const bool tf32 = d->compute != LKV_COMPUTE_FP32 && init_gdn_exact_tensor_supported(k, false);
+    if ((tf32 ? launch_init_gdn_exact_tensor(k, false, s, own_cut) : launch_init_gdn_exact_fp32(k, false, s)) != cudaSuccess) return LKV_ERR_CUDA;
     GdnArgs p3 = a;
-    ranges(p3, n, 0);
     p3.n_s0 = 1; p3.S0_more = init; p3.st_first = n - 1;
-    return launch_gdn_scan_tensor(p3, s) == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
+    return scan(p3, n, 0);
 }
 
 }  // namespace
@@ -330,14 +343,13 @@ int lkv_init_state_batched(const void *states, const void *transitions, const in
 
 // lkv_gdn_fwd, and with `transition` set the scan from S = I with v = 0 whose final state is the chunk transition
 // what: 0 = scan, 1 = chunk transitions (start from S = I, v read as zeros), 2 = one step of the online fold (v read as
-// zeros, S_add added to the final state), 3 = local states and transitions in one launch: d->n_seq = 2 m - 1 sequences,
-// the first m of them scans over the m ranges of d->cu_seqlens (m + 1 entries), the other m - 1 the transitions of ranges
-// 1 .. m-1 (the kernels' "transition sequences")
-// 4 = local states and transitions of every sequence in one launch: d->n_seq = 2 m sequences over the m ranges of
-// d->cu_seqlens, the last m of them transition sequences that write to tr_out
+// zeros, S_add added to the final state), 3 = local states and transitions of every sequence in one launch: d->n_seq = 2 m
+// sequences over the m ranges of d->cu_seqlens, the last m of them transition sequences that write to tr_out
+// segments (of a scan of one sequence): cut there, with this scratch, instead of where gdn_cut says
 static int gdn_impl(const void *q, const void *k, const void *v, const float *g, const float *beta,
                     const float *S0, void *o, void *S_T, const lkv_gdn_desc *d, void *stream, int what,
-                    const float *S_add = nullptr, float *tr_out = nullptr) {
+                    const float *S_add = nullptr, float *tr_out = nullptr, const std::vector<int32_t> *segments = nullptr,
+                    bool own_cut = true, void *scratch = nullptr) {
     const bool transition = what == 1;
     if (!d) return LKV_ERR_NULL;
     if (!dtype_ok(d->io_dtype) || !compute_ok(d->compute) || !dtype_ok(d->state_dtype)) return LKV_ERR_MODE;
@@ -345,11 +357,11 @@ static int gdn_impl(const void *q, const void *k, const void *v, const float *g,
     if (st_bf16 && S_T && S_T == S0) return LKV_ERR_OVERLAP;   // an fp32 input cannot be a bf16 output
     if (d->H_k < 1 || d->H_v < 1 || d->d_k < 1 || d->d_v < 1 || d->H_v % d->H_k != 0) return LKV_ERR_DIM;
     std::vector<int32_t> cu;
-    const int n_ranges = what == 3 ? (d->n_seq + 1) / 2 : what == 4 ? d->n_seq / 2 : d->n_seq;
+    const int n_ranges = what == 3 ? d->n_seq / 2 : d->n_seq;
     int st = check_seqs(d->T_total, n_ranges, d->cu_seqlens, cu);
     if (st != LKV_OK) return st;
     if (d->n_seq == 0) return LKV_OK;
-    if ((transition || what >= 3) && d->d_k != d->d_v) return LKV_ERR_DIM;
+    if ((transition || what == 3) && d->d_k != d->d_v) return LKV_ERR_DIM;
     if (d->T_total > 0 && (!q || !k || !g || !beta)) return LKV_ERR_NULL;
     if (what == 0 && d->T_total > 0 && !v) return LKV_ERR_NULL;
     if (!o && !S_T) return LKV_ERR_NULL;   // nothing to compute
@@ -362,7 +374,7 @@ static int gdn_impl(const void *q, const void *k, const void *v, const float *g,
         // outputs may not overlap inputs (S_T == S0 exactly is the one allowed alias) nor each other
         const size_t es = d->io_dtype == LKV_DTYPE_BF16 ? 2 : 4, T = static_cast<size_t>(d->T_total);
         const size_t qk_b = es * T * d->H_k * d->d_k, v_b = es * T * d->H_v * d->d_v, gb_b = sizeof(float) * T * d->H_v;
-        const size_t st_in = sizeof(float) * static_cast<size_t>(what == 4 ? n_ranges : d->n_seq) * d->H_v * d->d_k * d->d_v;
+        const size_t st_in = sizeof(float) * static_cast<size_t>(n_ranges) * d->H_v * d->d_k * d->d_v;
         const size_t st_b = st_bf16 ? st_in / 2 : st_in;
         const void *in[6] = {q, k, v, g, beta, S0};
         const size_t in_b[6] = {qk_b, qk_b, v ? v_b : 0, gb_b, gb_b, S0 ? st_in : 0};
@@ -379,7 +391,7 @@ static int gdn_impl(const void *q, const void *k, const void *v, const float *g,
     a.n_seq = d->n_seq; a.T_total = d->T_total; a.H_k = d->H_k; a.H_v = d->H_v; a.d_k = d->d_k; a.d_v = d->d_v;
     a.scale = d->scale != 0.f ? d->scale : 1.0f / sqrtf(static_cast<float>(d->d_k));
     a.s0_identity = transition ? 1 : 0;
-    a.n_ranges = n_ranges; a.tr_first = n_ranges; a.tr_src0 = what == 3 ? 1 : 0; a.tr_out = tr_out;
+    a.n_ranges = n_ranges; a.tr_first = n_ranges; a.tr_src0 = 0; a.tr_out = tr_out;
     a.n_s0 = d->n_seq; a.st_first = 0; a.S0_more = nullptr;
     a.status = static_cast<int32_t *>(d->workspace);
     const bool io_bf16 = d->io_dtype == LKV_DTYPE_BF16;
@@ -397,16 +409,26 @@ static int gdn_impl(const void *q, const void *k, const void *v, const float *g,
         use_tensor = tensor_fits;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (segments) {
+        // S_T on top of S0 is written while S0 is read: it goes through the scratch, behind what gdn_segmented uses of it
+        const bool alias = S_T && S_T == S0;
+        const size_t st_elems = static_cast<size_t>(d->H_v) * d->d_k * d->d_v;
+        if (alias) a.S_T = static_cast<float *>(scratch) + 3 * (segments->size() - 2) * st_elems;
+        st = gdn_segmented(a, d, *segments, own_cut, use_tensor, scratch, s);
+        if (st == LKV_OK && alias && cudaMemcpyAsync(S_T, a.S_T, sizeof(float) * st_elems, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+            st = LKV_ERR_CUDA;
+        return st;
+    }
     // A long sequence that leaves SMs idle runs in segments (a caller whose workspace is smaller than
     // lkv_workspace_bytes() asked for gets the plain scan; S_T on top of S0 would be written while S0 is read)
     const Cut cut = use_tensor && what == 0 && S_T != S0 && o ? gdn_cut(d, d->n_seq) : Cut{1, {0}};
     const size_t head = ws_bytes_for(2 * d->n_seq + 1, kScanIdxCap);
-    if (cut.n > 1 && d->workspace_bytes >= head + gdn_segment_scratch(d, cut))
-        return gdn_segmented(a, cut, static_cast<char *>(d->workspace) + head, s);
-    if (what >= 3) {
-        // launch order over all sequences, longest first; transition sequence j runs over range j - m + (1 or 0)
+    if (cut.n > 1 && d->workspace_bytes >= head + gdn_segment_scratch(d, cut.n))
+        return gdn_segmented(a, d, segment_tokens(cut, kGdnBlock, d->T_total), true, true, static_cast<char *>(d->workspace) + head, s);
+    if (what == 3) {
+        // launch order over all sequences, longest first; transition sequence j runs over range j - m
         std::vector<int32_t> order(d->n_seq);
-        auto len = [&](int sq) { const int r = sq < n_ranges ? sq : sq - n_ranges + (what == 3 ? 1 : 0); return cu[r + 1] - cu[r]; };
+        auto len = [&](int sq) { const int r = sq % n_ranges; return cu[r + 1] - cu[r]; };
         for (int i = 0; i < d->n_seq; ++i) order[i] = i;
         std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return len(x) > len(y); });
         cu.insert(cu.end(), order.begin(), order.end());
@@ -474,24 +496,27 @@ int lkv_init_state_fold(const void *states, const void *k, const float *g, const
     return LKV_OK;
 }
 
-// n_segments == 0: as many segments as keep both scanning passes within one round of CTAs on this GPU -- (2 n - 3) H_v and
-// n H_v CTAs, one per SM -- and no segment shorter than 512 tokens
-static int auto_segments(const lkv_gdn_desc *d) {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        cudaGetLastError();
-        sms = 148;
+// Where the sequence is cut.  n_segments == 0: as lkv_gdn_fwd cuts it; what runs in fp32 arithmetic into as many segments as keep
+// both scanning passes within one round of CTAs on this GPU -- (2 n - 3) H_v and n H_v CTAs, one per SM -- and none shorter
+// than 512 tokens.
+static std::vector<int32_t> segments_of(const lkv_gdn_desc *d, int n_segments) {
+    if (n_segments == 0) {
+        if (d->io_dtype == LKV_DTYPE_BF16 && d->compute != LKV_COMPUTE_FP32 && d->d_k == 128 && d->d_v == 128)
+            return segment_tokens(gdn_cut(d, 1), kGdnBlock, d->T_total);
+        n_segments = std::max(1, std::min((sm_count() / d->H_v + 3) / 2, d->T_total / 512));
     }
-    int n = (sms / (d->H_v > 0 ? d->H_v : 1) + 3) / 2;
-    if (n > d->T_total / 512) n = d->T_total / 512;
-    return n < 1 ? 1 : n;
+    // equal, on multiples of 64 tokens: every block of the segmented scan is a block of the plain one
+    const long long per = (static_cast<long long>(d->T_total) + n_segments - 1) / n_segments;
+    std::vector<int32_t> at(n_segments + 1);
+    for (int i = 0; i <= n_segments; ++i) at[i] = static_cast<int32_t>(std::min<long long>(i * ((per + 63) / 64 * 64), d->T_total));
+    return at;
 }
 
 size_t lkv_gdn_segmented_scratch_bytes(const lkv_gdn_desc *d, int n_segments) {
-    if (!d || n_segments < 0 || d->H_v < 1 || d->d_k < 1 || d->d_v < 1) return 0;
-    if (n_segments == 0) n_segments = auto_segments(d);
+    if (!d || n_segments < 0 || d->T_total < 0 || d->H_v < 1 || d->d_k < 1 || d->d_v < 1) return 0;
+    if (n_segments == 0) n_segments = static_cast<int>(segments_of(d, 0).size()) - 1;
     if (n_segments < 2) return 0;
-    return sizeof(float) * static_cast<size_t>(4 * n_segments - 3) * d->H_v * d->d_k * d->d_v;
+    return sizeof(float) * (4 * static_cast<size_t>(n_segments) - 3) * d->H_v * d->d_k * d->d_v;
 }
 
 int lkv_gdn_fwd_segmented(const void *q, const void *k, const void *v, const float *g, const float *beta,
@@ -499,9 +524,11 @@ int lkv_gdn_fwd_segmented(const void *q, const void *k, const void *v, const flo
                           void *scratch, size_t scratch_bytes, void *stream) {
     if (!d) return LKV_ERR_NULL;
     if (n_segments < 0) return LKV_ERR_DIM;
+    std::vector<int32_t> at;
     if (n_segments == 0) {
         if (d->H_v < 1 || d->T_total < 0) return LKV_ERR_DIM;
-        n_segments = auto_segments(d);
+        at = segments_of(d, 0);
+        n_segments = static_cast<int>(at.size()) - 1;
     }
     if (n_segments == 1) return lkv_gdn_fwd(q, k, v, g, beta, S0, o, S_T, d, stream);
     if (d->n_seq != 1 || d->state_dtype != LKV_DTYPE_F32) return LKV_ERR_UNSUPPORTED;   // one sequence, fp32 final state
@@ -510,55 +537,14 @@ int lkv_gdn_fwd_segmented(const void *q, const void *k, const void *v, const flo
     if (d->cu_seqlens && (d->cu_seqlens[0] != 0 || d->cu_seqlens[1] != d->T_total)) return LKV_ERR_INDEX;
     if (!scratch || scratch_bytes < lkv_gdn_segmented_scratch_bytes(d, n_segments)) return LKV_ERR_WORKSPACE;
     if (!aligned16(scratch)) return LKV_ERR_ALIGN;
-    if (!o && !S_T) return LKV_ERR_NULL;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int n_seg = n_segments, n_st = n_seg - 1;
-    const size_t slot = static_cast<size_t>(d->H_v) * d->d_k * d->d_v;   // floats per state of all heads
-    float *pool = static_cast<float *>(scratch);                        // S_local of segments 0 .. n_st-1, then T of 1 .. n_st-1
-    float *trans = pool + (static_cast<size_t>(n_st) - 1) * slot;       // T of segment j at trans + j slots (slot 0 is never read)
-    float *S_init = pool + (2 * static_cast<size_t>(n_st) - 1) * slot;  // [n_seg]
-    float *S_fin = S_init + static_cast<size_t>(n_seg) * slot;          // [n_seg]; first the initial states of pass 1
-    // segment boundaries on multiples of 64 tokens, so that every block of the segmented scan is a block of the plain one
-    const int per = ((d->T_total + n_seg - 1) / n_seg + 63) / 64 * 64;
-    std::vector<int32_t> bounds(n_seg + 1);
-    for (int i = 0; i <= n_seg; ++i) bounds[i] = std::min<long long>(static_cast<long long>(i) * per, d->T_total);
-    // ---- pass 1: local states of segments 0 .. n_st-1 (segment 0 from S0) and transitions of segments 1 .. n_st-1, one launch
-    if (cudaMemsetAsync(S_fin, 0, sizeof(float) * slot * n_st, s) != cudaSuccess) return LKV_ERR_CUDA;
-    if (S0 && cudaMemcpyAsync(S_fin, S0, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return LKV_ERR_CUDA;
-    lkv_gdn_desc d1 = *d;
-    d1.n_seq = 2 * n_st - 1;
-    d1.T_total = bounds[n_st];
-    d1.cu_seqlens = bounds.data();
-    int st = gdn_impl(q, k, v, g, beta, S_fin, nullptr, pool, &d1, stream, 3);
-    if (st != LKV_OK) return st;
-    // ---- pass 2: the state each segment starts from, by exact composition (Eq. 6) over the segments before it
-    if (S0) {
-        if (cudaMemcpyAsync(S_init, S0, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return LKV_ERR_CUDA;
-    } else if (cudaMemsetAsync(S_init, 0, sizeof(float) * slot, s) != cudaSuccess) {
-        return LKV_ERR_CUDA;
-    }
-    {
-        std::vector<int32_t> ids, cu_k(n_st + 1, 0);
-        for (int r = 0; r < n_st; ++r) {
-            for (int j = 0; j <= r; ++j) ids.push_back(j);
-            cu_k[r + 1] = static_cast<int32_t>(ids.size());
-        }
-        lkv_init_desc di{};
-        di.family = LKV_FAMILY_GDN; di.H = d->H_v; di.d_k = d->d_k; di.d_v = d->d_v; di.n_chunks = n_st;
-        di.state_dtype = LKV_DTYPE_F32; di.sel_index = 0; di.compute = d->compute; di.chunk_ids = nullptr;
-        di.workspace = d->workspace; di.workspace_bytes = d->workspace_bytes;
-        st = lkv_init_state_batched(pool, trans, ids.data(), cu_k.data(), n_st, LKV_INIT_EXACT, nullptr, S_init + slot, &di, stream);
-        if (st != LKV_OK) return st;
-    }
-    // ---- pass 3: every segment scanned from its initial state, all at once
-    lkv_gdn_desc d3 = *d;
-    d3.n_seq = n_seg;
-    d3.cu_seqlens = bounds.data();
-    st = gdn_impl(q, k, v, g, beta, S_init, o, S_fin, &d3, stream, 0);
-    if (st != LKV_OK) return st;
-    if (S_T && cudaMemcpyAsync(S_T, S_fin + static_cast<size_t>(n_seg - 1) * slot, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return LKV_ERR_CUDA;
-    return LKV_OK;
+    // the longest index lists of the three launches
+    const int n = n_segments;
+    if (n > (1 << 15) || !d->workspace || d->workspace_bytes < ws_bytes_for(2 * (2 * n - 3) + 1, kScanIdxCap) ||
+        d->workspace_bytes < ws_bytes_for(n + n * (n - 1) / 2, kInitIdxCap))
+        return LKV_ERR_WORKSPACE;
+    const bool own_cut = !at.empty();
+    if (!own_cut) at = segments_of(d, n);
+    return gdn_impl(q, k, v, g, beta, S0, o, S_T, d, stream, 0, nullptr, nullptr, &at, own_cut, scratch);
 }
 
 int lkv_stage_chunks(const void *host_states, const void *host_transitions, const int32_t *chunk_ids, int n_ids,
@@ -618,7 +604,7 @@ int lkv_gdn_chunk_artifacts(const void *k, const void *v, const float *g, const 
     lkv_gdn_desc d2 = *d;
     d2.n_seq = 2 * d->n_seq;   // every chunk twice: once as a scan from the empty state, once as a transition sequence
     // q is not needed for the states: the key tensor stands in for it (its read-outs are not written)
-    return gdn_impl(k, k, v, g, beta, nullptr, nullptr, states, &d2, stream, 4, nullptr, transitions);
+    return gdn_impl(k, k, v, g, beta, nullptr, nullptr, states, &d2, stream, 3, nullptr, transitions);
 }
 
 int lkv_mamba_chunk_logdecay(const float *dt, const float *A, float *logdecay, const lkv_ssd_desc *d, void *stream) {
@@ -730,7 +716,7 @@ size_t lkv_workspace_bytes(int which, const void *desc, int n_units, int n_index
         case LKV_WS_INIT: return ws_bytes_for(2 * n_units + 1 + n_index, kInitIdxCap);
         case LKV_WS_GDN: {
             const lkv_gdn_desc *d = static_cast<const lkv_gdn_desc *>(desc);
-            return ws_bytes_for(2 * n_units + 1, kScanIdxCap) + gdn_segment_scratch(d, gdn_cut(d, n_units));
+            return ws_bytes_for(2 * n_units + 1, kScanIdxCap) + gdn_segment_scratch(d, gdn_cut(d, n_units).n);
         }
         case LKV_WS_SSD: {
             const lkv_ssd_desc *d = static_cast<const lkv_ssd_desc *>(desc);

@@ -243,6 +243,31 @@ def test_segmented_prefill_equals_the_plain_scan_and_the_oracle(case):
     assert torch.equal(o[:per], o_p[:per])
 
 
+@pytest.mark.parametrize("T, n, d, io", [(3000, 0, 128, "bf16"), (1100, 5, 128, "bf16"), (640, 3, 64, "f32"), (6500, 100, 128, "bf16")])
+def test_segmented_prefill_shares_the_scan_own_segments(T, n, d, io):
+    """n = 0 is the cut of lkv_gdn_fwd, bit for bit; S_T may be S0; a list of segments too long for the kernel parameters travels
+    through the workspace."""
+    import torch
+    rng = np.random.default_rng(T)
+    H_k, H_v = 1, 2
+    tok = wl.gdn_tokens(rng, T, H_k, H_v, d, d, io=io, live_chunk_len=256)
+    dt = torch.bfloat16 if io == "bf16" else None
+    args = (dev(tok["q"], dt), dev(tok["k"], dt), dev(tok["v"], dt), dev(tok["g"]), dev(tok["beta"]))
+    S0 = dev(rng.standard_normal((1, H_v, d, d)).astype(np.float32))
+    ws = torch.zeros(1 << 16, dtype=torch.uint8, device="cuda")
+    o, ST = b.lkv_gdn_fwd_segmented(*args, S0, n_segments=n, workspace_t=ws)
+    o_p, ST_p = b.lkv_gdn_fwd(*args, S0)
+    if n == 0:
+        assert torch.equal(o, o_p) and torch.equal(ST, ST_p)
+        small = torch.zeros(4096, dtype=torch.uint8, device="cuda")
+        o_p, _ = b.lkv_gdn_fwd(*args, S0, workspace_t=small)
+        assert not torch.equal(o, o_p)                    # it does run in segments
+    tol = TOL_BF16 if io == "bf16" else TOL_F32
+    assert maxrel(host(o), host(o_p)) <= tol and maxrel(host(ST), host(ST_p)) <= tol
+    o2, ST2 = b.lkv_gdn_fwd_segmented(*args, S0, None, S0, n_segments=n, workspace_t=ws)
+    assert ST2 is S0 and torch.equal(o2, o) and torch.equal(ST2, ST)
+
+
 @pytest.mark.parametrize("family", ["gdn", "mamba2"])
 def test_staging_from_a_host_pool_feeds_the_initialisers(family):
     """The cache lives in (pinned) host memory; the chunks a batch names are staged once each into a compact device pool
