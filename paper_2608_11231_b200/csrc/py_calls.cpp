@@ -160,16 +160,16 @@ void check(int st, const char *where) {
 // of a long index list; the engine's other threads run on meanwhile.  The arguments are plain C values by then, what they
 // point to is held by the caller's frame.  A call may be several launches that pass data through the workspace, and threads that
 // share a stream share its workspace: calls on one workspace take turns (the lock is picked by the workspace's address).
+std::mutex g_turns[64];
 template <typename... P, typename... A>
 void call(const char *where, const void *workspace, int (*f)(P...), A... args) {
-    static std::mutex turns[64];
     int st;
     {
         struct Released {
             PyThreadState *state = PyEval_SaveThread();
             ~Released() { PyEval_RestoreThread(state); }
         } released;
-        std::lock_guard<std::mutex> turn(turns[(reinterpret_cast<uintptr_t>(workspace) >> 9) % 64]);
+        std::lock_guard<std::mutex> turn(g_turns[(reinterpret_cast<uintptr_t>(workspace) >> 9) % 64]);
         st = f(args...);
     }
     check(st, where);
