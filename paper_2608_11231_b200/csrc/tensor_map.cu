@@ -21,6 +21,22 @@ EncodeTiledFn encode_fn() {
     }();
     return fn;
 }
+
+// `encode` with a current context.  A driver call, unlike a runtime call, does not make the device's primary context current on a
+// thread that has made no CUDA call yet (an engine's worker whose tensors all came out of the caching allocator): there the
+// encode fails, the runtime is made to set the context up, and the encode runs again.
+template <typename F>
+bool with_context(F &&encode) {
+    CUresult r = encode();
+    if (r == CUDA_ERROR_INVALID_CONTEXT || r == CUDA_ERROR_NOT_INITIALIZED) {
+        if (cudaFree(nullptr) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        r = encode();
+    }
+    return r == CUDA_SUCCESS;
+}
 }  // namespace
 
 bool make_tensor_map_2d(CUtensorMap *map, const void *base, int elem_bytes, uint64_t inner, uint64_t rows,
@@ -32,10 +48,9 @@ bool make_tensor_map_2d(CUtensorMap *map, const void *base, int elem_bytes, uint
     const cuuint32_t box[2] = {box_inner, box_rows};
     const cuuint32_t estride[2] = {1, 1};
     const CUtensorMapDataType dt = elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-    const CUresult r = fn(map, dt, 2, const_cast<void *>(base), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    return with_context([&] { return fn(map, dt, 2, const_cast<void *>(base), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
                           swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE); });
 }
 
 bool make_tensor_map_cols64(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows, uint64_t row_stride_bytes,
@@ -46,10 +61,9 @@ bool make_tensor_map_cols64(CUtensorMap *map, const void *base, uint64_t inner, 
     const cuuint64_t gstride[2] = {row_stride_bytes, 128};
     const cuuint32_t box[3] = {64, box_rows, box_blocks};
     const cuuint32_t estride[3] = {1, 1, 1};
-    const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), gdim, gstride, box, estride,
+    return with_context([&] { return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), gdim, gstride, box, estride,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE); });
 }
 
 }  // namespace lkv

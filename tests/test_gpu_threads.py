@@ -2,6 +2,7 @@
 a workspace) do not mix."""
 import threading
 import time
+from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
 import pytest
@@ -56,18 +57,13 @@ def test_threads_that_share_a_stream():
     work = [(b.lkv_gdn_fwd, a) for a in gdn] + [(b.lkv_ssd_fwd, a) for a in ssd]
     alone = [f(*a) for f, a in work]
     torch.cuda.synchronize()
-    wrong = []
 
     def engine(i):
         f, a = work[i]
         for _ in range(20):
-            o, S = f(*a)
-            if not (torch.equal(o, alone[i][0]) and torch.equal(S, alone[i][1])):
-                wrong.append(i)
+            o, S = f(*a)   # the thread's first CUDA call
+            assert torch.equal(o, alone[i][0]) and torch.equal(S, alone[i][1])
 
-    threads = [threading.Thread(target=engine, args=(i,)) for i in range(len(work))]
-    for t in threads:
-        t.start()
-    for t in threads:
-        t.join()
-    assert not wrong
+    with ThreadPoolExecutor(len(work)) as pool:
+        for r in [pool.submit(engine, i) for i in range(len(work))]:
+            r.result()
