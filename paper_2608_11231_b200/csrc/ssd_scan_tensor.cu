@@ -1,6 +1,7 @@
 // Chunkwise Mamba-2 (SSD) scan on the 5th-generation tensor cores (Eq. 1 with Eq. 2), for
 // headdim P = 64, d_state N = 128 and bf16 x/B/C/y.  One CTA owns one sequence and TWO heads of one group and walks
-// the sequence in blocks of up to 128 tokens with the heads' states carried on chip.
+// the sequence in tiles of 128 tokens with the heads' states carried on chip.  A tile is one block of the scan unless its decay
+// is too strong (below).
 //
 // No decay appears inside a contraction.  With l the running sum of dt * A_h inside a block (in log2 units, n its last
 // token) and R a scale exponent of the block,
@@ -13,8 +14,15 @@
 // The state as held, S^ + B^T X^, is the next block's S^ with R - l_n for R: it is multiplied by a power of two only when
 // that would pass kMaxScale, every block to every seventh with decays as strong as the benchmark's.
 // Scaling by powers of two commutes with rounding, and fp32 and bf16 have the same exponent range, so nothing is lost
-// while the exponents stay in range: a block ends before the token at which |l| would pass kMaxRange (it always keeps one
-// token).
+// while the exponents stay in range.
+//
+// Where |l| would pass kMaxRange inside a tile, in either head, the tile is scanned in several blocks, each with its own R, that end on
+// multiples of 16 tokens: only the chain -- (Y2), (S), state pass -- runs once per block, 1.5 K cycles; loads, G, mask, X^ and
+// outputs run once per tile as before.  Where 16 tokens are still too many (12 log2 units a token and more) a block of fewer
+// tokens is a "unit" of its own, for which X^ is written and y read separately, 3 K cycles.  32 sequences x 2048 tokens x 80 heads, dt
+// of 0.14 on average: A = -0.02 or -1 .. -7.4 375 / 382 us, A uniform in -1 .. -16 475 us; dt of 0.8: A = -4 737 us, A uniform in
+// -1 .. -16 3200 us.  (Whole tiles loaded and scanned for every block: 370 / 378, 628, 1450, 3770 us.  The form with the decays
+// inside the mask: 622 / 620, 650, 660, 960 us.)
 //
 // Everything is held transposed so that the tiles have M = 128 rows = 2 heads x 64 features (all 128 TMEM lanes):
 //   (G)    G     = C B^T                     [128 t x 128 i], K = n        tcgen05; tril -> bf16 tile in shared memory (prep warps)
@@ -28,16 +36,16 @@
 // shared-memory port (128 bytes per clock, the scarcest thing on chip here) is spared the write-back and three reads.
 // The chain from block to block is (Y2), (S) -> state pass; X^, G and the outputs hang off it.
 //
-// Bound: per block the CTA takes in 96 KB (B, C, two X tiles) and writes 32 KB; an SM takes in about 40 bytes per clock
+// Bound: per tile the CTA takes in 96 KB (B, C, two X tiles) and writes 32 KB; an SM takes in about 40 bytes per clock
 // from L2, 2.4 K cycles, and the copy bandwidth of the memory gives 2.9 K for the X and y bytes alone.  Measured: 3.2 K
-// cycles a block on an idle GPU, 3.4 K on a full one, 2.0 K without outputs (one head per CTA and the decays inside the
+// cycles a tile on an idle GPU, 3.4 K on a full one, 2.0 K without outputs (one head per CTA and the decays inside the
 // mask took 7.7 K for the same two heads).  32 sequences x 4096 tokens x 80 heads: 1370 -> 725 us.
 //
-// The hot loops are rolled where they repeat: eight programs run side by side, each once per block, and fetched unrolled
+// The hot loops are rolled where they repeat: eight programs run side by side, each once per tile, and fetched unrolled
 // (60 KB of code) every role took three to five times as long as its instructions (the scalar warp 5300 cycles for 250).
 //
 // Warps 0-7 outputs (warpgroup = half of the tokens), 8-15 state (warpgroup = half of n), 16-23 X^ (warpgroup = half of the
-// tokens) and then the mask, 24 TMA loads, 25 MMA issue of (S), 26 MMA issue of (G), (Y2), (Y1), 27 block limits and scalars.
+// tokens) and then the mask, 24 TMA loads, 25 MMA issue of (S), 26 MMA issue of (G), (Y2), (Y1), 27 blocks and scalars.
 // All waits on mbarriers are bounded.
 #include <string.h>
 
@@ -52,7 +60,7 @@ using namespace tc;
 
 constexpr int kP = 64;     // headdim
 constexpr int kN = 128;    // d_state
-constexpr int kQ = 128;    // tokens per block
+constexpr int kQ = 128;    // tokens per tile
 constexpr int kThreads = 896;
 
 // shared-memory map (bytes, after 1024-byte alignment); every tile row is 128 bytes, 128-byte swizzle
@@ -63,17 +71,23 @@ constexpr int kOffY = kOffX + 2 * kTile;         // y likewise, staged for the T
 constexpr int kOffG = kOffY + 2 * kTile;         // tril(G) bf16: columns i < 64 of all rows t (16 KB), then i >= 64 of rows t >= 64 (8 KB)
 constexpr int kOffSlot = kOffG + kTile + kTile / 2;
 constexpr int kSlots = 4;
-struct Slot {            // block descriptor
-    uint2 s[2][kQ / 2];  // 2^{R - l_t} dt_t of two tokens per head (0 beyond the block), as two bf16 parts: {high pair, low pair}
+constexpr int kMaxBlocks = kQ / 16;
+// A unit: tokens o .. o + n - 1 of the tile that begins at token `row`, as a rule the whole tile.  It is scanned in nb blocks, block j
+// in steps of 16 tokens from kb[j - 1] (k0) to kb[j]
+struct Slot {            // its descriptor
+    uint2 s[2][kQ / 2];  // 2^{R - l_t} dt_t of two tokens per head (0 outside the unit), as two bf16 parts: {high pair, low pair}
     float e[2][kQ];      // 2^{l_t - R}
-    float f2[2], e2[2];  // exponents: R minus the R that the block before left, l_n - R
-    int start, n;        // first token, number of tokens
-    int pad[2];
+    int fin, last;       // the last unit of its tile; of the sequence
+    int row, o, n, k0, nb, pad;
+    int kb[kMaxBlocks];
+    float f2[2][kMaxBlocks], e2[2];   // exponents: R of a block minus the R that the one before left, l_n - R of the last one
+    int pad2[2];
 };
+static_assert(sizeof(Slot) % 16 == 0, "vector stores");
 constexpr int kSmemBytes = kOffSlot + kSlots * static_cast<int>(sizeof(Slot)) + 1024;
 static_assert(kSmemBytes + 512 <= 227 * 1024, "shared memory budget");
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kMaxRange = 200.f;               // log2 units of decay inside one block
+constexpr float kMaxRange = 200.f;               // log2 units of decay inside one block of the scan
 constexpr float kMaxScale = 104.f;               // R - l_n at most: X^ and S^ grow to about 2^104.  A state that is scaled back starts
                                                  // from R = 0, or from below (to -96) where the block's own decay leaves no other choice
 
@@ -94,8 +108,8 @@ struct Bars {
     uint64_t sc_ready[kSlots];
     // the eight output, state or prep warps
     uint64_t y_free, hb_ready, x_free, x2_ready, mask_done;
-    // readers of a block descriptor that nothing later waits for: the output and state warps (state warps alone when no outputs are
-    // wanted) and the TMA warp.  (The other readers are done before the products that the state and the outputs wait for.)
+    // output and state warps (state warps alone when no outputs are wanted), the last readers of a descriptor: the others are done
+    // before the products that these wait for
     uint64_t slot_free[kSlots];
 };
 constexpr int kBars1 = 9;
@@ -137,20 +151,78 @@ __device__ __forceinline__ void copy_state32(uint32_t lane_base, int n0, const u
     for (int c = 0; c < 16; ++c) w[c] = pack_bf16(__uint_as_float(rr[2 * c]), __uint_as_float(rr[2 * c + 1]));
     tmem_st16(lane_base + kTmSb + n0 / 2, w);
 }
-// 64 columns of the fp32 state multiplied by 2^ex in place, in two steps: the factor may lie below the fp32 range where its
-// product with the state does not.  Not inlined: one block in several needs it.
-__device__ __noinline__ void scale_state64(uint32_t taddr, float ex) {
-    const float f = ex2(0.5f * ex);
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
-        uint32_t rr[16];
-        tmem_ld16(taddr + 16 * q, rr);
-        tmem_ld_wait();
+// Scale exponent of a block of decay ln, R what the block before has left
+__device__ __forceinline__ float scale_into(float R, float ln) {
+    float Rn = R;
+    if (fabsf(R - ln) > kMaxScale) Rn = ln < 0.f ? fminf(0.f, floorf(kMaxScale + ln)) : fmaxf(0.f, ceilf(ln - kMaxScale));
+    if (fabsf(ln) > kMaxRange) Rn = rintf(ln);   // a single token of violent decay: nothing of the state is left
+    return Rn;
+}
+__device__ __forceinline__ void append_block(Slot &sl, int nb, int hd, float f2, float e2, int end) {
+    sl.f2[hd][nb] = f2;
+    sl.e2[hd] = e2;
+    sl.kb[nb] = (end + 15) / 16;
+}
+// The blocks of a unit whose decay leaves the range.  A block ends before the first token that does, in either head, on a multiple of 16
+// tokens: then the blocks of a unit share no step of the products, and X^ is written, G masked and y read once for all of
+// them.  Where 16 tokens are too many, they end the unit too.  Per lane, eight tokens: l from the first token of the unit ->
+// l - R of their block; dt and l zero beyond the unit.  Rare, and kept out of the scalar warp's loop.
+struct Cut {
+    float l[8], dt[8], keep[8];   // keep: dt of the tokens that the unit leaves
+    float R, total;
+    int o, end, nb;               // first token of the unit; end of the tile -> of the unit
+};
+__device__ __noinline__ void cut_unit(Slot &sl, Cut &c, int hd, int hl) {
+    float l[8], base = 0.f, R = c.R, total = c.total;
+    const int o = c.o, end = c.end;
+    int cur = o, nb = 0;
 #pragma unroll
-        for (int c = 0; c < 16; ++c) rr[c] = __float_as_uint(__uint_as_float(rr[c]) * f * f);
-        tmem_st16(taddr + 16 * q, rr);
+    for (int j = 0; j < 8; ++j) l[j] = c.l[j];
+#pragma unroll 1
+    for (bool open = true; open;) {
+        unsigned bad = end;
+#pragma unroll
+        for (int j = 7; j >= 0; --j)
+            if (8 * hl + j >= cur && !(fabsf(l[j] - base) <= kMaxRange)) bad = min(bad, 8 * hl + j);
+        int m = __reduce_min_sync(0xffffffffu, bad);
+        open = m < end;
+        if (open) {
+            if ((m & ~15) > cur) {
+                m &= ~15;
+            } else {
+                if (nb > 0) break;
+                m = max(m, o + 1);
+                open = false;
+            }
+        }
+        float lm = 0.f;   // l of the block's last token
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (j == ((m - 1) & 7)) lm = l[j];
+        lm = __shfl_sync(0xffffffffu, lm, (m - 1) >> 3, 16);
+        const float ln = lm - base, Rn = scale_into(R, ln);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (8 * hl + j >= cur && 8 * hl + j < m) l[j] -= base + Rn;   // (not looked at again)
+        if (hl == 0) append_block(sl, nb, hd, Rn - R, ln - Rn, m);
+        R = Rn - ln;
+        total += ln;
+        base = lm;
+        cur = m;
+        ++nb;
     }
-    tmem_st_wait();
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const bool out = 8 * hl + j >= cur;
+        const float dt = c.dt[j];
+        c.keep[j] = out ? dt : 0.f;
+        c.dt[j] = out ? 0.f : dt;
+        c.l[j] = out ? 0.f : l[j];
+    }
+    c.R = R;
+    c.total = total;
+    c.end = cur;
+    c.nb = nb;
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -193,7 +265,7 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
         for (int i = 0; i < 2; ++i) mbar_init(bp++, has_y ? 2 : 1);
         for (int i = 0; i < kSlots; ++i) mbar_init(bp++, 1);
         for (int i = 0; i < 5; ++i) mbar_init(bp++, 8);
-        for (int i = 0; i < kSlots; ++i) mbar_init(bp++, has_y ? 17 : 9);
+        for (int i = 0; i < kSlots; ++i) mbar_init(bp++, has_y ? 16 : 8);
         mbar_fence_init();
     }
     if (warp == 0) tmem_alloc(&tmem_base, kTmemCols);
@@ -211,109 +283,120 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
         const int hd = lane >> 4, hl = lane & 15;
         const float Ah = a.A[hd ? h1 : h0] * kLog2e;
         const float *dth = a.dt + (hd ? h1 : h0);
-        // dt of the next block and of the one after it (a load from DRAM takes as long as a block without outputs)
+        // dt of the next tile and of the one after it (a load from DRAM takes as long as a block without outputs)
         float dt[8], dt2[8];
         auto fetch_dt = [&](float (&d)[8], int t0) {
             const float *p = dth + static_cast<size_t>(t0 + 8 * hl) * a.H;
 #pragma unroll
             for (int j = 0; j < 8; ++j) d[j] = t0 + 8 * hl + j < t_end ? p[static_cast<size_t>(j) * a.H] : 0.f;
         };
-        int t0 = t_begin;
+        int t0 = t_begin, o = 0;   // tile, first token of the unit in it
         float R = 0.f, total = 0.f;
         fetch_dt(dt, t0);
         fetch_dt(dt2, t0 + kQ);
-        // (never leaves the loop early: every pass advances t0 whatever the waits say)
+        // (never leaves the loop early: every pass advances whatever the waits say)
 #pragma unroll 1
         for (int b = 0; t0 < t_end; ++b) {
-            float l2[8], dv[8];
+            Slot &sl = slots[b % kSlots];
+            float l2[8], run = 0.f, far = 0.f;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) dv[j] = dt[j];
-            int n = min(kQ, t_end - t0);
-            // the block ends before the first token whose decay leaves the range, in either head: then again without the rest
-#pragma unroll 1
-            for (;;) {
-                float run = 0.f;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    run = fmaf(dv[j], Ah, run);
-                    l2[j] = run;
-                }
-                float tot = run;
-#pragma unroll
-                for (int o = 1; o < 16; o <<= 1) {
-                    const float up = __shfl_up_sync(0xffffffffu, tot, o, 16);
-                    if (hl >= o) tot += up;
-                }
-                const float before = tot - run;
-                int bad = kQ;
-#pragma unroll
-                for (int j = 7; j >= 0; --j) {
-                    l2[j] += before;
-                    if (fabsf(l2[j]) > kMaxRange) bad = 8 * hl + j;
-                }
-                unsigned any = __ballot_sync(0xffffffffu, bad < n);
-                if (!any || n == 1) break;
-#pragma unroll 1
-                for (; any; any &= any - 1) n = min(n, __shfl_sync(0xffffffffu, bad, __ffs(any) - 1));
-                n = max(n, 1);
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (8 * hl + j >= n) dv[j] = 0.f;
+            for (int j = 0; j < 8; ++j) {
+                run = fmaf(dt[j], Ah, run);   // (the tokens before the unit have been set to zero)
+                l2[j] = run;
             }
-            const float ln = __shfl_sync(0xffffffffu, l2[7], 15, 16);   // tokens beyond the block have dt = 0
-            float Rn = R;
-            if (fabsf(R - ln) > kMaxScale) Rn = ln < 0.f ? fminf(0.f, floorf(kMaxScale + ln)) : fmaxf(0.f, ceilf(ln - kMaxScale));
-            if (fabsf(ln) > kMaxRange) Rn = rintf(ln);   // a single token of violent decay: nothing of the state is left
-            const int start = t0;
-            t0 += n;
+            float tot = run;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) dt[j] = dt2[j];
-            if (n < kQ && t0 < t_end) fetch_dt(dt, t0);
-            fetch_dt(dt2, t0 + kQ);
+            for (int k = 1; k < 16; k <<= 1) {
+                const float up = __shfl_up_sync(0xffffffffu, tot, k, 16);
+                if (hl >= k) tot += up;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                l2[j] += tot - run;
+                far = fmaxf(far, fabsf(l2[j]));
+            }
             if (b >= kSlots) mbar_wait(&bars.slot_free[b % kSlots], ((b - kSlots) / kSlots) & 1, &dead, a.status);
             __syncwarp();
-            Slot &sl = slots[b % kSlots];
+            int cur = min(kQ, t_end - t0), nb = 1;
+            Cut c;
+            if (__builtin_expect(__any_sync(0xffffffffu, !(far <= kMaxRange)), 0)) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    c.l[j] = l2[j];
+                    c.dt[j] = dt[j];
+                }
+                c.R = R;
+                c.total = total;
+                c.o = o;
+                c.end = cur;
+                cut_unit(sl, c, hd, hl);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    l2[j] = c.l[j];
+                    dt[j] = c.dt[j];
+                }
+                R = c.R;
+                total = c.total;
+                nb = c.nb;
+                cur = c.end;
+            } else {
+                const float ln = __shfl_sync(0xffffffffu, l2[7], 15, 16);   // tokens beyond the sequence have dt = 0
+                const float Rn = scale_into(R, ln);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) l2[j] -= Rn;
+                if (hl == 0) append_block(sl, 0, hd, Rn - R, ln - Rn, cur);
+                R = Rn - ln;
+                total += ln;
+            }
+            const bool last = t0 + cur == t_end, fin = cur == kQ || last;
+            if (lane == 0) {
+                *reinterpret_cast<int4 *>(&sl.fin) = make_int4(fin, last, t0, o);
+                *reinterpret_cast<int4 *>(&sl.n) = make_int4(cur - o, o / 16, nb, 0);
+            }
             uint32_t hi[4], lo[4];
 #pragma unroll
             for (int j = 0; j < 8; j += 2) {
-                const float s0 = dv[j] * ex2(Rn - l2[j]), s1 = dv[j + 1] * ex2(Rn - l2[j + 1]);
+                const float s0 = dt[j] * ex2(-l2[j]), s1 = dt[j + 1] * ex2(-l2[j + 1]);
                 hi[j / 2] = pack_bf16(s0, s1);
                 lo[j / 2] = pack_bf16(s0 - __uint_as_float(hi[j / 2] << 16), s1 - __uint_as_float(hi[j / 2] & 0xFFFF0000u));
             }
 #pragma unroll
             for (int j = 0; j < 8; j += 4) {
                 *reinterpret_cast<uint4 *>(&sl.s[hd][4 * hl + j / 2]) = make_uint4(hi[j / 2], lo[j / 2], hi[j / 2 + 1], lo[j / 2 + 1]);
-                *reinterpret_cast<float4 *>(&sl.e[hd][8 * hl + j]) = make_float4(ex2(l2[j] - Rn), ex2(l2[j + 1] - Rn), ex2(l2[j + 2] - Rn), ex2(l2[j + 3] - Rn));
+                *reinterpret_cast<float4 *>(&sl.e[hd][8 * hl + j]) = make_float4(ex2(l2[j]), ex2(l2[j + 1]), ex2(l2[j + 2]), ex2(l2[j + 3]));
             }
-            if (hl == 0) {
-                sl.f2[hd] = Rn - R;
-                sl.e2[hd] = ln - Rn;
-                sl.start = start;
-                sl.n = n;
-            }
-            R = Rn - ln;
-            total += ln;
             warp_arrive(&bars.sc_ready[b % kSlots]);
+            if (fin) {
+                o = 0;
+                t0 += kQ;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) dt[j] = dt2[j];
+                fetch_dt(dt2, t0 + kQ);
+            } else {
+                o = cur;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) dt[j] = c.keep[j];
+            }
         }
         if (a.lam && hl == 0 && (hd == 0 || two)) a.lam[static_cast<size_t>(seq) * a.H + h0 + hd] = total / kLog2e;
     } else if (warp >= 24) {
         // ======================================================= single-issue roles.  The whole warp walks the loop and one elected lane
         // issues: the operands of these instructions live in registers that the warp shares, so its lanes stay together.
-        int row = t_begin;
         if (warp == 24) {
             // ---- TMA: one load brings both 64-column halves of B or C, or X of both heads
+            int row = t_begin;
 #pragma unroll 1
-            for (int b = 0; row < t_end; ++b) {
+            for (int j = 0; row < t_end; ++j, row += kQ) {
                 if (warp_dead(&dead)) break;   // a wait ran out: nothing more is issued
-                const int st = b & 1;
-                if (b >= 2) mbar_wait(&bars.bc_free[st], ((b - 2) >> 1) & 1, &dead, a.status);
+                const int st = j & 1;
+                if (j >= 2) mbar_wait(&bars.bc_free[st], ((j - 2) >> 1) & 1, &dead, a.status);
                 __syncwarp();
                 if (elect_one()) {
                     unsigned char *bc = sm + st * kBCStage;
                     mbar_expect_tx(&bars.full_bc[st], has_y ? kBCStage : kBCStage / 2);
                     tma_load_3d(bc, &mapB, row, 2 * grp, &bars.full_bc[st]);
                     if (has_y) tma_load_3d(bc + 2 * kTile, &mapC, row, 2 * grp, &bars.full_bc[st]);
-                    // the ring cannot hide the DRAM latency of the tile loads: pull the tiles of block b+2 into L2 now
+                    // the ring cannot hide the DRAM latency of the tile loads: pull the tiles after the next into L2 now
                     if (row + 2 * kQ < t_end) {
                         tma_prefetch_l2_3d(&mapX, row + 2 * kQ, h0);
                         tma_prefetch_l2_3d(&mapB, row + 2 * kQ, 2 * grp);
@@ -321,88 +404,130 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
                     }
                 }
                 __syncwarp();
-                if (b >= 1) mbar_wait(&bars.x_free, (b - 1) & 1, &dead, a.status);
+                if (j >= 1) mbar_wait(&bars.x_free, (j - 1) & 1, &dead, a.status);
                 __syncwarp();
                 if (elect_one()) {
                     mbar_expect_tx(&bars.full_x, 2 * kTile);
                     tma_load_3d(sm + kOffX, &mapX, row, h0, &bars.full_x);
                 }
                 __syncwarp();
-                // where the next block starts
-                mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
-                row += slots[b % kSlots].n;
-                warp_arrive(&bars.slot_free[b % kSlots]);
             }
         } else if (warp == 25) {
             // ---- MMA issue of (S)
             constexpr uint32_t idS = umma_idesc(kFmtBF16, false, true, 128, 128);
+            bool last = false;
+            uint32_t par = 0;   // of the block
 #pragma unroll 1
-            for (int b = 0; row < t_end; ++b) {
+            for (int b = 0, tile = 0; !last; ++b) {
                 if (warp_dead(&dead)) break;
-                const int st = b & 1;
-                const uint64_t dB = umma_desc(smem_u32(sm + st * kBCStage), kTile, 1024);
                 mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
-                row += slots[b % kSlots].n;
-                mbar_wait(&bars.full_bc[st], (b >> 1) & 1, &dead, a.status);
+                const Slot &sl = slots[b % kSlots];
+                const int nb = sl.nb, fin = sl.fin;
+                last = sl.last;
+                const int st = tile & 1;
+                const uint64_t dB = umma_desc(smem_u32(sm + st * kBCStage), kTile, 1024);
+                mbar_wait(&bars.full_bc[st], (tile >> 1) & 1, &dead, a.status);
                 mbar_wait(&bars.x2_ready, b & 1, &dead, a.status);
-                mbar_wait(&bars.hb_ready, b & 1, &dead, a.status);
-                __syncwarp();
-                tc_fence_after_sync();
-                if (elect_one()) {
+                int k = sl.k0;
+#pragma unroll 1
+                for (int j = 0; j < nb; ++j, par ^= 1) {
+                    const int k1 = sl.kb[j];
+                    mbar_wait(&bars.hb_ready, par, &dead, a.status);
+                    __syncwarp();
+                    tc_fence_after_sync();
+                    if (elect_one()) {
+                        if (__builtin_expect(k1 - k == 8, 1)) {   // these instructions are on the chain: nothing is computed between them
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) umma_bf16_ts(tm + kTmS, tm + kTmX + 8 * k, dB + ((k * 16 * 128) >> 4), idS, true);
-                    umma_commit(&bars.h_done);
-                    umma_commit(&bars.xs_free);
-                    umma_commit(&bars.bc_free[st]);
+                            for (int i = 0; i < 8; ++i) umma_bf16_ts(tm + kTmS, tm + kTmX + 8 * i, dB + ((i * 16 * 128) >> 4), idS, true);
+                        } else {
+#pragma unroll 1
+                            for (int i = k; i < k1; ++i) umma_bf16_ts(tm + kTmS, tm + kTmX + 8 * i, dB + ((i * 16 * 128) >> 4), idS, true);
+                        }
+                        umma_commit(&bars.h_done);
+                        if (j == nb - 1) {
+                            umma_commit(&bars.xs_free);
+                            if (fin) umma_commit(&bars.bc_free[st]);
+                        }
+                    }
+                    k = k1;
+                    __syncwarp();
                 }
-                __syncwarp();
+                tile += fin;
             }
         } else if (has_y) {
-            // ---- MMA issue of (G) (both operands K-major; one block ahead), (Y2), (Y1)
+            // ---- MMA issue of (G) (both operands K-major; one tile ahead), (Y2), (Y1)
             constexpr uint32_t idG = umma_idesc(kFmtBF16, false, false, 128, 128);
-            constexpr uint32_t idY64 = umma_idesc(kFmtBF16, false, false, 128, 64);
+            auto id_cols = [](int k) { return umma_idesc(kFmtBF16, false, false, 128, 16 * k); };   // 16 k columns
             const uint64_t dG = umma_desc(smem_u32(sm + kOffG), 0, 1024);
+            int tile = 0;
+            uint32_t par = 0;   // of the block
+            bool last = false;
 #pragma unroll 1
-            for (int b = -1; b < 0 || row < t_end; ++b) {
+            for (int b = -1; !last; ++b) {
                 if (warp_dead(&dead)) break;
-                bool last = false;
+                bool next = true;
                 if (b >= 0) {
-                    const uint64_t dC = umma_desc(smem_u32(sm + (b & 1) * kBCStage + 2 * kTile), 0, 1024);
                     mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
-                    row += slots[b % kSlots].n;
-                    last = row >= t_end;
+                    const Slot &sl = slots[b % kSlots];
+                    const int nb = sl.nb, fin = sl.fin;
+                    last = sl.last;
+                    next = fin && !last;
+                    const uint64_t dC = umma_desc(smem_u32(sm + (tile & 1) * kBCStage + 2 * kTile), 0, 1024);
                     if (b >= 1) mbar_wait(&bars.y_free, (b - 1) & 1, &dead, a.status);
-                    mbar_wait(&bars.hb_ready, b & 1, &dead, a.status);
-                    __syncwarp();
-                    tc_fence_after_sync();
-                    if (elect_one()) {
+                    int k = sl.k0;
+#pragma unroll 1
+                    for (int j = 0; j < nb; ++j, par ^= 1) {
+                        const int k1 = sl.kb[j];
+                        mbar_wait(&bars.hb_ready, par, &dead, a.status);
+                        __syncwarp();
+                        tc_fence_after_sync();
+                        if (elect_one()) {
 #pragma unroll
-                        for (int k = 0; k < 8; ++k)
-                            umma_bf16_ts(tm + kTmY, tm + kTmSb + 8 * k, dC + (((k >> 2) * kTile + (k & 3) * 32) >> 4), idG, k > 0);
-                        umma_commit(&bars.y2_done);
-                        umma_commit(&bars.bc_free[b & 1]);
+                            for (int i = 0; i < 8; ++i)
+                                umma_bf16_ts(tm + kTmY + 16 * k, tm + kTmSb + 8 * i, dC + ((16 * k * 128 + (i >> 2) * kTile + (i & 3) * 32) >> 4), id_cols(k1 - k), i > 0);
+                            umma_commit(&bars.y2_done);
+                            if (fin && j == nb - 1) umma_commit(&bars.bc_free[tile & 1]);
+                        }
+                        k = k1;
+                        __syncwarp();
                     }
-                    __syncwarp();
                     mbar_wait(&bars.x2_ready, b & 1, &dead, a.status);
-                    mbar_wait(&bars.mask_done, b & 1, &dead, a.status);
+                    mbar_wait(&bars.mask_done, tile & 1, &dead, a.status);
                     __syncwarp();
                     tc_fence_after_sync();
                     if (elect_one()) {
-                        // tokens i < 64 onto all t, then i >= 64 onto t >= 64
+                        // tokens i < 64 onto all t of their block, those from 64 on onto t from 64 on
+                        if (__builtin_expect(nb == 1 && k - sl.k0 == 8, 1)) {
+                            constexpr uint32_t idY64 = umma_idesc(kFmtBF16, false, false, 128, 64);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) umma_bf16_ts(tm + kTmY, tm + kTmX + 8 * k, dG + ((k * 32) >> 4), idG, true);
+                            for (int i = 0; i < 4; ++i) umma_bf16_ts(tm + kTmY, tm + kTmX + 8 * i, dG + ((i * 32) >> 4), idG, true);
 #pragma unroll
-                        for (int k = 4; k < 8; ++k)
-                            umma_bf16_ts(tm + kTmY + 64, tm + kTmX + 8 * k, dG + ((kTile + (k - 4) * 32) >> 4), idY64, true);
+                            for (int i = 4; i < 8; ++i)
+                                umma_bf16_ts(tm + kTmY + 64, tm + kTmX + 8 * i, dG + ((kTile + (i - 4) * 32) >> 4), idY64, true);
+                        } else {
+                            k = sl.k0;
+#pragma unroll 1
+                            for (int j = 0; j < nb; ++j) {
+                                const int k1 = sl.kb[j], q = max(k, 4);
+#pragma unroll 1
+                                for (int i = k; i < k1; ++i) {
+                                    const int c = i < 4 ? k : q;
+                                    const uint32_t tile_at = i < 4 ? 16 * k * 128 + i * 32 : kTile + 16 * (q - 4) * 128 + (i - 4) * 32;
+                                    umma_bf16_ts(tm + kTmY + 16 * c, tm + kTmX + 8 * i, dG + (tile_at >> 4), id_cols(k1 - c), true);
+                                }
+                                k = k1;
+                            }
+                        }
                         umma_commit(&bars.y_done);
                         umma_commit(&bars.xy_free);
                     }
                     __syncwarp();
+                    tile += next;
                 }
-                if (!last) {   // (G) of block b+1: the mask warps have drained the G columns
-                    const uint32_t bc = smem_u32(sm + ((b + 1) & 1) * kBCStage);
+                if (next) {   // (G) of the next tile: the mask warps have drained the G columns
+                    const uint32_t bc = smem_u32(sm + (tile & 1) * kBCStage);
                     const uint64_t dB = umma_desc(bc, 0, 1024), dC = umma_desc(bc + 2 * kTile, 0, 1024);
-                    mbar_wait(&bars.full_bc[(b + 1) & 1], ((b + 1) >> 1) & 1, &dead, a.status);
+                    mbar_wait(&bars.full_bc[tile & 1], (tile >> 1) & 1, &dead, a.status);
                     __syncwarp();
                     tc_fence_after_sync();
                     if (elect_one()) {
@@ -432,12 +557,13 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
         }
         bool last = false;
 #pragma unroll 1
-        for (int b = 0; !last; ++b) {
+        for (int b = 0, tile = 0; !last; ++b) {
             if (warp_dead(&dead)) break;
             mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
             const Slot &sl = slots[b % kSlots];
-            last = sl.start + sl.n >= t_end;
-            mbar_wait(&bars.full_x, b & 1, &dead, a.status);
+            const bool first = sl.o == 0, fin = sl.fin;
+            last = sl.last;
+            mbar_wait(&bars.full_x, tile & 1, &dead, a.status);
             __syncwarp();
             uint32_t w[2][16];
 #pragma unroll
@@ -467,7 +593,7 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
 #pragma unroll
             for (int j = 0; j < 16; j += 4) any |= w[0][j] | w[1][j];
             const uint32_t odd = __ballot_sync(0xffffffffu, any & 1u);
-            if (lane == (odd ? __ffs(odd) - 1 : 0)) mbar_arrive(&bars.x_free);
+            if (fin && lane == (odd ? __ffs(odd) - 1 : 0)) mbar_arrive(&bars.x_free);
             if (b >= 1) {   // (S) and (Y1) have read the X^ before
                 mbar_wait(&bars.xs_free, (b - 1) & 1, &dead, a.status);
                 if (has_y) mbar_wait(&bars.xy_free, (b - 1) & 1, &dead, a.status);
@@ -479,10 +605,10 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
             tmem_st_wait();
             tc_fence_before_sync();
             warp_arrive(&bars.x2_ready);
-            if (has_y) {
+            if (has_y && first) {
                 // mask, 32 columns at a time: the two warps of a lane quarter take every other one; the last holds the diagonal.
                 // ((Y1) of the block before has read the tile: waited for above.)
-                mbar_wait(&bars.g_done, b & 1, &dead, a.status);
+                mbar_wait(&bars.g_done, tile & 1, &dead, a.status);
                 __syncwarp();
                 tc_fence_after_sync();
 #pragma unroll 1
@@ -505,13 +631,14 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
                 tc_fence_before_sync();
                 warp_arrive(&bars.mask_done);
             }
+            tile += fin;
         }
     } else if (wg >= 2) {
         // ======================================================= state: lane = (head, p), warpgroup = 64 columns n
         const int x = tid & 127, hd = x >> 6, n0 = 64 * (wg - 2);
         const size_t mine = (hd && two ? static_cast<size_t>(kN) * kP : 0) + static_cast<size_t>(n0) * kP + (x & 63);
         {
-            // initial state, scaled by 2^R of block 0
+            // initial state, scaled by 2^R of the first block
 #pragma unroll 1
             for (int q = 0; q < 2; ++q) {
                 uint32_t rr[32];
@@ -519,7 +646,7 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
                 for (int c = 0; c < 32; ++c) rr[c] = S0 ? __float_as_uint(S0[mine + (32 * q + c) * kP]) : 0u;
                 if (q == 0) mbar_wait(&bars.sc_ready[0], 0, &dead, a.status);
                 __syncwarp();
-                const float f = ex2(slots[0].f2[hd]);
+                const float f = ex2(slots[0].f2[hd][0]);
 #pragma unroll
                 for (int c = 0; c < 32; ++c) rr[c] = __float_as_uint(__uint_as_float(rr[c]) * f);
                 tmem_st32(lane_base + kTmS + n0 + 32 * q, rr);
@@ -530,23 +657,27 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
             warp_arrive(&bars.hb_ready);
         }
         bool last = false;
+        int b = 0, j = 0;   // unit, block
 #pragma unroll 1
-        for (int b = 0; !last; ++b) {
+        for (uint32_t par = 0; !last; par ^= 1) {
             if (warp_dead(&dead)) break;
             mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
             const Slot &sl = slots[b % kSlots];
-            last = sl.start + sl.n >= t_end;
+            const bool done = j + 1 == sl.nb;   // with the unit
+            last = done && sl.last;
             float ex = sl.e2[hd];
-            if (!last) {
+            if (!done) {
+                ex = sl.f2[hd][j + 1];
+            } else if (!last) {
                 mbar_wait(&bars.sc_ready[(b + 1) % kSlots], ((b + 1) / kSlots) & 1, &dead, a.status);
-                ex = slots[(b + 1) % kSlots].f2[hd];
+                ex = slots[(b + 1) % kSlots].f2[hd][0];
             }
-            mbar_wait(&bars.h_done, b & 1, &dead, a.status);
-            if (has_y) mbar_wait(&bars.y2_done, b & 1, &dead, a.status);   // the bf16 copy has been read
+            const float f = ex2(0.5f * ex);   // in two steps: the factor may lie below the fp32 range where its product with the state does not
+            const bool scale = __any_sync(0xffffffffu, ex != 0.f);
+            mbar_wait(&bars.h_done, par, &dead, a.status);
+            if (has_y) mbar_wait(&bars.y2_done, par, &dead, a.status);   // the bf16 copy has been read
             __syncwarp();
             tc_fence_after_sync();
-            if (ex != 0.f) scale_state64(lane_base + kTmS + n0, ex);
-            __syncwarp();
             if (last) {
                 const bool store = ST && (hd == 0 || two) && !warp_dead(&dead);
 #pragma unroll 1
@@ -556,7 +687,7 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
                     tmem_ld_wait();
 #pragma unroll
                     for (int c = 0; c < 8; ++c)
-                        if (store) store_state(ST, a.st_bf16, st_off + mine + static_cast<size_t>(8 * q + c) * kP, __uint_as_float(rr[c]));
+                        if (store) store_state(ST, a.st_bf16, st_off + mine + static_cast<size_t>(8 * q + c) * kP, __uint_as_float(rr[c]) * f * f);
                 }
             } else {
 #pragma unroll 1
@@ -564,13 +695,23 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
                     uint32_t rr[32];
                     tmem_ld32(lane_base + kTmS + n0 + 32 * q, rr);
                     tmem_ld_wait();
+                    if (scale) {
+#pragma unroll
+                        for (int c = 0; c < 32; ++c) rr[c] = __float_as_uint(__uint_as_float(rr[c]) * f * f);
+                        tmem_st32(lane_base + kTmS + n0 + 32 * q, rr);
+                    }
                     copy_state32(lane_base, n0 + 32 * q, rr);
                 }
                 tmem_st_wait();
                 tc_fence_before_sync();
                 warp_arrive(&bars.hb_ready);
             }
-            warp_arrive(&bars.slot_free[b % kSlots]);
+            ++j;
+            if (done) {
+                warp_arrive(&bars.slot_free[b % kSlots]);
+                ++b;
+                j = 0;
+            }
         }
     } else if (has_y) {
         // ======================================================= outputs of 64 tokens; this warp: 32 features of one head
@@ -585,8 +726,8 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
         for (int b = 0; !last; ++b) {
             mbar_wait(&bars.sc_ready[b % kSlots], (b / kSlots) & 1, &dead, a.status);
             const Slot &sl = slots[b % kSlots];
-            const int start = sl.start, n = sl.n;
-            last = start + n >= t_end;
+            const int row = sl.row, o = sl.o, n = sl.n;
+            last = sl.last;
             mbar_wait(&bars.y_done, b & 1, &dead, a.status);
             __syncwarp();
             tc_fence_after_sync();
@@ -621,24 +762,25 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
                 for (int kk = 0; kk < 4; ++kk)   // 16 tokens
                     stmatrix_x4_trans(srow + 16 * kk * 128 + (((4 * (wq & 1) + 2 * lh + (m & 1)) ^ i) << 4), w[lh][4 * kk], w[lh][4 * kk + 1],
                                       w[lh][4 * kk + 2], w[lh][4 * kk + 3]);
-            if (n == kQ && two) {
+            if (__builtin_expect(n == kQ && two, 1)) {
                 fence_async_smem();
                 named_bar_sync(2, 256);
                 if (warp == 0 && elect_one()) {
-                    tma_store_3d(&mapY, sm + kOffY, start, h0);
+                    tma_store_3d(&mapY, sm + kOffY, row, h0);
                     tma_store_commit();
                 }
             } else if (hd == 0 || two) {
-                // a block that is not whole, or whose second head is not wanted: rows straight to global memory
+                // a block that is not a whole tile, or whose second head is not wanted: rows straight to global memory; lane = row i
+                // of eight, piece m of this warp's four
                 __syncwarp();
+                const int lo = max(o - 64 * th, 0), hi = min(o + n - 64 * th, 64), row0 = (lo & ~7) + i;
                 const size_t tstride = static_cast<size_t>(a.H) * kP;
-                __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(a.y) + static_cast<size_t>(start + 64 * th + i) * tstride +
+                __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(a.y) + static_cast<size_t>(row + 64 * th + row0) * tstride +
                                      static_cast<size_t>(h0 + hd) * kP + 32 * (wq & 1) + 8 * m;
-                const unsigned char *src = ys + i * 128 + (((4 * (wq & 1) + m) ^ i) << 4);
-                const int left = min(64, n - 64 * th);
+                const unsigned char *src = ys + row0 * 128 + (((4 * (wq & 1) + m) ^ i) << 4);
 #pragma unroll 1
-                for (int j = i; j < left; j += 8, src += 8 * 128, dst += 8 * tstride)   // lane = row i of 8, piece m of this warp's four
-                    *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(src);
+                for (int r = row0; r < hi; r += 8, src += 8 * 128, dst += 8 * tstride)
+                    if (r >= lo) *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(src);
                 fence_async_smem();
             }
         }

@@ -17,6 +17,9 @@ pytestmark = pytest.mark.gpu
     (4, 1, [700, 130], np.array([0.05, 20.0, 1.0, 200.0])),      # mild and violent heads in one CTA: blocks end early
     (80, 1, [300], 0.02),                                        # benchmark shape, weak decay
     (4, 1, [3333], 0.3),                                         # one long sequence: segments
+    (4, 1, [700, 130, 128, 1], np.array([2.0, 3.0, 5.0, 9.0])),  # tiles of several blocks
+    (3, 1, [257, 384], np.array([6.0, 0.1, 12.0])),              # the same beside a mild head, and the last head alone
+    (4, 1, [3333], np.array([3.0, 8.0, 20.0, 0.5])),             # the same in segments
 ])
 @pytest.mark.parametrize("outputs", [True, False])
 def test_ssd_scan_block_edges(H, G, lens, decay, outputs):
@@ -38,6 +41,54 @@ def test_ssd_scan_block_edges(H, G, lens, decay, outputs):
         assert maxrel_per_head(ST[s], ST_ref, 0) <= TOL_BF16
         if outputs:
             assert maxrel_per_head(y[sl], y_ref, 1) <= TOL_BF16
+
+
+@pytest.mark.parametrize("every, dt", [(37, 60.0), (16, 1000.0), (5, 30.0)])
+def test_ssd_scan_with_tokens_that_forget_everything(every, dt):
+    """Single tokens whose own decay is beyond the range of a block's scale, among mild ones: they cut tiles at any offset."""
+    import torch
+    rng = np.random.default_rng(every)
+    H, T = 4, 500
+    A = wl.ssd_A(rng, H).astype(np.float32)
+    tok = wl.ssd_tokens(rng, T, H, 64, 128, 1)
+    tok["dt"][every - 1::every, ::2] = dt
+    S0 = rng.standard_normal((1, H, 128, 64)).astype(np.float32)
+    bf = torch.bfloat16
+    y, ST = b.lkv_ssd_fwd(dev(tok["x"], bf), dev(tok["dt"]), dev(A), dev(tok["B"], bf), dev(tok["C"], bf), dev(S0))
+    y_ref, ST_ref = oracle.ssd_seq(tok["x"], tok["dt"], A, tok["B"], tok["C"], S0[0])
+    assert maxrel_per_head(host(ST)[0], ST_ref, 0) <= TOL_BF16
+    y = host(y)
+    forget = np.arange(T) % every == every - 1   # their outputs are as large as dt: scored apart
+    for rows in (forget, ~forget):
+        assert maxrel_per_head(y[rows], y_ref[rows], 1) <= TOL_BF16
+
+
+def test_ssd_scan_time_bends_with_the_decays_but_does_not_break():
+    """Decays of 600 log2 units a tile: the chain runs several times per tile, everything else once (every block a tile of its own
+    took four times as long as mild decays)."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rn = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    H, n, L = 80, 16, 2048
+    T = n * L
+    bf = torch.bfloat16
+    x, B, C = rn(T, H, 64).to(bf), (rn(T, 1, 128) / 128 ** 0.5).to(bf), (rn(T, 1, 128) / 128 ** 0.5).to(bf)
+    dt = torch.nn.functional.softplus(0.2 + 0.3 * rn(T, H))
+    cu = (np.arange(n + 1) * L).astype(np.int32)
+
+    def us(A):
+        best = float("inf")
+        for _ in range(5):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            b.lkv_ssd_fwd(x, dt, A, B, C, cu_seqlens=cu)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        return best
+
+    mild, strong = us(torch.full((H,), -0.05, device="cuda")), us(torch.full((H,), -4.0, device="cuda"))
+    assert strong < 3 * mild
 
 
 @pytest.mark.parametrize("decay, outputs", [(1.0, True), (40.0, True), (40.0, False)])
