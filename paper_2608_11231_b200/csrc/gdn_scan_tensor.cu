@@ -25,7 +25,10 @@
 // identity step.
 // R goes back to 0 when 2^R would leave its range (the state is rescaled then), and a block whose own decay is beyond 2^80 runs
 // in an "exact" form: R = 0, A and Ps carry 2^{l_t - l_i} element by element, X2 takes 2^{l_i}, Q is scaled in its tile, and (5)
-// and (7) get an operand each.  Same roles, same barriers; the rare code is in functions that are not inlined.
+// and (7) get an operand each.  Same roles, same barriers.  What the mask warps add for it sits in their loops (the loads, packing and
+// stores around it are shared: as functions beside the loops it cost instruction fetch, 740 -> 720 us on the case below), Q
+// is scaled by the mask warps, off the chain.  32 sequences x 2048 tokens, 32 heads, log2 units of decay per token: 0.1 481 us, 0.5 503,
+// 1.0 575, 1.3 (both forms in turn) 793, 4 758, 8 728; with the exact form written for rare use 485, 565, 639, 1382, 1438, 1438.
 //
 // Warps 0-7 chain (lane = state column, warpgroup = half of the tokens / state rows), 8-11 mask epilogue of (1), 12-15 prep
 // (the inverse), 16 TMA loads of V and the stores of the output tiles, 17 MMA issue of the chain, 18 MMA issue of (1) and (W),
@@ -76,7 +79,7 @@ constexpr int kOffGb = kOffD + kC * kLdD * 4;          // per-block scalars, fou
 // arrays of a block's scalars (l = running sum of g in log2 units, R = the block's scale exponent), 64 floats each
 constexpr int kGbL = 0;                                // l
 constexpr int kGbX1 = kC, kGbX2 = 2 * kC;              // column factors of X1, X2: beta 2^{R - l}, -beta (exact block: beta, -beta 2^l)
-constexpr int kGbE = 3 * kC, kGbW = 4 * kC;            // output factor scale 2^{l - R} (exact block: 1), 2^{l_C - l} (exact block only)
+constexpr int kGbE = 3 * kC, kGbW = 4 * kC;            // output factor scale 2^{l - R} (exact block: scale), 2^{l_C - l} (exact block only)
 constexpr int kGbExp = 5 * kC;                         // exponents into the block: bf16 copy, fp32 state; exponent out of it; exact flag
 constexpr int kGbFloats = 5 * kC + 4;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -111,20 +114,22 @@ struct Bars {
 constexpr int kBars1 = 18, kBars4 = 8, kBars2 = 8, kBarsS = 4, kBars8 = 6;
 static_assert(sizeof(Bars) == 8 * (kBars1 + kBars4 + kBars2 + kBarsS + kBars8), "barrier table");
 
-// Exact block: a quarter row of the Q tile (token tid & 63, 16-byte chunks 4 * (part & 1) .. + 3 of K-block part >> 1,
-// part = tid >> 6) multiplied in place by f.
-static __device__ __noinline__ void scale_q_quarter(unsigned char *stage, int tid, float f) {
-    const int tq = tid & 63, part = tid >> 6;
-    unsigned char *qt = stage + (part >> 1) * (2 * kC * 128) + tq * 128;
+// Exact block: row t of the Q tile multiplied in place by f.
+static __device__ __noinline__ void scale_q_row(unsigned char *stage, int t, float f) {
+    unsigned char *qt = stage + t * 128;
     const __nv_bfloat162 f2 = __float2bfloat162_rn(f);
 #pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-        uint4 *p = reinterpret_cast<uint4 *>(qt + (((4 * (part & 1) + c) ^ (tq & 7)) << 4));
-        uint4 v = *p;
-        __nv_bfloat162 *e = reinterpret_cast<__nv_bfloat162 *>(&v);
+    for (int kb = 0; kb < 2; ++kb, qt += 2 * kC * 128) {
+        uint4 v[8];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) e[i] = __hmul2(e[i], f2);
-        *p = v;
+        for (int c = 0; c < 8; ++c) v[c] = *reinterpret_cast<uint4 *>(qt + ((c ^ (t & 7)) << 4));
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            __nv_bfloat162 *e = reinterpret_cast<__nv_bfloat162 *>(&v[c]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) e[i] = __hmul2(e[i], f2);
+            *reinterpret_cast<uint4 *>(qt + ((c ^ (t & 7)) << 4)) = v[c];
+        }
     }
 }
 
@@ -262,29 +267,20 @@ __device__ __forceinline__ void pack16(const float (&v)[16], uint32_t (&w)[8]) {
 #pragma unroll
     for (int e = 0; e < 8; ++e) w[e] = pack_bf16(v[2 * e], v[2 * e + 1]);
 }
-// Mask of one group of 16 columns of one row of G, exact form for a block whose decay is too violent for the
-// per-group factors: one exponential per element.  Rare, kept out of the hot loop as a whole (load from tensor
-// memory, mask, store) so that no register array crosses the call.  ps: bf16 row of Ps; else the group's place in the row
-// of F and, if not null, in that of D.
-__device__ __noinline__ void mask_group_exact(uint32_t taddr, const float *sc, float cgt, float coef, int i0, int lim, unsigned char *ps, int t,
-                                              unsigned char *frow, float *drow) {
-    uint32_t rr[16];
-    tmem_ld16(taddr, rr);
-    tmem_ld_wait();
-    float v[16];
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// Exact block: W entries of a row of G times 2^{l_t - l_i}, l = the columns' l in shared memory.  What lies above the diagonal may
+// overflow; nobody reads it unmasked.
+template <int W>
+__device__ __forceinline__ void apply_decay(float (&v)[W], const float *l, float lt) {
 #pragma unroll
-    for (int c = 0; c < 16; ++c) v[c] = (i0 + c <= lim) ? coef * exp2f(cgt - sc[i0 + c]) * __uint_as_float(rr[c]) : 0.f;
-    if (ps) {
-        store_row_chunks(ps, t, i0 >> 3, v);
-        return;
+    for (int c = 0; c < W; c += 4) {
+        const float4 li = *reinterpret_cast<const float4 *>(l + c);
+        v[c] *= ex2(lt - li.x); v[c + 1] *= ex2(lt - li.y); v[c + 2] *= ex2(lt - li.z); v[c + 3] *= ex2(lt - li.w);
     }
-#pragma unroll
-    for (int c = 0; c < 16; c += 8)
-        *reinterpret_cast<uint4 *>(frow + 2 * c) =
-            make_uint4(pack_f16(v[c], v[c + 1]), pack_f16(v[c + 2], v[c + 3]), pack_f16(v[c + 4], v[c + 5]), pack_f16(v[c + 6], v[c + 7]));
-    if (drow)
-#pragma unroll
-        for (int c = 0; c < 16; c += 4) *reinterpret_cast<float4 *>(drow + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
 }
 // Rows of a ragged last block go straight to global memory: 16 tokens of one state column per call, read from
 // tensor memory and scaled here.
@@ -296,26 +292,23 @@ __device__ __noinline__ void store_o_partial(uint32_t taddr, const float *e, __n
     for (int c = 0; c < 16; ++c)
         if (c < n_left) orow[c * tstride] = __float2bfloat16_rn(__uint_as_float(pu[c]) * e[c]);
 }
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-// 64 rows of the state from row 64 half on: fp32 values times 2^acc_exp in place, times 2^copy_exp as bf16 pairs beside them (each in two
-// steps: the factor may lie below the fp32 range where its product with the state does not).  One block in several needs it.
+// 64 rows of the state from row 64 half on: times 2^copy_exp as bf16 pairs beside them, times 2^acc_exp in place (2^copy_exp brings it back
+// to a small scale, what an exact block takes off on top of that may vanish).  One block in several needs it.
 __device__ __noinline__ void rescale_state(uint32_t tm_s, uint32_t tm_sb, float copy_exp, float acc_exp) {
-    const float fc = ex2(0.5f * copy_exp), fa = ex2(0.5f * acc_exp);
+    const float fc = ex2(copy_exp), fa = ex2(acc_exp - copy_exp);
 #pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
-        uint32_t rr[16], w[8];
-        tmem_ld16(tm_s + 16 * q, rr);
+    for (int q = 0; q < 2; ++q) {
+        uint32_t rr[32], w[16];
+        tmem_ld32(tm_s + 32 * q, rr);
         tmem_ld_wait();
 #pragma unroll
-        for (int e = 0; e < 8; ++e) w[e] = pack_bf16(__uint_as_float(rr[2 * e]) * fc * fc, __uint_as_float(rr[2 * e + 1]) * fc * fc);
-        tmem_st8(tm_sb + 8 * q, w);
+        for (int c = 0; c < 32; ++c) rr[c] = __float_as_uint(__uint_as_float(rr[c]) * fc);
 #pragma unroll
-        for (int c = 0; c < 16; ++c) rr[c] = __float_as_uint(__uint_as_float(rr[c]) * fa * fa);
-        tmem_st16(tm_s + 16 * q, rr);
+        for (int e = 0; e < 16; ++e) w[e] = pack_bf16(__uint_as_float(rr[2 * e]), __uint_as_float(rr[2 * e + 1]));
+        tmem_st16(tm_sb + 16 * q, w);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) rr[c] = __float_as_uint(__uint_as_float(rr[c]) * fa);
+        tmem_st32(tm_s + 32 * q, rr);
     }
 }
 // Empty sequence: the initial state (the identity, S0, or zero) and what is to be added, as the final state
@@ -324,22 +317,22 @@ __device__ __noinline__ void hand_through(float *ST, size_t obase, int st_bf16, 
     for (int e = threadIdx.x; e < kD * kD; e += kThreads)
         store_state(ST, st_bf16, obase + e, (id ? (e / kD == e % kD ? 1.f : 0.f) : (S0 ? S0[e] : 0.f)) + (add ? add[e] : 0.f));
 }
-// Exact block: u_t[j] of 32 tokens -> Uw = w o u as bf16 pairs over the first 16 of these 32 columns, u over the rest
-__device__ __noinline__ void u_operands_exact(uint32_t taddr, const float *w) {
-    uint32_t rr[32], p[8];
+// Exact block: u_t[j] of 32 tokens -> Uw = w o u as bf16 pairs over the first 16 of these 32 columns, u (if wanted) over the rest
+__device__ __noinline__ void u_operands_exact(uint32_t taddr, const float *w, bool both) {
+    uint32_t rr[32], p[16];
     tmem_ld32(taddr, rr);
     tmem_ld_wait();
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int k = q & 1;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int c = 16 * k + 2 * e;
-            const float w0 = q < 2 ? w[c] : 1.f, w1 = q < 2 ? w[c + 1] : 1.f;
-            p[e] = pack_bf16(__uint_as_float(rr[c]) * w0, __uint_as_float(rr[c + 1]) * w1);
-        }
-        tmem_st8(taddr + 8 * q, p);
+    for (int e = 0; e < 16; e += 2) {
+        const float4 f = *reinterpret_cast<const float4 *>(w + 2 * e);
+        p[e] = pack_bf16(__uint_as_float(rr[2 * e]) * f.x, __uint_as_float(rr[2 * e + 1]) * f.y);
+        p[e + 1] = pack_bf16(__uint_as_float(rr[2 * e + 2]) * f.z, __uint_as_float(rr[2 * e + 3]) * f.w);
     }
+    tmem_st16(taddr, p);
+    if (!both) return;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) p[e] = pack_bf16(__uint_as_float(rr[2 * e]), __uint_as_float(rr[2 * e + 1]));
+    tmem_st16(taddr + 16, p);
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -509,7 +502,7 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
             *reinterpret_cast<float2 *>(sc + kGbL + t) = make_float2(c0, c1);
             *reinterpret_cast<float2 *>(sc + kGbX1 + t) = exact ? bv : make_float2(bv.x * ex2(Rn - c0), bv.y * ex2(Rn - c1));
             *reinterpret_cast<float2 *>(sc + kGbX2 + t) = exact ? make_float2(-bv.x * ex2(c0), -bv.y * ex2(c1)) : make_float2(-bv.x, -bv.y);
-            *reinterpret_cast<float2 *>(sc + kGbE + t) = exact ? make_float2(1.f, 1.f) : make_float2(a.scale * ex2(c0 - Rn), a.scale * ex2(c1 - Rn));
+            *reinterpret_cast<float2 *>(sc + kGbE + t) = exact ? make_float2(a.scale, a.scale) : make_float2(a.scale * ex2(c0 - Rn), a.scale * ex2(c1 - Rn));
             if (exact) *reinterpret_cast<float2 *>(sc + kGbW + t) = make_float2(ex2(last - c0), ex2(last - c1));
             const float in = Rn - R;
             R = exact ? 0.f : Rn - last;
@@ -604,10 +597,10 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
             }
             __syncwarp();
             // (2Q) O = S^T Q^T while the chain warps work on U: O columns drained with the outputs of block b-2.  An exact
-            // block has its Q tile scaled first.
+            // block has had its Q tile scaled.
             const bool exact = gb[(b & 3) * kGbFloats + kGbExp + 3] != 0.f;
-            if (exact) mbar_wait(&bars.uw_ready, par, &dead, a.status);
             if (has_o) {
+                if (exact) mbar_wait(&bars.p_ready[par], (b >> 1) & 1, &dead, a.status);   // with Ps its Q tile is ready
                 if (b >= 2) mbar_wait(&bars.o_done[(b - 2) & 3], ((b - 2) >> 2) & 1, &dead, a.status);
                 __syncwarp();
                 tc_fence_after_sync();
@@ -835,21 +828,23 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
 #pragma unroll 1
                     for (int q = 0; 16 * q <= row_hi; ++q) {
                         const int i0 = 16 * q;
-                        if (exact) {
-                            mask_group_exact(lane_base + kTmG + i0, sc, sc[kGbL + t], a.scale, i0, t, ps, t, nullptr, nullptr);
-                            continue;
-                        }
                         uint32_t rr[16];
                         tmem_ld16(lane_base + kTmG + i0, rr);
                         tmem_ld_wait();
                         float v[16];
 #pragma unroll
                         for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(rr[c]);
+                        if (exact) apply_decay(v, sc + kGbL + i0, sc[kGbL + t]);
                         if (i0 + 31 >= row_hi) {   // the groups that the diagonal of this warp's rows passes through
 #pragma unroll
                             for (int c = 0; c < 16; ++c) v[c] = (i0 + c <= t) ? v[c] : 0.f;
                         }
                         store_row_chunks(ps, t, 2 * q, v);
+                    }
+                    // an exact block's row of the Q tile times 2^l for (2Q), which waits for it; (1) has read the tile
+                    if (exact) {
+                        mbar_wait(&bars.full_qk[b % kQKStages], (b / kQKStages) & 1, &dead, a.status);   // this thread reads what the TMA wrote
+                        scale_q_row(sm + (b % kQKStages) * kQKStage, t, ex2(sc[kGbL + t]));
                     }
                 }
                 tc_fence_before_sync();
@@ -872,18 +867,13 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
                 for (int q = 0; 32 * q <= row_hi; ++q) {
                     const int i0 = 32 * q;
                     unsigned char *frow = fb + (i0 + 31 == row_hi ? q : 2) * kFTile;
-                    if (exact) {
-#pragma unroll 1
-                        for (int i1 = i0; i1 < i0 + 32; i1 += 16)
-                            mask_group_exact(lane_base + kTmG + i1, sc, sc[kGbL + t], bt, i1, t - 1, nullptr, t, frow + 2 * (i1 - i0), i1 == (t & ~15) ? drow : nullptr);
-                        continue;
-                    }
                     uint32_t rr[32];
                     tmem_ld32(lane_base + kTmG + i0, rr);
                     tmem_ld_wait();
                     float v[32];
 #pragma unroll
                     for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(rr[c]) * bt;
+                    if (exact) apply_decay(v, sc + kGbL + i0, sc[kGbL + t]);
 #pragma unroll
                     for (int c = 0; c < 32; c += 8)
                         *reinterpret_cast<uint4 *>(frow + 2 * c) =
@@ -969,16 +959,8 @@ gdn_scan_tensor_kernel(const __grid_constant__ GdnArgs a, const __grid_constant_
             mbar_wait(&bars.u_done, par, &dead, a.status);
             __syncwarp();
             tc_fence_after_sync();
-            if (exact && has_o) {
-                // the Q tile scaled in place by scale 2^l for (2Q), which waits for it; (1) has read the tile: W came after it.
-                // Thread = (token, quarter of the row).
-                mbar_wait(&bars.full_qk[b % kQKStages], (b / kQKStages) & 1, &dead, a.status);   // this thread reads what the TMA wrote
-                scale_q_quarter(sm + (b % kQKStages) * kQKStage, tid, a.scale * ex2(sc[kGbL + (tid & 63)]));
-                fence_async_smem();
-                __syncwarp();
-            }
             if (exact) {
-                u_operands_exact(lane_base + kTmU + 32 * half, sc + kGbW + 32 * half);
+                u_operands_exact(lane_base + kTmU + 32 * half, sc + kGbW + 32 * half, has_o);
             } else {
                 uint32_t rr[32], w[16];
                 tmem_ld32(lane_base + kTmU + 32 * half, rr);

@@ -19,6 +19,9 @@ def _decays(kind, rng, T, H):
         g[blk % 3 == 1] *= 200.0
     elif kind == "reset":        # the running scale passes its limit every few blocks
         g *= 40.0
+    elif kind == "edge":         # blocks on either side of the limit of the exact form, in turn and within a block
+        g *= 85.0 * (1.0 + 0.1 * np.sin(blk))[:, None]
+        g[:, 1] *= 3.0
     return g.astype(np.float32)
 
 
@@ -26,6 +29,7 @@ def _decays(kind, rng, T, H):
     ([1, 63, 64, 65, 127, 128, 129, 191, 193], "mild"),
     ([257, 320, 321, 640], "violent"),
     ([1000, 64], "reset"),
+    ([1000, 65, 130], "edge"),
     ([3000], "mild"),                                            # one long sequence: segments
     ([2943], "reset"),
 ])
@@ -49,6 +53,34 @@ def test_gdn_scan_block_edges(lens, kind, outputs):
         assert maxrel_per_head(ST[s], ST_ref, 0) <= TOL_BF16
         if outputs:
             assert maxrel_per_head(o[sl], o_ref, 1) <= TOL_BF16
+
+
+def test_gdn_scan_time_bends_with_the_decays_but_does_not_break():
+    """Decays of 250 log2 units a block (the exact form, whose mask takes an exponential per element) against mild ones: it took three
+    times as long while that form was written for rare use."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rn = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    n, L = 16, 2048
+    T = n * L
+    bf = torch.bfloat16
+    unit = lambda x: torch.nn.functional.normalize(x, dim=-1).to(bf)
+    q, k, v, beta = unit(rn(T, 16, 128)), unit(rn(T, 16, 128)), rn(T, 32, 128).to(bf), torch.rand(T, 32, generator=gen, device="cuda")
+    cu = (np.arange(n + 1) * L).astype(np.int32)
+
+    def us(scale):
+        g = -scale * torch.rand(T, 32, generator=gen, device="cuda")
+        best = float("inf")
+        for _ in range(5):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            b.lkv_gdn_fwd(q, k, v, g, beta, cu_seqlens=cu)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        return best
+
+    assert us(5.4) < 2.2 * us(0.1)
 
 
 @pytest.mark.parametrize("outputs", [True, False])
