@@ -277,6 +277,16 @@ int lkv_device_status_static(void *stream);
  * S_T == NULL skips the final-state write; S_T may alias S0; o == NULL skips
  * the outputs (final states only; S_T is then required).  Sequences of
  * any length >= 0 are accepted (no padding is required).
+ *
+ * Range of the tensor-core scans (this one and lkv_ssd_fwd): inside, states and updates are held times a power of two
+ * that follows the decays.  What is carried on from S0 has the range of fp32.  Updates (beta_t v_t; dt_t x_t) keep their
+ * precision up to 2^46 in magnitude here, and in lkv_ssd_fwd between 2^-60 and 2^60, or 2^-25 and 2^25 in heads whose decay
+ * over 128 tokens is beyond 2^-128; what is larger may become infinite, what is smaller may vanish.
+ * LKV_COMPUTE_FP32 has the range of fp32 throughout.
+ *
+ * One long sequence in a call of its own may be scanned in segments whose initial states are composed (Eq. 6; the workspace
+ * size of lkv_workspace_bytes allows for that, with less the plain scan runs): its results then differ in rounding from
+ * those of the same sequence in a batch.  Equal calls with equal workspace sizes give equal bits.
  */
 int lkv_gdn_fwd(const void *q, const void *k, const void *v, const float *g, const float *beta,
                 const float *S0, void *o, void *S_T, const lkv_gdn_desc *d, void *stream);

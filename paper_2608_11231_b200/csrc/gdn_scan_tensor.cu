@@ -84,8 +84,10 @@ constexpr int kGbExp = 5 * kC;                         // exponents into the blo
 constexpr int kGbFloats = 5 * kC + 4;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kMaxRange = 80.f;                      // log2 units of decay inside a block: beyond that the block is "exact"
-constexpr float kMaxScale = 100.f;                     // R - l_C at most; then the state goes back to R = 0 (never below: a state that
-                                                       // only decays, as a transition does, keeps the whole fp32 range)
+constexpr float kMaxScale = 80.f;                      // R - l_C at most; then the state goes back to R = 0 (never below: a state that
+                                                       // only decays, as a transition does, keeps the whole fp32 range).  fp32 and bf16
+                                                       // then hold pseudo-values u up to 2^46; a state that is only carried on has no
+                                                       // upper limit (it decays as R grows)
 constexpr int kSmemUsed = kOffGb + 4 * kGbFloats * 4;  // from the 1024-byte aligned base
 constexpr int kSmemBytes = kSmemUsed + 1024;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");

@@ -12,9 +12,9 @@
 // nothing but the causal mask applied.  (The form with the decays inside, G'_ti = G_ti e^{l_t - l_i} dt_i, costs a mask of
 // 128 x 128 / 2 products and exponent factors per head and block; that, not the tensor cores, set the pace of this scan.)
 // The state as held, S^ + B^T X^, is the next block's S^ with R - l_n for R: it is multiplied by a power of two only when
-// that would pass kMaxScale, every block to every seventh with decays as strong as the benchmark's.
+// that would leave the window of kMaxScale, every block to every fifth with decays as strong as the benchmark's.
 // Scaling by powers of two commutes with rounding, and fp32 and bf16 have the same exponent range, so nothing is lost
-// while the exponents stay in range.
+// while the exponents stay in range (see kMaxScale).
 //
 // Where |l| would pass kMaxRange inside a tile, in either head, the tile is scanned in several blocks, each with its own R, that end on
 // multiples of 16 tokens: only the chain -- (Y2), (S), state pass -- runs once per block, 1.5 K cycles; loads, G, mask, X^ and
@@ -88,8 +88,10 @@ constexpr int kSmemBytes = kOffSlot + kSlots * static_cast<int>(sizeof(Slot)) + 
 static_assert(kSmemBytes + 512 <= 227 * 1024, "shared memory budget");
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kMaxRange = 200.f;               // log2 units of decay inside one block of the scan
-constexpr float kMaxScale = 104.f;               // R - l_n at most: X^ and S^ grow to about 2^104.  A state that is scaled back starts
-                                                 // from R = 0, or from below (to -96) where the block's own decay leaves no other choice
+constexpr float kMaxScale = 64.f;                // R and R - l_n stay within -64 .. 64, or where the block's own decay leaves no other
+                                                 // choice within -100 .. 100.  fp32 and bf16 then hold what lies between 2^-60 and 2^60, in
+                                                 // those blocks 2^-25 and 2^25; a state that is only carried on has no upper limit
+                                                 // (it decays as R grows)
 
 // tensor-memory map (columns)
 constexpr uint32_t kTmS = 0;        // 128: S^^T fp32
@@ -151,10 +153,12 @@ __device__ __forceinline__ void copy_state32(uint32_t lane_base, int n0, const u
     for (int c = 0; c < 16; ++c) w[c] = pack_bf16(__uint_as_float(rr[2 * c]), __uint_as_float(rr[2 * c + 1]));
     tmem_st16(lane_base + kTmSb + n0 / 2, w);
 }
-// Scale exponent of a block of decay ln, R what the block before has left
+// Scale exponent of a block of decay ln, R what the block before has left.  It is kept while it stays in the window, and then goes to the
+// window's other end: the longest way until the state has to be scaled again.
 __device__ __forceinline__ float scale_into(float R, float ln) {
+    const float W = fmaxf(kMaxScale, ceilf(0.5f * fabsf(ln)));
     float Rn = R;
-    if (fabsf(R - ln) > kMaxScale) Rn = ln < 0.f ? fminf(0.f, floorf(kMaxScale + ln)) : fmaxf(0.f, ceilf(ln - kMaxScale));
+    if (fmaxf(fabsf(R), fabsf(R - ln)) > W) Rn = copysignf(W, ln);
     if (fabsf(ln) > kMaxRange) Rn = rintf(ln);   // a single token of violent decay: nothing of the state is left
     return Rn;
 }

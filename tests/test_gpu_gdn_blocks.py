@@ -55,6 +55,24 @@ def test_gdn_scan_block_edges(lens, kind, outputs):
             assert maxrel_per_head(o[sl], o_ref, 1) <= TOL_BF16
 
 
+@pytest.mark.parametrize("decay", [0.01, 0.6, 1.0, 3.0])
+def test_gdn_scan_is_homogeneous(decay):
+    """Values and states times a power of two: the results times that power, bit for bit.  (A held state times 2^100 became infinite
+    from 2^27 on.)"""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    rn = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    T = 1000
+    bf = torch.bfloat16
+    unit = lambda x: torch.nn.functional.normalize(x, dim=-1).to(bf)
+    q, k, v, S0 = unit(rn(T, 2, 128)), unit(rn(T, 2, 128)), rn(T, 4, 128).to(bf), rn(1, 4, 128, 128)
+    beta, g = torch.rand(T, 4, generator=gen, device="cuda"), -2 * decay * torch.rand(T, 4, generator=gen, device="cuda")
+    o, S = b.lkv_gdn_fwd(q, k, v, g, beta, S0)
+    for f in (2.0 ** 42, 2.0 ** -80):
+        of, Sf = b.lkv_gdn_fwd(q, k, v * f, g, beta, S0 * f)
+        assert torch.equal(of, o * f) and torch.equal(Sf, S * f)
+
+
 def test_gdn_scan_time_bends_with_the_decays_but_does_not_break():
     """Decays of 250 log2 units a block (the exact form, whose mask takes an exponential per element) against mild ones: it took three
     times as long while that form was written for rare use."""

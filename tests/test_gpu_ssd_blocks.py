@@ -43,6 +43,29 @@ def test_ssd_scan_block_edges(H, G, lens, decay, outputs):
             assert maxrel_per_head(y[sl], y_ref, 1) <= TOL_BF16
 
 
+@pytest.mark.parametrize("A, power", [(-0.2, 50), (-3.0, 50), (-5.0, 24), (-60.0, 24)])
+def test_ssd_scan_is_homogeneous(A, power):
+    """Inputs and states times a power of two: the results times that power, upwards bit for bit.  (A held state times 2^100 became
+    infinite from 2^27 on.)  Downwards the low halves of the factors of x leave the range first: one more rounding to bf16."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    rn = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    T, H = 1000, 4
+    bf = torch.bfloat16
+    x, B, C = rn(T, H, 64).to(bf), (rn(T, 1, 128) / 128 ** 0.5).to(bf), (rn(T, 1, 128) / 128 ** 0.5).to(bf)
+    dt, S0 = torch.nn.functional.softplus(-2.0 + 0.5 * rn(T, H)), rn(1, H, 128, 64)
+    a = torch.full((H,), A, device="cuda")
+    y, S = b.lkv_ssd_fwd(x, dt, a, B, C, S0)
+    f = 2.0 ** power
+    yf, Sf = b.lkv_ssd_fwd(x * f, dt, a, B, C, S0 * f)
+    assert torch.equal(yf, y * f) and torch.equal(Sf, S * f)
+    yf, Sf = b.lkv_ssd_fwd(x / f, dt, a, B, C, S0 / f)
+    assert maxrel_per_head(host(yf * f), host(y), 1) <= 2.0 ** -8 and maxrel_per_head(host(Sf * f), host(S), 1) <= 2.0 ** -8
+    yf, Sf = b.lkv_ssd_fwd(x * 0.0, dt, a, B, C, S0 * 2.0 ** 110)   # a state that is only carried on
+    y0, S1 = b.lkv_ssd_fwd(x * 0.0, dt, a, B, C, S0)
+    assert torch.isfinite(yf).all() and torch.equal(yf[:8], y0[:8] * 2.0 ** 110)
+
+
 @pytest.mark.parametrize("every, dt", [(37, 60.0), (16, 1000.0), (5, 30.0)])
 def test_ssd_scan_with_tokens_that_forget_everything(every, dt):
     """Single tokens whose own decay is beyond the range of a block's scale, among mild ones: they cut tiles at any offset."""
