@@ -4,8 +4,6 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
-#include <string.h>
-
 #include <type_traits>
 
 #include "../../include/lkv.h"
@@ -75,23 +73,11 @@ struct IndexBlock {
 };
 constexpr int kInitIdxCap = 4000;  // ints: cu_k | sel | ids
 constexpr int kScanIdxCap = 1000;  // ints: cu_seqlens[n_seq + 1] | launch order[n_seq]
-// Most calls have short lists, and a launch is the slower the more parameter bytes it carries (16 KB: 1.1 us).  The initialisers and
-// the fp32 scans therefore exist with a short list too, and with_args() hands the launch whichever form of the arguments fits.
-// Not the tensor-core scans: as one of two instantiations in their module the GDN scan ran 27 % slower with every SM busy
-// (instruction fetch), with either list.
-constexpr int kSmallIdxCap = 96;   // ints: 32 requests with one chunk each, scans of 47 sequences
-template <template <int> class Args, int CAP, typename F>
-cudaError_t with_args(const Args<CAP> &a, F &&launch) {
-    const auto &idx = a.index();
-    if (!idx.ptr && idx.n > kSmallIdxCap) return launch(a);
-    Args<kSmallIdxCap> s;
-    static_cast<typename Args<CAP>::Base &>(s) = a;
-    auto &small = s.index();
-    small.ptr = idx.ptr;
-    small.n = idx.n;
-    if (!idx.ptr) memcpy(small.v, idx.v, sizeof(int32_t) * idx.n);
-    return launch(s);
-}
+// A launch is the slower the more parameter bytes it carries.  It shows where the kernel is next to nothing and the kernel after it waits for
+// no more than its launch: the copy of one cached state followed by the scan of a 37-token suffix takes 10.1 us with this short
+// list and 10.9 with the long one (in turn on one GPU, twice); composition and the fp32 kernels take the same time with either.  So
+// the copy exists with a short list too.
+constexpr int kSmallIdxCap = 96;   // ints: 32 requests with one chunk each
 
 // Launch-side records shared by the entry points and the kernels.  Passed by value as
 // __grid_constant__ kernel parameters.
@@ -106,10 +92,7 @@ struct InitArgsBase {
 };
 template <int CAP>
 struct InitArgsT : InitArgsBase {
-    using Base = InitArgsBase;
     IndexBlock<CAP> idx;
-    const IndexBlock<CAP> &index() const { return idx; }
-    IndexBlock<CAP> &index() { return idx; }
     __device__ __forceinline__ int cu_k(int r) const { return idx[r]; }
     __device__ __forceinline__ int id(int i) const { return idx[off_ids + i]; }
     __device__ __forceinline__ int sel(int r, int K) const { return off_sel < 0 ? K - 1 : idx[off_sel + r]; }
@@ -118,7 +101,7 @@ using InitArgs = InitArgsT<kInitIdxCap>;
 
 int sm_count();   // of the current device
 
-struct GdnArgsBase {
+struct GdnArgs {
     const void *q, *k, *v;
     const float *g, *beta, *S0;
     void *o;
@@ -140,17 +123,10 @@ struct GdnArgsBase {
     int32_t n_s0, st_first;
     const float *S0_more;
     int32_t *status;
+    IndexBlock<kScanIdxCap> cu;  // cu_seqlens[n_seq + 1], then the launch order: sequence of grid row y at [n_seq + 1 + y]
 };
-template <int CAP>
-struct GdnArgsT : GdnArgsBase {
-    using Base = GdnArgsBase;
-    IndexBlock<CAP> cu;  // cu_seqlens[n_seq + 1], then the launch order: sequence of grid row y at [n_seq + 1 + y]
-    const IndexBlock<CAP> &index() const { return cu; }
-    IndexBlock<CAP> &index() { return cu; }
-};
-using GdnArgs = GdnArgsT<kScanIdxCap>;
 
-struct SsdArgsBase {
+struct SsdArgs {
     const void *x, *B, *C;
     const float *dt, *A, *S0;
     void *y;
@@ -164,15 +140,8 @@ struct SsdArgsBase {
     float *lam;
     int32_t n_seq, T_total, H, P, N, G;
     int32_t *status;
+    IndexBlock<kScanIdxCap> cu;  // cu_seqlens[n_seq + 1]
 };
-template <int CAP>
-struct SsdArgsT : SsdArgsBase {
-    using Base = SsdArgsBase;
-    IndexBlock<CAP> cu;  // cu_seqlens[n_seq + 1]
-    const IndexBlock<CAP> &index() const { return cu; }
-    IndexBlock<CAP> &index() { return cu; }
-};
-using SsdArgs = SsdArgsT<kScanIdxCap>;
 
 // Kernel launchers (one translation unit each); all return a cudaError_t from the launch.
 cudaError_t launch_init_single(const InitArgs &a, bool pool_bf16, cudaStream_t s);

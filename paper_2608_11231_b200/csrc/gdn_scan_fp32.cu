@@ -29,8 +29,8 @@ constexpr int kC = 32;  // tokens per block
 __host__ __device__ constexpr int row_stride(int dk) { return (((dk + 3) / 4) | 1) * 4; }
 constexpr int kLdA = kC + 4;   // row stride of the coupling matrix A (read by lane = row)
 
-template <typename T, int VC, class Args>
-__global__ void __launch_bounds__(256) gdn_scan_fp32_kernel(const __grid_constant__ Args a) {
+template <typename T, int VC>
+__global__ void __launch_bounds__(256) gdn_scan_fp32_kernel(const __grid_constant__ GdnArgs a) {
     constexpr int NG = 256 / VC;   // thread groups along tokens / state rows
     constexpr int TPER = kC / NG;  // tokens per thread in the token-parallel steps
     static_assert(kC % NG == 0 && TPER >= 1, "block shape");
@@ -269,12 +269,10 @@ size_t smem_bytes(int dk, int vc) {
 template <typename T, int VC>
 cudaError_t launch(const GdnArgs &a, cudaStream_t s) {
     const size_t smem = smem_bytes(a.d_k, VC);
-    return with_args(a, [&](const auto &x) {
-        auto kernel = gdn_scan_fp32_kernel<T, VC, std::decay_t<decltype(x)>>;
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        return launch_chained(kernel, dim3(a.H_v, a.n_seq, a.d_v / VC), 256, smem, s, x);
-    });
+    auto kernel = gdn_scan_fp32_kernel<T, VC>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_chained(kernel, dim3(a.H_v, a.n_seq, a.d_v / VC), 256, smem, s, a);
 }
 
 // Columns per CTA: all of them when heads and sequences fill the GPU; otherwise halved as long as that still finds idle SMs.

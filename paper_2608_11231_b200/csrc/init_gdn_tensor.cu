@@ -62,9 +62,9 @@ __device__ __forceinline__ int stage_of(int j) { return (j - 1) % kStages; }
 __device__ __forceinline__ uint32_t phase_of(int j) { return static_cast<uint32_t>((j - 1) / kStages) & 1u; }
 
 // SBF16: the cached states are stored as bf16 (the transitions are fp32 either way); S0 is written as fp32.
-template <bool SBF16, class Args>
+template <bool SBF16>
 __global__ void __launch_bounds__(kThreads, 1)
-init_gdn_exact_tensor_kernel(const __grid_constant__ Args a, const __grid_constant__ CUtensorMap mapT) {
+init_gdn_exact_tensor_kernel(const __grid_constant__ InitArgs a, const __grid_constant__ CUtensorMap mapT) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *sm = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);   // an offset, not a cast: the compiler keeps shared-memory addressing
     // fullT: TMA transactions; roundT: the rounding warps are done with the stage; freeT: the MMAs of the step have read it;
@@ -245,13 +245,10 @@ cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cuda
     CUtensorMap mapT;
     const uint64_t rows = static_cast<uint64_t>(a.n_chunks) * a.H * kD;
     if (!make_tensor_map_2d(&mapT, a.transitions, 4, kD, rows, kD * 4, 32, kD, true)) return cudaErrorInvalidValue;
-    return with_args(a, [&](const auto &x) {
-        using Args = std::decay_t<decltype(x)>;
-        auto kernel = pool_bf16 ? init_gdn_exact_tensor_kernel<true, Args> : init_gdn_exact_tensor_kernel<false, Args>;
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        return launch_kernel(early, kernel, dim3(a.H, a.n_req), kThreads, kSmemBytes, s, x, mapT);
-    });
+    auto kernel = pool_bf16 ? init_gdn_exact_tensor_kernel<true> : init_gdn_exact_tensor_kernel<false>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e != cudaSuccess) return e;
+    return launch_kernel(early, kernel, dim3(a.H, a.n_req), kThreads, kSmemBytes, s, a, mapT);
 }
 
 }  // namespace lkv

@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(256) init_single_kernel(const __grid_constant_
 // S <- S_{c_1};  S <- exp(lambda_{c_j,h}) S + S_{c_j}.  Pure streaming: every thread owns
 // one 16-byte vector of the state and walks the K chunks with kUnroll independent loads
 // in flight; the decays are K scalars per head.  grid = (vectors per state / 256, n_req).
-template <bool BF16, class Args>
-__global__ void __launch_bounds__(256) init_mamba_exact_kernel(const __grid_constant__ Args a, size_t state_elems, int head_elems) {
+template <bool BF16>
+__global__ void __launch_bounds__(256) init_mamba_exact_kernel(const __grid_constant__ InitArgs a, size_t state_elems, int head_elems) {
     using PV = PoolVec<BF16>;
     constexpr int E = PV::kElems;
     constexpr int kUnroll = 8;
@@ -122,8 +122,8 @@ constexpr int kMaxStages = 6;
 // row stride (floats) of a staged transition: 16-byte rows, successive rows four banks apart
 __host__ __device__ constexpr int t_stride(int dk) { return (((dk + 3) / 4) | 1) * 4; }
 
-template <bool BF16, int TN, class Args>
-__global__ void __launch_bounds__(256) init_gdn_exact_fp32_kernel(const __grid_constant__ Args a, int stages) {
+template <bool BF16, int TN>
+__global__ void __launch_bounds__(256) init_gdn_exact_fp32_kernel(const __grid_constant__ InitArgs a, int stages) {
     constexpr int RG = 256 / TN, U = kTM / RG;   // thread (rg, c) has rows rg, rg + RG, ... of column c
     extern __shared__ __align__(16) float smem[];
     const int dk = a.d_k, dv = a.d_v, ts = t_stride(dk);
@@ -225,12 +225,10 @@ cudaError_t launch_gdn_fp32(const InitArgs &a, cudaStream_t s) {
     const size_t state = 2 * static_cast<size_t>(a.d_k) * TN * sizeof(float), stage = static_cast<size_t>(kTM) * t_stride(a.d_k) * sizeof(float);
     const int stages = static_cast<int>(std::min<size_t>(kMaxStages, (227 * 1024 - state) / stage));
     const size_t smem = state + stages * stage;
-    return with_args(a, [&](const auto &x) {
-        auto kernel = init_gdn_exact_fp32_kernel<BF16, TN, std::decay_t<decltype(x)>>;
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        return launch_chained(kernel, dim3((a.d_v + TN - 1) / TN, a.H, a.n_req), 256, smem, s, x, stages);
-    });
+    auto kernel = init_gdn_exact_fp32_kernel<BF16, TN>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_chained(kernel, dim3((a.d_v + TN - 1) / TN, a.H, a.n_req), 256, smem, s, a, stages);
 }
 
 }  // namespace
@@ -239,20 +237,24 @@ cudaError_t launch_init_single(const InitArgs &a, bool pool_bf16, cudaStream_t s
     const size_t elems = static_cast<size_t>(a.H) * a.d_k * a.d_v;
     const int per = pool_bf16 ? 8 : 4;
     dim3 grid(static_cast<unsigned>((elems / per + 255) / 256), a.n_req);
-    return with_args(a, [&](const auto &x) {
+    auto launch = [&](const auto &x) {
         using Args = std::decay_t<decltype(x)>;
         return launch_chained(pool_bf16 ? init_single_kernel<true, Args> : init_single_kernel<false, Args>, grid, 256, 0, s, x, elems);
-    });
+    };
+    if (!a.idx.ptr && a.idx.n > kSmallIdxCap) return launch(a);
+    InitArgsT<kSmallIdxCap> small;
+    static_cast<InitArgsBase &>(small) = a;
+    small.idx.ptr = a.idx.ptr;
+    small.idx.n = a.idx.n;
+    if (!a.idx.ptr) std::copy(a.idx.v, a.idx.v + a.idx.n, small.idx.v);
+    return launch(small);
 }
 
 cudaError_t launch_init_mamba_exact(const InitArgs &a, bool pool_bf16, cudaStream_t s) {
     const size_t elems = static_cast<size_t>(a.H) * a.d_k * a.d_v;
     const int per = pool_bf16 ? 8 : 4;
     dim3 grid(static_cast<unsigned>((elems / per + 255) / 256), a.n_req);
-    return with_args(a, [&](const auto &x) {
-        using Args = std::decay_t<decltype(x)>;
-        return launch_chained(pool_bf16 ? init_mamba_exact_kernel<true, Args> : init_mamba_exact_kernel<false, Args>, grid, 256, 0, s, x, elems, a.d_k * a.d_v);
-    });
+    return launch_chained(pool_bf16 ? init_mamba_exact_kernel<true> : init_mamba_exact_kernel<false>, grid, 256, 0, s, a, elems, a.d_k * a.d_v);
 }
 
 // 32 columns of the state per CTA, or 8 where that many CTAs still find an SM each (a step is then a quarter of the work: what
@@ -268,8 +270,7 @@ namespace {
 
 // One warp per (sequence, group of 32 heads): lanes walk consecutive heads, so every token's dt row is read with
 // coalesced 128-byte accesses; four partial sums per lane keep several loads in flight.
-template <class Args>
-__global__ void mamba_logdecay_kernel(const __grid_constant__ Args a, float *__restrict__ out) {
+__global__ void mamba_logdecay_kernel(const __grid_constant__ SsdArgs a, float *__restrict__ out) {
     const int seq = blockIdx.y;
     const int h = blockIdx.x * 32 + (threadIdx.x & 31);
     const int part = threadIdx.x >> 5, nparts = blockDim.x >> 5;
@@ -292,9 +293,7 @@ __global__ void mamba_logdecay_kernel(const __grid_constant__ Args a, float *__r
 }  // namespace
 
 cudaError_t launch_mamba_logdecay(const SsdArgs &a, float *logdecay, cudaStream_t s) {
-    return with_args(a, [&](const auto &x) {
-        return launch_chained(mamba_logdecay_kernel<std::decay_t<decltype(x)>>, dim3((a.H + 31) / 32, a.n_seq), 256, 0, s, x, logdecay);
-    });
+    return launch_chained(mamba_logdecay_kernel, dim3((a.H + 31) / 32, a.n_seq), 256, 0, s, a, logdecay);
 }
 
 namespace {

@@ -34,9 +34,9 @@ __device__ __forceinline__ void bulk_load(void *smem_dst, const void *gmem_src, 
                  : "memory");
 }
 
-template <bool BF16, int PER, class Args>
+template <bool BF16, int PER>
 __global__ void __launch_bounds__(kConsumers + 32, 1)
-init_mamba_exact_stream_kernel(const __grid_constant__ Args a, size_t state_elems, int head_elems, int tiles_per_state) {
+init_mamba_exact_stream_kernel(const __grid_constant__ InitArgs a, size_t state_elems, int head_elems, int tiles_per_state) {
     constexpr int kElemBytes = BF16 ? 2 : 4;
     constexpr int kPieceElems = kPieceBytes / kElemBytes;
     constexpr int kTileBytes = PER * kPieceBytes;
@@ -177,12 +177,10 @@ static cudaError_t launch_stream(const InitArgs &a, int sms, cudaStream_t s) {
     const int tiles = static_cast<int>((pieces + PER - 1) / PER);
     const long long units = static_cast<long long>(a.n_req) * tiles;
     const int grid = static_cast<int>(units < sms ? units : sms);
-    return with_args(a, [&](const auto &x) {
-        auto kernel = init_mamba_exact_stream_kernel<BF16, PER, std::decay_t<decltype(x)>>;
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        return launch_chained(kernel, grid, kConsumers + 32, kSmemBytes, s, x, elems, a.d_k * a.d_v, tiles);
-    });
+    auto kernel = init_mamba_exact_stream_kernel<BF16, PER>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e != cudaSuccess) return e;
+    return launch_chained(kernel, grid, kConsumers + 32, kSmemBytes, s, a, elems, a.d_k * a.d_v, tiles);
 }
 
 cudaError_t launch_init_mamba_exact_stream(const InitArgs &a, bool pool_bf16, cudaStream_t s) {

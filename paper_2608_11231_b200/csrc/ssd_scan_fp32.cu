@@ -14,8 +14,8 @@ namespace {
 
 constexpr int kQ = 32;
 
-template <typename T, int P, class Args>
-__global__ void __launch_bounds__(256) ssd_scan_fp32_kernel(const __grid_constant__ Args a) {
+template <typename T, int P>
+__global__ void __launch_bounds__(256) ssd_scan_fp32_kernel(const __grid_constant__ SsdArgs a) {
     constexpr int NG = 256 / P;
     constexpr int TPER = kQ / NG;
     static_assert(kQ % NG == 0 && TPER >= 1, "block shape");
@@ -121,12 +121,10 @@ size_t smem_bytes(int N, int P) {
 template <typename T, int P>
 cudaError_t launch(const SsdArgs &a, cudaStream_t s) {
     const size_t smem = smem_bytes(a.N, P);
-    return with_args(a, [&](const auto &x) {
-        auto kernel = ssd_scan_fp32_kernel<T, P, std::decay_t<decltype(x)>>;
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        return launch_chained(kernel, dim3(a.H, a.n_seq), 256, smem, s, x);
-    });
+    auto kernel = ssd_scan_fp32_kernel<T, P>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_chained(kernel, dim3(a.H, a.n_seq), 256, smem, s, a);
 }
 
 template <typename T>

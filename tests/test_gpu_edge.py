@@ -234,3 +234,14 @@ def test_long_index_list_is_refused_under_stream_capture():
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(S0[:10], ref[:10])
+
+
+@pytest.mark.parametrize("n_req", [1, 47, 48, 60, 1999, 2000])
+def test_single_state_init_with_index_lists_of_every_kind(n_req):
+    """2 n + 1 indices: the short kernel parameters (up to 96), the long ones (up to 4000), the workspace."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(n_req)
+    states = torch.randn((50, 2, 16, 8), generator=gen, device="cuda")
+    ids = np.random.default_rng(n_req).integers(0, 50, n_req).astype(np.int32)
+    S0 = b.lkv_init_state_batched(states, None, ids, np.arange(n_req + 1, dtype=np.int32), n_req, b.LKV_INIT_LAST, family=b.LKV_FAMILY_GDN)
+    assert torch.equal(S0, states[torch.from_numpy(ids).long().cuda()])
