@@ -16,6 +16,7 @@ input copied host->device from pinned memory and every result copied back inside
 from __future__ import annotations
 
 import argparse
+import ctypes
 import json
 import os
 import statistics
@@ -128,7 +129,7 @@ class Family:
         self.host_out = torch.empty(self.out_shape, dtype=bf).pin_memory()
         self.host_S_T = torch.empty(self.S_T.shape, dtype=torch.float32).pin_memory()
         self.ws_init = torch.zeros(1 << 20, dtype=torch.uint8, device="cuda")
-        self.ws_scan = torch.zeros(1 << 16, dtype=torch.uint8, device="cuda")
+        self.ws_scan = self.scan_workspace(T, self.n_req)
         self.h2d_bytes = sum(t.numel() * t.element_size() for t in self.host.values())
         self.d2h_bytes = self.host_out.numel() * 2 + self.host_S_T.numel() * 4
         # bytes an exact composition must move at least once: every pool state and transition that some request reads
@@ -139,7 +140,21 @@ class Family:
         per_trans = h["trans"][0].numel() * 4
         self.compose_bytes = len(first | later) * per_state + len(later) * per_trans + self.n_req * per_state
         self.set_bytes = self.h2d_bytes
-        self.launches = 3
+        # one long sequence is scanned in segments: two launches more
+        self.launches = 5 if self.n_req == 1 and self.ws_scan.numel() > self.scan_workspace(T, 2).numel() else 3
+
+    def scan_workspace(self, tokens, n_seq):
+        """The workspace that the library asks for: what a caller of the public API has without passing one."""
+        b = self.b
+        if self.fam == "gdn":
+            s = GDN_SHAPE
+            d = b.lkv_gdn_desc(T_total=tokens, n_seq=n_seq, H_k=s["H_k"], H_v=s["H_v"], d_k=s["d_k"], d_v=s["d_v"], io_dtype=b.LKV_DTYPE_BF16)
+            which = b.LKV_WS_GDN
+        else:
+            s = SSD_SHAPE
+            d = b.lkv_ssd_desc(T_total=tokens, n_seq=n_seq, H=s["H"], P=s["P"], N=s["N"], G=s["G"], io_dtype=b.LKV_DTYPE_BF16)
+            which = b.LKV_WS_SSD
+        return self.torch.zeros(b.lkv_workspace_bytes(which, d, n_seq), dtype=self.torch.uint8, device="cuda")
 
     def cold_copy(self):
         """A second instance over the same host data with device buffers of its own (inputs and outputs): launches
@@ -174,7 +189,7 @@ class Family:
             for n in ("S0_last", "S0", "S_T", "host_S_T"):
                 setattr(c, n, getattr(self, n)[r0:r1])
             c.out, c.host_out = self.out[t0:t1], self.host_out[t0:t1]
-            c.ws_init, c.ws_scan = self.ws_init.clone(), self.ws_scan.clone()
+            c.ws_init, c.ws_scan = self.ws_init.clone(), self.scan_workspace(t1 - t0, c.n_req)
             out.append(c)
         return out
 
@@ -231,23 +246,29 @@ class Family:
             self.full_ST = torch.empty((1,) + self.state_shape, dtype=torch.float32, device="cuda")
             self.full_out = torch.empty((tokens, s["H"], s["P"]), dtype=bf, device="cuda")
         self.full_tokens = tokens
+        self.ws_full = self.scan_workspace(tokens, 1)
 
     def full_prefill_segmented(self):
-        """The same full prefill with the sequence cut into segments scanned in parallel (GDN; the library picks the count)."""
+        """The same full prefill through the call that takes a number of segments and scratch of its own (GDN; the library picks both)."""
         b, d = self.b, self.full
         if getattr(self, "seg_scratch", None) is None:
             s = GDN_SHAPE
             self.seg_scratch = self.torch.empty(64 * s["H_v"] * s["d_k"] * s["d_v"] * 4, dtype=self.torch.uint8, device="cuda")
         b.lkv_gdn_fwd_segmented(d["q"], d["k"], d["v"], d["g"], d["beta"], None, self.full_out, self.full_ST, n_segments=0,
-                                scratch=self.seg_scratch, workspace_t=self.ws_scan)
+                                scratch=self.seg_scratch, workspace_t=self.ws_full)
+
+    def segment_scratch_bytes(self):
+        b, s = self.b, GDN_SHAPE
+        d = b.lkv_gdn_desc(T_total=self.full_tokens, n_seq=1, H_k=s["H_k"], H_v=s["H_v"], d_k=s["d_k"], d_v=s["d_v"], io_dtype=b.LKV_DTYPE_BF16)
+        return int(b.load().lkv_gdn_segmented_scratch_bytes(ctypes.byref(d), 0))
 
     def full_prefill(self):
         b, d = self.b, self.full
         if self.fam == "gdn":
-            b.lkv_gdn_fwd(d["q"], d["k"], d["v"], d["g"], d["beta"], None, self.full_out, self.full_ST, workspace_t=self.ws_scan)
+            b.lkv_gdn_fwd(d["q"], d["k"], d["v"], d["g"], d["beta"], None, self.full_out, self.full_ST, workspace_t=self.ws_full)
         else:
             b.lkv_ssd_fwd(d["x"], d["dt"], self.dev["A"], d["B"], d["C"], None, self.full_out, self.full_ST,
-                          workspace_t=self.ws_scan)
+                          workspace_t=self.ws_full)
 
 
 class ClockSampler:
@@ -542,11 +563,12 @@ def measure_workload(name, rank, world, args, torch, b, dist, timer, peaks, with
             full[f.fam] = dict(tokens=f.full_tokens, us=1e3 * t, tokens_per_s=f.full_tokens / (t * 1e-3),
                                cached_path_us_per_request=1e3 * t_cached, cached_over_full=t_cached / t)
             if f.fam == "gdn":
-                # the same prefill as a sequence-parallel scan (lkv_gdn_fwd_segmented, segment count chosen by the library)
+                # the same prefill with the scratch of its segments passed separately (lkv_gdn_fwd_segmented)
                 g2 = timer.graph_of(f.full_prefill_segmented)
                 t2 = 1e-3 * statistics.median(1e3 * x for x in timer.flushed(g2.replay, max(steps, 5)))
                 full[f.fam]["segmented_us"] = 1e3 * t2
-                full[f.fam]["segments"] = max(1, min((148 // GDN_SHAPE["H_v"] + 3) // 2, f.full_tokens // 512))
+                slot = 4 * int(np.prod(f.state_shape))
+                full[f.fam]["segments"] = max(1, (f.segment_scratch_bytes() // slot + 3) // 4)   # scratch: 4 n - 3 states
                 f.seg_scratch = None
             del f.full, f.full_out
 
