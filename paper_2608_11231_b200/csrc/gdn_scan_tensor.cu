@@ -36,11 +36,12 @@
 //
 // What bounds it: neither a pipe (tensor 36 %, issue slots 39 % with every SM busy) nor one chain, but the latency of about
 // 6 K instructions per block in ten programs that share an SM: mask 1.7 K cycles, inverse 3.0 K, chain 2.1 K of a block period of
-// 3.3 K -- and instruction fetch: 5 KB less code in the issuing and scalar warps (each piece of code once, its loop started a
-// block early instead of a copy before it) took 32 x 4096 tokens from 992 to 940 us.  Hence small rolled loops, fp16 storage of what is an fp16 operand, ldmatrix / movmatrix instead of fp32 round trips, and
-// few warps: outputs in a warpgroup of their own, or the last merge of the inverse moved to the W warps, made every program slower
-// (8 % and 17 % on one sequence).  Measured on B200, 32 value heads: one sequence of 8192 tokens 311 -> 254 us, 32 x 4096 tokens
-// 1172 -> 982 us against the form that gates the products and solves for u in the chain (three conversions).
+// 3.3 K -- and instruction fetch: 7 KB less code in the issuing and scalar warps (each piece of code once, its loop started a
+// block early instead of a copy before it) took 32 x 4096 tokens from 992 to 940 us.  Hence small rolled loops, fp16 storage of what
+// is an fp16 operand, ldmatrix / movmatrix instead of fp32 round trips, and few warps: outputs in a warpgroup of their own, or the last
+// merge of the inverse moved to the W warps, made every program slower (8 % and 17 % on one sequence).  Measured on B200, 32
+// value heads: one sequence of 8192 tokens 311 -> 237 us as one chain, 32 x 4096 tokens 1172 -> 940 us against the form that gates
+// the products and solves for u in the chain (three conversions).
 #include <cuda_fp16.h>
 #include <string.h>
 

@@ -268,8 +268,8 @@ cudaError_t launch_init_gdn_exact_fp32(const InitArgs &a, bool pool_bf16, cudaSt
 
 namespace {
 
-// One warp per (sequence, group of 32 heads): lanes walk consecutive heads, so every token's dt row is read with
-// coalesced 128-byte accesses; four partial sums per lane keep several loads in flight.
+// One CTA per (sequence, group of 32 heads): lanes walk consecutive heads, so every token's dt row is read with coalesced
+// 128-byte accesses; each of the eight warps sums every eighth token, and their sums are added in a fixed order.
 __global__ void mamba_logdecay_kernel(const __grid_constant__ SsdArgs a, float *__restrict__ out) {
     const int seq = blockIdx.y;
     const int h = blockIdx.x * 32 + (threadIdx.x & 31);
