@@ -172,23 +172,32 @@ _ws_replaced = []
 _err_ws_cache = {}
 
 
-def workspace(device, nbytes: int) -> torch.Tensor:
-    """A zero-initialised, cached device workspace of at least nbytes (one per device and stream).
+def _cached(cache, device, nbytes: int) -> torch.Tensor:
+    """The zero-initialised buffer of at least nbytes that `cache` holds for this device and the current stream.
 
-    A workspace that has become too small is replaced but not given back: a CUDA graph captured with it, or a call that another
+    A buffer that has become too small is replaced but not given back: a CUDA graph captured with it, or a call that another
     thread has in flight, still writes there.  Sizes at least double, so that all the replaced ones together are smaller than
     the one in use.
     """
     key = (torch.device(device).index, torch.cuda.current_stream().cuda_stream)
-    ws = _ws_cache.get(key)
+    ws = cache.get(key)
     if ws is None or ws.numel() < nbytes:
         size = max(int(nbytes), 4096)
         if ws is not None:
             size = max(size, 2 * ws.numel())
             _ws_replaced.append(ws)
-        ws = torch.zeros(size, dtype=torch.uint8, device=device)
-        _ws_cache[key] = ws
+        ws = cache[key] = torch.zeros(size, dtype=torch.uint8, device=device)
     return ws
+
+
+def workspace(device, nbytes: int) -> torch.Tensor:
+    """A zero-initialised, cached device workspace of at least nbytes (one per device and stream)."""
+    return _cached(_ws_cache, device, nbytes)
+
+
+def error_workspace(device, nbytes: int) -> torch.Tensor:
+    """The same for lkv_state_rel_error, which keeps partial sums from byte 0 on and has no status header."""
+    return _cached(_err_ws_cache, device, nbytes)
 
 
 def lkv_workspace_bytes(which: int, desc, n_units: int, n_index: int = 0) -> int:
@@ -393,11 +402,7 @@ def lkv_state_rel_error(S_init, S_ref, n_states: Optional[int] = None, rel_err=N
     if rel_err is None:
         rel_err = torch.empty((n,), dtype=torch.float32, device=S_init.device)
     nbytes = load().lkv_state_rel_error_workspace_bytes(n, elems)
-    # scratch of its own: this call keeps partial sums from byte 0 on, it has no status header
-    key = torch.device(S_init.device).index
-    ws_t = _err_ws_cache.get(key)
-    if ws_t is None or ws_t.numel() < nbytes:
-        ws_t = _err_ws_cache[key] = torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=S_init.device)
+    ws_t = error_workspace(S_init.device, nbytes)
     st = load().lkv_state_rel_error(_ptr(S_init), _ptr(S_ref), _ptr(rel_err), n, elems, ws_t.data_ptr(), ws_t.numel(),
                                     _stream(stream))
     if st != LKV_OK:

@@ -303,23 +303,29 @@ def test_chunk_artifacts_argument_errors(lib):
     assert f(_gdn_desc(workspace_bytes=8)) == b.LKV_ERR_WORKSPACE
 
 
-def test_replaced_workspaces_stay_alive(monkeypatch):
-    """A captured graph keeps the address of the workspace it was recorded with: growing must not give that memory back."""
+@pytest.mark.parametrize("make, cache", [("workspace", "_ws_cache"), ("error_workspace", "_err_ws_cache")])
+def test_replaced_workspaces_stay_alive(monkeypatch, make, cache):
+    """A captured graph keeps the address of the workspace it was recorded with: growing must not give that memory back.  And
+    streams do not share one."""
     import gc
     import types
     import weakref
 
     import torch
-    monkeypatch.setattr(b, "_ws_cache", {})
+    monkeypatch.setattr(b, cache, {})
     monkeypatch.setattr(b, "_ws_replaced", [])
-    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0))
-    first = weakref.ref(b.workspace("cpu", 100))
+    stream = types.SimpleNamespace(cuda_stream=0)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: stream)
+    get = getattr(b, make)
+    first = weakref.ref(get("cpu", 100))
     sizes = [first().numel()]
     for need in (5000, 6000, 40_000, 10):
-        ws = b.workspace("cpu", need)
+        ws = get("cpu", need)
         assert ws.numel() >= need and not ws.any()
         if ws.numel() != sizes[-1]:
             sizes.append(ws.numel())
     gc.collect()
     assert first() is not None
     assert sum(sizes[:-1]) <= sizes[-1]
+    stream.cuda_stream = 7
+    assert get("cpu", 10).data_ptr() != ws.data_ptr()
