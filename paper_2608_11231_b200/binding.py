@@ -9,6 +9,7 @@ missing, the first call raises.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 from typing import Optional, Sequence
@@ -172,32 +173,37 @@ _ws_replaced = []
 _err_ws_cache = {}
 
 
-def _cached(cache, device, nbytes: int) -> torch.Tensor:
-    """The zero-initialised buffer of at least nbytes that `cache` holds for this device and the current stream.
+def _cached(cache, device, nbytes: int, stream=None) -> torch.Tensor:
+    """The zero-initialised buffer of at least nbytes that `cache` holds for this device and the stream of the call (a stream, its
+    raw handle, or None for the current one): calls on different streams may overlap, so they do not share one.
 
     A buffer that has become too small is replaced but not given back: a CUDA graph captured with it, or a call that another
     thread has in flight, still writes there.  Sizes at least double, so that all the replaced ones together are smaller than
     the one in use.
     """
-    key = (torch.device(device).index, torch.cuda.current_stream().cuda_stream)
+    current = torch.cuda.current_stream().cuda_stream
+    raw = current if stream is None else getattr(stream, "cuda_stream", stream)
+    key = (torch.device(device).index, raw)
     ws = cache.get(key)
     if ws is None or ws.numel() < nbytes:
         size = max(int(nbytes), 4096)
         if ws is not None:
             size = max(size, 2 * ws.numel())
             _ws_replaced.append(ws)
-        ws = cache[key] = torch.zeros(size, dtype=torch.uint8, device=device)
+        # filled on the stream that will use it
+        with contextlib.nullcontext() if raw == current else torch.cuda.stream(torch.cuda.ExternalStream(raw)):
+            ws = cache[key] = torch.zeros(size, dtype=torch.uint8, device=device)
     return ws
 
 
-def workspace(device, nbytes: int) -> torch.Tensor:
+def workspace(device, nbytes: int, stream=None) -> torch.Tensor:
     """A zero-initialised, cached device workspace of at least nbytes (one per device and stream)."""
-    return _cached(_ws_cache, device, nbytes)
+    return _cached(_ws_cache, device, nbytes, stream)
 
 
-def error_workspace(device, nbytes: int) -> torch.Tensor:
+def error_workspace(device, nbytes: int, stream=None) -> torch.Tensor:
     """The same for lkv_state_rel_error, which keeps partial sums from byte 0 on and has no status header."""
-    return _cached(_err_ws_cache, device, nbytes)
+    return _cached(_err_ws_cache, device, nbytes, stream)
 
 
 def lkv_workspace_bytes(which: int, desc, n_units: int, n_index: int = 0) -> int:
@@ -218,14 +224,14 @@ def lkv_selftest_bounded_wait(poll_limit: int, ws: torch.Tensor, stream=None) ->
     return int(load().lkv_selftest_bounded_wait(int(poll_limit), _ptr(ws), _stream(stream)))
 
 
-def _init_desc(states, family, compute, ws_t, n_units, n_index, chunk_ids_np=None, sel_index=0):
+def _init_desc(states, family, compute, ws_t, n_units, n_index, chunk_ids_np=None, sel_index=0, stream=None):
     n, H, d_k, d_v = states.shape
     d = lkv_init_desc(family=family, H=H, d_k=d_k, d_v=d_v, n_chunks=n, state_dtype=_dtype_code(states),
                       sel_index=int(sel_index), compute=compute,
                       chunk_ids=None if chunk_ids_np is None else chunk_ids_np.ctypes.data, workspace=None,
                       workspace_bytes=0)
     if ws_t is None:
-        ws_t = workspace(states.device, lkv_workspace_bytes(LKV_WS_INIT, d, n_units, n_index))
+        ws_t = workspace(states.device, lkv_workspace_bytes(LKV_WS_INIT, d, n_units, n_index), stream)
     d.workspace = ws_t.data_ptr()
     d.workspace_bytes = ws_t.numel()
     return d, ws_t
@@ -293,7 +299,7 @@ def lkv_gdn_fwd_segmented(q, k, v, g, beta, S0=None, o=None, S_T=None, *, n_segm
     _, H_v, d_v = v.shape
     d = lkv_gdn_desc(T_total=T, n_seq=1, cu_seqlens=None, H_k=H_k, H_v=H_v, d_k=d_k, d_v=d_v, io_dtype=_dtype_code(v),
                      compute=compute, scale=float(scale), state_dtype=0, workspace=None, workspace_bytes=0)
-    ws_t = workspace_t if workspace_t is not None else workspace(v.device, lkv_workspace_bytes(LKV_WS_GDN, d, 2 * n_segments))
+    ws_t = workspace_t if workspace_t is not None else workspace(v.device, lkv_workspace_bytes(LKV_WS_GDN, d, 2 * n_segments), stream)
     d.workspace, d.workspace_bytes = ws_t.data_ptr(), ws_t.numel()
     need = int(load().lkv_gdn_segmented_scratch_bytes(ctypes.byref(d), int(n_segments)))
     if scratch is None:
@@ -329,7 +335,7 @@ def lkv_init_state_fold(states: torch.Tensor, k, g, beta, cu_tokens, K: int, chu
     cu_tokens: host int32[n_chunks + 1].  Returns S0 [H, d, d] fp32.
     """
     ids, cu = _host_i32(chunk_ids), _host_i32(cu_tokens)
-    d, ws_t = _init_desc(states, LKV_FAMILY_GDN, compute, workspace_t, 1, int(K), ids)
+    d, ws_t = _init_desc(states, LKV_FAMILY_GDN, compute, workspace_t, 1, int(K), ids, stream=stream)
     if S0 is None:
         S0 = torch.empty(tuple(states.shape[1:]), dtype=torch.float32, device=states.device)
     st = load().lkv_init_state_fold(_ptr(states), _ptr(k), _ptr(g), _ptr(beta), _hp(cu), int(K), _ptr(S0),
@@ -370,7 +376,7 @@ def lkv_gdn_chunk_transition(k, g, beta, transitions=None, *, cu_seqlens=None, H
     d = lkv_gdn_desc(T_total=T, n_seq=n_seq, cu_seqlens=None if cu is None else cu.ctypes.data, H_k=H_k, H_v=H_v,
                      d_k=d_k, d_v=d_k, io_dtype=_dtype_code(k), compute=compute, scale=0.0, state_dtype=0,
                      workspace=None, workspace_bytes=0)
-    ws_t = workspace_t if workspace_t is not None else workspace(k.device, lkv_workspace_bytes(LKV_WS_GDN, d, n_seq))
+    ws_t = workspace_t if workspace_t is not None else workspace(k.device, lkv_workspace_bytes(LKV_WS_GDN, d, n_seq), stream)
     d.workspace, d.workspace_bytes = ws_t.data_ptr(), ws_t.numel()
     if transitions is None:
         transitions = torch.empty((n_seq, H_v, d_k, d_k), dtype=torch.float32, device=k.device)
@@ -402,7 +408,7 @@ def lkv_state_rel_error(S_init, S_ref, n_states: Optional[int] = None, rel_err=N
     if rel_err is None:
         rel_err = torch.empty((n,), dtype=torch.float32, device=S_init.device)
     nbytes = load().lkv_state_rel_error_workspace_bytes(n, elems)
-    ws_t = error_workspace(S_init.device, nbytes)
+    ws_t = error_workspace(S_init.device, nbytes, stream)
     st = load().lkv_state_rel_error(_ptr(S_init), _ptr(S_ref), _ptr(rel_err), n, elems, ws_t.data_ptr(), ws_t.numel(),
                                     _stream(stream))
     if st != LKV_OK:

@@ -25,7 +25,7 @@ namespace {
 
 // handed over once by binding.py
 PyObject *g_error = nullptr;      // LkvError(status, where)
-PyObject *g_workspace = nullptr;  // workspace(device, nbytes): makes and caches a workspace
+PyObject *g_workspace = nullptr;  // workspace(device, nbytes, raw stream): makes and caches a workspace
 PyObject *g_ws_cache = nullptr;   // its cache: {(device index, raw stream): tensor}
 PyObject *g_host_i32 = nullptr;   // any index sequence -> contiguous int32 numpy array
 
@@ -112,9 +112,9 @@ void *stream_of(PyObject *o) {
     return s;
 }
 
-// The caller's workspace tensor, or the cached one of this device and the current stream (binding.workspace).
+// The caller's workspace tensor, or the cached one of this device and the call's stream (binding.workspace).
 template <typename Desc>
-void set_workspace(Desc &d, PyObject *given, const at::Tensor &like, int which, int n_units, int n_index) {
+void set_workspace(Desc &d, PyObject *given, const at::Tensor &like, void *stream, int which, int n_units, int n_index) {
     if (given != Py_None) {
         const at::Tensor &t = tensor_of(given);
         d.workspace = t.data_ptr();
@@ -123,8 +123,8 @@ void set_workspace(Desc &d, PyObject *given, const at::Tensor &like, int which, 
     }
     const size_t need = lkv_workspace_bytes(which, &d, n_units, n_index);
     const int dev = like.device().index();
-    PyObject *key = Py_BuildValue("(iK)", dev, static_cast<unsigned long long>(
-                                                   reinterpret_cast<uintptr_t>(c10::cuda::getCurrentCUDAStream().stream())));
+    const auto raw = static_cast<unsigned long long>(reinterpret_cast<uintptr_t>(stream));
+    PyObject *key = Py_BuildValue("(iK)", dev, raw);
     if (!key) throw Failed{};
     PyObject *hit = PyDict_GetItemWithError(g_ws_cache, key);   // borrowed; the cache keeps it
     Py_DECREF(key);
@@ -138,7 +138,7 @@ void set_workspace(Desc &d, PyObject *given, const at::Tensor &like, int which, 
     } else if (PyErr_Occurred()) {
         throw Failed{};
     }
-    PyObject *made = PyObject_CallFunction(g_workspace, "in", dev, static_cast<Py_ssize_t>(need));
+    PyObject *made = PyObject_CallFunction(g_workspace, "inK", dev, static_cast<Py_ssize_t>(need), raw);
     if (!made) throw Failed{};
     const at::Tensor &t = tensor_of(made);
     d.workspace = t.data_ptr();
@@ -270,12 +270,13 @@ PyObject *init_state(PyObject *, PyObject *const *a, Py_ssize_t n) {
         HostInts ids(a[6]);
         d.sel_index = to_int(a[7]);
         d.chunk_ids = ids.data();
-        set_workspace(d, a[9], states, LKV_WS_INIT, 1, K);
+        void *stream = stream_of(a[10]);
+        set_workspace(d, a[9], states, stream, LKV_WS_INIT, 1, K);
         Output S0;
         if (a[4] != Py_None) S0.given(a[4]);
         else S0.make(new_tensor(states.sizes().slice(1), at::kFloat, states));
         call("lkv_init_state", d.workspace, lkv_init_state, ptr_of(a[0]), ptr_of(a[1]), K, to_int(a[3]), S0.ptr, &d,
-             stream_of(a[10]));
+             stream);
         return S0.take();
     });
 }
@@ -288,12 +289,13 @@ PyObject *init_state_batched(PyObject *, PyObject *const *a, Py_ssize_t n) {
         lkv_init_desc d = init_desc(states, a[8], a[9]);
         HostInts ids(a[2]), cu(a[3]), sel(a[6]);
         const int n_req = to_int(a[4]);
-        set_workspace(d, a[10], states, LKV_WS_INIT, n_req, ids.size());
+        void *stream = stream_of(a[11]);
+        set_workspace(d, a[10], states, stream, LKV_WS_INIT, n_req, ids.size());
         Output S0;
         if (a[7] != Py_None) S0.given(a[7]);
         else S0.make(new_tensor({n_req, states.size(1), states.size(2), states.size(3)}, at::kFloat, states));
         call("lkv_init_state_batched", d.workspace, lkv_init_state_batched, ptr_of(a[0]), ptr_of(a[1]), ids.data(), cu.data(),
-             n_req, to_int(a[5]), sel.data(), S0.ptr, &d, stream_of(a[11]));
+             n_req, to_int(a[5]), sel.data(), S0.ptr, &d, stream);
         return S0.take();
     });
 }
@@ -325,7 +327,8 @@ PyObject *gdn_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
         d.io_dtype = dtype_code(v);
         d.scale = static_cast<float>(PyFloat_AsDouble(a[9]));
         if (PyErr_Occurred()) throw Failed{};
-        set_workspace(d, a[14], v, LKV_WS_GDN, d.n_seq, 0);
+        void *stream = stream_of(a[15]);
+        set_workspace(d, a[14], v, stream, LKV_WS_GDN, d.n_seq, 0);
         Output o, S_T;
         if (a[6] != Py_None) o.given(a[6]);
         else if (PyObject_IsTrue(a[12]) == 1) o.make(new_tensor(v.sizes(), v.scalar_type(), v));
@@ -334,7 +337,7 @@ PyObject *gdn_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
         if (S_T.obj) d.state_dtype = dtype_code(THPVariable_Unpack(S_T.obj));
         call("lkv_gdn_fwd", d.workspace, lkv_gdn_fwd, ptr_of(a[0]), ptr_of(a[1]), ptr_of(a[2]),
              static_cast<float *>(ptr_of(a[3])), static_cast<float *>(ptr_of(a[4])), static_cast<float *>(ptr_of(a[5])), o.ptr,
-             S_T.ptr, &d, stream_of(a[15]));
+             S_T.ptr, &d, stream);
         return pair(o, S_T);
     });
 }
@@ -348,7 +351,8 @@ PyObject *gdn_chunk_artifacts(PyObject *, PyObject *const *a, Py_ssize_t n) {
         HostInts cu(a[6]);
         lkv_gdn_desc d = gdn_desc(k, v.size(1), v.size(2), cu, a[7]);
         d.io_dtype = dtype_code(k);
-        set_workspace(d, a[8], k, LKV_WS_GDN, 2 * d.n_seq, 0);
+        void *stream = stream_of(a[9]);
+        set_workspace(d, a[8], k, stream, LKV_WS_GDN, 2 * d.n_seq, 0);
         Output S, T;
         if (a[4] != Py_None) S.given(a[4]);
         else S.make(new_tensor({d.n_seq, d.H_v, d.d_k, d.d_v}, at::kFloat, k));
@@ -356,7 +360,7 @@ PyObject *gdn_chunk_artifacts(PyObject *, PyObject *const *a, Py_ssize_t n) {
         else T.make(new_tensor({d.n_seq, d.H_v, d.d_k, d.d_k}, at::kFloat, k));
         call("lkv_gdn_chunk_artifacts", d.workspace, lkv_gdn_chunk_artifacts, ptr_of(a[0]), ptr_of(a[1]),
              static_cast<float *>(ptr_of(a[2])), static_cast<float *>(ptr_of(a[3])), static_cast<float *>(S.ptr),
-             static_cast<float *>(T.ptr), &d, stream_of(a[9]));
+             static_cast<float *>(T.ptr), &d, stream);
         return pair(S, T);
     });
 }
@@ -379,7 +383,8 @@ PyObject *ssd_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
         d.N = static_cast<int32_t>(B.size(2));
         d.io_dtype = dtype_code(x);
         d.compute = to_int(a[9]);
-        set_workspace(d, a[13], x, LKV_WS_SSD, d.n_seq, 0);
+        void *stream = stream_of(a[14]);
+        set_workspace(d, a[13], x, stream, LKV_WS_SSD, d.n_seq, 0);
         Output y, S_T;
         if (a[6] != Py_None) y.given(a[6]);
         else if (PyObject_IsTrue(a[11]) == 1) y.make(new_tensor(x.sizes(), x.scalar_type(), x));
@@ -388,7 +393,7 @@ PyObject *ssd_fwd(PyObject *, PyObject *const *a, Py_ssize_t n) {
         if (S_T.obj) d.state_dtype = dtype_code(THPVariable_Unpack(S_T.obj));
         call("lkv_ssd_fwd", d.workspace, lkv_ssd_fwd, ptr_of(a[0]), static_cast<float *>(ptr_of(a[1])),
              static_cast<float *>(ptr_of(a[2])), ptr_of(a[3]), ptr_of(a[4]), static_cast<float *>(ptr_of(a[5])), y.ptr,
-             S_T.ptr, &d, stream_of(a[14]));
+             S_T.ptr, &d, stream);
         return pair(y, S_T);
     });
 }
@@ -406,12 +411,13 @@ PyObject *mamba_chunk_logdecay(PyObject *, PyObject *const *a, Py_ssize_t n) {
         d.cu_seqlens = cu.data();
         d.H = static_cast<int32_t>(dt.size(1));
         d.P = d.N = d.G = 1;
-        set_workspace(d, a[4], dt, LKV_WS_SSD, d.n_seq, 0);
+        void *stream = stream_of(a[5]);
+        set_workspace(d, a[4], dt, stream, LKV_WS_SSD, d.n_seq, 0);
         Output out;
         if (a[2] != Py_None) out.given(a[2]);
         else out.make(new_tensor({d.n_seq, d.H}, at::kFloat, dt));
         call("lkv_mamba_chunk_logdecay", d.workspace, lkv_mamba_chunk_logdecay, static_cast<float *>(ptr_of(a[0])),
-             static_cast<float *>(ptr_of(a[1])), static_cast<float *>(out.ptr), &d, stream_of(a[5]));
+             static_cast<float *>(ptr_of(a[1])), static_cast<float *>(out.ptr), &d, stream);
         return out.take();
     });
 }

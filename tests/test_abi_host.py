@@ -327,5 +327,10 @@ def test_replaced_workspaces_stay_alive(monkeypatch, make, cache):
     gc.collect()
     assert first() is not None
     assert sum(sizes[:-1]) <= sizes[-1]
+    monkeypatch.setattr(torch.cuda, "ExternalStream", lambda raw: raw)
+    monkeypatch.setattr(torch.cuda, "stream", lambda s: __import__("contextlib").nullcontext())
+    other = types.SimpleNamespace(cuda_stream=7)
+    mine = get("cpu", 10, other)                      # the stream that the call runs on, not the current one
+    assert mine.data_ptr() != ws.data_ptr() and get("cpu", 10, 7) is mine
     stream.cuda_stream = 7
-    assert get("cpu", 10).data_ptr() != ws.data_ptr()
+    assert get("cpu", 10) is mine

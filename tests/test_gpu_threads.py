@@ -67,3 +67,25 @@ def test_threads_that_share_a_stream():
     with ThreadPoolExecutor(len(work)) as pool:
         for r in [pool.submit(engine, i) for i in range(len(work))]:
             r.result()
+
+
+def test_calls_on_streams_passed_explicitly():
+    """The segments' states travel through the workspace: calls that may overlap have one each, whatever stream is current."""
+    import torch
+    bf = torch.bfloat16
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    rn = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    T = 8192
+    unit = lambda x: torch.nn.functional.normalize(x, dim=-1).to(bf)
+    work = [(unit(rn(T, 2, 128)), unit(rn(T, 2, 128)), rn(T, 2, 128).to(bf), -0.01 * torch.rand(T, 2, generator=gen, device="cuda"),
+             torch.rand(T, 2, generator=gen, device="cuda")) for _ in range(2)]
+    alone = [b.lkv_gdn_fwd(*a) for a in work]
+    streams = [torch.cuda.Stream() for _ in work]
+    outs = [[(torch.empty_like(a[2]), torch.empty((1, 2, 128, 128), device="cuda")) for _ in range(10)] for a in work]
+    torch.cuda.synchronize()
+    for i in range(10):
+        for s, a, o in zip(streams, work, outs):
+            b.lkv_gdn_fwd(*a, None, *o[i], stream=s)
+    torch.cuda.synchronize()
+    for ref, o in zip(alone, outs):
+        assert all(torch.equal(x, ref[0]) and torch.equal(S, ref[1]) for x, S in o)
