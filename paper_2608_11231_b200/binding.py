@@ -12,6 +12,7 @@ from __future__ import annotations
 import contextlib
 import ctypes
 import os
+import threading
 from typing import Optional, Sequence
 
 import numpy as np
@@ -170,6 +171,7 @@ def _hp(a: Optional[np.ndarray]):
 
 _ws_cache = {}
 _ws_replaced = []
+_ws_lock = threading.Lock()
 _err_ws_cache = {}
 
 
@@ -184,15 +186,16 @@ def _cached(cache, device, nbytes: int, stream=None) -> torch.Tensor:
     current = torch.cuda.current_stream().cuda_stream
     raw = current if stream is None else getattr(stream, "cuda_stream", stream)
     key = (torch.device(device).index, raw)
-    ws = cache.get(key)
-    if ws is None or ws.numel() < nbytes:
-        size = max(int(nbytes), 4096)
-        if ws is not None:
-            size = max(size, 2 * ws.numel())
-            _ws_replaced.append(ws)
-        # filled on the stream that will use it
-        with contextlib.nullcontext() if raw == current else torch.cuda.stream(torch.cuda.ExternalStream(raw)):
-            ws = cache[key] = torch.zeros(size, dtype=torch.uint8, device=device)
+    with _ws_lock:   # (torch.zeros lets other threads run: two that both found nothing would each keep one, and one be given back)
+        ws = cache.get(key)
+        if ws is None or ws.numel() < nbytes:
+            size = max(int(nbytes), 4096)
+            if ws is not None:
+                size = max(size, 2 * ws.numel())
+                _ws_replaced.append(ws)
+            # filled on the stream that will use it
+            with contextlib.nullcontext() if raw == current else torch.cuda.stream(torch.cuda.ExternalStream(raw)):
+                ws = cache[key] = torch.zeros(size, dtype=torch.uint8, device=device)
     return ws
 
 

@@ -334,3 +334,23 @@ def test_replaced_workspaces_stay_alive(monkeypatch, make, cache):
     assert mine.data_ptr() != ws.data_ptr() and get("cpu", 10, 7) is mine
     stream.cuda_stream = 7
     assert get("cpu", 10) is mine
+
+
+def test_threads_that_need_a_workspace_at_once_get_the_same(monkeypatch):
+    import time
+    import types
+    from concurrent.futures import ThreadPoolExecutor
+
+    import torch
+    monkeypatch.setattr(b, "_ws_cache", {})
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0))
+    zeros = torch.zeros
+
+    def slow_zeros(*a, **k):
+        time.sleep(0.05)
+        return zeros(*a, **k)
+
+    monkeypatch.setattr(torch, "zeros", slow_zeros)
+    with ThreadPoolExecutor(4) as pool:
+        got = list(pool.map(lambda _: b.workspace("cpu", 100), range(4)))
+    assert all(w is got[0] for w in got)
