@@ -366,7 +366,7 @@ ssd_scan_tensor_kernel(const __grid_constant__ SsdArgs a, const __grid_constant_
 #pragma unroll
             for (int j = 0; j < 8; j += 4) {
                 *reinterpret_cast<uint4 *>(&sl.s[hd][4 * hl + j / 2]) = make_uint4(hi[j / 2], lo[j / 2], hi[j / 2 + 1], lo[j / 2 + 1]);
-                *reinterpret_cast<float4 *>(&sl.e[hd][8 * hl + j]) = make_float4(ex2(l2[j]), ex2(l2[j + 1]), ex2(l2[j + 2]), ex2(l2[j + 3]));
+                if (has_y) *reinterpret_cast<float4 *>(&sl.e[hd][8 * hl + j]) = make_float4(ex2(l2[j]), ex2(l2[j + 1]), ex2(l2[j + 2]), ex2(l2[j + 3]));
             }
             warp_arrive(&bars.sc_ready[b % kSlots]);
             if (fin) {
