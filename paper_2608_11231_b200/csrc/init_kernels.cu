@@ -4,11 +4,15 @@
 // d_k = d_v = 128 lives in init_gdn_tensor.cu).
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 
 namespace lkv {
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 // 16 bytes of pool state -> 4 (fp32 pool) or 8 (bf16 pool) floats.
 template <bool BF16>
@@ -268,32 +272,59 @@ cudaError_t launch_init_gdn_exact_fp32(const InitArgs &a, bool pool_bf16, cudaSt
 
 namespace {
 
-// One CTA per (sequence, group of 32 heads): lanes walk consecutive heads, so every token's dt row is read with coalesced
-// 128-byte accesses; each of the eight warps sums every eighth token, and their sums are added in a fixed order.
-__global__ void mamba_logdecay_kernel(const __grid_constant__ SsdArgs a, float *__restrict__ out) {
-    const int seq = blockIdx.y;
-    const int h = blockIdx.x * 32 + (threadIdx.x & 31);
-    const int part = threadIdx.x >> 5, nparts = blockDim.x >> 5;
-    __shared__ float red[8][32];
+// A cluster of eight CTAs per (sequence, group of 32 heads), an eighth of the tokens each: lanes walk consecutive heads, so every
+// token's dt row is read with coalesced 128-byte accesses.  What bounds it is the latency of the loads, not their bytes: each of
+// a CTA's eight warps has eight tokens in flight, in eight sums of their own, and the cluster puts 768 CTAs on the 32 chunks of
+// 256 .. 2048 tokens x 80 heads that one CTA per (sequence, 32 heads), one load after the other into one sum, took 38.9 us
+// for; behind the scan that makes the states of these chunks 201 -> 174 us for both.  All partial sums are added in a fixed order.
+constexpr int kDecayParts = 8, kDecayWarps = 8, kDecayLoads = 8;
+__global__ void __cluster_dims__(kDecayParts, 1, 1) __launch_bounds__(32 * kDecayWarps)
+mamba_logdecay_kernel(const __grid_constant__ SsdArgs a, float *__restrict__ out) {
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int seq = blockIdx.y, part = blockIdx.x % kDecayParts;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int h = (blockIdx.x / kDecayParts) * 32 + lane;
+    __shared__ float red[kDecayWarps][32], sum[32];
     pdl_launch();
     pdl_wait();
-    const int t0 = a.cu[seq], t1 = a.cu[seq + 1];
-    float acc = 0.f;
-    if (h < a.H)
-        for (int t = t0 + part; t < t1; t += nparts) acc += a.dt[static_cast<size_t>(t) * a.H + h];
-    red[part][threadIdx.x & 31] = acc;
-    __syncthreads();
-    if (part == 0 && h < a.H) {
-        float sum = 0.f;
-        for (int p = 0; p < nparts; ++p) sum += red[p][threadIdx.x];
-        out[static_cast<size_t>(seq) * a.H + h] = a.A[h] * sum;
+    const int t0 = a.cu[seq], n = a.cu[seq + 1] - t0;
+    const int per = (n + kDecayParts - 1) / kDecayParts;
+    const long long end = min(static_cast<long long>(per) * (part + 1), static_cast<long long>(n));
+    float acc[kDecayLoads];
+#pragma unroll
+    for (int i = 0; i < kDecayLoads; ++i) acc[i] = 0.f;
+    if (h < a.H) {
+        const float *p = a.dt + static_cast<size_t>(t0) * a.H + h;
+        for (long long t = static_cast<long long>(per) * part + warp; t < end; t += kDecayWarps * kDecayLoads) {
+            float v[kDecayLoads];
+#pragma unroll
+            for (int i = 0; i < kDecayLoads; ++i) v[i] = t + i * kDecayWarps < end ? p[static_cast<size_t>(t + i * kDecayWarps) * a.H] : 0.f;
+#pragma unroll
+            for (int i = 0; i < kDecayLoads; ++i) acc[i] += v[i];
+        }
     }
+    red[warp][lane] = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]));
+    __syncthreads();
+    if (warp == 0) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < kDecayWarps; ++w) s += red[w][lane];
+        sum[lane] = s;
+    }
+    cluster.sync();
+    if (part == 0 && warp == 0 && h < a.H) {
+        float s = 0.f;
+#pragma unroll
+        for (int r = 0; r < kDecayParts; ++r) s += cluster.map_shared_rank(sum, r)[lane];
+        out[static_cast<size_t>(seq) * a.H + h] = a.A[h] * s;
+    }
+    cluster.sync();   // the sums stay where they are until they have been read
 }
 
 }  // namespace
 
 cudaError_t launch_mamba_logdecay(const SsdArgs &a, float *logdecay, cudaStream_t s) {
-    return launch_chained(mamba_logdecay_kernel, dim3((a.H + 31) / 32, a.n_seq), 256, 0, s, a, logdecay);
+    return launch_chained(mamba_logdecay_kernel, dim3(kDecayParts * ((a.H + 31) / 32), a.n_seq), 32 * kDecayWarps, 0, s, a, logdecay);
 }
 
 namespace {
