@@ -151,8 +151,8 @@ bool init_mamba_stream_supported(const InitArgs &a, bool pool_bf16);
 cudaError_t launch_init_mamba_exact_stream(const InitArgs &a, bool pool_bf16, cudaStream_t s);
 cudaError_t launch_init_gdn_exact_fp32(const InitArgs &a, bool pool_bf16, cudaStream_t s);
 bool init_gdn_exact_tensor_supported(const InitArgs &a, bool pool_bf16);
-// early = false: not before the kernel ahead of it on the stream has left the GPU
-cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cudaStream_t s, bool early = true);
+// early = false: not before the kernel ahead of it on the stream has left the GPU; shared: the requests name the same chunks
+cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cudaStream_t s, bool early = true, bool shared = false);
 
 bool gdn_scan_fp32_supported(int d_k, int d_v);
 cudaError_t launch_gdn_scan_fp32(const GdnArgs &a, bool io_bf16, cudaStream_t s);

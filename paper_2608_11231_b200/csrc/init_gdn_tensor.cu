@@ -40,6 +40,11 @@ constexpr int kEpiThreads = 256;             // two epilogue warpgroups
 constexpr int kRoundThreads = 128;           // warps that round the transitions
 constexpr int kThreads = kEpiThreads + kRoundThreads + 64;   // + MMA warp + TMA warp
 constexpr int kSmemBytes = kStages * kTStageBytes + 1024;
+// Where the requests share chunks and more than L2 holds at once, CTAs are launched in groups of up to eight requests, those of a group next
+// to each other for one head: the chunks of some 18 heads, not of all, are then in use at a time, and each is read from DRAM once.  Eight
+// requests over one pool of 32 chunks (134 MB), each in its own order, composition and scan: 305 -> 285 us (where nothing is
+// shared the order by heads is level to 1 % better).
+constexpr int kMaxGroupLog2 = 3;
 constexpr uint32_t kTmemCols = 512;          // D buffers: 0..127 and 128..255, A buffers: 256..383 and 384..511
 
 // fp32 -> nearest tf32 (ties away from zero, as cvt.rna.tf32.f32 rounds), in integer arithmetic: the conversion
@@ -64,7 +69,7 @@ __device__ __forceinline__ uint32_t phase_of(int j) { return static_cast<uint32_
 // SBF16: the cached states are stored as bf16 (the transitions are fp32 either way); S0 is written as fp32.
 template <bool SBF16>
 __global__ void __launch_bounds__(kThreads, 1)
-init_gdn_exact_tensor_kernel(const __grid_constant__ InitArgs a, const __grid_constant__ CUtensorMap mapT) {
+init_gdn_exact_tensor_kernel(const __grid_constant__ InitArgs a, const __grid_constant__ CUtensorMap mapT, int group_log2) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *sm = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);   // an offset, not a cast: the compiler keeps shared-memory addressing
     // fullT: TMA transactions; roundT: the rounding warps are done with the stage; freeT: the MMAs of the step have read it;
@@ -74,8 +79,9 @@ init_gdn_exact_tensor_kernel(const __grid_constant__ InitArgs a, const __grid_co
     __shared__ volatile int dead;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int h = blockIdx.x, r = blockIdx.y;
+    const int h = blockIdx.x >> group_log2, r = (blockIdx.y << group_log2) + (blockIdx.x & ((1 << group_log2) - 1));
     pdl_launch();
+    if (r >= a.n_req) return;
     if (a.idx.ptr) pdl_wait();   // the index list is in global memory
     const int k0 = a.cu_k(r), K = a.cu_k(r + 1) - k0;
     constexpr size_t ss = static_cast<size_t>(kD) * kD;
@@ -241,14 +247,17 @@ bool init_gdn_exact_tensor_supported(const InitArgs &a, bool) {
            static_cast<long long>(a.n_chunks) * a.H * kD < (1ll << 31);
 }
 
-cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cudaStream_t s, bool early) {
+cudaError_t launch_init_gdn_exact_tensor(const InitArgs &a, bool pool_bf16, cudaStream_t s, bool early, bool shared) {
     CUtensorMap mapT;
     const uint64_t rows = static_cast<uint64_t>(a.n_chunks) * a.H * kD;
     if (!make_tensor_map_2d(&mapT, a.transitions, 4, kD, rows, kD * 4, 32, kD, true)) return cudaErrorInvalidValue;
     auto kernel = pool_bf16 ? init_gdn_exact_tensor_kernel<true> : init_gdn_exact_tensor_kernel<false>;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
-    return launch_kernel(early, kernel, dim3(a.H, a.n_req), kThreads, kSmemBytes, s, a, mapT);
+    int group_log2 = 0;
+    while (shared && group_log2 < kMaxGroupLog2 && (2 << group_log2) <= a.n_req) ++group_log2;
+    const int group = 1 << group_log2;
+    return launch_kernel(early, kernel, dim3(a.H << group_log2, (a.n_req + group - 1) / group), kThreads, kSmemBytes, s, a, mapT, group_log2);
 }
 
 }  // namespace lkv

@@ -80,6 +80,20 @@ int check_init_desc(const lkv_init_desc *d) {
     return LKV_OK;
 }
 
+// Do the requests name the chunks 1.5 times on average or more, and more of them than L2 holds at once?  Then the order of the
+// composition's CTAs matters (kMaxGroupLog2 in init_gdn_tensor.cu).
+bool shares_chunks(const int32_t *ids, int total, const lkv_init_desc *d) {
+    constexpr double kL2Bytes = 126e6;
+    if (2.0 * sizeof(float) * total * d->H * d->d_k * d->d_v <= kL2Bytes) return false;
+    std::vector<bool> seen(d->n_chunks, false);
+    int distinct = 0;
+    for (int i = 0; i < total; ++i) {
+        distinct += !seen[ids[i]];
+        seen[ids[i]] = true;
+    }
+    return 2LL * total >= 3LL * distinct;
+}
+
 int init_impl(const void *states, const void *transitions, const int32_t *chunk_ids, const int32_t *cu_k,
               int n_req, int mode, const int32_t *sel_index, void *S0, const lkv_init_desc *d, void *stream) {
     int st = check_init_desc(d);
@@ -171,7 +185,7 @@ int init_impl(const void *states, const void *transitions, const int32_t *chunk_
                                                           : launch_init_mamba_exact(a, pool_bf16, s);
             break;
         case kGdnFp32: e = launch_init_gdn_exact_fp32(a, pool_bf16, s); break;
-        case kGdnTensor: e = launch_init_gdn_exact_tensor(a, pool_bf16, s); break;
+        case kGdnTensor: e = launch_init_gdn_exact_tensor(a, pool_bf16, s, true, shares_chunks(chunk_ids, total, d)); break;
     }
     return e == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
 }
