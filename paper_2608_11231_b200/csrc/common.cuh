@@ -158,6 +158,8 @@ bool gdn_scan_fp32_supported(int d_k, int d_v);
 cudaError_t launch_gdn_scan_fp32(const GdnArgs &a, bool io_bf16, cudaStream_t s);
 bool gdn_scan_tensor_supported(const GdnArgs &a, bool io_bf16);
 cudaError_t launch_gdn_scan_tensor(const GdnArgs &a, cudaStream_t s);
+// states (S_T) and transitions (tr_out) of the n_seq sequences, from nothing; shapes as for the scan, v not null
+cudaError_t launch_gdn_build_tensor(const GdnArgs &a, cudaStream_t s);
 
 bool ssd_scan_fp32_supported(int N, int P);
 cudaError_t launch_ssd_scan_fp32(const SsdArgs &a, bool io_bf16, cudaStream_t s);

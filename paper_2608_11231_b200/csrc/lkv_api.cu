@@ -439,7 +439,14 @@ static int gdn_impl(const void *q, const void *k, const void *v, const float *g,
     const size_t head = ws_bytes_for(2 * d->n_seq + 1, kScanIdxCap);
     if (cut.n > 1 && d->workspace_bytes >= head + gdn_segment_scratch(d, cut.n))
         return gdn_segmented(a, d, segment_tokens(cut, kGdnBlock, d->T_total), true, true, static_cast<char *>(d->workspace) + head, s);
-    if (what == 3) {
+    // States and transitions: one CTA for both of a chunk and head, once two CTAs would no longer find an SM each (32 heads, 3 x 1024 tokens
+    // 57 -> 39 us); up to there they are faster side by side (2 x 2048 tokens 55 us, in one CTA 67).  Without v, read as zeros, or
+    // in fp32 arithmetic the scan runs twice.
+    const bool both = what == 3 && use_tensor && v && static_cast<long long>(a.n_seq) * a.H_v > sm_count();
+    if (both) {
+        a.n_seq = n_ranges;
+        append_launch_order(cu, n_ranges);
+    } else if (what == 3) {
         // launch order over all sequences, longest first; transition sequence j runs over range j - m
         std::vector<int32_t> order(d->n_seq);
         auto len = [&](int sq) { const int r = sq % n_ranges; return cu[r + 1] - cu[r]; };
@@ -451,7 +458,7 @@ static int gdn_impl(const void *q, const void *k, const void *v, const float *g,
     }
     st = place_indices(a.cu, cu, d->workspace, s);
     if (st != LKV_OK) return st;
-    const cudaError_t e = use_tensor ? launch_gdn_scan_tensor(a, s) : launch_gdn_scan_fp32(a, io_bf16, s);
+    const cudaError_t e = both ? launch_gdn_build_tensor(a, s) : use_tensor ? launch_gdn_scan_tensor(a, s) : launch_gdn_scan_fp32(a, io_bf16, s);
     return e == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
 }
 
