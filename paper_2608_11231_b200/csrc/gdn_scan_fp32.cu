@@ -17,16 +17,22 @@
 // by shuffles instead of leaving 31 dependent sums to one thread.  Measured on B200 with two heads of
 // 64 x 64: the composition of four chunks and a scan of 64 tokens, 69.7 -> 28.7 us for the two calls (register tiles and four
 // times the CTAs).
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 
 namespace lkv {
 
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int kC = 32;  // tokens per block
 
 // row stride (floats) of the q and k tiles: 16-byte rows, successive rows four banks apart
 __host__ __device__ constexpr int row_stride(int dk) { return (((dk + 3) / 4) | 1) * 4; }
+// the same for products in steps of 16 channels: rows of a multiple of 16, every fourth row 16 banks on
+__host__ __device__ constexpr int cluster_stride(int dk) { return (dk + 15) / 16 * 16 + 4; }
 constexpr int kLdA = kC + 4;   // row stride of the coupling matrix A (read by lane = row)
 
 template <typename T, int VC>
@@ -262,8 +268,225 @@ __global__ void __launch_bounds__(256) gdn_scan_fp32_kernel(const __grid_constan
     }
 }
 
+// The same for calls of few heads and sequences, where the time of a block is all that counts: eight columns a CTA, and the CTAs of a head
+// in clusters of CS (d_v = 16, 32, 64 and more: 2, 4, 8), which form a part of the coupling matrices each and write it to one another.
+// What bounds the products is what shared memory returns, a value a lane and warp a cycle, so they are one product in register tiles:
+// the 64 rows [k; q] of the block against 32 / CS rows of k and the eight columns of S (kept transposed), 4 x (8 + 32 / CS) / 4 values a
+// thread, the contraction split over four lanes (every other four channels of 16).  After that nothing leaves a warp: lane = token, warp =
+// column for the right-hand side, the substitution and the outputs, lane = channel for the state.  Tokens of the next block are copied
+// (fp32) while the other CTAs' parts are waited for.  Two heads of 64 x 64: a block 5.2 -> 3.1 us (product 0.7, substitution 0.5, outputs and
+// state 0.8, the rest barriers and hand-overs); 64, 512 tokens 12.7, 85.4 -> 9.6, 53.3 us.  Slower: 16 columns a CTA, a row of k and
+// q a lane and no cluster 13.9, 78; the tokens by bulk copies, a row each, 12.5, 78.5; copied at the start of a block 11.1, 62.5.
+template <typename T, int CS>
+__global__ void __cluster_dims__(1, 1, CS) __launch_bounds__(256) gdn_scan_fp32_cluster_kernel(const __grid_constant__ GdnArgs a) {
+    constexpr int VC = 8, kOwn = kC / CS, NCT = (kOwn + VC) / 4;   // columns of the coupling matrices; product columns a thread
+    const cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ __align__(16) float smem[];
+    const int dk = a.d_k, dv = a.d_v, ks = cluster_stride(dk), dkp = ks - 4;
+    float *KQ = smem;                         // two stages: [k; q] [2 kC][ks], zero beyond dk
+    float *St = KQ + 4 * kC * ks;             // [VC][ks]: S^T, zero beyond dk
+    float *Am = St + VC * ks;                 // two copies (of successive blocks) of A, P: [kC i][kC t] each
+    float *sS = Am + 4 * kC * kC;             // S^T k, S^T q: [2][VC][kC]
+    float *cgs = sS + 2 * VC * kC, *bs = cgs + 2 * kC;   // two copies each: running sum of g, beta
+    float2 *U = reinterpret_cast<float2 *>(bs + 2 * kC);   // [VC][kC]: u, u times e^{cg_C - cg_i}
+    pdl_launch();
+    pdl_wait();
+    const int h = blockIdx.x, seq = a.cu[a.n_ranges + 1 + blockIdx.y];   // launch order: longest sequence first
+    const bool tr = seq >= a.tr_first;                                    // transition sequence
+    const int rg = tr ? seq - a.tr_first + a.tr_src0 : seq;
+    const int hk = h / (a.H_v / a.H_k);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = blockIdx.z % CS;
+    const int j = blockIdx.z * VC + warp;     // this warp's column
+    const int t_begin = a.cu[rg], t_end = a.cu[rg + 1];
+    const T *q = static_cast<const T *>(a.q);
+    const T *k = static_cast<const T *>(a.k);
+    const T *v = tr ? nullptr : static_cast<const T *>(a.v);
+    T *o = tr ? nullptr : static_cast<T *>(a.o);
+    auto state_at = [&](int i) { return (static_cast<size_t>(i) * a.H_v + h) * dk * dv + j; };
+    const bool more = seq >= a.n_s0, own = tr && a.tr_out != nullptr, id = a.s0_identity || tr;
+    const float *S0 = more ? a.S0_more : a.S0;
+    float *ST = own ? a.tr_out : seq >= a.st_first ? a.S_T : nullptr;
+    const size_t obase = state_at(own ? seq - a.tr_first : seq - a.st_first);
+
+    auto async16 = [](float *dst, const void *src) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
+    };
+    // k, q of the block at t0 into a stage; g, beta and v of it into registers
+    const bool async = std::is_same<T, float>::value && dk % 4 == 0;
+    float g_next = 0.f, b_next = 0.f, v_next = 0.f;
+    auto fetch = [&](int t0, int stage) {
+        float *st = KQ + stage * 2 * kC * ks;
+        if (async) {
+            for (int m = 4 * lane; m < dk; m += 128) {   // warp = tokens warp, warp + 8, ..
+                const size_t off = (static_cast<size_t>(t0 + warp) * a.H_k + hk) * dk + m, step = static_cast<size_t>(8) * a.H_k * dk;
+                float *dst = st + warp * ks + m;
+#pragma unroll
+                for (int u = 0; u < kC / 8; ++u) {
+                    if (t0 + warp + 8 * u < t_end) {
+                        async16(dst + 8 * u * ks, k + off + u * step);
+                        async16(dst + (kC + 8 * u) * ks, q + off + u * step);
+                    } else {
+                        *reinterpret_cast<float4 *>(dst + 8 * u * ks) = *reinterpret_cast<float4 *>(dst + (kC + 8 * u) * ks) = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        } else {
+#pragma unroll 4
+            for (int row = warp; row < 2 * kC; row += 8) {
+                const int t = row & (kC - 1);
+                const T *src = (row < kC ? k : q) + (static_cast<size_t>(t0 + t) * a.H_k + hk) * dk;
+                for (int m = lane; m < dk; m += 32) st[row * ks + m] = t0 + t < t_end ? to_f32<T>(src[m]) : 0.f;
+            }
+        }
+        const int t = t0 + lane;   // a padded token is the identity step: g = 0, beta = 0
+        const bool ok = t < t_end;
+        g_next = ok ? a.g[static_cast<size_t>(t) * a.H_v + h] : 0.f;
+        b_next = ok ? a.beta[static_cast<size_t>(t) * a.H_v + h] : 0.f;
+        v_next = v && ok ? to_f32<T>(v[(static_cast<size_t>(t) * a.H_v + h) * dv + j]) : 0.f;
+    };
+    if (t_begin < t_end) fetch(t_begin, 0);
+    // the state, and zeros beyond dk
+    if (!id && S0) S0 += state_at(more ? seq - a.n_s0 : seq);
+    for (int m = lane; m < dkp; m += 32) {
+        float x = 0.f;
+        if (m < dk) x = id ? (m == j ? 1.f : 0.f) : S0 ? S0[static_cast<size_t>(m) * dv] : 0.f;
+        St[warp * ks + m] = x;
+    }
+    for (int row = warp; row < 4 * kC; row += 8)
+        for (int m = dk + lane; m < dkp; m += 32) KQ[row * ks + m] = 0.f;
+    cluster.sync();   // the others have started: their shared memory may be written
+
+    // the product's tile of this thread, shared by four lanes: rows row0 .., columns col0, col0 + 4, ..
+    const int part = lane & 3, row0 = 4 * ((tid >> 2) & 15), col0 = tid >> 6;
+    int odd = 0;
+    for (int t0 = t_begin; t0 < t_end; t0 += kC, odd ^= 1) {
+        const float *Ks = KQ + odd * 2 * kC * ks;
+        float *A = Am + odd * 2 * kC * kC, *P = A + kC * kC;
+        const float bt = b_next, vt = v_next;
+        float cg = g_next;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const float up = __shfl_up_sync(0xffffffffu, cg, d);
+            if (lane >= d) cg += up;
+        }
+        if (warp == 0) {
+            cgs[odd * kC + lane] = cg;
+            bs[odd * kC + lane] = bt;
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();   // this block's k, q and the state are there; everybody has left the other stage
+        float acc[4][NCT];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int c = 0; c < NCT; ++c) acc[u][c] = 0.f;
+        const float *rp = Ks + row0 * ks + 4 * part;
+        const float *cp[NCT];
+#pragma unroll
+        for (int c = 0; c < NCT; ++c) cp[c] = (4 * c < kOwn ? Ks + (rank * kOwn + col0 + 4 * c) * ks : St + (col0 + 4 * c - kOwn) * ks) + 4 * part;
+#pragma unroll 2
+        for (int m = 0; m < dkp; m += 16) {
+            float4 x[4], y[NCT];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = *reinterpret_cast<const float4 *>(rp + u * ks + m);
+#pragma unroll
+            for (int c = 0; c < NCT; ++c) y[c] = *reinterpret_cast<const float4 *>(cp[c] + m);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int c = 0; c < NCT; ++c) {
+                    acc[u][c] = fmaf(x[u].x, y[c].x, acc[u][c]);
+                    acc[u][c] = fmaf(x[u].y, y[c].y, acc[u][c]);
+                    acc[u][c] = fmaf(x[u].z, y[c].z, acc[u][c]);
+                    acc[u][c] = fmaf(x[u].w, y[c].w, acc[u][c]);
+                }
+        }
+        // the four parts added up: lane `part` keeps row row0 + part
+        const int row = row0 + part, t = row & (kC - 1);
+        const float cgt = cgs[odd * kC + t], bst = bs[odd * kC + t];
+#pragma unroll
+        for (int c = 0; c < NCT; ++c) {
+            const float g0 = part & 2 ? acc[0][c] : acc[2][c], g1 = part & 2 ? acc[1][c] : acc[3][c];
+            float k0 = part & 2 ? acc[2][c] : acc[0][c], k1 = part & 2 ? acc[3][c] : acc[1][c];
+            k0 += __shfl_xor_sync(0xffffffffu, g0, 2);
+            k1 += __shfl_xor_sync(0xffffffffu, g1, 2);
+            const float give = part & 1 ? k0 : k1;
+            const float x = (part & 1 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, give, 1);
+            const int col = col0 + 4 * c;
+            if (4 * c < kOwn) {
+                const int i = rank * kOwn + col;
+                const bool in = row < kC ? i < t : i <= t;
+                const float dec = in ? expf(cgt - cgs[odd * kC + i]) : 0.f;
+                const float y = in ? (row < kC ? bst * dec * x : dec * x) : 0.f;
+                float *dst = (row < kC ? A : P) + i * kC + t;
+#pragma unroll
+                for (int r = 0; r < CS; ++r) *cluster.map_shared_rank(dst, r) = y;
+            } else {
+                sS[((row < kC ? 0 : VC) + col - kOwn) * kC + t] = x;
+            }
+        }
+        // the others' parts, and the next block's tokens while they are waited for
+        cluster.barrier_arrive();
+        if (t0 + kC < t_end) fetch(t0 + kC, odd ^ 1);
+        cluster.barrier_wait();
+        // forward substitution down the block: lane = token
+        const float et = expf(cg);
+        float r = bt * (vt - et * sS[warp * kC + lane]);
+        {
+            float ar[kC];
+#pragma unroll
+            for (int i = 0; i < kC - 1; ++i) ar[i] = A[i * kC + lane];
+#pragma unroll
+            for (int i = 0; i < kC - 1; ++i)   // A is zero in the lanes up to i: u_i is final there
+                r = fmaf(-ar[i], __shfl_sync(0xffffffffu, r, i), r);
+        }
+        const float last = __shfl_sync(0xffffffffu, cg, 31), gam = expf(last);
+        float2 *u = U + warp * kC;
+        u[lane] = make_float2(r, expf(last - cg) * r);
+        __syncwarp();
+        // outputs (P is zero above the diagonal) and new state, two channels a lane, in one loop: their reads are in flight together
+        float x = et * sS[(VC + warp) * kC + lane];
+        for (int mb = 0; mb < dkp; mb += 64) {   // (all lanes: each has a token's outputs)
+            const int m0 = min(mb + lane, dkp - 1), m1 = min(mb + lane + 32, dkp - 1);
+            float y0 = gam * St[warp * ks + m0], y1 = gam * St[warp * ks + m1];
+#pragma unroll 8
+            for (int i = 0; i < kC; ++i) {
+                const float2 uw = u[i];
+                if (mb == 0) x = fmaf(P[i * kC + lane], uw.x, x);
+                y0 = fmaf(Ks[i * ks + m0], uw.y, y0);
+                y1 = fmaf(Ks[i * ks + m1], uw.y, y1);
+            }
+            __syncwarp();   // (the last channel may have been read by several lanes)
+            if (mb + lane < dkp) St[warp * ks + m0] = y0;
+            if (mb + lane + 32 < dkp) St[warp * ks + m1] = y1;
+        }
+        if (o && t0 + lane < t_end) o[(static_cast<size_t>(t0 + lane) * a.H_v + h) * dv + j] = from_f32<T>(a.scale * x);
+        __syncwarp();
+    }
+    if (ST)
+        for (int m = lane; m < dk; m += 32) {
+            const size_t e = static_cast<size_t>(m) * dv;
+            float x = St[warp * ks + m];
+            if (a.S_add) x += a.S_add[state_at(seq) + e];
+            store_state(ST, a.st_bf16, obase + e, x);
+        }
+}
+
 size_t smem_bytes(int dk, int vc) {
     return sizeof(float) * (2 * static_cast<size_t>(kC) * row_stride(dk) + kC * kLdA + kC * kC + 3 * kC + static_cast<size_t>(dk) * vc + kC * (vc + 1));
+}
+
+size_t cluster_smem_bytes(int dk) {
+    return sizeof(float) * ((4 * kC + 8) * static_cast<size_t>(cluster_stride(dk)) + 4 * kC * kC + 2 * 8 * kC + 4 * kC + 8 * 2 * kC);
+}
+template <typename T, int CS>
+cudaError_t launch_cluster(const GdnArgs &a, cudaStream_t s) {
+    const size_t smem = cluster_smem_bytes(a.d_k);
+    auto kernel = gdn_scan_fp32_cluster_kernel<T, CS>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_chained(kernel, dim3(a.H_v, a.n_seq, a.d_v / 8), 256, smem, s, a);
 }
 
 template <typename T, int VC>
@@ -279,6 +502,9 @@ cudaError_t launch(const GdnArgs &a, cudaStream_t s) {
 // The coupling matrices are then computed once per part, side by side.
 template <typename T>
 cudaError_t dispatch(const GdnArgs &a, cudaStream_t s) {
+    // clusters while every CTA of theirs finds an SM
+    if (static_cast<long long>(a.H_v) * a.n_seq * (a.d_v / 8) <= sm_count() && cluster_smem_bytes(a.d_k) <= 227 * 1024)
+        return a.d_v == 16 ? launch_cluster<T, 2>(a, s) : a.d_v == 32 ? launch_cluster<T, 4>(a, s) : launch_cluster<T, 8>(a, s);
     int vc = a.d_v;
     const long long units = static_cast<long long>(a.H_v) * a.n_seq;
     while (vc > 16 && units * (a.d_v / vc) * 2 <= sm_count()) vc /= 2;
