@@ -88,6 +88,7 @@ struct InitArgsBase {
     int32_t n_req, H, d_k, d_v, n_chunks;
     int32_t off_sel;           // offset of sel[n_req] in idx, or -1 (= last block)
     int32_t off_ids;           // offset of ids[total_K] in idx; cu_k[n_req + 1] sits at 0
+    int32_t product = -1;      // GDN on the tensor cores: this request is the product of its chunks' transitions, with no states in it
     int32_t *status;           // device status word
 };
 template <int CAP>

@@ -185,14 +185,21 @@ init_gdn_exact_tensor_kernel(const __grid_constant__ InitArgs a, const __grid_co
         // this thread's 64 values of chunk j's cached state (column c, rows i0..i0+63): a warp reads whole 128-byte
         // (fp32) or 64-byte (bf16) row pieces; issued before the wait for the MMAs, which hides their latency
         float sv[64];
+        const bool prod = r == a.product;   // starts from the first chunk's transition, and nothing is added
         auto fetch_S = [&](int j) {
+            if (prod) {
+                const float *src = a.transitions + (static_cast<size_t>(prow(j)) + i0) * kD + c;
+#pragma unroll
+                for (int i = 0; i < 64; ++i) sv[i] = j == 0 ? src[static_cast<size_t>(i) * kD] : 0.f;
+                return;
+            }
             const PoolT *src = pool + (static_cast<size_t>(prow(j)) + i0) * kD + c;
 #pragma unroll
             for (int i = 0; i < 64; ++i) sv[i] = to_f32<PoolT>(src[static_cast<size_t>(i) * kD]);
         };
         // the rows of the chunk after next, pulled into L2 (64 rows of 512 or 256 bytes per warpgroup)
         auto prefetch_S = [&](int j) {
-            if (j >= K) return;
+            if (j >= K || prod) return;
             const char *src = reinterpret_cast<const char *>(pool + (static_cast<size_t>(prow(j)) + i0) * kD);
             constexpr int bytes = 64 * kD * static_cast<int>(sizeof(PoolT));
             for (int o = (tid & 127) * 128; o < bytes; o += 128 * 128) prefetch_l2(src + o);

@@ -94,6 +94,42 @@ bool shares_chunks(const int32_t *ids, int total, const lkv_init_desc *d) {
     return 2LL * total >= 3LL * distinct;
 }
 
+// One request's chain of K steps in two halves side by side, where three CTAs a head find an SM each: the state A of the first half, and of
+// the second the state B that it reaches from nothing and the product P of its transitions; then S0 = P A + B.  The second launch costs
+// about four steps.  32 heads: K = 10 19.6 -> 17.1 us, 16 30.3 -> 22.8, 64 120.6 -> 69.7 (8 chunks are 16.2 as one chain); the error against
+// 64 bits is that of the chain (7.3e-4 with transitions of norm 0.97).
+constexpr int kSplitChunks = 10;
+bool gdn_splits(const lkv_init_desc *d, int n_req, int total) {
+    return n_req == 1 && total >= kSplitChunks && total + total <= kInitIdxCap - 4 && d->family == LKV_FAMILY_GDN && d->compute != LKV_COMPUTE_FP32 && d->d_k == 128 &&
+           d->d_v == 128 && 3LL * d->H <= sm_count();
+}
+size_t gdn_split_scratch(const lkv_init_desc *d, int n_req, int total) {
+    return gdn_splits(d, n_req, total) ? 3 * sizeof(float) * static_cast<size_t>(d->H) * d->d_k * d->d_v : 0;
+}
+int gdn_split(InitArgs a, const int32_t *ids, int K, bool pool_bf16, float *scratch, cudaStream_t s) {
+    const int half = (K + 1) / 2;
+    float *S0 = a.S0;
+    const size_t slot = static_cast<size_t>(a.H) * a.d_k * a.d_v;
+    a.S0 = scratch;   // A, B, P
+    a.n_req = 3;
+    a.product = 2;
+    a.off_ids = 4;
+    a.idx.ptr = nullptr;
+    a.idx.n = 4 + half + 2 * (K - half);
+    const int32_t cu[4] = {0, half, K, K + (K - half)};
+    std::copy(cu, cu + 4, a.idx.v);
+    std::copy(ids, ids + K, a.idx.v + 4);
+    std::copy(ids + half, ids + K, a.idx.v + 4 + K);
+    if (launch_init_gdn_exact_tensor(a, pool_bf16, s) != cudaSuccess) return LKV_ERR_CUDA;
+    InitArgs b = a;   // chunks A, B of a pool whose second transition is P
+    b.states = scratch; b.transitions = scratch + slot; b.S0 = S0; b.n_req = 1; b.n_chunks = 2; b.product = -1;
+    const int32_t list[4] = {0, 2, 0, 1};
+    b.off_ids = 2;
+    b.idx.n = 4;
+    std::copy(list, list + 4, b.idx.v);
+    return launch_init_gdn_exact_tensor(b, false, s) == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
+}
+
 int init_impl(const void *states, const void *transitions, const int32_t *chunk_ids, const int32_t *cu_k,
               int n_req, int mode, const int32_t *sel_index, void *S0, const lkv_init_desc *d, void *stream) {
     int st = check_init_desc(d);
@@ -175,6 +211,10 @@ int init_impl(const void *states, const void *transitions, const int32_t *chunk_
         if (which == kGdnFp32 && (2 * d->d_k * 32 + 32 * (d->d_k + 1)) * sizeof(float) > 227 * 1024) return LKV_ERR_UNSUPPORTED;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // (a caller whose workspace is smaller than lkv_workspace_bytes() asks for gets the chain in one)
+    const size_t head = ws_bytes_for(n_ints, kInitIdxCap);
+    if (which == kGdnTensor && gdn_splits(d, n_req, total) && d->workspace_bytes >= head + gdn_split_scratch(d, n_req, total))
+        return gdn_split(a, chunk_ids, total, pool_bf16, reinterpret_cast<float *>(static_cast<char *>(d->workspace) + head), s);
     st = place_indices(a.idx, ints, d->workspace, s);
     if (st != LKV_OK) return st;
     cudaError_t e = cudaSuccess;
@@ -734,7 +774,8 @@ int lkv_ssd_fwd(const void *x, const float *dt, const float *A, const void *B, c
 size_t lkv_workspace_bytes(int which, const void *desc, int n_units, int n_index) {
     if (!desc || n_units < 0 || n_index < 0) return 0;
     switch (which) {
-        case LKV_WS_INIT: return ws_bytes_for(2 * n_units + 1 + n_index, kInitIdxCap);
+        case LKV_WS_INIT:
+            return ws_bytes_for(2 * n_units + 1 + n_index, kInitIdxCap) + gdn_split_scratch(static_cast<const lkv_init_desc *>(desc), n_units, n_index);
         case LKV_WS_GDN: {
             const lkv_gdn_desc *d = static_cast<const lkv_gdn_desc *>(desc);
             return ws_bytes_for(2 * n_units + 1, kScanIdxCap) + gdn_segment_scratch(d, gdn_cut(d, n_units).n);

@@ -22,5 +22,7 @@ def test_shared_chunks_equal_single_requests(n_req):
     got = b.lkv_init_state_batched(states, trans, ids, cu_k, n_req, b.LKV_INIT_EXACT, family=b.LKV_FAMILY_GDN)
     for r in range(n_req):
         own = ids[cu_k[r]:cu_k[r + 1]]
-        ref = b.lkv_init_state(states, trans, len(own), b.LKV_INIT_EXACT, family=b.LKV_FAMILY_GDN, chunk_ids=own)
+        # (as one chain: with room for it a single request is composed in two halves)
+        ref = b.lkv_init_state(states, trans, len(own), b.LKV_INIT_EXACT, family=b.LKV_FAMILY_GDN, chunk_ids=own,
+                               workspace_t=torch.zeros(256, dtype=torch.uint8, device="cuda"))
         assert torch.equal(got[r], ref), r
