@@ -128,7 +128,7 @@ class Family:
         self.out = torch.empty(self.out_shape, dtype=bf, device="cuda")
         self.host_out = torch.empty(self.out_shape, dtype=bf).pin_memory()
         self.host_S_T = torch.empty(self.S_T.shape, dtype=torch.float32).pin_memory()
-        self.ws_init = torch.zeros(1 << 20, dtype=torch.uint8, device="cuda")
+        self.ws_init = self.init_workspace(self.n_req, len(self.ids))
         self.ws_scan = self.scan_workspace(T, self.n_req)
         self.h2d_bytes = sum(t.numel() * t.element_size() for t in self.host.values())
         self.d2h_bytes = self.host_out.numel() * 2 + self.host_S_T.numel() * 4
@@ -142,6 +142,14 @@ class Family:
         self.set_bytes = self.h2d_bytes
         # one long sequence is scanned in segments: two launches more
         self.launches = 5 if self.n_req == 1 and self.ws_scan.numel() > self.scan_workspace(T, 2).numel() else 3
+        # and one long chain of chunks is composed in two halves: one more
+        self.launches += self.n_req == 1 and self.ws_init.numel() > self.init_workspace(2, len(self.ids)).numel()
+
+    def init_workspace(self, n_req, n_ids):
+        b = self.b
+        H, d_k, d_v = self.state_shape
+        d = b.lkv_init_desc(family=self.family_code, H=H, d_k=d_k, d_v=d_v, n_chunks=n_ids, state_dtype=b.LKV_DTYPE_F32)
+        return self.torch.zeros(b.lkv_workspace_bytes(b.LKV_WS_INIT, d, n_req, n_ids), dtype=self.torch.uint8, device="cuda")
 
     def scan_workspace(self, tokens, n_seq):
         """The workspace that the library asks for: what a caller of the public API has without passing one."""
