@@ -216,6 +216,10 @@ class Family:
 
     def init_exact(self):
         b, d = self.b, self.dev
+        if self.n_req == 1:   # the call for one request may compose a long chain in halves
+            b.lkv_init_state(d["states"], d["trans"], len(self.ids), b.LKV_INIT_EXACT, self.S0[0], family=self.family_code,
+                             chunk_ids=self.ids, workspace_t=self.ws_init)
+            return
         b.lkv_init_state_batched(d["states"], d["trans"], self.ids, self.cu_k, self.n_req, b.LKV_INIT_EXACT, None,
                                  self.S0, family=self.family_code, workspace_t=self.ws_init)
 

@@ -214,7 +214,8 @@ int lkv_init_state(const void *states, const void *transitions, int K, int mode,
  *   cu_k       HOST int32[n_req + 1]    request r owns chunk_ids[cu_k[r] .. cu_k[r+1])
  *   sel_index  HOST int32[n_req]        mode INDEX: position within each request; ignored otherwise (may be NULL)
  *   S0         out, float [n_req, H, d_k, d_v]
- * d->chunk_ids and d->sel_index are ignored.
+ * d->chunk_ids and d->sel_index are ignored.  A request's bits depend on its own chunks only: not on the other requests,
+ * their number or the size of the workspace.
  */
 int lkv_init_state_batched(const void *states, const void *transitions, const int32_t *chunk_ids,
                            const int32_t *cu_k, int n_req, int mode, const int32_t *sel_index, void *S0,

@@ -97,7 +97,8 @@ bool shares_chunks(const int32_t *ids, int total, const lkv_init_desc *d) {
 // One request's chain of K steps in two halves side by side, where three CTAs a head find an SM each: the state A of the first half, and of
 // the second the state B that it reaches from nothing and the product P of its transitions; then S0 = P A + B.  The second launch costs
 // about four steps.  32 heads: K = 10 19.6 -> 17.1 us, 16 30.3 -> 22.8, 64 120.6 -> 69.7 (8 chunks are 16.2 as one chain); the error against
-// 64 bits is that of the chain (7.3e-4 with transitions of norm 0.97).
+// 64 bits is that of the chain (7.3e-4 with transitions of norm 0.97).  Only lkv_init_state does this: a request of a batch is rounded as
+// one chain, whatever else is in the batch and wherever the scratch lies.
 constexpr int kSplitChunks = 10;
 bool gdn_splits(const lkv_init_desc *d, int n_req, int total) {
     return n_req == 1 && total >= kSplitChunks && total + total <= kInitIdxCap - 4 && d->family == LKV_FAMILY_GDN && d->compute != LKV_COMPUTE_FP32 && d->d_k == 128 &&
@@ -130,8 +131,9 @@ int gdn_split(InitArgs a, const int32_t *ids, int K, bool pool_bf16, float *scra
     return launch_init_gdn_exact_tensor(b, false, s) == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
 }
 
+// may_split: lkv_init_state, whose one request may be composed in halves
 int init_impl(const void *states, const void *transitions, const int32_t *chunk_ids, const int32_t *cu_k,
-              int n_req, int mode, const int32_t *sel_index, void *S0, const lkv_init_desc *d, void *stream) {
+              int n_req, int mode, const int32_t *sel_index, void *S0, const lkv_init_desc *d, void *stream, bool may_split = false) {
     int st = check_init_desc(d);
     if (st != LKV_OK) return st;
     if (mode != LKV_INIT_LAST && mode != LKV_INIT_INDEX && mode != LKV_INIT_EXACT) return LKV_ERR_MODE;
@@ -213,7 +215,7 @@ int init_impl(const void *states, const void *transitions, const int32_t *chunk_
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // (a caller whose workspace is smaller than lkv_workspace_bytes() asks for gets the chain in one)
     const size_t head = ws_bytes_for(n_ints, kInitIdxCap);
-    if (which == kGdnTensor && gdn_splits(d, n_req, total) && d->workspace_bytes >= head + gdn_split_scratch(d, n_req, total))
+    if (may_split && which == kGdnTensor && gdn_splits(d, n_req, total) && d->workspace_bytes >= head + gdn_split_scratch(d, n_req, total))
         return gdn_split(a, chunk_ids, total, pool_bf16, reinterpret_cast<float *>(static_cast<char *>(d->workspace) + head), s);
     st = place_indices(a.idx, ints, d->workspace, s);
     if (st != LKV_OK) return st;
@@ -386,7 +388,7 @@ int lkv_init_state(const void *states, const void *transitions, int K, int mode,
     }
     const int32_t cu_k[2] = {0, K};
     const int32_t sel[1] = {d->sel_index};
-    return init_impl(states, transitions, idp, cu_k, 1, mode, sel, S0, d, stream);
+    return init_impl(states, transitions, idp, cu_k, 1, mode, sel, S0, d, stream, true);
 }
 
 int lkv_init_state_batched(const void *states, const void *transitions, const int32_t *chunk_ids,

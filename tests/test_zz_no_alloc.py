@@ -91,3 +91,21 @@ def test_static_scratch_gdn_exact_on_the_tensor_cores_and_its_status_word():
     assert e.value.status == b.LKV_ERR_INDEX
     torch.cuda.synchronize()
     assert torch.equal(out, keep) and b.lkv_device_status_static() == b.LKV_OK
+
+
+@pytest.mark.parametrize("n_req, K", [(1, 16), (1, 64), (2, 16)])
+def test_static_scratch_gdn_long_chains_are_those_of_the_batched_call(n_req, K):
+    """A request of a batch is one chain of products, also where it is the only one and long (lkv_init_state may cut such a chain)."""
+    import torch
+    rng = np.random.default_rng(K)
+    pool = torch.from_numpy(wl.synthetic_states(rng, K, 2, 128, 128)).cuda()
+    tr = torch.from_numpy(wl.synthetic_gdn_transitions(rng, K, 2, 128)).cuda()
+    ids = np.concatenate([rng.permutation(K) for _ in range(n_req)]).astype(np.int32)
+    cu = (np.arange(n_req + 1) * K).astype(np.int32)
+    kw = dict(family=b.LKV_FAMILY_GDN)
+    ref = b.lkv_init_state_batched(pool, tr, ids, cu, n_req, b.LKV_INIT_EXACT, **kw)
+    assert torch.equal(b.lkv_init_state_batched_static(pool, tr, ids, cu, n_req, b.LKV_INIT_EXACT, **kw), ref)
+    for r in range(n_req):   # without room for anything but the chain, the call for one request gives the same bits
+        own = b.lkv_init_state(pool, tr, K, b.LKV_INIT_EXACT, chunk_ids=ids[cu[r]:cu[r + 1]],
+                               workspace_t=torch.zeros(256, dtype=torch.uint8, device="cuda"), **kw)
+        assert torch.equal(own, ref[r])
