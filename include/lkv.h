@@ -34,8 +34,9 @@
  *     nothing and keeps no pointer after a call returns; scratch lives in a
  *     caller-provided workspace whose size lkv_workspace_bytes() reports.  For
  *     a scan of one long sequence that size includes room for the states of
- *     the segments it is cut into when SMs would be idle; with a smaller
- *     workspace such a call runs as one piece.
+ *     the segments it is cut into when SMs would be idle, and for
+ *     lkv_init_state with a long chain of GDN chunks room for the three states
+ *     of its halves; with a smaller workspace such a call runs as one piece.
  *     A workspace must not be shared by calls that can overlap on the GPU.
  *   - Calls are asynchronous on `stream` (a cudaStream_t passed as void*,
  *     NULL = the legacy default stream).  They do not synchronise.
@@ -200,6 +201,15 @@ typedef struct lkv_ssd_desc {
  * for j = 2..K (Eq. 5 applied in context order); the transition of the first
  * chunk is never read.  K == 1 returns S_{c_1} untouched in every mode;
  * K == 0 returns the zero state.
+ * On the tensor cores (GDN, d_k = d_v = 128) a chain of 10 chunks or more may
+ * be computed in two halves, S0 = P A + B with A the state of the first half, B
+ * what the second half reaches from nothing and P the product of its
+ * transitions: where three CTAs a head find an SM each and the workspace has the
+ * size that lkv_workspace_bytes() states.  The error is that of the chain, the
+ * rounding is another one: bits then depend on the number of SMs and on whether
+ * the workspace is that large, and differ from those of
+ * lkv_init_state_batched.  Equal calls with equal workspace sizes on equal
+ * GPUs give equal bits.
  * Errors: NULL states/S0/desc (or transitions in EXACT with K >= 2), bad
  * mode/family/dtype, K < 0, id outside [0, n_chunks), sel_index outside
  * [0, K), misaligned pointers, unsupported dims, workspace too small.

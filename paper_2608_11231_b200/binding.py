@@ -243,7 +243,10 @@ def _init_desc(states, family, compute, ws_t, n_units, n_index, chunk_ids_np=Non
 def lkv_init_state(states: torch.Tensor, transitions: Optional[torch.Tensor], K: int, mode: int,
                    S0: Optional[torch.Tensor] = None, *, family: int, chunk_ids=None, sel_index: int = 0,
                    compute: int = LKV_COMPUTE_AUTO, workspace_t: Optional[torch.Tensor] = None, stream=None):
-    """State initialisation for one request.  states: pool [n, H, d_k, d_v]; returns S0 [H, d_k, d_v] fp32."""
+    """State initialisation for one request.  states: pool [n, H, d_k, d_v]; returns S0 [H, d_k, d_v] fp32.
+
+    A long GDN chain may be composed in two halves: other rounding than in lkv_init_state_batched, the same error.
+    """
     return (_calls or calls()).init_state(states, transitions, K, mode, S0, family, chunk_ids, sel_index, compute, workspace_t,
                                           stream)
 
