@@ -111,6 +111,8 @@ extern "C" {
 #define LKV_WS_INIT 0
 #define LKV_WS_GDN 1
 #define LKV_WS_SSD 2
+#define LKV_WS_INIT_LIST 3 /* an initialiser call that composes nothing in halves: lkv_init_state in the modes LAST and INDEX,
+                              lkv_init_state_batched, lkv_init_state_fold */
 
 /*
  * Descriptor of lkv_init_state / lkv_init_state_batched.
@@ -419,7 +421,9 @@ size_t lkv_state_rel_error_workspace_bytes(int n_states, size_t state_elems);
 
 /*
  * Workspace size in bytes for a call described by `desc` (lkv_init_desc, lkv_gdn_desc or
- * lkv_ssd_desc according to `which`).  n_units is the number of requests (init) or
+ * lkv_ssd_desc according to `which`).  LKV_WS_INIT is enough for every initialiser call; a long
+ * GDN chain makes it three states larger than LKV_WS_INIT_LIST, which lkv_init_state uses in mode
+ * EXACT only.  n_units is the number of requests (init) or
  * sequences (scans) and n_index the total number of chunk ids over all requests
  * (init; 0 for the scans).  Returns 0 for a NULL or invalid descriptor.
  */

@@ -29,7 +29,7 @@ LKV_FAMILY_MAMBA2, LKV_FAMILY_GDN = 0, 1
 LKV_DTYPE_F32, LKV_DTYPE_BF16 = 0, 1
 LKV_INIT_LAST, LKV_INIT_INDEX, LKV_INIT_EXACT = 0, 1, 2
 LKV_COMPUTE_AUTO, LKV_COMPUTE_FP32, LKV_COMPUTE_TENSOR = 0, 1, 2
-LKV_WS_INIT, LKV_WS_GDN, LKV_WS_SSD = 0, 1, 2
+LKV_WS_INIT, LKV_WS_GDN, LKV_WS_SSD, LKV_WS_INIT_LIST = 0, 1, 2, 3
 
 EXPORTS = ("lkv_init_state", "lkv_init_state_batched", "lkv_init_state_batched_static", "lkv_gdn_fwd", "lkv_ssd_fwd",
            "lkv_gdn_chunk_transition", "lkv_mamba_chunk_logdecay", "lkv_init_state_fold", "lkv_gdn_fwd_segmented",
@@ -234,7 +234,7 @@ def _init_desc(states, family, compute, ws_t, n_units, n_index, chunk_ids_np=Non
                       chunk_ids=None if chunk_ids_np is None else chunk_ids_np.ctypes.data, workspace=None,
                       workspace_bytes=0)
     if ws_t is None:
-        ws_t = workspace(states.device, lkv_workspace_bytes(LKV_WS_INIT, d, n_units, n_index), stream)
+        ws_t = workspace(states.device, lkv_workspace_bytes(LKV_WS_INIT_LIST, d, n_units, n_index), stream)
     d.workspace = ws_t.data_ptr()
     d.workspace_bytes = ws_t.numel()
     return d, ws_t

@@ -776,6 +776,8 @@ int lkv_ssd_fwd(const void *x, const float *dt, const float *A, const void *B, c
 size_t lkv_workspace_bytes(int which, const void *desc, int n_units, int n_index) {
     if (!desc || n_units < 0 || n_index < 0) return 0;
     switch (which) {
+        case LKV_WS_INIT_LIST:
+            return ws_bytes_for(2 * n_units + 1 + n_index, kInitIdxCap);
         case LKV_WS_INIT:
             return ws_bytes_for(2 * n_units + 1 + n_index, kInitIdxCap) + gdn_split_scratch(static_cast<const lkv_init_desc *>(desc), n_units, n_index);
         case LKV_WS_GDN: {

@@ -271,11 +271,12 @@ PyObject *init_state(PyObject *, PyObject *const *a, Py_ssize_t n) {
         d.sel_index = to_int(a[7]);
         d.chunk_ids = ids.data();
         void *stream = stream_of(a[10]);
-        set_workspace(d, a[9], states, stream, LKV_WS_INIT, 1, K);
+        const int mode = to_int(a[3]);
+        set_workspace(d, a[9], states, stream, mode == LKV_INIT_EXACT ? LKV_WS_INIT : LKV_WS_INIT_LIST, 1, K);
         Output S0;
         if (a[4] != Py_None) S0.given(a[4]);
         else S0.make(new_tensor(states.sizes().slice(1), at::kFloat, states));
-        call("lkv_init_state", d.workspace, lkv_init_state, ptr_of(a[0]), ptr_of(a[1]), K, to_int(a[3]), S0.ptr, &d,
+        call("lkv_init_state", d.workspace, lkv_init_state, ptr_of(a[0]), ptr_of(a[1]), K, mode, S0.ptr, &d,
              stream);
         return S0.take();
     });
@@ -290,7 +291,7 @@ PyObject *init_state_batched(PyObject *, PyObject *const *a, Py_ssize_t n) {
         HostInts ids(a[2]), cu(a[3]), sel(a[6]);
         const int n_req = to_int(a[4]);
         void *stream = stream_of(a[11]);
-        set_workspace(d, a[10], states, stream, LKV_WS_INIT, n_req, ids.size());
+        set_workspace(d, a[10], states, stream, LKV_WS_INIT_LIST, n_req, ids.size());
         Output S0;
         if (a[7] != Py_None) S0.given(a[7]);
         else S0.make(new_tensor({n_req, states.size(1), states.size(2), states.size(3)}, at::kFloat, states));

@@ -209,6 +209,17 @@ def test_workspace_bytes(lib):
     assert b.lkv_workspace_bytes(17, d, 1, 1) == 0
 
 
+@pytest.mark.parametrize("K", [1, 9, 10, 64, 4100])
+def test_workspace_of_calls_that_compose_nothing_in_halves(lib, K):
+    """Their workspace is the status word and the index list; the states of the halves are asked for by the one call that uses them."""
+    d = _desc(H=32, d_k=128, d_v=128, n_chunks=K)
+    lists = 256 + (0 if K + 3 <= 4000 else (4 * (K + 3) + 255) // 256 * 256)
+    assert b.lkv_workspace_bytes(b.LKV_WS_INIT_LIST, d, 1, K) == lists
+    # (4000 indices travel in the kernel parameters; the halves name the chunks of the second one twice)
+    assert b.lkv_workspace_bytes(b.LKV_WS_INIT, d, 1, K) - lists == (3 * 32 * 128 * 128 * 4 if 10 <= K <= 1998 else 0)
+    assert b.lkv_workspace_bytes(b.LKV_WS_INIT, d, 2, K) == b.lkv_workspace_bytes(b.LKV_WS_INIT_LIST, d, 2, K)
+
+
 def test_missing_library_fails_loudly(tmp_path, monkeypatch):
     monkeypatch.setattr(b, "_lib", None)
     monkeypatch.setattr(b, "LIB_PATH", str(tmp_path / "liblkv.so"))

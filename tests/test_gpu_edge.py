@@ -245,3 +245,29 @@ def test_single_state_init_with_index_lists_of_every_kind(n_req):
     ids = np.random.default_rng(n_req).integers(0, 50, n_req).astype(np.int32)
     S0 = b.lkv_init_state_batched(states, None, ids, np.arange(n_req + 1, dtype=np.int32), n_req, b.LKV_INIT_LAST, family=b.LKV_FAMILY_GDN)
     assert torch.equal(S0, states[torch.from_numpy(ids).long().cuda()])
+
+
+def test_workspaces_are_as_large_as_the_call_needs():
+    """Only an exact composition of one request asks for the states of its halves: the copies, the batched call and the fold do not."""
+    import torch
+    K, H = 12, 4
+    states, trans = torch.randn((K, H, 128, 128), device="cuda"), 0.05 * torch.randn((K, H, 128, 128), device="cuda")
+    k = torch.nn.functional.normalize(torch.randn((K * 8, H, 128), device="cuda"), dim=-1).bfloat16()
+    gate = torch.zeros((K * 8, H), device="cuda")
+    ids, cu = np.arange(K, dtype=np.int32), np.array([0, K], dtype=np.int32)
+    fam = dict(family=b.LKV_FAMILY_GDN)
+    size = {}
+    calls = dict(last=lambda s: b.lkv_init_state(states, None, K, b.LKV_INIT_LAST, stream=s, **fam),
+                 index=lambda s: b.lkv_init_state(states, None, K, b.LKV_INIT_INDEX, sel_index=3, stream=s, **fam),
+                 batched=lambda s: b.lkv_init_state_batched(states, trans, ids, cu, 1, b.LKV_INIT_EXACT, stream=s, **fam),
+                 fold=lambda s: b.lkv_init_state_fold(states, k, gate, gate, 8 * np.arange(K + 1, dtype=np.int32), K, stream=s),
+                 exact=lambda s: b.lkv_init_state(states, trans, K, b.LKV_INIT_EXACT, stream=s, **fam))
+    torch.cuda.synchronize()
+    for name, f in calls.items():
+        s = torch.cuda.Stream()
+        b._ws_cache.pop((0, s.cuda_stream), None)   # (streams come from a pool: another test may have used this one)
+        f(s)
+        s.synchronize()
+        size[name] = b._ws_cache[(0, s.cuda_stream)].numel()
+    assert size.pop("exact") == 256 + 3 * 4 * H * 128 * 128
+    assert set(size.values()) == {4096}
