@@ -26,3 +26,86 @@ def test_composition_in_halves(K, H, bf16):
     chain = err(b.lkv_init_state(pool, trans, K, b.LKV_INIT_EXACT, workspace_t=torch.zeros(256, dtype=torch.uint8, device="cuda"), **kw))
     # tf32 operands, rounded to nearest: 2^-12 a step and operand at most, added in squares
     assert chain <= 2 ** -12 * (2 * K) ** 0.5 and cut <= 1.02 * chain, (cut, chain)
+
+
+def _cached_chunks(K, H, decay, seed):
+    """States and transitions that the library makes from tokens whose decays leave a share of the carried state."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    F, L = torch.nn.functional, 96
+    rn = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    k, v = F.normalize(rn(K * L, H, 128), dim=-1).bfloat16(), rn(K * L, H, 128).bfloat16()
+    return b.lkv_gdn_chunk_artifacts(k, v, -decay * F.softplus(rn(K * L, H)), torch.sigmoid(rn(K * L, H)) / 4, cu_seqlens=(np.arange(K + 1) * L).astype(np.int32))
+
+
+@pytest.mark.parametrize("K", [10, 17, 40])
+@pytest.mark.parametrize("decay", [1e-4, 1e-3, 1e-2])   # of the state, a chunk of 96 tokens leaves all, nine tenths, half
+def test_composition_in_halves_of_chunks_from_tokens(K, decay):
+    import torch
+    states, trans = _cached_chunks(K, 2, decay, K)
+    ref = states[0].double()
+    for j in range(1, K):
+        ref = trans[j].double() @ ref + states[j].double()
+    kw = dict(family=b.LKV_FAMILY_GDN)
+    err = lambda x: float((x.double() - ref).norm() / ref.norm())
+    cut = err(b.lkv_init_state(states, trans, K, b.LKV_INIT_EXACT, **kw))
+    chain = err(b.lkv_init_state(states, trans, K, b.LKV_INIT_EXACT, workspace_t=torch.zeros(256, dtype=torch.uint8, device="cuda"), **kw))
+    # the other order of the products rounds otherwise, not worse (within 2 % here; 15 % are left for other draws)
+    assert chain <= 2 ** -12 * (2 * K) ** 0.5 and cut <= 1.15 * chain, (cut, chain)
+
+
+def test_composition_in_halves_from_a_graph():
+    """Two kernels that hand three states on through the workspace: a replay on new inputs gives the bits of the plain call."""
+    import torch
+    K, H = 16, 4
+    sets = [_cached_chunks(K, H, 1e-3, seed) for seed in (1, 2)]
+    states, trans = (x.clone() for x in sets[0])
+    S0 = torch.empty((H, 128, 128), device="cuda")
+    f = lambda s, t, out=None: b.lkv_init_state(s, t, K, b.LKV_INIT_EXACT, out, family=b.LKV_FAMILY_GDN)
+    want = [f(*x) for x in sets]
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(side):
+        f(states, trans, S0)   # the stream's workspace exists before the capture
+        with torch.cuda.graph(graph, stream=side):
+            f(states, trans, S0)
+            f(states, trans, S0)
+    for i in (1, 0, 1):
+        states.copy_(sets[i][0])
+        trans.copy_(sets[i][1])
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(S0, want[i])
+
+
+def test_composition_in_halves_by_threads_that_share_a_stream():
+    import torch
+    from concurrent.futures import ThreadPoolExecutor
+    sets = [_cached_chunks(K, 8, 1e-3, K) for K in (10, 16, 33)]
+    f = lambda i: b.lkv_init_state(*sets[i], sets[i][0].shape[0], b.LKV_INIT_EXACT, family=b.LKV_FAMILY_GDN)
+    want = [f(i) for i in range(3)]
+    torch.cuda.synchronize()
+
+    def engine(i):
+        for _ in range(30):
+            assert torch.equal(f(i), want[i])
+
+    with ThreadPoolExecutor(3) as pool:
+        for r in [pool.submit(engine, i) for i in range(3)]:
+            r.result()
+
+
+def test_composition_in_halves_on_several_streams():
+    import torch
+    sets = [_cached_chunks(16, 8, 1e-3, seed) for seed in (5, 6)]
+    f = lambda i, out, stream: b.lkv_init_state(*sets[i], 16, b.LKV_INIT_EXACT, out, family=b.LKV_FAMILY_GDN, stream=stream)
+    want = [f(i, None, None) for i in range(2)]
+    outs = torch.empty((2, 20, 8, 128, 128), device="cuda")
+    streams = [torch.cuda.Stream() for _ in sets]
+    torch.cuda.synchronize()
+    for n in range(20):
+        for i in range(2):
+            f(i, outs[i, n], streams[i])
+    torch.cuda.synchronize()
+    assert all(torch.equal(outs[i, n], want[i]) for i in range(2) for n in range(20))
