@@ -498,12 +498,25 @@ cudaError_t launch(const GdnArgs &a, cudaStream_t s) {
     return launch_chained(kernel, dim3(a.H_v, a.n_seq, a.d_v / VC), 256, smem, s, a);
 }
 
+// Does a call go to the clusters?  Yes where each of their CTAs finds an SM.  The SMs of a cluster belong to one GPC, which leaves some
+// without: 15, 33 and 74 clusters of 8, 4 and 2 are resident at a time with one CTA an SM, 120, 132 and 148 of the 148 SMs (as numbers
+// and not as a query, so that equal calls take the same kernel, and give the same bits, whichever SMs a GPU has).  One cluster more and
+// there is a second round: 64 tokens of 15, 16 heads of 176 x 64 16.2, 30.9 us against 24.4 without clusters.  Up to d_k = 160 two CTAs share
+// an SM instead.  A block then takes longer and the start is dearer, which pays in long sequences only: 18 heads of 64 x 64 13.7 us
+// (64 tokens), 23.9 (128), 81 (512) against 13.1, 23.7, 86; of 160 x 64 23.4, 41.4, 144 against 22.5, 41.6, 156.
+bool clusters_pay(const GdnArgs &a) {
+    const long long ctas = static_cast<long long>(a.H_v) * a.n_seq * (a.d_v / 8);
+    const size_t smem = cluster_smem_bytes(a.d_k);
+    if (ctas > sm_count() || smem > 227 * 1024) return false;
+    const int without = a.d_v == 16 ? 0 : a.d_v == 32 ? 16 : 28;   // SMs
+    return ctas <= sm_count() - without || (2 * (smem + 1024) <= 228 * 1024 && a.T_total >= 256LL * a.n_ranges);
+}
+
 // Columns per CTA: all of them when heads and sequences fill the GPU; otherwise halved as long as that still finds idle SMs.
 // The coupling matrices are then computed once per part, side by side.
 template <typename T>
 cudaError_t dispatch(const GdnArgs &a, cudaStream_t s) {
-    // clusters while every CTA of theirs finds an SM
-    if (static_cast<long long>(a.H_v) * a.n_seq * (a.d_v / 8) <= sm_count() && cluster_smem_bytes(a.d_k) <= 227 * 1024)
+    if (clusters_pay(a))
         return a.d_v == 16 ? launch_cluster<T, 2>(a, s) : a.d_v == 32 ? launch_cluster<T, 4>(a, s) : launch_cluster<T, 8>(a, s);
     int vc = a.d_v;
     const long long units = static_cast<long long>(a.H_v) * a.n_seq;
