@@ -402,59 +402,110 @@ cudaError_t launch_init_gdn_exact_fp32(const InitArgs &a, bool pool_bf16, cudaSt
 
 namespace {
 
-// A cluster of eight CTAs per (sequence, group of 32 heads), an eighth of the tokens each: lanes walk consecutive heads, so every
-// token's dt row is read with coalesced 128-byte accesses.  What bounds it is the latency of the loads, not their bytes: each of
-// a CTA's eight warps has eight tokens in flight, in eight sums of their own, and the cluster puts 768 CTAs on the 32 chunks of
-// 256 .. 2048 tokens x 80 heads that one CTA per (sequence, 32 heads), one load after the other into one sum, took 38.9 us
-// for; behind the scan that makes the states of these chunks 201 -> 174 us for both.  All partial sums are added in a fixed order.
-constexpr int kDecayParts = 8, kDecayWarps = 8, kDecayLoads = 8;
-__global__ void __cluster_dims__(kDecayParts, 1, 1) __launch_bounds__(32 * kDecayWarps)
-mamba_logdecay_kernel(const __grid_constant__ SsdArgs a, float *__restrict__ out) {
-    const cg::cluster_group cluster = cg::this_cluster();
-    const int seq = blockIdx.y, part = blockIdx.x % kDecayParts;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int h = (blockIdx.x / kDecayParts) * 32 + lane;
-    __shared__ float red[kDecayWarps][32], sum[32];
-    pdl_launch();
-    pdl_wait();
-    const int t0 = a.cu[seq], n = a.cu[seq + 1] - t0;
-    const int per = (n + kDecayParts - 1) / kDecayParts;
-    const long long end = min(static_cast<long long>(per) * (part + 1), static_cast<long long>(n));
+// Lanes walk consecutive heads, so every token's dt row is read with coalesced 128-byte accesses.  What bounds it is the latency of the
+// loads, not their bytes.  A sequence of up to kDecayShort tokens is summed by one CTA of eight warps, a warp every eighth token,
+// 16 loads in flight; a longer one in eight parts of its tokens, a part by eight warps with eight loads in flight.  The parts are
+// side by side in a cluster or one after the other in a CTA: all sums are added in an order that the sequence's own length sets,
+// whatever else is in the call.
+// 80 heads: 1 x 16, 256, 512 tokens 1.4, 1.9, 2.6 us; 64 x 64 1.7, 256 x 64 3.6 (all in clusters 2.1, 2.2, 2.4, 7.7, 27.6; one load after
+// the other in one CTA 1.6, 2.8, 4.4, 2.0, 3.2); 1 x 8192 18.5 and 32 x 2048 13.1 in clusters (144, 38).
+constexpr int kDecayParts = 8, kDecayWarps = 8, kDecayLoads = 8, kDecayShort = 512;
+
+__device__ __forceinline__ float decay_tree(const float (&x)[kDecayLoads]) {
+    return ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
+}
+// dt of every eighth token, n of them, in eight running sums
+__device__ __forceinline__ float decay_short(const float *dt, int H, int n) {
+    const size_t step = static_cast<size_t>(kDecayWarps) * H;
     float acc[kDecayLoads];
 #pragma unroll
     for (int i = 0; i < kDecayLoads; ++i) acc[i] = 0.f;
-    if (h < a.H) {
-        const float *p = a.dt + static_cast<size_t>(t0) * a.H + h;
-        for (long long t = static_cast<long long>(per) * part + warp; t < end; t += kDecayWarps * kDecayLoads) {
-            float v[kDecayLoads];
+    for (; n > 0; n -= 2 * kDecayLoads, dt += 2 * kDecayLoads * step) {
+        float v[2 * kDecayLoads];
 #pragma unroll
-            for (int i = 0; i < kDecayLoads; ++i) v[i] = t + i * kDecayWarps < end ? p[static_cast<size_t>(t + i * kDecayWarps) * a.H] : 0.f;
+        for (int i = 0; i < 2 * kDecayLoads; ++i) v[i] = i < n ? dt[i * step] : 0.f;
 #pragma unroll
-            for (int i = 0; i < kDecayLoads; ++i) acc[i] += v[i];
-        }
+        for (int i = 0; i < 2 * kDecayLoads; ++i) acc[i % kDecayLoads] += v[i];
     }
-    red[warp][lane] = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]));
-    __syncthreads();
-    if (warp == 0) {
-        float s = 0.f;
-#pragma unroll
-        for (int w = 0; w < kDecayWarps; ++w) s += red[w][lane];
-        sum[lane] = s;
-    }
-    cluster.sync();
-    if (part == 0 && warp == 0 && h < a.H) {
-        float s = 0.f;
-#pragma unroll
-        for (int r = 0; r < kDecayParts; ++r) s += cluster.map_shared_rank(sum, r)[lane];
-        out[static_cast<size_t>(seq) * a.H + h] = a.A[h] * s;
-    }
-    cluster.sync();   // the sums stay where they are until they have been read
+    return decay_tree(acc);
 }
+// dt of every eighth of the tokens t .. end, in eight running sums
+__device__ __forceinline__ float decay_part(const float *dt, int H, long long t, long long end) {
+    float acc[kDecayLoads];
+#pragma unroll
+    for (int i = 0; i < kDecayLoads; ++i) acc[i] = 0.f;
+    for (; t < end; t += kDecayWarps * kDecayLoads) {
+        float v[kDecayLoads];
+#pragma unroll
+        for (int i = 0; i < kDecayLoads; ++i) v[i] = t + i * kDecayWarps < end ? dt[static_cast<size_t>(t + i * kDecayWarps) * H] : 0.f;
+#pragma unroll
+        for (int i = 0; i < kDecayLoads; ++i) acc[i] += v[i];
+    }
+    return decay_tree(acc);
+}
+__device__ __forceinline__ float decay_column(const float (*x)[32], int lane) {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s += x[i][lane];
+    return s;
+}
+
+template <bool kCluster>
+__device__ __forceinline__ void logdecay(const SsdArgs &a, float *__restrict__ out) {
+    const int seq = blockIdx.y, part = kCluster ? blockIdx.x % kDecayParts : 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int h = (kCluster ? blockIdx.x / kDecayParts : blockIdx.x) * 32 + lane;
+    __shared__ float red[kCluster ? 1 : kDecayParts][kDecayWarps][32], sum[kDecayParts][32];
+    pdl_launch();
+    pdl_wait();
+    const int t0 = a.cu[seq], n = a.cu[seq + 1] - t0;
+    const float *dt = a.dt + static_cast<size_t>(t0) * a.H + h;
+    const bool in = h < a.H;
+    if (n <= kDecayShort) {
+        if (part > 0) return;   // (and so do the others of the cluster: nobody is waited for)
+        sum[warp][lane] = in ? decay_short(dt + static_cast<size_t>(warp) * a.H, a.H, (n - warp + kDecayWarps - 1) / kDecayWarps) : 0.f;
+        __syncthreads();
+        if (warp == 0 && in) out[static_cast<size_t>(seq) * a.H + h] = a.A[h] * decay_column(sum, lane);
+        return;
+    }
+    const long long per = (n + kDecayParts - 1) / kDecayParts;
+    auto partial = [&](int p) { return in ? decay_part(dt, a.H, per * p + warp, min(per * (p + 1), static_cast<long long>(n))) : 0.f; };
+    if (kCluster) {
+        const cg::cluster_group cluster = cg::this_cluster();
+        red[0][warp][lane] = partial(part);
+        __syncthreads();
+        if (warp == 0) sum[0][lane] = decay_column(red[0], lane);
+        cluster.sync();
+        if (part == 0 && warp == 0 && in) {
+            float s = 0.f;
+#pragma unroll
+            for (int r = 0; r < kDecayParts; ++r) s += cluster.map_shared_rank(sum[0], r)[lane];
+            out[static_cast<size_t>(seq) * a.H + h] = a.A[h] * s;
+        }
+        cluster.sync();   // the sums stay where they are until they have been read
+    } else {
+#pragma unroll 1
+        for (int p = 0; p < kDecayParts; ++p) red[p][warp][lane] = partial(p);
+        __syncthreads();
+        sum[warp][lane] = decay_column(red[warp], lane);
+        __syncthreads();
+        if (warp == 0 && in) out[static_cast<size_t>(seq) * a.H + h] = a.A[h] * decay_column(sum, lane);
+    }
+}
+__global__ void __cluster_dims__(kDecayParts, 1, 1) __launch_bounds__(32 * kDecayWarps)
+mamba_logdecay_cluster_kernel(const __grid_constant__ SsdArgs a, float *__restrict__ out) { logdecay<true>(a, out); }
+__global__ void __launch_bounds__(32 * kDecayWarps, 4)
+mamba_logdecay_kernel(const __grid_constant__ SsdArgs a, float *__restrict__ out) { logdecay<false>(a, out); }
 
 }  // namespace
 
-cudaError_t launch_mamba_logdecay(const SsdArgs &a, float *logdecay, cudaStream_t s) {
-    return launch_chained(mamba_logdecay_kernel, dim3(kDecayParts * ((a.H + 31) / 32), a.n_seq), 32 * kDecayWarps, 0, s, a, logdecay);
+cudaError_t launch_mamba_logdecay(const SsdArgs &a, float *logdecay, int longest, cudaStream_t s) {
+    const int groups = (a.H + 31) / 32;
+    // A launch of clusters costs 3.5 ns a CTA; in one CTA the longest sequence takes 4 (dt in L2) to 10 ns a token.  80 heads, clusters, CTAs:
+    // 32 x 1024 tokens (768 CTAs in clusters) 8.7, 13.8 us; 64 x 1024 13.4, 14.5; 128 x 1024 22.8, 17.1; 400 x 1024 65, 40.
+    if (longest > kDecayShort && static_cast<long long>(kDecayParts) * groups * a.n_seq <= 2LL * longest)
+        return launch_chained(mamba_logdecay_cluster_kernel, dim3(kDecayParts * groups, a.n_seq), 32 * kDecayWarps, 0, s, a, logdecay);
+    return launch_chained(mamba_logdecay_kernel, dim3(groups, a.n_seq), 32 * kDecayWarps, 0, s, a, logdecay);
 }
 
 namespace {

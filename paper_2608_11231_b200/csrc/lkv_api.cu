@@ -685,9 +685,11 @@ int lkv_mamba_chunk_logdecay(const float *dt, const float *A, float *logdecay, c
     a.dt = dt; a.A = A; a.n_seq = d->n_seq; a.T_total = d->T_total; a.H = d->H; a.P = d->P; a.N = d->N; a.G = d->G;
     a.status = static_cast<int32_t *>(d->workspace);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    int longest = 0;
+    for (int i = 0; i < d->n_seq; ++i) longest = std::max(longest, cu[i + 1] - cu[i]);
     st = place_indices(a.cu, cu, d->workspace, s);
     if (st != LKV_OK) return st;
-    return launch_mamba_logdecay(a, logdecay, s) == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
+    return launch_mamba_logdecay(a, logdecay, longest, s) == cudaSuccess ? LKV_OK : LKV_ERR_CUDA;
 }
 
 size_t lkv_state_rel_error_workspace_bytes(int n_states, size_t state_elems) {
