@@ -353,8 +353,8 @@ __global__ void __cluster_dims__(1, 1, CS) __launch_bounds__(256) gdn_scan_fp32_
         if (m < dk) x = id ? (m == j ? 1.f : 0.f) : S0 ? S0[static_cast<size_t>(m) * dv] : 0.f;
         St[warp * ks + m] = x;
     }
-    for (int row = warp; row < 4 * kC; row += 8)
-        for (int m = dk + lane; m < dkp; m += 32) KQ[row * ks + m] = 0.f;
+    for (int e = tid; e < 4 * kC * 16; e += 256)   // (at most 15 zeros a row)
+        if (dk + (e & 15) < dkp) KQ[(e >> 4) * ks + dk + (e & 15)] = 0.f;
     cluster.sync();   // the others have started: their shared memory may be written
 
     // the product's tile of this thread, shared by four lanes: rows row0 .., columns col0, col0 + 4, ..
