@@ -311,34 +311,43 @@ __global__ void __cluster_dims__(1, 1, CS) __launch_bounds__(256) gdn_scan_fp32_
     auto async16 = [](float *dst, const void *src) {
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
     };
-    // k, q of the block at t0 into a stage; g, beta and v of it into registers
-    const bool async = std::is_same<T, float>::value && dk % 4 == 0;
+    // k, q of the block at t0 into a stage (warp = tokens warp, warp + 8, ..); g, beta and v of it into registers
+    constexpr bool async = std::is_same<T, float>::value;
     float g_next = 0.f, b_next = 0.f, v_next = 0.f;
     auto fetch = [&](int t0, int stage) {
-        float *st = KQ + stage * 2 * kC * ks;
-        if (async) {
-            for (int m = 4 * lane; m < dk; m += 128) {   // warp = tokens warp, warp + 8, ..
-                const size_t off = (static_cast<size_t>(t0 + warp) * a.H_k + hk) * dk + m, step = static_cast<size_t>(8) * a.H_k * dk;
-                float *dst = st + warp * ks + m;
+        float *st = KQ + (stage * 2 * kC + warp) * ks;
+        const size_t first = (static_cast<size_t>(t0 + warp) * a.H_k + hk) * dk, step = static_cast<size_t>(8) * a.H_k * dk;
+        if (async && dk % 4 == 0) {
+            for (int m = 4 * lane; m < dk; m += 128) {
+                float *dst = st + m;
 #pragma unroll
                 for (int u = 0; u < kC / 8; ++u) {
                     if (t0 + warp + 8 * u < t_end) {
-                        async16(dst + 8 * u * ks, k + off + u * step);
-                        async16(dst + (kC + 8 * u) * ks, q + off + u * step);
+                        async16(dst + 8 * u * ks, k + first + m + u * step);
+                        async16(dst + (kC + 8 * u) * ks, q + first + m + u * step);
                     } else {
                         *reinterpret_cast<float4 *>(dst + 8 * u * ks) = *reinterpret_cast<float4 *>(dst + (kC + 8 * u) * ks) = make_float4(0.f, 0.f, 0.f, 0.f);
                     }
                 }
             }
-            asm volatile("cp.async.commit_group;" ::: "memory");
         } else {
-#pragma unroll 4
-            for (int row = warp; row < 2 * kC; row += 8) {
-                const int t = row & (kC - 1);
-                const T *src = (row < kC ? k : q) + (static_cast<size_t>(t0 + t) * a.H_k + hk) * dk;
-                for (int m = lane; m < dk; m += 32) st[row * ks + m] = t0 + t < t_end ? to_f32<T>(src[m]) : 0.f;
+            for (int m = lane; m < dk; m += 32) {
+                float *dst = st + m;
+                float kr[kC / 8], qr[kC / 8];
+#pragma unroll
+                for (int u = 0; u < kC / 8; ++u) {
+                    const bool in = t0 + warp + 8 * u < t_end;
+                    kr[u] = in ? to_f32<T>(k[first + m + u * step]) : 0.f;
+                    qr[u] = in ? to_f32<T>(q[first + m + u * step]) : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < kC / 8; ++u) {
+                    dst[8 * u * ks] = kr[u];
+                    dst[(kC + 8 * u) * ks] = qr[u];
+                }
             }
         }
+        if (async) asm volatile("cp.async.commit_group;" ::: "memory");
         const int t = t0 + lane;   // a padded token is the identity step: g = 0, beta = 0
         const bool ok = t < t_end;
         g_next = ok ? a.g[static_cast<size_t>(t) * a.H_v + h] : 0.f;
