@@ -19,6 +19,8 @@
 // times the CTAs).
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace lkv {
@@ -275,7 +277,7 @@ __global__ void __launch_bounds__(256) gdn_scan_fp32_kernel(const __grid_constan
 // thread, the contraction split over four lanes (every other four channels of 16).  After that nothing leaves a warp: lane = token, warp =
 // column for the right-hand side, the substitution and the outputs, lane = channel for the state.  Tokens of the next block are copied
 // (fp32) while the other CTAs' parts are waited for.  Two heads of 64 x 64: a block 5.2 -> 3.1 us (product 0.7, substitution 0.5, outputs and
-// state 0.8, the rest barriers and hand-overs); 64, 512 tokens 12.7, 85.4 -> 9.6, 53.3 us.  Slower: 16 columns a CTA, a row of k and
+// state 0.8, the rest barriers and hand-overs); 64, 512 tokens 12.7, 85.4 -> 9.1, 52.8 us.  Slower: 16 columns a CTA, a row of k and
 // q a lane and no cluster 13.9, 78; the tokens by bulk copies, a row each, 12.5, 78.5; copied at the start of a block 11.1, 62.5.
 template <typename T, int CS>
 __global__ void __cluster_dims__(1, 1, CS) __launch_bounds__(256) gdn_scan_fp32_cluster_kernel(const __grid_constant__ GdnArgs a) {
@@ -490,8 +492,7 @@ size_t cluster_smem_bytes(int dk) {
     return sizeof(float) * ((4 * kC + 8) * static_cast<size_t>(cluster_stride(dk)) + 4 * kC * kC + 2 * 8 * kC + 4 * kC + 8 * 2 * kC);
 }
 template <typename T, int CS>
-cudaError_t launch_cluster(const GdnArgs &a, cudaStream_t s) {
-    const size_t smem = cluster_smem_bytes(a.d_k);
+cudaError_t launch_cluster(const GdnArgs &a, size_t smem, cudaStream_t s) {
     auto kernel = gdn_scan_fp32_cluster_kernel<T, CS>;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -507,26 +508,34 @@ cudaError_t launch(const GdnArgs &a, cudaStream_t s) {
     return launch_chained(kernel, dim3(a.H_v, a.n_seq, a.d_v / VC), 256, smem, s, a);
 }
 
-// Does a call go to the clusters?  Yes where each of their CTAs finds an SM.  The SMs of a cluster belong to one GPC, which leaves some
-// without: 15, 33 and 74 clusters of 8, 4 and 2 are resident at a time with one CTA an SM, 120, 132 and 148 of the 148 SMs (as numbers
-// and not as a query, so that equal calls take the same kernel, and give the same bits, whichever SMs a GPU has).  One cluster more and
-// there is a second round: 64 tokens of 15, 16 heads of 176 x 64 16.2, 30.9 us against 24.4 without clusters.  Up to d_k = 160 two CTAs share
-// an SM instead.  A block then takes longer and the start is dearer, which pays in long sequences only: 18 heads of 64 x 64 13.7 us
-// (64 tokens), 23.9 (128), 81 (512) against 13.1, 23.7, 86; of 160 x 64 23.4, 41.4, 144 against 22.5, 41.6, 156.
-bool clusters_pay(const GdnArgs &a) {
+// Shared memory of the CTAs of a call that goes to the clusters, or 0 for one that does not.
+// - Where each CTA finds an SM.  The SMs of a cluster belong to one GPC, which leaves some without: 15, 33 and 74 clusters of 8, 4 and 2 are
+//   resident at a time with one CTA an SM, 120, 132 and 148 of the 148 SMs (as numbers and not as a query, so that equal calls take the
+//   same kernel, and give the same bits, whichever SMs a GPU has).  One cluster more and there is a second round: 64 tokens of 15,
+//   16 heads of 176 x 64 15.9, 30.9 us against 24.4 without clusters.  CTAs that take less than half of an SM are packed two to an SM
+//   although others are idle, so they ask for more: 64, 512 tokens of 15 heads of 64 x 64 12.6, 74 -> 9.9, 55 us (13.1, 87
+//   without clusters).
+// - Two to an SM a block takes longer, which only pays in long sequences and larger heads: 18 heads of 64 x 64 13.7 us (64 tokens), 23.9
+//   (128), 43.0 (256), 95 (600) against 13.1, 23.6, 44.5, 102; 18 of 128 x 64 58, 130 (256, 600) against 67, 155; 16 of 32 x 64 38
+//   (256) against 34.
+// - Small heads have little to share: one head of 4 x 64 9.9 us (64 tokens) against 8.0; of 16 x 64 9.0, 25.4 (64, 256) against 9.0, 29.5.
+constexpr size_t kOwnSmBytes = 116 * 1024;   // more than half of the 228 KB of an SM
+size_t cluster_smem(const GdnArgs &a) {
     const long long ctas = static_cast<long long>(a.H_v) * a.n_seq * (a.d_v / 8);
     const size_t smem = cluster_smem_bytes(a.d_k);
-    if (ctas > sm_count() || smem > 227 * 1024) return false;
+    if (ctas > sm_count() || smem > 227 * 1024 || a.d_k < 16) return 0;
     const int without = a.d_v == 16 ? 0 : a.d_v == 32 ? 16 : 28;   // SMs
-    return ctas <= sm_count() - without || (2 * (smem + 1024) <= 228 * 1024 && a.T_total >= 256LL * a.n_ranges);
+    const bool own = ctas <= sm_count() - without, longs = a.T_total >= 256LL * a.n_ranges;
+    if (own && (a.d_k > 16 || longs)) return std::max(smem, kOwnSmBytes);
+    return longs && a.d_k >= 64 && a.d_k % 16 == 0 && 2 * (smem + 1024) <= 228 * 1024 ? smem : 0;
 }
 
 // Columns per CTA: all of them when heads and sequences fill the GPU; otherwise halved as long as that still finds idle SMs.
 // The coupling matrices are then computed once per part, side by side.
 template <typename T>
 cudaError_t dispatch(const GdnArgs &a, cudaStream_t s) {
-    if (clusters_pay(a))
-        return a.d_v == 16 ? launch_cluster<T, 2>(a, s) : a.d_v == 32 ? launch_cluster<T, 4>(a, s) : launch_cluster<T, 8>(a, s);
+    if (const size_t smem = cluster_smem(a))
+        return a.d_v == 16 ? launch_cluster<T, 2>(a, smem, s) : a.d_v == 32 ? launch_cluster<T, 4>(a, smem, s) : launch_cluster<T, 8>(a, smem, s);
     int vc = a.d_v;
     const long long units = static_cast<long long>(a.H_v) * a.n_seq;
     while (vc > 16 && units * (a.d_v / vc) * 2 <= sm_count()) vc /= 2;

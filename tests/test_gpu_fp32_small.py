@@ -61,13 +61,17 @@ def test_small_scan(H_k, H_v, d_k, d_v, lens, io, init):
         assert np.abs(host(ST)[s] - ST_ref).max() <= 1e-5 * max(1.0, np.abs(ST_ref).max())
 
 
-@pytest.mark.parametrize("H, d_k, d_v", [(15, 176, 64), (16, 176, 64), (33, 168, 32), (34, 168, 32), (18, 64, 64), (74, 16, 16), (18, 160, 64)])
-@pytest.mark.parametrize("T", [40, 256])   # clusters that share SMs are taken from 256 tokens up
-def test_scan_around_the_calls_that_go_to_clusters(H, d_k, d_v, T):
+@pytest.mark.parametrize("H, d_k, d_v", [(15, 176, 64), (16, 176, 64), (33, 168, 32), (34, 168, 32), (18, 64, 64), (74, 16, 16), (18, 160, 64),
+                                         (15, 20, 64), (60, 130, 16), (17, 130, 64)])
+@pytest.mark.parametrize("T, io", [(40, "f32"), (256, "f32"), (70, "bf16")])   # clusters that share SMs are taken from 256 tokens up
+def test_scan_around_the_calls_that_go_to_clusters(H, d_k, d_v, T, io):
+    import torch
     rng = np.random.default_rng(H + T)
-    tok = wl.gdn_tokens(rng, T, H, H, d_k, d_v, io="f32")
+    tok = wl.gdn_tokens(rng, T, H, H, d_k, d_v, io=io)
     S0 = rng.standard_normal((1, H, d_k, d_v)).astype(np.float32)
-    o, ST = b.lkv_gdn_fwd(*(dev(tok[n]) for n in ("q", "k", "v", "g", "beta")), dev(S0), compute=b.LKV_COMPUTE_FP32)
+    t = torch.bfloat16 if io == "bf16" else None
+    o, ST = b.lkv_gdn_fwd(*(dev(tok[n], t) for n in ("q", "k", "v")), dev(tok["g"]), dev(tok["beta"]), dev(S0), compute=b.LKV_COMPUTE_FP32)
     o_ref, ST_ref = oracle.gdn_seq(tok["q"], tok["k"], tok["v"], tok["g"], tok["beta"], S0[0])
-    assert np.abs(host(o) - o_ref).max() <= 1e-5 * max(1.0, np.abs(o_ref).max())
+    # outputs in bf16 round by 2^-9 of themselves
+    assert np.abs(host(o.float()) - o_ref).max() <= (4e-3 if t else 1e-5) * max(1.0, np.abs(o_ref).max())
     assert np.abs(host(ST)[0] - ST_ref).max() <= 1e-5 * max(1.0, np.abs(ST_ref).max())
