@@ -40,10 +40,13 @@ constexpr int kEpiThreads = 256;             // two epilogue warpgroups
 constexpr int kRoundThreads = 128;           // warps that round the transitions
 constexpr int kThreads = kEpiThreads + kRoundThreads + 64;   // + MMA warp + TMA warp
 constexpr int kSmemBytes = kStages * kTStageBytes + 1024;
-// Where the requests share chunks and more than L2 holds at once, CTAs are launched in groups of up to eight requests, those of a group next
-// to each other for one head: the chunks of some 18 heads, not of all, are then in use at a time, and each is read from DRAM once.  Eight
-// requests over one pool of 32 chunks (134 MB), each in its own order, composition and scan: 305 -> 285 us (where nothing is
-// shared the order by heads is level to 1 % better).
+// Where the requests share chunks, CTAs are launched in groups of up to eight requests, those of a group next to each other for one head:
+// the chunks of some 18 heads, not of all, are then in use at a time, and each is read from DRAM once.  That gains most where the pool
+// does not fit L2, and something where it does (its 126 MB are two halves, and a chunk that is read on both sides is in both).
+// 32 heads, every request over the whole pool in an order of its own, composition alone, by heads -> in groups: 8 requests over 4, 20,
+// 28, 32, 40 chunks (17, 84, 117, 134, 168 MB) 27.9 -> 26.0, 89 -> 87, 127 -> 115, 140 -> 130, 177 -> 159 us; 16 requests over 20, 28, 40
+// 165 -> 159, 228 -> 214, 337 -> 302; bf16 states, 8 over 4, 28, 40 27.6 -> 25.6, 119 -> 115, 162 -> 156.  Where nothing is shared
+// the order by heads is level to 1 % better.
 constexpr int kMaxGroupLog2 = 3;
 constexpr uint32_t kTmemCols = 512;          // D buffers: 0..127 and 128..255, A buffers: 256..383 and 384..511
 

@@ -80,8 +80,9 @@ int check_init_desc(const lkv_init_desc *d) {
     return LKV_OK;
 }
 
-// Do the requests name the chunks 1.5 times on average or more, and more of them than L2 holds at once?  Then the order of the
-// composition's CTAs matters (kMaxGroupLog2 in init_gdn_tensor.cu).
+// Do the requests name the chunks 1.5 times on average or more, and is all that they name, repeats included and every state counted as
+// fp32, more than L2 holds?  Then the order of the composition's CTAs matters (kMaxGroupLog2 in init_gdn_tensor.cu).  Below that
+// many bytes it does not: 4 requests over 4 chunks (67 MB) 17.4 us in either order.
 bool shares_chunks(const int32_t *ids, int total, const lkv_init_desc *d) {
     constexpr double kL2Bytes = 126e6;
     if (2.0 * sizeof(float) * total * d->H * d->d_k * d->d_v <= kL2Bytes) return false;
