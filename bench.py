@@ -926,6 +926,15 @@ def run_profile_case(args):
         cu = (np.arange(n_seq + 1) * L).astype(np.int32)
         fn = lambda: b.lkv_ssd_fwd(x, dt, A, Bm, Cm, S0, y, ST, cu_seqlens=cu, workspace_t=ws)
         work = dict(tokens=T, flops=ssd_scan_flops(T))
+    elif name == "gdn_build":
+        s, n_seq, L = GDN_SHAPE, 16, 1024
+        T = n_seq * L
+        k = torch.nn.functional.normalize(rn(T, s["H_k"], s["d_k"]), dim=-1).to(bf)
+        v, g, beta = rn(T, s["H_v"], s["d_v"]).to(bf), -0.012 * torch.nn.functional.softplus(rn(T, s["H_v"])), torch.sigmoid(rn(T, s["H_v"])) / 8
+        ST, P = rn(n_seq, s["H_v"], s["d_k"], s["d_v"]), rn(n_seq, s["H_v"], s["d_k"], s["d_k"])
+        cu = (np.arange(n_seq + 1) * L).astype(np.int32)
+        fn = lambda: b.lkv_gdn_chunk_artifacts(k, v, g, beta, ST, P, cu_seqlens=cu, workspace_t=ws)
+        work = dict(tokens=T, chunks=n_seq)
     elif name in ("gdn_compose", "mamba_compose"):
         n_req, K = (32, 8) if name == "gdn_compose" else (32, 16)
         if name == "gdn_compose":
@@ -963,7 +972,7 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--sweep", action="store_true", help="composition time against K instead of the step benchmark")
     ap.add_argument("--artifacts", action="store_true", help="time of building chunk states and transitions")
-    ap.add_argument("--profile-case", default=None, choices=["gdn_scan", "ssd_scan", "gdn_compose", "mamba_compose"],
+    ap.add_argument("--profile-case", default=None, choices=["gdn_scan", "ssd_scan", "gdn_build", "gdn_compose", "mamba_compose"],
                     help="three launches of one kernel on a small fixed case, for an ncu capture")
     ap.add_argument("--no-configs", action="store_true", help="leave the cfg1-cfg3 object out of the default line")
     ap.add_argument("--dry-run", action="store_true",
