@@ -227,7 +227,8 @@ int lkv_init_state(const void *states, const void *transitions, int K, int mode,
  *   sel_index  HOST int32[n_req]        mode INDEX: position within each request; ignored otherwise (may be NULL)
  *   S0         out, float [n_req, H, d_k, d_v]
  * d->chunk_ids and d->sel_index are ignored.  A request's bits depend on its own chunks only: not on the other requests,
- * their number or the size of the workspace.
+ * their number or the size of the workspace.  (GDN in fp32 arithmetic: small calls have a kernel of their own, which adds in
+ * another order; there the number of requests is a part of what the bits depend on.)
  */
 int lkv_init_state_batched(const void *states, const void *transitions, const int32_t *chunk_ids,
                            const int32_t *cu_k, int n_req, int mode, const int32_t *sel_index, void *S0,
@@ -299,7 +300,8 @@ int lkv_device_status_static(void *stream);
  *
  * One long sequence in a call of its own may be scanned in segments whose initial states are composed (Eq. 6; the workspace
  * size of lkv_workspace_bytes allows for that, with less the plain scan runs): its results then differ in rounding from
- * those of the same sequence in a batch.  Equal calls with equal workspace sizes give equal bits.
+ * those of the same sequence in a batch.  In fp32 arithmetic small calls have kernels of their own: heads, sequences and
+ * lengths of the call decide which, and the rounding differs.  Equal calls with equal workspace sizes give equal bits.
  */
 int lkv_gdn_fwd(const void *q, const void *k, const void *v, const float *g, const float *beta,
                 const float *S0, void *o, void *S_T, const lkv_gdn_desc *d, void *stream);
@@ -369,7 +371,7 @@ int lkv_ssd_fwd(const void *x, const float *dt, const float *A, const void *B, c
  *
  * lkv_mamba_chunk_logdecay: for every sequence c and head h, lambda[c][h] = A_h * sum_t dt_t (fp32, device,
  * n_seq x H): exp(lambda) is the scalar T_c of Eq. 2 / Eq. 5, kept as a logarithm because it underflows
- * fp32 for long chunks.  `d` is the descriptor of lkv_ssd_fwd on the same tokens (P, N, G unused).
+ * fp32 for long chunks.  Its bits depend on the chunk's own tokens only.  `d` is the descriptor of lkv_ssd_fwd on the same tokens (P, N, G unused).
  *
  * Errors as for the scans (LKV_ERR_DIM if d_v != d_k).  Both need the scan workspace.
  */
