@@ -468,7 +468,7 @@ __device__ __forceinline__ void logdecay(const SsdArgs &a, float *__restrict__ o
         if (warp == 0 && in) out[static_cast<size_t>(seq) * a.H + h] = a.A[h] * decay_column(sum, lane);
         return;
     }
-    const long long per = (n + kDecayParts - 1) / kDecayParts;
+    const long long per = (static_cast<long long>(n) + kDecayParts - 1) / kDecayParts;
     auto partial = [&](int p) { return in ? decay_part(dt, a.H, per * p + warp, min(per * (p + 1), static_cast<long long>(n))) : 0.f; };
     if (kCluster) {
         const cg::cluster_group cluster = cg::this_cluster();
