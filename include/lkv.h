@@ -427,7 +427,8 @@ size_t lkv_state_rel_error_workspace_bytes(int n_states, size_t state_elems);
  * GDN chain makes it three states larger than LKV_WS_INIT_LIST, which lkv_init_state uses in mode
  * EXACT only.  n_units is the number of requests (init) or
  * sequences (scans) and n_index the total number of chunk ids over all requests
- * (init; 0 for the scans).  Returns 0 for a NULL or invalid descriptor.
+ * (init; 0 for the scans).  Returns 0 for a NULL descriptor, an unknown `which` or an invalid
+ * lkv_init_desc; of a scan descriptor only what the size depends on is looked at.
  */
 size_t lkv_workspace_bytes(int which, const void *desc, int n_units, int n_index);
 

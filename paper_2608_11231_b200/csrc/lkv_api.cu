@@ -780,9 +780,12 @@ size_t lkv_workspace_bytes(int which, const void *desc, int n_units, int n_index
     if (!desc || n_units < 0 || n_index < 0) return 0;
     switch (which) {
         case LKV_WS_INIT_LIST:
-            return ws_bytes_for(2 * n_units + 1 + n_index, kInitIdxCap);
-        case LKV_WS_INIT:
-            return ws_bytes_for(2 * n_units + 1 + n_index, kInitIdxCap) + gdn_split_scratch(static_cast<const lkv_init_desc *>(desc), n_units, n_index);
+        case LKV_WS_INIT: {
+            const lkv_init_desc *d = static_cast<const lkv_init_desc *>(desc);
+            const long long ints = 2LL * n_units + 1 + n_index;
+            if (check_init_desc(d) != LKV_OK || ints > INT32_MAX) return 0;
+            return ws_bytes_for(static_cast<int>(ints), kInitIdxCap) + (which == LKV_WS_INIT ? gdn_split_scratch(d, n_units, n_index) : 0);
+        }
         case LKV_WS_GDN: {
             const lkv_gdn_desc *d = static_cast<const lkv_gdn_desc *>(desc);
             return ws_bytes_for(2 * n_units + 1, kScanIdxCap) + gdn_segment_scratch(d, gdn_cut(d, n_units).n);

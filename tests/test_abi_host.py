@@ -220,6 +220,12 @@ def test_workspace_of_calls_that_compose_nothing_in_halves(lib, K):
     assert b.lkv_workspace_bytes(b.LKV_WS_INIT, d, 2, K) == b.lkv_workspace_bytes(b.LKV_WS_INIT_LIST, d, 2, K)
 
 
+@pytest.mark.parametrize("bad", [dict(H=-1), dict(H=0), dict(d_k=0), dict(n_chunks=-1), dict(family=2), dict(state_dtype=5), dict(compute=9)])
+def test_workspace_of_an_invalid_initialiser_descriptor(lib, bad):
+    d = _desc(**{**dict(H=32, d_k=128, d_v=128, n_chunks=16), **bad})
+    assert b.lkv_workspace_bytes(b.LKV_WS_INIT, d, 1, 16) == 0 and b.lkv_workspace_bytes(b.LKV_WS_INIT_LIST, d, 1, 16) == 0
+
+
 def test_missing_library_fails_loudly(tmp_path, monkeypatch):
     monkeypatch.setattr(b, "_lib", None)
     monkeypatch.setattr(b, "LIB_PATH", str(tmp_path / "liblkv.so"))
