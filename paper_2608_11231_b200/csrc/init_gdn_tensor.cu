@@ -52,9 +52,17 @@ constexpr uint32_t kTmemCols = 512;          // D buffers: 0..127 and 128..255, 
 
 // fp32 -> nearest tf32 (ties away from zero, as cvt.rna.tf32.f32 rounds), in integer arithmetic: the conversion
 // instruction runs at a fraction of the integer rate, and one step rounds 32 K values per CTA.  Adding half a tf32 ulp
-// to the magnitude and dropping the 13 low bits is that rounding (a carry out of the mantissa bumps the exponent, which
-// is the right result; infinities and NaNs keep their class).
-__device__ __forceinline__ uint32_t rn_tf32_bits(float x) { return (__float_as_uint(x) + 0x1000u) & 0xFFFFE000u; }
+// to the magnitude is that rounding (a carry out of the mantissa bumps the exponent, which is the right result): the tensor
+// cores drop the 13 low bits, of infinities too.  A NaN whose payload begins with ten ones must not carry into the sign and
+// become a number.  The NaN that arithmetic makes, 0x7fffffff, is one: as signed integers the larger of sum and value is
+// it, in one instruction.  What is read from memory may have the sign set as well (buffers filled with 0xff): it is lowered first, which
+// leaves it a NaN.  K = 16, one chain, 32 heads: 30.7 us with an addition and a mask, which lost such NaNs, 29.8 so; 8 x 32
+// chunks 127.4, 128.8; 16 x 16 170.2, 169.8.
+__device__ __forceinline__ uint32_t rn_tf32_bits(float x) {
+    const int b = __float_as_int(x);
+    return static_cast<uint32_t>(__viaddmax_s32(b, 0x1000, b));
+}
+__device__ __forceinline__ uint32_t rn_tf32_any(uint32_t x) { return rn_tf32_bits(__uint_as_float(umin(x, 0xFFFFEFFFu))); }
 
 __device__ __forceinline__ void umma_tf32_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, bool accumulate) {
     asm volatile(
@@ -170,8 +178,8 @@ init_gdn_exact_tensor_kernel(const __grid_constant__ InitArgs a, const __grid_co
 #pragma unroll 8
             for (int q = 0; q < kTStageBytes / 16 / kRoundThreads; ++q) {
                 uint4 v = t4[q * kRoundThreads + x];
-                v.x = rn_tf32_bits(__uint_as_float(v.x)); v.y = rn_tf32_bits(__uint_as_float(v.y));
-                v.z = rn_tf32_bits(__uint_as_float(v.z)); v.w = rn_tf32_bits(__uint_as_float(v.w));
+                v.x = rn_tf32_any(v.x); v.y = rn_tf32_any(v.y);
+                v.z = rn_tf32_any(v.z); v.w = rn_tf32_any(v.w);
                 t4[q * kRoundThreads + x] = v;
             }
             fence_async_smem();
@@ -214,6 +222,9 @@ init_gdn_exact_tensor_kernel(const __grid_constant__ InitArgs a, const __grid_co
             if (j > 0) {
                 mbar_wait(&bar_mma[half], (j - 1) & 1, &dead, a.status);
                 tc_fence_after_sync();
+            } else if (K > 1) {   // an operand only: as it is in memory (later values come from an addition)
+#pragma unroll
+                for (int i = 0; i < 64; ++i) sv[i] = __uint_as_float(umin(__float_as_uint(sv[i]), 0xFFFFEFFFu));
             }
             const uint32_t dbuf = lane_base + 128 * (j & 1) + i0;
             const uint32_t abuf = lane_base + 256 + 128 * (j & 1) + i0;

@@ -109,3 +109,22 @@ def test_composition_in_halves_on_several_streams():
             f(i, outs[i, n], streams[i])
     torch.cuda.synchronize()
     assert all(torch.equal(outs[i, n], want[i]) for i in range(2) for n in range(20))
+
+
+@pytest.mark.parametrize("bits", [0x7f800000, 0x7fc00000, 0x7fffffff, 0xffffffff])   # infinity, NaNs: torch's, the one arithmetic makes, memory filled with 0xff
+@pytest.mark.parametrize("K", [3, 12])
+@pytest.mark.parametrize("where", ["states", "transitions"])
+def test_infinities_and_nans_stay(where, K, bits):
+    """They are in the result where 64-bit arithmetic has them, whichever chunk holds them, in one chain and in halves."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    clean = [torch.randn((K, 1, 128, 128), generator=gen, device="cuda") * s for s in (1.0, 0.05)]
+    for j in range(1 if where == "transitions" else 0, K):   # (the first chunk's transition is not read)
+        pools = dict(zip(("states", "transitions"), (x.clone() for x in clean)))
+        pools[where].view(torch.int32)[j, 0, 5, 77] = bits - (1 << 32) if bits >> 31 else bits
+        ref = pools["states"][0].double()
+        for i in range(1, K):
+            ref = pools["transitions"][i].double() @ ref + pools["states"][i].double()
+        for ws in (None, torch.zeros(256, dtype=torch.uint8, device="cuda")):
+            got = b.lkv_init_state(pools["states"], pools["transitions"], K, b.LKV_INIT_EXACT, family=b.LKV_FAMILY_GDN, workspace_t=ws)
+            assert torch.equal(got.isfinite(), ref.isfinite()), (j, ws is None)
