@@ -4,7 +4,8 @@
 // one call in Python (about sixty interpreted operations: ctypes structures and pointers, per-tensor checks, stream and
 // workspace look-up) took 25 us, so the GPU waited for the host.  Here the same work reads the tensors' C++ objects.
 // One request with a 37-token suffix (state copy + Mamba-2 scan): 53.3 -> 16.4 us per pass; one 8K Mamba-2 request
-// (composition of 8 chunks + 1024-token scan): 55.2 -> 35.6 us, both now paced by the GPU.
+// (composition of 8 chunks + 1024-token scan): 55.2 -> 35.6 us.  With today's kernels 11 and 29 us: the second is paced by the GPU, the
+// first by the host again (10.3-11.2 us, 3.6 of them for three new tensors; 8.9 us from a graph).
 //
 // The functions mirror the Python wrappers of binding.py one to one (same arguments, results, checks and exceptions);
 // binding.py keeps the signatures, the constants and everything that is not on the request path.
